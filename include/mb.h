@@ -175,7 +175,8 @@ mb_status mb_measure_fma_rate(mb_context *ctx, mb_precision prec, double *flops_
  * memory makes the copies faster).  Mixing kinds is MB_EINVAL.  With the
  * wall, every z must be > 0 (blobs at z < a are computed as written but the
  * matrix need not be positive definite); this is not checked.  N = 0 is a
- * no-op.
+ * no-op.  u may be f or r.  MB_FP64 and MB_DF64 add partial sums with FP64
+ * atomics, so results may differ between calls in the last FP64 bits.
  */
 mb_status mb_mobility_matvec(mb_context *ctx, const double *r, const double *f, int64_t n,
                              double a, double eta, int wall, mb_precision prec, double *u,

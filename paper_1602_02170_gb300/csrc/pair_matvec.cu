@@ -9,7 +9,9 @@
 // then reads the same source, a shared-memory broadcast) and accumulates the
 // tile in FP32 registers, folding each tile sum into a Kahan-compensated
 // accumulator.  Chunk partials go to an FP64 buffer that a second kernel sums
-// in a fixed order, so results are deterministic.
+// in a fixed order, so results are deterministic.  The symmetric kernels (each
+// unordered pair evaluated once for both blobs) add to u with FP64 atomics
+// instead: their results agree to FP64 rounding from call to call.
 //
 // FP32 positions carry a hi/lo split: d = (hi_i - hi_j) + (lo_i - lo_j); the
 // hi difference is exact for nearby blobs (Sterbenz), so near pairs keep full
@@ -251,45 +253,36 @@ __global__ void __launch_bounds__(kNT, 2) pair_sym_kernel(
     }
 }
 
-template <bool WALL, int NT = kNT>
-__global__ void __launch_bounds__(NT) pair_f64_kernel(
-    const double *__restrict__ r, const double *__restrict__ f, int64_t n, int64_t chunk,
-    int n_tblocks, int64_t n_items, PairConsts<double> k, double *__restrict__ out, double scale,
-    int direct)
+// FP64 kernel: one warp per CTA and item, an item being a block of 32
+// targets against C sources of a block at or after it (f64sym_item).  The
+// FP64 pipe (one instruction per ~19 cycles and SM) is the only resource in
+// use, so a warp or two per scheduler keep it busy and what matters is that
+// every scheduler gets the same number of pair steps: the items are far more
+// than the warps in flight and the hardware deals them out as CTAs end.
+// launch_f64sym picks C.  2,730 blobs: 1,276 -> 632 us against every ordered
+// pair once in one-warp CTAs; 16,384 blobs: 28.3 -> 21.3 ms against 256-thread
+// symmetric items of the ungrouped formula (1.36 TFLOP/s in the method's 108
+// flop per ordered pair, of 1.06 measured: each pair is evaluated once).
+template <bool WALL, int C>
+__global__ void __launch_bounds__(32) pair_f64sym_kernel(
+    const double *__restrict__ r, const double *__restrict__ f, int64_t n, int64_t n_items,
+    MobConsts<double> k, double *__restrict__ u, double scale)
 {
-    __shared__ double sm[6 * NT];
+    __shared__ double sm[6 * C];
+    constexpr int kParts = 32 / C;
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const int tb = (int)(item % n_tblocks);
-        const int64_t sc = item / n_tblocks;
-        const int64_t j_begin = sc * chunk;
-        const int64_t j_end = j_begin + chunk < n ? j_begin + chunk : n;
-        f64_item<WALL, NT>(sm, r, n, r, f, tb, j_begin, j_end, k, direct ? out : out + 3 * sc * n,
-                           direct ? scale : 1.0);
+        // pair t = J (J + 1) / 2 + I of the triangle I <= J
+        const int64_t t = item / kParts;
+        int64_t J = (int64_t)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+        while (J * (J + 1) / 2 > t) --J;
+        while ((J + 1) * (J + 2) / 2 <= t) ++J;
+        const int64_t I = t - J * (J + 1) / 2;
+        const int64_t j0 = J * 32 + (item - t * kParts) * C;
+        if (j0 < n) f64sym_item<WALL, C>(sm, r, f, n, I, j0, I == J, k, u, scale);
+        __syncwarp();  // the item is done with sm
     }
 }
 
-// FP64 kernel for larger problems: symmetric over the upper-triangular
-// pairs of blocks of kNT blobs (one target per thread); see f64sym_item.
-template <bool WALL>
-__global__ void __launch_bounds__(kNT) pair_f64sym_kernel(
-    const double *__restrict__ r, const double *__restrict__ f, int64_t n, int64_t nb,
-    int64_t n_items, PairConsts<double> k, double *__restrict__ u, double scale)
-{
-    __shared__ double sm[9 * kNT];
-    for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-        int64_t lo_r = 0, hi_r = nb;
-        while (hi_r - lo_r > 1) {
-            const int64_t mid = (lo_r + hi_r) >> 1;
-            if (mid * nb - mid * (mid - 1) / 2 <= item) lo_r = mid;
-            else hi_r = mid;
-        }
-        const int64_t I = lo_r, J = I + (item - (I * nb - I * (I - 1) / 2));
-        f64sym_item<WALL, kNT>(sm, r, f, n, I, J, k, u, scale);
-    }
-}
-
-// Double-float kernel: symmetric over the upper-triangular pairs of blocks
-// of kNT blobs (one target per thread); see dfsym_item.
 // Flow evaluation at points other than the blobs (targets != sources):
 // packed FP32 and FP64 items over (target block, source chunk), partials
 // reduced like the matvec's.  The targets are tracers of the blob radius a
@@ -316,7 +309,7 @@ template <bool WALL>
 __global__ void __launch_bounds__(kNT) eval_f64_kernel(
     const double *__restrict__ x, int64_t nt, const double *__restrict__ r,
     const double *__restrict__ f, int64_t ns, int64_t chunk, int n_tblocks, int64_t n_items,
-    PairConsts<double> k, double *__restrict__ out, double scale, int direct)
+    MobConsts<double> k, double *__restrict__ out, double scale, int direct)
 {
     __shared__ double sm[6 * kNT];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
@@ -397,6 +390,8 @@ __global__ void __launch_bounds__(NT) pair_dfx_kernel(
     }
 }
 
+// Double-float kernel: symmetric over the upper-triangular pairs of blocks of
+// NT blobs (one target per thread); see dfsym_item.
 // box (optional, spatial order): the bounding boxes of the sort's blocks of
 // 2 kNT blobs (two blocks of this kernel each); block pairs whose boxes are
 // 64 a or more apart take the FAR instance of the item.
@@ -506,9 +501,8 @@ constexpr int kTPT = MB_PAIR_TPT;  // targets per thread
 //   2: packed f32x2 kernel, 4 targets per thread
 constexpr int kF32Variants = 5;
 constexpr int kSmallNT = 32;        // CTA size of the small-problem kernels
-constexpr int64_t kSmallN = 8192;   // below this the FP64 and double-float paths use them
+constexpr int64_t kSmallN = 8192;   // below this the double-float path uses them
 constexpr int64_t kDfxMaxN = 1024;  // up to this the double-float product is forward only
-constexpr int kSmallF64Chunk = 8;   // smallest source chunk of the small FP64 kernel
 
 int f32_targets_per_cta(int v)
 {
@@ -1070,6 +1064,34 @@ mb_status matvec_pack_positions(mb_context *ctx, const double *r, int64_t n, cud
     return MB_OK;
 }
 
+// Sources per item of the FP64 kernel: 32 unless that leaves fewer than
+// kF64ItemsPerWarp items for each of an SM's four schedulers, then 16, 8 or 4.
+// Every scheduler takes a whole number of items, so with m items each about
+// 1/(2 m) of the time is lost to the last one; smaller items cost more
+// reductions and atomics (C = 4: 12% of the FP64 instructions).
+constexpr int kF64ItemsPerWarp = 16;
+
+template <bool WALL, int C>
+void launch_f64sym_c(const double *r, const double *f, int64_t n, int64_t pairs, double a,
+                     double *u, double scale, cudaStream_t s)
+{
+    const int64_t items = pairs * (32 / C);
+    pair_f64sym_kernel<WALL, C><<<(unsigned)std::min<int64_t>(items, 1 << 30), 32, 0, s>>>(
+        r, f, n, items, MobConsts<double>::make(a), u, scale);
+}
+
+template <bool WALL>
+void launch_f64sym(mb_context *ctx, const double *r, const double *f, int64_t n, double a,
+                   double *u, double scale, cudaStream_t s)
+{
+    const int64_t nb = ceil_div(n, 32), pairs = nb * (nb + 1) / 2;
+    const int64_t want = (int64_t)kF64ItemsPerWarp * 4 * ctx->sm_count;
+    if (pairs >= want) launch_f64sym_c<WALL, 32>(r, f, n, pairs, a, u, scale, s);
+    else if (2 * pairs >= want) launch_f64sym_c<WALL, 16>(r, f, n, pairs, a, u, scale, s);
+    else if (4 * pairs >= want) launch_f64sym_c<WALL, 8>(r, f, n, pairs, a, u, scale, s);
+    else launch_f64sym_c<WALL, 4>(r, f, n, pairs, a, u, scale, s);
+}
+
 mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64_t n, double a,
                         double eta, int wall, mb_precision prec, double *u, cudaStream_t s,
                         MatvecPartials *defer)
@@ -1147,77 +1169,47 @@ mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64
         MB_CUDA_TRY(ctx, cudaGetLastError());
         return MB_OK;
     }
-    const bool small = n < kSmallN;
-    if (!small) {
-        // symmetric FP64 kernel: zero u, one launch over the block-pair triangle
-        const int res = wall ? resident_ctas(ctx, pair_f64sym_kernel<true>)
-                             : resident_ctas(ctx, pair_f64sym_kernel<false>);
-        const int64_t nb = ceil_div(n, kNT);
-        const int64_t items = nb * (nb + 1) / 2;
-        const int grid = (int)std::min<int64_t>(items, res);
-        MB_CUDA_TRY(ctx, cudaMemsetAsync(u, 0, sizeof(double) * 3 * (size_t)n, s));
-        auto *ev = profile_begin(ctx, s);
-        const PairConsts<double> k = PairConsts<double>::make(a);
-        if (wall)
-            pair_f64sym_kernel<true><<<grid, kNT, 0, s>>>(r, f, n, nb, items, k, u, scale);
-        else
-            pair_f64sym_kernel<false><<<grid, kNT, 0, s>>>(r, f, n, nb, items, k, u, scale);
-        profile_end(ev, s);
-        count_launch();
-        MB_CUDA_TRY(ctx, cudaGetLastError());
-        return MB_OK;
+    // FP64: u (or, deferred, the one partial sum the caller scales) zeroed,
+    // then one launch over the block-pair triangle
+    double *uk = u, sk = mob_scale(eta);
+    if (defer) {
+        MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)n, "matvec partials"));
+        uk = (double *)ctx->partial.ptr;
+        *defer = MatvecPartials{uk, 1, sk};
+        sk = 1.0;
     }
-    Plan p;
-    if (small) {
-        const int res = wall ? resident_ctas(ctx, pair_f64_kernel<true, kSmallNT>, kSmallNT)
-                             : resident_ctas(ctx, pair_f64_kernel<false, kSmallNT>, kSmallNT);
-        // source chunks down to 8 blobs: several one-warp CTAs per SM, since
-        // a single warp leaves the FP64 pipe mostly idle
-        p = make_plan(n, kSmallNT, res, 1024, kSmallF64Chunk, kSmallF64Chunk);
-    } else {
-        const int res = wall ? resident_ctas(ctx, pair_f64_kernel<true>)
-                             : resident_ctas(ctx, pair_f64_kernel<false>);
-        p = make_plan(n, kNT, res);
-    }
-    double *out = u;
-    const int direct = p.S == 1;
-    if (!direct) {
-        MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)n * p.S, "matvec partials"));
-        out = (double *)ctx->partial.ptr;
-    }
+    MB_CUDA_TRY(ctx, cudaMemsetAsync(uk, 0, sizeof(double) * 3 * (size_t)n, s));
     auto *ev = profile_begin(ctx, s);
-    const PairConsts<double> k = PairConsts<double>::make(a);
-    if (small && wall)
-        pair_f64_kernel<true, kSmallNT><<<p.grid, kSmallNT, 0, s>>>(r, f, n, p.chunk, p.n_tblocks,
-                                                                   p.items, k, out, scale, direct);
-    else if (small)
-        pair_f64_kernel<false, kSmallNT><<<p.grid, kSmallNT, 0, s>>>(r, f, n, p.chunk, p.n_tblocks,
-                                                                    p.items, k, out, scale, direct);
-    else if (wall)
-        pair_f64_kernel<true><<<p.grid, kNT, 0, s>>>(r, f, n, p.chunk, p.n_tblocks, p.items, k, out,
-                                                     scale, direct);
-    else
-        pair_f64_kernel<false><<<p.grid, kNT, 0, s>>>(r, f, n, p.chunk, p.n_tblocks, p.items, k,
-                                                      out, scale, direct);
+    if (wall) launch_f64sym<true>(ctx, r, f, n, a, uk, sk, s);
+    else launch_f64sym<false>(ctx, r, f, n, a, uk, sk, s);
     profile_end(ev, s);
     count_launch();
     MB_CUDA_TRY(ctx, cudaGetLastError());
-    if (!direct && defer) {
-        *defer = MatvecPartials{out, p.S, scale};
-        return MB_OK;
-    }
-    if (!direct) {
-        const int grid = (int)std::min<int64_t>(ceil_div(3 * n, 256), 8 * (int64_t)ctx->sm_count);
-        reduce_partials_kernel<<<grid, 256, 0, s>>>(out, n, p.S, scale, u);
-        count_launch();
-        MB_CUDA_TRY(ctx, cudaGetLastError());
-    }
     return MB_OK;
+}
+
+// Whether two arrays of n blob vectors share memory.
+bool overlap(const double *x, const double *y, int64_t n)
+{
+    return x < y + 3 * n && y < x + 3 * n;
 }
 
 mb_status matvec_device(mb_context *ctx, const double *r, const double *f, int64_t n, double a,
                         double eta, int wall, mb_precision prec, double *u, cudaStream_t s)
 {
+    // The symmetric kernels zero u and add to it while they read f (FP64: and
+    // r), so a product in place works on copies.
+    const size_t bytes = sizeof(double) * 3 * (size_t)n;
+    if (overlap(u, f, n)) {
+        MB_TRY(ensure(ctx, ctx->stage_f, bytes, "in-place product"));
+        MB_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->stage_f.ptr, f, bytes, cudaMemcpyDeviceToDevice, s));
+        f = (const double *)ctx->stage_f.ptr;
+    }
+    if (prec == MB_FP64 && overlap(u, r, n)) {
+        MB_TRY(ensure(ctx, ctx->stage_r, bytes, "in-place product"));
+        MB_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->stage_r.ptr, r, bytes, cudaMemcpyDeviceToDevice, s));
+        r = (const double *)ctx->stage_r.ptr;
+    }
     if (prec != MB_FP64) MB_TRY(matvec_pack_positions(ctx, r, n, s));
     return matvec_packed(ctx, r, f, n, a, eta, wall, prec, u, s);
 }
@@ -1226,7 +1218,7 @@ mb_status matvec_eval(mb_context *ctx, const double *x, int64_t nt, const double
                       const double *f, int64_t ns, double a, double eta, int wall,
                       mb_precision prec, double *u, cudaStream_t s)
 {
-    const double scale = 1.0 / (6.0 * kPi * eta * a);
+    const double scale = prec == MB_FP64 ? mob_scale(eta) : 1.0 / (6.0 * kPi * eta * a);
     if (prec == MB_FP64) {
         const int res = wall ? resident_ctas(ctx, eval_f64_kernel<true>)
                              : resident_ctas(ctx, eval_f64_kernel<false>);
@@ -1237,7 +1229,7 @@ mb_status matvec_eval(mb_context *ctx, const double *x, int64_t nt, const double
             MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)nt * p.S, "eval partials"));
             out = (double *)ctx->partial.ptr;
         }
-        const PairConsts<double> k = PairConsts<double>::make(a);
+        const MobConsts<double> k = MobConsts<double>::make(a);
         if (wall)
             eval_f64_kernel<true><<<p.grid, kNT, 0, s>>>(x, nt, r, f, ns, p.chunk, p.n_tblocks,
                                                          p.items, k, out, scale, direct);

@@ -133,7 +133,7 @@ __device__ __forceinline__ void f64_item(double *__restrict__ sm, const double *
                                          int64_t n, const double *__restrict__ r,
                                          const double *__restrict__ f, int tb,
                                          int64_t j_begin, int64_t j_end,
-                                         const PairConsts<double> &k, double *__restrict__ out,
+                                         const MobConsts<double> &k, double *__restrict__ out,
                                          double m)
 {
     double *sx = sm, *sy = sm + NT, *sz = sm + 2 * NT, *sfx = sm + 3 * NT, *sfy = sm + 4 * NT,
@@ -159,9 +159,11 @@ __device__ __forceinline__ void f64_item(double *__restrict__ sm, const double *
         // the staged sources of this tile (chunks may be shorter than NT)
         const int cnt = j_end - jt < NT ? (int)(j_end - jt) : NT;
 #pragma unroll 2
-        for (int s = 0; s < cnt; ++s)
-            pair_accumulate<WALL, double>(xi - sx[s], yi - sy[s], zi - sz[s], zi, sz[s], sfx[s],
-                                          sfy[s], sfz[s], k, ux, uy, uz);
+        for (int s = 0; s < cnt; ++s) {
+            const double dx = xi - sx[s], dy = yi - sy[s], dz = zi - sz[s];
+            const Mob<double> m = mob_coefs<WALL>(dx, dy, dz, zi, sz[s], k);
+            mob_apply<WALL>(m, dx, dy, dz, sfx[s], sfy[s], sfz[s], ux, uy, uz);
+        }
     }
     if (i < n) {
         out[3 * i] = m * ux;
@@ -522,72 +524,69 @@ __device__ __forceinline__ void dfsym_item(float4 *__restrict__ sD, double *__re
     }
 }
 
-// FP64 symmetric item over block pair (I, J), I <= J, blocks of NT blobs,
-// one target per thread: the scheme of dfsym_item in FP64.  Sources are
-// staged as six FP64 arrays (lanes read consecutive sources: no bank
-// conflicts); each unordered pair is evaluated once for both blobs, the
-// reverse sums rotate through the warp (lane l holds source l's sum after 32
-// steps) and reach u with FP64 atomics, so u must be zeroed beforehand.
-// Diagonal items run forward only over all ordered pairs.
-template <bool WALL, int NT>
+// FP64 symmetric item of one warp: blob block I (32 targets, one per lane)
+// against C sources (C divides 32) starting at j0, a part of block J >= I.
+// Sources are staged as six FP64 arrays in sm (6 C).  Each unordered pair is
+// evaluated once for both blobs: at step t lane l meets source (l + t) mod C,
+// and the reverse sums move to lane l - 1 within the groups of C lanes after
+// each step, so that after C steps lane l holds source (l mod C)'s sum over
+// its group's targets; the groups are then added.  All sums reach u with FP64
+// atomics, so u must be zeroed beforehand.  A diagonal item (I == J) runs
+// forward only over all ordered pairs.
+template <bool WALL, int C>
 __device__ __forceinline__ void f64sym_item(double *__restrict__ sm, const double *__restrict__ r,
                                             const double *__restrict__ f, int64_t n, int64_t I,
-                                            int64_t J, const PairConsts<double> &k,
+                                            int64_t j0, bool diag, const MobConsts<double> &k,
                                             double *__restrict__ u, double scale)
 {
-    double *sx = sm, *sy = sm + NT, *sz = sm + 2 * NT, *sfx = sm + 3 * NT, *sfy = sm + 4 * NT,
-           *sfz = sm + 5 * NT, *sRev = sm + 6 * NT;
     const int lane = threadIdx.x & 31;
-    const bool diag = I == J;
-    const int64_t i = I * NT + threadIdx.x;
-    const int64_t ic = i < n ? i : n - 1;
+    const int64_t i = I * 32 + lane, ic = i < n ? i : n - 1;
     const double xi = r[3 * ic], yi = r[3 * ic + 1], zi = r[3 * ic + 2];
+    // padding targets and sources carry no force, so they add nothing
     const double gx = i < n ? f[3 * i] : 0.0, gy = i < n ? f[3 * i + 1] : 0.0,
                  gz = i < n ? f[3 * i + 2] : 0.0;
-    double ux = 0.0, uy = 0.0, uz = 0.0;
-    const int64_t j0 = J * NT;
-    __syncthreads();
-    {
-        const int64_t j = j0 + threadIdx.x;
-        const bool valid = j < n;
-        const int64_t jc = valid ? j : j0;
-        sx[threadIdx.x] = r[3 * jc];
-        sy[threadIdx.x] = r[3 * jc + 1];
-        sz[threadIdx.x] = r[3 * jc + 2];
-        sfx[threadIdx.x] = valid ? f[3 * jc] : 0.0;
-        sfy[threadIdx.x] = valid ? f[3 * jc + 1] : 0.0;
-        sfz[threadIdx.x] = valid ? f[3 * jc + 2] : 0.0;
-        sRev[3 * threadIdx.x] = sRev[3 * threadIdx.x + 1] = sRev[3 * threadIdx.x + 2] = 0.0;
+    if (lane < C) {
+        const int64_t j = j0 + lane, jc = j < n ? j : j0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            sm[c * C + lane] = r[3 * jc + c];
+            sm[(3 + c) * C + lane] = j < n ? f[3 * jc + c] : 0.0;
+        }
     }
-    __syncthreads();
+    __syncwarp();
+    double ux = 0.0, uy = 0.0, uz = 0.0;
     if (diag) {
 #pragma unroll 1
-        for (int s = 0; s < NT; ++s)
-            pair_accumulate<WALL, double>(xi - sx[s], yi - sy[s], zi - sz[s], zi, sz[s], sfx[s],
-                                          sfy[s], sfz[s], k, ux, uy, uz);
-    } else {
-        for (int g = 0; g < NT / 32; ++g) {
-            double vx = 0.0, vy = 0.0, vz = 0.0;
-#pragma unroll 1
-            for (int t = 0; t < 32; ++t) {
-                const int s = g * 32 + ((lane + t) & 31);
-                pair_sym_rg<WALL, double>(xi - sx[s], yi - sy[s], zi - sz[s], zi, sz[s], sfx[s],
-                                          sfy[s], sfz[s], gx, gy, gz, k, ux, uy, uz, vx, vy, vz);
-                const int from = (lane + 1) & 31;
-                vx = __shfl_sync(0xffffffffu, vx, from);
-                vy = __shfl_sync(0xffffffffu, vy, from);
-                vz = __shfl_sync(0xffffffffu, vz, from);
-            }
-            double *o3 = sRev + 3 * (g * 32 + lane);
-            atomicAdd(o3, vx);
-            atomicAdd(o3 + 1, vy);
-            atomicAdd(o3 + 2, vz);
+        for (int s = 0; s < C; ++s) {
+            const double dx = xi - sm[s], dy = yi - sm[C + s], zj = sm[2 * C + s], dz = zi - zj;
+            const Mob<double> m = mob_coefs<WALL>(dx, dy, dz, zi, zj, k);
+            mob_apply<WALL>(m, dx, dy, dz, sm[3 * C + s], sm[4 * C + s], sm[5 * C + s], ux, uy, uz);
         }
-        __syncthreads();
-        const int64_t j = j0 + threadIdx.x;
-        if (j < n) {
+    } else {
+        double vx = 0.0, vy = 0.0, vz = 0.0;
+        const int from = (lane & ~(C - 1)) | ((lane + 1) & (C - 1));
+#pragma unroll 1
+        for (int t = 0; t < C; ++t) {
+            const int s = (lane + t) & (C - 1);
+            const double dx = xi - sm[s], dy = yi - sm[C + s], zj = sm[2 * C + s], dz = zi - zj;
+            const Mob<double> m = mob_coefs<WALL>(dx, dy, dz, zi, zj, k);
+            mob_apply<WALL>(m, dx, dy, dz, sm[3 * C + s], sm[4 * C + s], sm[5 * C + s], ux, uy, uz);
+            mob_apply<WALL, true>(m, dx, dy, dz, gx, gy, gz, vx, vy, vz);
+            vx = __shfl_sync(0xffffffffu, vx, from);
+            vy = __shfl_sync(0xffffffffu, vy, from);
+            vz = __shfl_sync(0xffffffffu, vz, from);
+        }
 #pragma unroll
-            for (int c = 0; c < 3; ++c) atomicAdd(u + 3 * j + c, scale * sRev[3 * threadIdx.x + c]);
+        for (int o = C; o < 32; o <<= 1) {
+            vx += __shfl_xor_sync(0xffffffffu, vx, o);
+            vy += __shfl_xor_sync(0xffffffffu, vy, o);
+            vz += __shfl_xor_sync(0xffffffffu, vz, o);
+        }
+        const int64_t j = j0 + lane;
+        if (lane < C && j < n) {
+            atomicAdd(u + 3 * j, scale * vx);
+            atomicAdd(u + 3 * j + 1, scale * vy);
+            atomicAdd(u + 3 * j + 2, scale * vz);
         }
     }
     if (i < n) {
@@ -598,4 +597,3 @@ __device__ __forceinline__ void f64sym_item(double *__restrict__ sm, const doubl
 }
 
 }  // namespace mb
-

@@ -154,7 +154,7 @@ __device__ __forceinline__ void tri_index(int e, int &i, int &j)
 template <bool WALL, bool L_SMEM>
 __global__ void __launch_bounds__(kSetupThreads) precond_setup_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
-    const int64_t *__restrict__ start, const int64_t *__restrict__ poff, PairConsts<double> k,
+    const int64_t *__restrict__ start, const int64_t *__restrict__ poff, MobConsts<double> k,
     double scale, double *__restrict__ P, double *__restrict__ scratch, int64_t scratch_stride,
     int *__restrict__ flag, int flag_slot, int schur, const double *__restrict__ shift)
 {
@@ -458,7 +458,7 @@ int64_t split_stride(int nmax) { return (int64_t)nmax * nmax + 19 * (int64_t)nma
 template <bool WALL>
 __global__ void __launch_bounds__(256) pc_assemble_kernel(
     int64_t nb, const double *__restrict__ r, const int64_t *__restrict__ start,
-    const int64_t *__restrict__ poff, PairConsts<double> k, double scale, double *__restrict__ P,
+    const int64_t *__restrict__ poff, MobConsts<double> k, double scale, double *__restrict__ P,
     const double *__restrict__ shift)
 {
     const int lane = threadIdx.x & 31;
@@ -1689,8 +1689,8 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
     const int64_t group = std::max<int64_t>(1, std::min<int64_t>(nb, cap_bytes / (8 * stride)));
     MB_TRY(ensure(ctx, ctx->sol_dots, sizeof(double) * stride * group, "preconditioner scratch"));
     SplitScratch scr{(double *)ctx->sol_dots.ptr, stride, nmax};
-    const PairConsts<double> k = PairConsts<double>::make(a);
-    const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
+    const MobConsts<double> k = MobConsts<double>::make(a);
+    const double scale = mob_scale(eta);
     const bool lsmem = nmax <= kSmemMaxRows;
     const size_t fsmem =
         sizeof(double) * (lsmem ? (size_t)nmax * nmax + (7 + kPanel) * (size_t)nmax + 72
@@ -1881,8 +1881,8 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
     const bool lsmem = nmax <= kSmemMaxRows;
     const size_t small = sizeof(double) * (13 * (size_t)nmax + 72);
     const size_t smem = small + (lsmem ? sizeof(double) * (size_t)nmax * nmax : 0);
-    const PairConsts<double> k = PairConsts<double>::make(a);
-    const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
+    const MobConsts<double> k = MobConsts<double>::make(a);
+    const double scale = mob_scale(eta);
     int grid = (int)std::min<int64_t>(nb, 4 * (int64_t)ctx->sm_count);
     double *scratch = nullptr;
     int64_t stride = 0;
@@ -1950,8 +1950,8 @@ mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, cons
     const bool lsmem = nmax <= kSmemMaxRows;
     const size_t small = sizeof(double) * (13 * (size_t)nmax + 72);
     const size_t smem = small + (lsmem ? sizeof(double) * (size_t)nmax * nmax : 0);
-    const PairConsts<double> k = PairConsts<double>::make(a);
-    const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
+    const MobConsts<double> k = MobConsts<double>::make(a);
+    const double scale = mob_scale(eta);
     int grid = (int)std::min<int64_t>(nb, 4 * (int64_t)ctx->sm_count);
     double *scratch = nullptr;
     int64_t stride = 0;

@@ -115,88 +115,173 @@ __device__ __forceinline__ void pair_accumulate(T dx, T dy, T dz, T zi, T zj, T 
     uz += Cx * fz + g * dz + s * (gw * R3 + kz);
 }
 
-// Both directions of one unordered pair (scalar types: FP64, double-float):
-// u_i += M_ij f_j and v_j += M_ij^T f_i (f3 and f4 exchange roles in the
-// transpose).
-template <bool WALL, typename T>
-__device__ __forceinline__ void pair_sym(T dx, T dy, T dz, T zi, T zj, T fx, T fy, T fz, T gx,
-                                         T gy, T gz, const PairConsts<T> &k, T &ux, T &uy, T &uz,
-                                         T &vx, T &vy, T &vz)
+// The regrouped form of the same interaction, in units of (4 pi eta)^-1 (1.5 a
+// times the ones above: the wall prefactor (3a/4)/rho becomes 1/(2 rho), so
+// that u = 1/rho itself multiplies the halved polynomials).  With w = u^2,
+// X = a^2 w, Q = X^2 / 3, E = R3^2 w, V = X E, S = V + Q and
+// c = zi zj w + X / 3, the polynomials f1..f5 of the header are
+//   f1 / 2     = -1/2 - c + S - 5 E Q
+//   f2 / 2     = -1/2 + 3 c - 5 S + 35 E Q
+//   f3 rho / 2 = zj - R3 (2 (f2/2) + 1 - 10 Q)
+//   f4 rho / 2 = zj - R3 10 Q
+//   f5 / 2     = -2 zj^2 w - 2 S - 2 Q + 30 E Q
+// Every coefficient but the two thirds is a small integer, exact in any
+// precision, and hs, ht, e3 (three products by 1/rho) are not formed.  The
+// interaction is then
+//   u_i = Cx f + G d (x, y);  Cz f_z + A4 RF + gw R3 + g d_z (z)
+//   g = D (d.f),  RF = d_xy.f_xy + R3 f_z,  gw = A2 RF + A3 f_z,  G = g + gw
+// with Cx = C + u f1/2, Cz = Cx + u f5/2 and A2, A3, A4 = u w times f2/2,
+// f3 rho/2, f4 rho/2; the transpose (M_ji = M_ij^T) exchanges A3 and A4.
+// 78 instructions for both directions of a pair besides the two reciprocal
+// square roots, where the form above takes 103.
+template <typename T>
+struct MobConsts {
+    T a2;       // a^2
+    T a2_3;     // a^2 / 3: far C = inv (1/2 + a^2/3 inv^2)
+    T ma2;      // -a^2:    far D = inv^3 (1/2 - a^2 inv^2)
+    T third;    // 1/3
+    T four_a2;  // 4 a^2: r^2 below this takes the overlap branch
+    T n0, n1, n2;  // near C = n0 - n1 r, D = n2 / r
+    T tiny;     // floor on r^2 (coincident blobs, including i = j)
+
+    __host__ static MobConsts make(double a)
+    {
+        MobConsts k;
+        k.a2 = T(a * a);
+        k.a2_3 = T(a * a / 3.0);
+        k.ma2 = T(-a * a);
+        k.third = T(1.0 / 3.0);
+        k.four_a2 = T(4.0 * a * a);
+        k.n0 = T(2.0 / (3.0 * a));
+        k.n1 = T(3.0 / (16.0 * a * a));
+        k.n2 = T(1.0 / (16.0 * a * a));
+        k.tiny = std::is_same<T, double>::value ? T(1e-300) : T(1e-30);
+        return k;
+    }
+};
+
+// Factor of the sums formed with MobConsts.
+__host__ inline double mob_scale(double eta) { return 1.0 / (4.0 * 3.14159265358979323846 * eta); }
+
+// 1/sqrt(x) in FP64 for x > 0.  FP64 instructions are what the FP64 kernels
+// wait for (one per ~19 cycles and SM), conversions between FP32 and FP64
+// among them, so the FP32 estimate is taken from x's truncated bits and
+// returned to FP64 by integer operations (both exact), and one cubic step
+// (Householder's iteration of third order) y + y e (1/2 + 3/8 e),
+// e = 1 - x y^2, finishes it in five FP64 instructions: |e| <= 2^-21.4 leaves
+// a truncation error of (5/16) e^3 < 2^-65.  x outside the FP32 range (and
+// NaN, infinities, zero) takes rsqrt().
+__device__ __forceinline__ double rsqrt_pos(double x)
 {
-    const T dxy2 = dx * dx + dy * dy;
-    const T r2 = mb_max(dz * dz + dxy2, k.tiny);
-    const T inv = mb_rsqrt(r2);
-    const T inv2 = inv * inv;
-    T C = inv * (k.c1 + k.c2 * inv2);
-    T D = inv * inv2 * (k.c3 + k.c4 * inv2);
-    if (r2 < k.four_a2) {
-        C = T(1) - k.k1 * (r2 * inv);
-        D = k.k2 * inv;
-    }
-    const T rf_xy = dx * fx + dy * fy;
-    const T g = D * (rf_xy + dz * fz);
-    const T rb_xy = dx * gx + dy * gy;
-    const T gb = D * (rb_xy + dz * gz);
-    if (!WALL) {
-        ux += C * fx + g * dx;
-        uy += C * fy + g * dy;
-        uz += C * fz + g * dz;
-        vx += C * gx + gb * dx;
-        vy += C * gy + gb * dy;
-        vz += C * gz + gb * dz;
-        return;
-    }
-    const T R3 = zi + zj;
-    const T invR = mb_rsqrt(R3 * R3 + dxy2);
-    const T hs = zj * invR;
-    const T ht = zi * invR;
-    const T e3 = hs + ht;
-    const T E = e3 * e3;
-    const T t2 = k.a2 * (invR * invR);
-    const T t4 = t2 * t2;
-    const T p = hs * ht;
-    const T f1 = T(-1) - T(2) * p + t2 * (T(2) * E - T(2.0 / 3.0)) + t4 * (T(2.0 / 3.0) - T(10.0 / 3.0) * E);
-    const T f2 = T(-1) + T(6) * p + t2 * (T(2) - T(10) * E) + t4 * (T(70.0 / 3.0) * E - T(10.0 / 3.0));
-    const T f3 = T(2) * hs + e3 * (t2 * (T(20) * E - T(4)) + t4 * (T(40.0 / 3.0) - T(140.0 / 3.0) * E) - T(12) * p);
-    const T f4 = T(2) * hs - T(20.0 / 3.0) * e3 * t4;
-    const T f5 = T(-4) * hs * hs - T(4) * E * t2 + t4 * (T(20) * E - T(8.0 / 3.0));
-    const T s = k.sw * invR;
-    const T Cx = C + s * f1;
-    const T eF = (rf_xy + R3 * fz) * invR;
-    const T gw = (f2 * eF + f3 * fz) * invR;
-    const T kz = f4 * eF + f5 * fz;
-    const T Gx = g + s * gw;
-    ux += Cx * fx + Gx * dx;
-    uy += Cx * fy + Gx * dy;
-    uz += Cx * fz + g * dz + s * (gw * R3 + kz);
-    const T eB = (rb_xy + R3 * gz) * invR;
-    const T gwb = (f2 * eB + f4 * gz) * invR;
-    const T kzb = f3 * eB + f5 * gz;
-    const T Gb = gb + s * gwb;
-    vx += Cx * gx + Gb * dx;
-    vy += Cx * gy + Gb * dy;
-    vz += Cx * gz + gb * dz + s * (gwb * R3 + kzb);
+    const int h = __double2hiint(x);
+    if ((unsigned)(h - 0x38100000) >= 0x47e00000u - 0x38100000u) return rsqrt(x);
+    const float xf =
+        __int_as_float(((h - 0x38000000) << 3) | (int)((unsigned)__double2loint(x) >> 29));
+    float yf;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(xf));
+    const int b = __float_as_int(yf);
+    const double y = __hiloint2double((b >> 3) + 0x38000000, b << 29);
+    const double e = fma(-x, y * y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
-// Full 3x3 block M_ij in FP64, units of (6 pi eta a)^-1, row-major
+// x < bound for x >= 0 on the bit patterns: an FP64 comparison is an FP64
+// instruction.
+__device__ __forceinline__ bool below(double x, double bound)
+{
+    return __double_as_longlong(x) < __double_as_longlong(bound);
+}
+
+template <typename T>
+struct Mob {
+    T Cx, Cz, D, A2, A3, A4, R3;
+};
+
+// Coefficients of one pair at separation d = r_i - r_j, heights zi, zj.
+template <bool WALL>
+__device__ __forceinline__ Mob<double> mob_coefs(double dx, double dy, double dz, double zi,
+                                                 double zj, const MobConsts<double> &k)
+{
+    Mob<double> m;
+    const double dxy2 = fma(dx, dx, dy * dy);
+    const double r2 = fma(dz, dz, dxy2);
+    const double inv = rsqrt_pos(r2), inv2 = inv * inv;
+    m.Cx = inv * fma(k.a2_3, inv2, 0.5);
+    m.D = (inv * inv2) * fma(k.ma2, inv2, 0.5);
+    if (below(r2, k.four_a2)) {  // overlapping blobs (rare): regularised branch
+        const double rr = fmax(r2, k.tiny), ir = rsqrt(rr);
+        m.Cx = fma(-k.n1, rr * ir, k.n0);
+        m.D = k.n2 * ir;
+    }
+    if (!WALL) return m;
+    m.R3 = zi + zj;
+    const double H2 = m.R3 * m.R3;
+    const double u = rsqrt_pos(H2 + dxy2), w = u * u;
+    const double X = k.a2 * w, X3 = X * k.third, Q = X3 * X, E = H2 * w;
+    const double c = fma(zi * zj, w, X3);
+    const double EQ = E * Q, S = fma(X, E, Q);
+    const double f1 = fma(-5.0, EQ, S) - (c + 0.5);
+    const double f2 = fma(35.0, EQ, fma(-5.0, S, fma(3.0, c, -0.5)));
+    const double Qm = -10.0 * Q, br = fma(2.0, f2, Qm + 1.0);
+    const double t3 = fma(-m.R3, br, zj), t4 = fma(m.R3, Qm, zj);
+    const double f5 = fma(30.0, EQ, -2.0 * fma(zj * zj, w, S + Q));
+    const double uw = u * w;
+    m.A2 = uw * f2;
+    m.A3 = uw * t3;
+    m.A4 = uw * t4;
+    m.Cx = fma(u, f1, m.Cx);
+    m.Cz = fma(u, f5, m.Cx);
+    return m;
+}
+
+// u += M f from the coefficients; TRANS: u += M^T f.
+template <bool WALL, bool TRANS = false, typename T>
+__device__ __forceinline__ void mob_apply(const Mob<T> &m, T dx, T dy, T dz, T fx, T fy, T fz,
+                                          T &ux, T &uy, T &uz)
+{
+    const T rf = fma(dx, fx, dy * fy);
+    const T g = m.D * fma(dz, fz, rf);
+    if (!WALL) {
+        ux = fma(m.Cx, fx, fma(g, dx, ux));
+        uy = fma(m.Cx, fy, fma(g, dy, uy));
+        uz = fma(m.Cx, fz, fma(g, dz, uz));
+        return;
+    }
+    const T RF = fma(m.R3, fz, rf);
+    const T gw = fma(m.A2, RF, (TRANS ? m.A4 : m.A3) * fz);
+    const T G = g + gw;
+    ux = fma(m.Cx, fx, fma(G, dx, ux));
+    uy = fma(m.Cx, fy, fma(G, dy, uy));
+    uz = fma(m.Cz, fz, fma(TRANS ? m.A3 : m.A4, RF, fma(gw, m.R3, fma(g, dz, uz))));
+}
+
+// Full 3x3 block M_ij in FP64, units of (4 pi eta)^-1, row-major
 // m[3*alpha + beta] (alpha = velocity component of i, beta = force
 // component of j).  Used to assemble the per-body blocks of the
 // preconditioner.
 template <bool WALL>
 __device__ __forceinline__ void block_f64(const double *ri, const double *rj,
-                                          const PairConsts<double> &k, double m[9])
+                                          const MobConsts<double> &k, double m[9])
 {
-    const double d[3] = {ri[0] - rj[0], ri[1] - rj[1], ri[2] - rj[2]};
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        double u[3] = {0.0, 0.0, 0.0};
-        const double f[3] = {b == 0 ? 1.0 : 0.0, b == 1 ? 1.0 : 0.0, b == 2 ? 1.0 : 0.0};
-        pair_accumulate<WALL, double>(d[0], d[1], d[2], ri[2], rj[2], f[0], f[1], f[2], k, u[0],
-                                      u[1], u[2]);
-        m[b] = u[0];
-        m[3 + b] = u[1];
-        m[6 + b] = u[2];
+    const double dx = ri[0] - rj[0], dy = ri[1] - rj[1], dz = ri[2] - rj[2];
+    const Mob<double> c = mob_coefs<WALL>(dx, dy, dz, ri[2], rj[2], k);
+    const double h = WALL ? c.D + c.A2 : c.D;  // factor of d_a d_b in the plane
+    const double hx = h * dx, hy = h * dy, Dz = c.D * dz;
+    m[0] = fma(hx, dx, c.Cx);
+    m[1] = m[3] = hx * dy;
+    m[4] = fma(hy, dy, c.Cx);
+    if (!WALL) {
+        m[2] = m[6] = dx * Dz;
+        m[5] = m[7] = dy * Dz;
+        m[8] = fma(dz, Dz, c.Cx);
+        return;
     }
+    const double AR = c.A2 * c.R3, v = Dz + AR;
+    m[2] = dx * (v + c.A3);
+    m[5] = dy * (v + c.A3);
+    m[6] = dx * (v + c.A4);
+    m[7] = dy * (v + c.A4);
+    m[8] = fma(c.R3, AR + (c.A3 + c.A4), fma(dz, Dz, c.Cz));
 }
 
 // ---------------------------------------------------------------------------

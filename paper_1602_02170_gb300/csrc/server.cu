@@ -344,7 +344,7 @@ template <bool WALL>
 __global__ void __launch_bounds__(kNT) eng_f64_kernel(const Work *__restrict__ W,
                                                       const int64_t *__restrict__ item_off, int nw,
                                                       int64_t n_items, const int *__restrict__ mask,
-                                                      PairConsts<double> k, double scale)
+                                                      MobConsts<double> k, double scale)
 {
     __shared__ double sm[6 * kNT];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
@@ -1021,7 +1021,8 @@ struct Engine {
                      const int *zero_mask = nullptr)
     {
         if (list.empty()) return MB_OK;
-        const double scale = 1.0 / (6.0 * kPi * prm.eta * prm.a);
+        const double scale =
+            prec == MB_FP64 ? mob_scale(prm.eta) : 1.0 / (6.0 * kPi * prm.eta * prm.a);
         const bool x2 = prec == MB_FP32_KAHAN;
         const bool dfs = prec == MB_DF64;          // symmetric double-float
         const bool sym = (x2 && np_variant == 3) || dfs;
@@ -1124,7 +1125,7 @@ struct Engine {
                 else eng_x2_kernel<false, 2><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
             }
         } else {
-            const PairConsts<double> k = PairConsts<double>::make(prm.a);
+            const MobConsts<double> k = MobConsts<double>::make(prm.a);
             if (wall) eng_f64_kernel<true><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
             else eng_f64_kernel<false><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
         }

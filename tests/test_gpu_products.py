@@ -1,0 +1,48 @@
+"""Products with the mobility at the sizes where their kernels change shape.
+
+Tolerances: FP64 1e-12 relative L2 (a sum of n terms of about a hundred
+roundings each, n eps ~ 1e-12 at the sizes here)."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1602_02170_gb300 import inputs as I
+from tests.gpu_common import ctx, dev, host, rel_l2  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp64": 1e-12}
+
+
+def _cloud(seed, n):
+    return I.blob_cloud(seed, n, 0.5, 2.0 * max(1.0, n ** 0.5), 0.5, 1.5)
+
+
+@pytest.mark.parametrize("wall", [True, False])
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 2209, 3140, 4420])
+def test_fp64_items_of_every_size(ctx, n, wall):
+    """The FP64 kernel's items hold 4, 8, 16 or 32 sources (the last three
+    from about 2,200, 3,140 and 4,420 blobs); ragged and full blocks."""
+    r, f = _cloud(n, n)
+    got = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, wall, "fp64"))
+    assert rel_l2(got, O.matvec(r, f, 0.5, 1.0, wall)) <= TOL["fp64"]
+
+
+def test_fp64_length_scale_outside_fp32_range(ctx):
+    """Lengths of 1e-25 put r^2 outside the FP32 range, where the FP64
+    reciprocal square root takes its general form: M scales as 1 / length."""
+    r, f = _cloud(5, 200)
+    ref = O.matvec(r, f, 0.5, 1.0, True)
+    got = host(ctx.mobility_matvec(dev(r * 1e-25), dev(f), 0.5e-25, 1.0, True, "fp64"))
+    assert rel_l2(got * 1e-25, ref) <= TOL["fp64"]
+
+
+@pytest.mark.parametrize("target", ["f", "r"])
+def test_fp64_product_in_place(ctx, target):
+    """The velocities may overwrite the forces or the positions."""
+    r, f = _cloud(6, 700)
+    R, F = dev(r), dev(f)
+    want = host(ctx.mobility_matvec(R, F, 0.5, 1.0, True, "fp64"))
+    out = F if target == "f" else R
+    ctx.mobility_matvec(R, F, 0.5, 1.0, True, "fp64", out=out)
+    assert rel_l2(host(out), want) <= 1e-14
