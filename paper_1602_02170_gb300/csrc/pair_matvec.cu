@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256) pack_hilo_kernel(const double *__restrict
 template <bool WALL, int TPT>
 __global__ void __launch_bounds__(kNT) pair_f32_kernel(
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
-    int64_t n, int64_t chunk, int n_tblocks, int64_t n_items, PairConsts<float> k,
+    int64_t n, int64_t chunk, int n_tblocks, int64_t n_items, MobConsts<float> k,
     double *__restrict__ out, double scale, int direct)
 {
     __shared__ float4 sA[kNT];  // (x_hi, y_hi, z_hi, f_x)
@@ -159,8 +159,8 @@ __global__ void __launch_bounds__(kNT) pair_f32_kernel(
                     const float dx = (xh[t] - A.x) + (xl[t] - B.x);
                     const float dy = (yh[t] - A.y) + (yl[t] - B.y);
                     const float dz = (zh[t] - A.z) + (zl[t] - B.z);
-                    pair_accumulate<WALL, float>(dx, dy, dz, zh[t], A.z, A.w, B.w, fz, k, ax[t],
-                                                 ay[t], az[t]);
+                    const Mob<float> m = mob_coefs<WALL>(dx, dy, dz, zh[t], A.z, k);
+                    mob_apply<WALL>(m, dx, dy, dz, A.w, B.w, fz, ax[t], ay[t], az[t]);
                 }
             }
 #pragma unroll
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kNT) pair_f32_kernel(
 template <bool WALL, int NP, int NT = kNT>
 __global__ void __launch_bounds__(NT, NT == kNT ? (NP == 1 ? 3 : 2) : 16) pair_f32x2_kernel(
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
-    int64_t n, int64_t chunk, int n_tblocks, int64_t n_items, PairConsts2 k,
+    int64_t n, int64_t chunk, int n_tblocks, int64_t n_items, MobConsts2 k,
     double *__restrict__ out, double scale, int direct)
 {
     __shared__ float4 sP[kX2SmemFloat4PerSource * NT];
@@ -211,7 +211,8 @@ __global__ void __launch_bounds__(NT, NT == kNT ? (NP == 1 ? 3 : 2) : 16) pair_f
 //
 // box (optional): the bounding box of every block, (min x, y, z, max x, y, z),
 // and grid->far2, the squared distance beyond which a block pair is far (see
-// x2sym_item); such pairs take the FAR instance.
+// x2sym_item); such pairs take the kFar instance, and the kVeryFar one from
+// kVeryFarRadii radii on.
 struct SortGrid {
     float lo[3], inv_h[3];  // cell of x: (x - lo) * inv_h per axis
     int bits[3];            // bits of the cell index per axis (nbits in all)
@@ -221,12 +222,13 @@ struct SortGrid {
 template <bool WALL>
 __global__ void __launch_bounds__(kNT, 2) pair_sym_kernel(
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
-    int64_t n, int64_t nb, int64_t n_items, PairConsts2 k, double *__restrict__ u, double scale,
+    int64_t n, int64_t nb, int64_t n_items, MobConsts2 k, double *__restrict__ u, double scale,
     const float *__restrict__ box, const SortGrid *__restrict__ grid)
 {
     __shared__ float4 sP[kX2SmemFloat4PerSource * kNT];
     __shared__ float sRev[3 * kNT * (kNT / 32)];
     const float far2 = box ? fmaxf(grid->far2, 1.5625f * k.four_a2) : 0.f;
+    const float vfar2 = 0.25f * kVeryFarRadii * kVeryFarRadii * k.four_a2;
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         // row I holds nb - I items; rowoff(I) = I*nb - I*(I-1)/2
         int64_t lo_r = 0, hi_r = nb;
@@ -237,7 +239,7 @@ __global__ void __launch_bounds__(kNT, 2) pair_sym_kernel(
         }
         const int64_t I = lo_r;
         const int64_t J = I + (item - (I * nb - I * (I - 1) / 2));
-        bool far = false;
+        int level = kNear;  // the same in every thread
         if (box && I != J) {
             const float *bi = box + 6 * I, *bj = box + 6 * J;
             float d2 = 0.f;
@@ -246,10 +248,13 @@ __global__ void __launch_bounds__(kNT, 2) pair_sym_kernel(
                 const float g = fmaxf(fmaxf(bj[c] - bi[3 + c], bi[c] - bj[3 + c]), 0.f);
                 d2 = fmaf(g, g, d2);
             }
-            far = d2 > far2;  // the same in every thread
+            if (d2 > far2) level = d2 > vfar2 ? kVeryFar : kFar;
         }
-        if (far) x2sym_item<WALL, kNT, true>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
-        else x2sym_item<WALL, kNT, false>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
+        if (level == kVeryFar)
+            x2sym_item<WALL, kNT, kVeryFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
+        else if (level == kFar)
+            x2sym_item<WALL, kNT, kFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
+        else x2sym_item<WALL, kNT, kNear>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
     }
 }
 
@@ -291,7 +296,7 @@ template <bool WALL>
 __global__ void __launch_bounds__(kNT, 3) eval_f32x2_kernel(
     const float4 *__restrict__ thi, const float4 *__restrict__ tlo, int64_t nt,
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
-    int64_t ns, int64_t chunk, int n_tblocks, int64_t n_items, PairConsts2 k,
+    int64_t ns, int64_t chunk, int n_tblocks, int64_t n_items, MobConsts2 k,
     double *__restrict__ out, double scale, int direct)
 {
     __shared__ float4 sP[kX2SmemFloat4PerSource * kNT];
@@ -525,17 +530,17 @@ void f32_launch(int v, const Plan &p, cudaStream_t s, const float4 *hi, const fl
 {
     if (v == 0) {
         pair_f32_kernel<WALL, kTPT><<<p.grid, kNT, 0, s>>>(
-            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, PairConsts<float>::make(a), out, scale,
+            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, MobConsts<float>::make(a), out, scale,
             direct);
     } else if (v == 1) {
         pair_f32x2_kernel<WALL, 1><<<p.grid, kNT, 0, s>>>(
-            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, PairConsts2::make(a), out, scale, direct);
+            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, MobConsts2::make(a), out, scale, direct);
     } else if (v == 4) {
         pair_f32x2_kernel<WALL, 1, kSmallNT><<<p.grid, kSmallNT, 0, s>>>(
-            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, PairConsts2::make(a), out, scale, direct);
+            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, MobConsts2::make(a), out, scale, direct);
     } else {
         pair_f32x2_kernel<WALL, 2><<<p.grid, kNT, 0, s>>>(
-            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, PairConsts2::make(a), out, scale, direct);
+            hi, lo, f, n, p.chunk, p.n_tblocks, p.items, MobConsts2::make(a), out, scale, direct);
     }
 }
 
@@ -950,7 +955,7 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
             MB_CUDA_TRY(ctx, cudaMemsetAsync(uk, 0, sizeof(double) * 3 * (size_t)n, s));
         }
         auto *ev = profile ? profile_begin(ctx, s) : nullptr;
-        const PairConsts2 k = PairConsts2::make(a);
+        const MobConsts2 k = MobConsts2::make(a);
         if (wall)
             pair_sym_kernel<true><<<grid, kNT, 0, s>>>(hi, lo, fk, n, nb, items, k, uk, scale, box, sg);
         else
@@ -1171,7 +1176,7 @@ mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64
     }
     // FP64: u (or, deferred, the one partial sum the caller scales) zeroed,
     // then one launch over the block-pair triangle
-    double *uk = u, sk = mob_scale(eta);
+    double *uk = u, sk = scale;
     if (defer) {
         MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)n, "matvec partials"));
         uk = (double *)ctx->partial.ptr;
@@ -1218,7 +1223,7 @@ mb_status matvec_eval(mb_context *ctx, const double *x, int64_t nt, const double
                       const double *f, int64_t ns, double a, double eta, int wall,
                       mb_precision prec, double *u, cudaStream_t s)
 {
-    const double scale = prec == MB_FP64 ? mob_scale(eta) : 1.0 / (6.0 * kPi * eta * a);
+    const double scale = 1.0 / (6.0 * kPi * eta * a);
     if (prec == MB_FP64) {
         const int res = wall ? resident_ctas(ctx, eval_f64_kernel<true>)
                              : resident_ctas(ctx, eval_f64_kernel<false>);
@@ -1267,7 +1272,7 @@ mb_status matvec_eval(mb_context *ctx, const double *x, int64_t nt, const double
         MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)nt * p.S, "eval partials"));
         out = (double *)ctx->partial.ptr;
     }
-    const PairConsts2 k = PairConsts2::make(a);
+    const MobConsts2 k = MobConsts2::make(a);
     const float4 *thi = (const float4 *)ctx->eval_hi.ptr, *tlo = (const float4 *)ctx->eval_lo.ptr;
     const float4 *hi = (const float4 *)ctx->pos_hi.ptr, *lo = (const float4 *)ctx->pos_lo.ptr;
     if (wall)
@@ -1430,7 +1435,7 @@ extern "C" mb_status mb_mobility_matvec_noalloc(const double *r, const double *f
                              kNoallocMaxChunks);
     const int direct = p.S == 1;
     double *out = direct ? u : partial;
-    const PairConsts<float> k = PairConsts<float>::make(a);
+    const MobConsts<float> k = MobConsts<float>::make(a);
     if (wall)
         pair_f32_kernel<true, kTPT><<<p.grid, kNT, 0, s>>>(hi, lo, f, n, p.chunk, p.n_tblocks,
                                                            p.items, k, out, scale, direct);

@@ -26,10 +26,20 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x)
 // Shared-memory floats per source in the packed kernel (5 float4).
 constexpr int kX2SmemFloat4PerSource = 5;
 
+__device__ __forceinline__ void stage_x2(float4 *d, float4 h, float4 l, float fx, float fy, float fz)
+{
+    const float zz = -2.f * h.z * h.z;
+    d[0] = make_float4(-h.x, -h.x, -h.y, -h.y);
+    d[1] = make_float4(h.z, h.z, zz, zz);
+    d[2] = make_float4(-l.x, -l.x, -l.y, -l.y);
+    d[3] = make_float4(-l.z, -l.z, fx, fx);
+    d[4] = make_float4(fy, fy, fz, fz);
+}
+
 // Packed FP32 item: each thread owns 2*NP targets, held as NP float2 pairs;
 // target of pair q, half h: tb*NT*2*NP + (2q + h)*NT + threadIdx.x.
 // Sources are staged once per tile as duplicated float2 operands:
-//   sP[5s+0] = (-x_hi, -x_hi, -y_hi, -y_hi)   sP[5s+1] = (-z_hi, -z_hi, z_hi, z_hi)
+//   sP[5s+0] = (-x_hi, -x_hi, -y_hi, -y_hi)   sP[5s+1] = (z_hi, z_hi, zz, zz), zz = -2 z_hi^2
 //   sP[5s+2] = (-x_lo, -x_lo, -y_lo, -y_lo)   sP[5s+3] = (-z_lo, -z_lo, f_x, f_x)
 //   sP[5s+4] = (f_y, f_y, f_z, f_z)
 template <bool WALL, int NP, int NT>
@@ -38,7 +48,7 @@ __device__ __forceinline__ void x2_item(float4 *__restrict__ sP, const float4 *_
                                         const float4 *__restrict__ hi,
                                         const float4 *__restrict__ lo,
                                         const double *__restrict__ f, int tb,
-                                        int64_t j_begin, int64_t j_end, const PairConsts2 &k,
+                                        int64_t j_begin, int64_t j_end, const MobConsts2 &k,
                                         double *__restrict__ out, double m)
 {
     float2 xh[NP], yh[NP], zh[NP], xl[NP], yl[NP], zl[NP];
@@ -74,12 +84,7 @@ __device__ __forceinline__ void x2_item(float4 *__restrict__ sP, const float4 *_
             const float fx = valid ? (float)f[3 * jc] : 0.f;
             const float fy = valid ? (float)f[3 * jc + 1] : 0.f;
             const float fz = valid ? (float)f[3 * jc + 2] : 0.f;
-            float4 *d = sP + kX2SmemFloat4PerSource * threadIdx.x;
-            d[0] = make_float4(-h.x, -h.x, -h.y, -h.y);
-            d[1] = make_float4(-h.z, -h.z, h.z, h.z);
-            d[2] = make_float4(-l.x, -l.x, -l.y, -l.y);
-            d[3] = make_float4(-l.z, -l.z, fx, fx);
-            d[4] = make_float4(fy, fy, fz, fz);
+            stage_x2(sP + kX2SmemFloat4PerSource * threadIdx.x, h, l, fx, fy, fz);
         }
         __syncthreads();
         float2 ax[NP], ay[NP], az[NP];
@@ -92,7 +97,7 @@ __device__ __forceinline__ void x2_item(float4 *__restrict__ sP, const float4 *_
             const float4 *P = sP + kX2SmemFloat4PerSource * s;
             const float4 P0 = P[0], P1 = P[1], P2 = P[2], P3 = P[3], P4 = P[4];
             const float2 nxh = make_float2(P0.x, P0.y), nyh = make_float2(P0.z, P0.w);
-            const float2 nzh = make_float2(P1.x, P1.y), zj = make_float2(P1.z, P1.w);
+            const float2 zj = make_float2(P1.x, P1.y), zz = make_float2(P1.z, P1.w);
             const float2 nxl = make_float2(P2.x, P2.y), nyl = make_float2(P2.z, P2.w);
             const float2 nzl = make_float2(P3.x, P3.y), fx = make_float2(P3.z, P3.w);
             const float2 fy = make_float2(P4.x, P4.y), fz = make_float2(P4.z, P4.w);
@@ -100,10 +105,10 @@ __device__ __forceinline__ void x2_item(float4 *__restrict__ sP, const float4 *_
             for (int q = 0; q < NP; ++q) {
                 const float2 dx = add2(add2(xh[q], nxh), add2(xl[q], nxl));
                 const float2 dy = add2(add2(yh[q], nyh), add2(yl[q], nyl));
-                const float2 dz = add2(add2(zh[q], nzh), add2(zl[q], nzl));
+                const float2 dz = add2(fma2(zj, k.m1, zh[q]), add2(zl[q], nzl));
                 const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
-                pair_accumulate2<WALL>(dx, dy, dz, dxy2, zh[q], zj, fx, fy, fz, k, ax[q], ay[q],
-                                       az[q]);
+                const Mob<float2> m = mob_coefs2<WALL, kNear>(dz, dxy2, zh[q], zj, zz, k);
+                mob_apply2<WALL>(m, dx, dy, dz, fx, fy, fz, ax[q], ay[q], az[q]);
             }
         }
 #pragma unroll
@@ -185,16 +190,15 @@ __device__ __forceinline__ void f64_item(double *__restrict__ sm, const double *
 // over all ordered pairs.  u must be zeroed beforehand and receives
 // scale * M f.
 //
-// FAR (off-diagonal block pairs whose bounding boxes are farther apart than
-// both 2a and 2^18 ulp of the largest coordinate): the separations take the
-// hi parts alone, whose rounding then moves a separation by at most 2^-18 of
-// itself, and the overlap test is left out.
-template <bool WALL, int NT, bool FAR = false>
+// LEVEL: how far apart the blocks' bounding boxes are known to be (mob_coefs2).
+// From kFar on the separations take the hi parts alone, whose rounding then
+// moves a separation by at most 2^-18 of itself.
+template <bool WALL, int NT, int LEVEL = kNear>
 __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__restrict__ sRev,
                                            const float4 *__restrict__ hi,
                                            const float4 *__restrict__ lo,
                                            const double *__restrict__ f, int64_t n, int64_t I,
-                                           int64_t J, const PairConsts2 &k,
+                                           int64_t J, const MobConsts2 &k,
                                            double *__restrict__ u, double scale)
 {
     constexpr int NW = NT / 32;
@@ -229,12 +233,7 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
             const float fx = valid ? (float)f[3 * jc] : 0.f;
             const float fy = valid ? (float)f[3 * jc + 1] : 0.f;
             const float fz = valid ? (float)f[3 * jc + 2] : 0.f;
-            float4 *d = sP + kX2SmemFloat4PerSource * threadIdx.x;
-            d[0] = make_float4(-h.x, -h.x, -h.y, -h.y);
-            d[1] = make_float4(-h.z, -h.z, h.z, h.z);
-            d[2] = make_float4(-l.x, -l.x, -l.y, -l.y);
-            d[3] = make_float4(-l.z, -l.z, fx, fx);
-            d[4] = make_float4(fy, fy, fz, fz);
+            stage_x2(sP + kX2SmemFloat4PerSource * threadIdx.x, h, l, fx, fy, fz);
         }
         __syncthreads();
         float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
@@ -243,13 +242,15 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
             for (int s = 0; s < NT; ++s) {
                 const float4 *P = sP + kX2SmemFloat4PerSource * s;
                 const float4 P0 = P[0], P1 = P[1], P2 = P[2], P3 = P[3], P4 = P[4];
+                const float2 zj = make_float2(P1.x, P1.y);
                 const float2 dx = add2(add2(xh, make_float2(P0.x, P0.y)), add2(xl, make_float2(P2.x, P2.y)));
                 const float2 dy = add2(add2(yh, make_float2(P0.z, P0.w)), add2(yl, make_float2(P2.z, P2.w)));
-                const float2 dz = add2(add2(zh, make_float2(P1.x, P1.y)), add2(zl, make_float2(P3.x, P3.y)));
+                const float2 dz = add2(fma2(zj, k.m1, zh), add2(zl, make_float2(P3.x, P3.y)));
                 const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
-                pair_accumulate2<WALL>(dx, dy, dz, dxy2, zh, make_float2(P1.z, P1.w),
-                                       make_float2(P3.z, P3.w), make_float2(P4.x, P4.y),
-                                       make_float2(P4.z, P4.w), k, ax, ay, az);
+                const Mob<float2> m =
+                    mob_coefs2<WALL, kNear>(dz, dxy2, zh, zj, make_float2(P1.z, P1.w), k);
+                mob_apply2<WALL>(m, dx, dy, dz, make_float2(P3.z, P3.w), make_float2(P4.x, P4.y),
+                                 make_float2(P4.z, P4.w), ax, ay, az);
             }
         } else {
             for (int g = 0; g < NT / 32; ++g) {
@@ -259,22 +260,23 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
                     const int s = g * 32 + ((lane + t) & 31);
                     const float4 *P = sP + kX2SmemFloat4PerSource * s;
                     const float4 P0 = P[0], P1 = P[1], P3 = P[3], P4 = P[4];
-                    float2 dx, dy, dz;
-                    if (FAR) {
-                        dx = add2(xh, make_float2(P0.x, P0.y));
-                        dy = add2(yh, make_float2(P0.z, P0.w));
-                        dz = add2(zh, make_float2(P1.x, P1.y));
-                    } else {
+                    const float2 zj = make_float2(P1.x, P1.y);
+                    float2 dx = add2(xh, make_float2(P0.x, P0.y));
+                    float2 dy = add2(yh, make_float2(P0.z, P0.w));
+                    float2 dz = fma2(zj, k.m1, zh);
+                    if (LEVEL == kNear) {
                         const float4 P2 = P[2];
-                        dx = add2(add2(xh, make_float2(P0.x, P0.y)), add2(xl, make_float2(P2.x, P2.y)));
-                        dy = add2(add2(yh, make_float2(P0.z, P0.w)), add2(yl, make_float2(P2.z, P2.w)));
-                        dz = add2(add2(zh, make_float2(P1.x, P1.y)), add2(zl, make_float2(P3.x, P3.y)));
+                        dx = add2(dx, add2(xl, make_float2(P2.x, P2.y)));
+                        dy = add2(dy, add2(yl, make_float2(P2.z, P2.w)));
+                        dz = add2(dz, add2(zl, make_float2(P3.x, P3.y)));
                     }
-                    const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
-                    pair_sym2<WALL, FAR>(dx, dy, dz, dxy2, zh, make_float2(P1.z, P1.w),
-                                         make_float2(P3.z, P3.w), make_float2(P4.x, P4.y),
-                                         make_float2(P4.z, P4.w), fix, fiy, fiz, k, ax, ay, az, rx,
-                                         ry, rz);
+                    const float2 dxy2 = fma2(dy, dy, LEVEL == kNear ? fma2(dx, dx, k.tiny)
+                                                                    : mul2(dx, dx));
+                    const Mob<float2> m =
+                        mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, zj, make_float2(P1.z, P1.w), k);
+                    mob_apply2<WALL>(m, dx, dy, dz, make_float2(P3.z, P3.w),
+                                     make_float2(P4.x, P4.y), make_float2(P4.z, P4.w), ax, ay, az);
+                    mob_apply2<WALL, true>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
                     // hand the accumulator to lane - 1, which meets this source next step
                     const int from = (lane + 1) & 31;
                     rx.x = __shfl_sync(0xffffffffu, rx.x, from);

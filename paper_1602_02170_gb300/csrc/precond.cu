@@ -1690,7 +1690,7 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
     MB_TRY(ensure(ctx, ctx->sol_dots, sizeof(double) * stride * group, "preconditioner scratch"));
     SplitScratch scr{(double *)ctx->sol_dots.ptr, stride, nmax};
     const MobConsts<double> k = MobConsts<double>::make(a);
-    const double scale = mob_scale(eta);
+    const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
     const bool lsmem = nmax <= kSmemMaxRows;
     const size_t fsmem =
         sizeof(double) * (lsmem ? (size_t)nmax * nmax + (7 + kPanel) * (size_t)nmax + 72
@@ -1882,7 +1882,7 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
     const size_t small = sizeof(double) * (13 * (size_t)nmax + 72);
     const size_t smem = small + (lsmem ? sizeof(double) * (size_t)nmax * nmax : 0);
     const MobConsts<double> k = MobConsts<double>::make(a);
-    const double scale = mob_scale(eta);
+    const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
     int grid = (int)std::min<int64_t>(nb, 4 * (int64_t)ctx->sm_count);
     double *scratch = nullptr;
     int64_t stride = 0;
@@ -1951,7 +1951,7 @@ mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, cons
     const size_t small = sizeof(double) * (13 * (size_t)nmax + 72);
     const size_t smem = small + (lsmem ? sizeof(double) * (size_t)nmax * nmax : 0);
     const MobConsts<double> k = MobConsts<double>::make(a);
-    const double scale = mob_scale(eta);
+    const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
     int grid = (int)std::min<int64_t>(nb, 4 * (int64_t)ctx->sm_count);
     double *scratch = nullptr;
     int64_t stride = 0;

@@ -259,7 +259,7 @@ __global__ void eng_rhs_kernel(const Seg *__restrict__ segs, int nseg, int64_t n
 template <bool WALL, int NP>
 __global__ void __launch_bounds__(kNT, NP == 1 ? 3 : 2) eng_x2_kernel(
     const Work *__restrict__ W, const int64_t *__restrict__ item_off, int nw, int64_t n_items,
-    const int *__restrict__ mask, PairConsts2 k, double scale)
+    const int *__restrict__ mask, MobConsts2 k, double scale)
 {
     __shared__ float4 sP[kX2SmemFloat4PerSource * kNT];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kNT, NP == 1 ? 3 : 2) eng_x2_kernel(
 template <bool WALL>
 __global__ void __launch_bounds__(kNT, 2) eng_sym_kernel(
     const Work *__restrict__ W, const int64_t *__restrict__ item_off, int nw, int64_t n_items,
-    const int *__restrict__ mask, PairConsts2 k, double scale)
+    const int *__restrict__ mask, MobConsts2 k, double scale)
 {
     __shared__ float4 sP[kX2SmemFloat4PerSource * kNT];
     __shared__ float sRev[3 * kNT * (kNT / 32)];
@@ -1021,8 +1021,7 @@ struct Engine {
                      const int *zero_mask = nullptr)
     {
         if (list.empty()) return MB_OK;
-        const double scale =
-            prec == MB_FP64 ? mob_scale(prm.eta) : 1.0 / (6.0 * kPi * prm.eta * prm.a);
+        const double scale = 1.0 / (6.0 * kPi * prm.eta * prm.a);
         const bool x2 = prec == MB_FP32_KAHAN;
         const bool dfs = prec == MB_DF64;          // symmetric double-float
         const bool sym = (x2 && np_variant == 3) || dfs;
@@ -1112,11 +1111,11 @@ struct Engine {
             if (wall) eng_df_kernel<true><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
             else eng_df_kernel<false><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
         } else if (sym) {
-            const PairConsts2 k = PairConsts2::make(prm.a);
+            const MobConsts2 k = MobConsts2::make(prm.a);
             if (wall) eng_sym_kernel<true><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
             else eng_sym_kernel<false><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
         } else if (prec == MB_FP32_KAHAN) {
-            const PairConsts2 k = PairConsts2::make(prm.a);
+            const MobConsts2 k = MobConsts2::make(prm.a);
             if (np_variant == 1) {
                 if (wall) eng_x2_kernel<true, 1><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
                 else eng_x2_kernel<false, 1><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);

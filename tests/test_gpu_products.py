@@ -1,7 +1,8 @@
 """Products with the mobility at the sizes where their kernels change shape.
 
 Tolerances: FP64 1e-12 relative L2 (a sum of n terms of about a hundred
-roundings each, n eps ~ 1e-12 at the sizes here)."""
+roundings each, n eps ~ 1e-12 at the sizes here); FP32 1e-5 of the largest
+velocity, the bar of the FP32 products, unless a test derives its own."""
 import numpy as np
 import pytest
 
@@ -11,7 +12,7 @@ from tests.gpu_common import ctx, dev, host, rel_l2  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
-TOL = {"fp64": 1e-12}
+TOL = {"fp64": 1e-12, "fp32": 1e-5}
 
 
 def _cloud(seed, n):
@@ -46,3 +47,26 @@ def test_fp64_product_in_place(ctx, target):
     out = F if target == "f" else R
     ctx.mobility_matvec(R, F, 0.5, 1.0, True, "fp64", out=out)
     assert rel_l2(host(out), want) <= 1e-14
+
+
+@pytest.mark.parametrize("gap", [90.0, 95.9, 96.1, 400.0])
+def test_fp32_far_and_very_far_blocks(ctx, gap):
+    """Two clusters of blobs a = 0.5 high above the wall, forces on one of
+    them only: the other's velocities come from block pairs around the
+    distance of 192 a = 96 from which the FP32 kernel leaves out the terms in
+    (a / rho)^4.  Expected: some twenty roundings of 2^-24 a pair, separations
+    from hi parts (2^-24 of coordinates up to 420 against 90 and more) and
+    dropped terms below 2^-26, so 4e-6 of the FP64 product."""
+    rng = np.random.default_rng(int(gap))
+    n = 9216  # 18 blocks of 512 in each cluster
+    r = rng.uniform([0, 0, 40], [10, 10, 50], (2 * n, 3))
+    r[n:, 0] += 10.0 + gap
+    f = rng.standard_normal((2 * n, 3))
+    f[n:] = 0.0
+    ctx.set_pair_variant(3)
+    try:
+        got = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, True, "fp32"))
+    finally:
+        ctx.set_pair_variant(-1)
+    ref = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, True, "fp64"))
+    assert rel_l2(got[n:], ref[n:]) <= 4e-6
