@@ -122,7 +122,7 @@ def parse():
     p.add_argument("--bodies", type=int, default=4096,
                    help="setup: monolayer bodies (at the monolayer's area density)")
     p.add_argument("--pair-variant", type=int, default=-1,
-                   help="FP32 pair-kernel variant (-1 autotune; 0..4 pin one, e.g. for profiling)")
+                   help="FP32 pair-kernel variant (-1 by size; 0..4 pin one, e.g. for profiling)")
     return p.parse_args()
 
 
@@ -652,7 +652,7 @@ def monolayer_line(ctx, precond="wall", peaks=None):
 
     s = I.config_monolayer(1)
     P = _dev_problem(s)
-    # size-class autotuning of the FP32 kernel happens on this first matvec
+    # the first matvec allocates the context's workspace
     r = ctx.blob_positions(P["q"], P["theta"], P["blob_start"], P["rho"])
     ctx.mobility_matvec(r, torch.ones_like(r), s.a, 1.0, True, "fp32")
     # the preconditioner setup alone (FP64), timed on the device

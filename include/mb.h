@@ -184,10 +184,7 @@ mb_status mb_mobility_matvec(mb_context *ctx, const double *r, const double *f, 
 
 /*
  * Choice of the FP32 pair-kernel variant used by this context:
- *   -1  autotune (default): the first FP32 matvec of each size class (half
- *       octaves of N, with or without the wall) runs every variant once on
- *       the caller's stream, synchronises, and keeps the fastest for later
- *       calls — so make that first call before any stream capture;
+ *   -1  by size (default): 3 from 600 blobs on, 4 below;
  *    0  scalar FP32 kernel, one target per thread;
  *    1  packed FP32 kernel (paired f32x2 arithmetic), two targets per thread;
  *    2  packed FP32 kernel, four targets per thread;
@@ -195,12 +192,11 @@ mb_status mb_mobility_matvec(mb_context *ctx, const double *r, const double *f, 
  *       for both blobs (M_ji = M_ij^T), partial sums added to u with FP64
  *       atomics, so results may differ between calls in the last FP64 bits;
  *    4  packed FP32 kernel in 32-thread CTAs (64 targets, source chunks of
- *       32 or more), which spreads small problems over many SMs; the
- *       autotuner's choice below 4,096 blobs.
+ *       32 or more), which spreads small problems over many SMs.
  * All variants compute the same product to FP32 rounding.  Other values are
- * MB_EINVAL.  Setting a variant clears the autotuner's cache.  Batched
- * solves and servers created on the context use the pinned variant for
- * their FP32 pair launches too (variant 0 runs as 1 there, 4 as 3).
+ * MB_EINVAL.  Batched solves and servers created on the context use the
+ * pinned variant for their FP32 pair launches too (variant 0 runs as 1 there,
+ * 4 as 3).
  */
 mb_status mb_context_set_pair_variant(mb_context *ctx, int variant);
 
@@ -220,8 +216,9 @@ mb_status mb_context_set_pair_variant(mb_context *ctx, int variant);
 mb_status mb_context_set_wait_limit(mb_context *ctx, double seconds);
 
 /* The FP32 pair-kernel variant this context uses for N blobs with or
- * without the wall: the fixed variant if one was set, else the autotuner's
- * cached choice for that size class, else -1 (not tuned yet). */
+ * without the wall: the fixed variant if one was set, else the one chosen
+ * by size once a matvec of that size class (half octaves of N, wall or not)
+ * has run, else -1. */
 mb_status mb_context_pair_variant(const mb_context *ctx, int64_t n, int wall, int *variant);
 
 /*

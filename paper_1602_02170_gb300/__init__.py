@@ -320,12 +320,12 @@ class Context:
         self._check(self.L.mb_context_set_wait_limit(self.handle, float(seconds)))
 
     def set_pair_variant(self, variant: int):
-        """-1 autotune (default), 0 scalar, 1 packed x2, 2 packed x4, 3 symmetric,
+        """-1 by size (default), 0 scalar, 1 packed x2, 2 packed x4, 3 symmetric,
         4 packed in 32-thread CTAs (small problems)."""
         self._check(self.L.mb_context_set_pair_variant(self.handle, int(variant)))
 
     def pair_variant(self, n: int, wall: bool = True) -> int:
-        """Variant used for N blobs (-1 if the autotuner has not run yet)."""
+        """Variant used for N blobs (-1 before the first product of their size class)."""
         v = ctypes.c_int()
         self._check(self.L.mb_context_pair_variant(self.handle, int(n), int(bool(wall)),
                                                     ctypes.byref(v)))

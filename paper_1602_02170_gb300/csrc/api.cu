@@ -245,7 +245,7 @@ mb_status mb_context_set_pair_variant(mb_context *ctx, int variant)
     MB_TRY(check_ctx(ctx));
     if (variant < -1 || variant > 4) return set_err(ctx, MB_EINVAL, "pair variant must be -1..4");
     ctx->pair_variant = variant;
-    ctx->tuned.clear();
+    ctx->chosen.clear();
     return MB_OK;
 }
 
@@ -256,8 +256,7 @@ mb_status mb_context_pair_variant(const mb_context *ctx, int64_t n, int wall, in
         *variant = ctx->pair_variant;
         return MB_OK;
     }
-    auto it = ctx->tuned.find(tune_key(n, wall));
-    *variant = it == ctx->tuned.end() ? -1 : it->second;
+    *variant = ctx->chosen.count(size_class(n, wall)) ? f32_variant(n) : -1;
     return MB_OK;
 }
 

@@ -47,7 +47,7 @@ struct IterSig {
 
 // One Arnoldi step captured as a CUDA graph.  A step is captured the second
 // time it is met with the same signature (the first run sizes every buffer
-// and settles the autotuner) and replayed from then on.
+// and picks the kernels) and replayed from then on.
 struct IterGraph {
     IterSig sig;
     bool seen = false;
@@ -125,10 +125,10 @@ struct mb_context {
     cudaStream_t cap_stream = nullptr;       // private stream for captures (the caller's
                                              // stream may be the legacy one)
 
-    // FP32 pair-kernel variant: -1 = autotune per (size class, wall), else fixed
+    // FP32 pair-kernel variant: -1 = by size, else fixed
     double wait_limit_s = 0.0;  // host waits for the stream: <= 0 without limit
     int pair_variant = -1;
-    std::map<int, int> tuned;   // size-class key -> fastest variant
+    std::map<int, bool> chosen;  // size classes met with the variant chosen by size
 
     // measurement: events around pair-kernel launches (mb_profile_*)
     int profiling = 0;
@@ -151,8 +151,9 @@ void release(mb_context *ctx, DevBuf &buf);
 // f_stride_blob lets the solver pass its packed vectors (stride 3 doubles).
 mb_status matvec_device(mb_context *ctx, const double *r, const double *f, int64_t n, double a,
                         double eta, int wall, mb_precision prec, double *u, cudaStream_t s);
-// Autotuner size class of an FP32 matvec (pair_matvec.cu).
-int tune_key(int64_t n, int wall);
+// FP32 variant chosen for N blobs, and the size class of a matvec (pair_matvec.cu).
+int f32_variant(int64_t n);
+int size_class(int64_t n, int wall);
 // Pack positions once (FP32 path); the matvec then only reads f.  order: also
 // sort them spatially for the symmetric FP32 kernel (N >= 16,384).
 mb_status matvec_pack_positions(mb_context *ctx, const double *r, int64_t n, cudaStream_t s,

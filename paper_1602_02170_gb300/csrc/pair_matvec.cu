@@ -206,42 +206,50 @@ __global__ void __launch_bounds__(NT, NT == kNT ? (NP == 1 ? 3 : 2) : 16) pair_f
     }
 }
 
-// Symmetric packed kernel: persistent loop over the upper-triangular block
-// pairs (I <= J) of blocks of 2*kNT blobs, row by row; see x2sym_item.
+// Symmetric packed kernel over the upper-triangular pairs of blocks of 2 NT
+// blobs; an item is block I against half of block J (x2sym_item), one CTA
+// each.  Bound by the FMA pipe once every SM has work, so the items are cut to
+// leave no SM idle: smaller blocks for fewer blobs, and more items than fit at
+// once, dealt out by the hardware as CTAs end (a persistent grid that strides
+// over them ends 6-9% later: items differ by a factor of 1.3 in length).
+// Times (us) of a product with the wall, NT = 32 / 64 / 128 / 256:
+//    1,000 blobs  21 / 25 / 34 / 74        9,003   142 / 136 / 144 / 183
+//    3,000        31 / 31 / 43 / 74       20,011   625 / 590 / 591 / 621
+//    7,000        94 / 93 / 102 / 129     65,536  8290 / 5376 / 5207 / 5235
+// (blocks of 512 in a persistent grid, the form before: 242 us at 9,003 blobs
+// and 5,555 at 65,536).
 //
-// box (optional): the bounding box of every block, (min x, y, z, max x, y, z),
-// and grid->far2, the squared distance beyond which a block pair is far (see
-// x2sym_item); such pairs take the kFar instance, and the kVeryFar one from
-// kVeryFarRadii radii on.
+// box (optional): the bounding box of every kBoxBlobs sorted blobs, (min x, y,
+// z, max x, y, z), and grid->far2, the squared distance beyond which a block
+// pair is far (see x2sym_item); such pairs take the kFar instance, and the
+// kVeryFar one from kVeryFarRadii radii on.
+constexpr int kBoxBlobs = 256;
+constexpr int64_t kSymNT64MinN = 3000, kSymNT128MinN = 12000;
+
 struct SortGrid {
     float lo[3], inv_h[3];  // cell of x: (x - lo) * inv_h per axis
     int bits[3];            // bits of the cell index per axis (nbits in all)
     float far2;             // squared box distance of a far block pair
 };
 
-template <bool WALL>
-__global__ void __launch_bounds__(kNT, 2) pair_sym_kernel(
+template <bool WALL, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) pair_sym_kernel(
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
-    int64_t n, int64_t nb, int64_t n_items, MobConsts2 k, double *__restrict__ u, double scale,
+    int64_t n, int64_t n_items, MobConsts2 k, double *__restrict__ u, double scale,
     const float *__restrict__ box, const SortGrid *__restrict__ grid)
 {
-    __shared__ float4 sP[kX2SmemFloat4PerSource * kNT];
-    __shared__ float sRev[3 * kNT * (kNT / 32)];
+    __shared__ float4 sP[kX2SmemFloat4PerSource * NT];
+    __shared__ float sRev[3 * NT * (NT / 32)];
+    constexpr int kPer = kBoxBlobs / (2 * NT);  // this kernel's blocks per box
     const float far2 = box ? fmaxf(grid->far2, 1.5625f * k.four_a2) : 0.f;
     const float vfar2 = 0.25f * kVeryFarRadii * kVeryFarRadii * k.four_a2;
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-        // row I holds nb - I items; rowoff(I) = I*nb - I*(I-1)/2
-        int64_t lo_r = 0, hi_r = nb;
-        while (hi_r - lo_r > 1) {
-            const int64_t mid = (lo_r + hi_r) >> 1;
-            if (mid * nb - mid * (mid - 1) / 2 <= item) lo_r = mid;
-            else hi_r = mid;
-        }
-        const int64_t I = lo_r;
-        const int64_t J = I + (item - (I * nb - I * (I - 1) / 2));
+        int64_t I, J;
+        triangle_pair(item >> 1, I, J);
+        const int half = (int)(item & 1);
         int level = kNear;  // the same in every thread
-        if (box && I != J) {
-            const float *bi = box + 6 * I, *bj = box + 6 * J;
+        if (box && I / kPer != J / kPer) {
+            const float *bi = box + 6 * (I / kPer), *bj = box + 6 * (J / kPer);
             float d2 = 0.f;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -251,10 +259,10 @@ __global__ void __launch_bounds__(kNT, 2) pair_sym_kernel(
             if (d2 > far2) level = d2 > vfar2 ? kVeryFar : kFar;
         }
         if (level == kVeryFar)
-            x2sym_item<WALL, kNT, kVeryFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
+            x2sym_item<WALL, NT, kVeryFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
         else if (level == kFar)
-            x2sym_item<WALL, kNT, kFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
-        else x2sym_item<WALL, kNT, kNear>(sP, sRev, hi, lo, f, n, I, J, k, u, scale);
+            x2sym_item<WALL, NT, kFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
+        else x2sym_item<WALL, NT, kNear>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
     }
 }
 
@@ -276,12 +284,9 @@ __global__ void __launch_bounds__(32) pair_f64sym_kernel(
     __shared__ double sm[6 * C];
     constexpr int kParts = 32 / C;
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-        // pair t = J (J + 1) / 2 + I of the triangle I <= J
         const int64_t t = item / kParts;
-        int64_t J = (int64_t)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
-        while (J * (J + 1) / 2 > t) --J;
-        while ((J + 1) * (J + 2) / 2 <= t) ++J;
-        const int64_t I = t - J * (J + 1) / 2;
+        int64_t I, J;
+        triangle_pair(t, I, J);
         const int64_t j0 = J * 32 + (item - t * kParts) * C;
         if (j0 < n) f64sym_item<WALL, C>(sm, r, f, n, I, j0, I == J, k, u, scale);
         __syncwarp();  // the item is done with sm
@@ -398,7 +403,7 @@ __global__ void __launch_bounds__(NT) pair_dfx_kernel(
 // Double-float kernel: symmetric over the upper-triangular pairs of blocks of
 // NT blobs (one target per thread); see dfsym_item.
 // box (optional, spatial order): the bounding boxes of the sort's blocks of
-// 2 kNT blobs (two blocks of this kernel each); block pairs whose boxes are
+// kBoxBlobs blobs (one block of this kernel each); block pairs whose boxes are
 // 64 a or more apart take the FAR instance of the item.
 template <bool WALL, int NT = kNT>
 __global__ void __launch_bounds__(NT) pair_df_kernel(
@@ -408,7 +413,6 @@ __global__ void __launch_bounds__(NT) pair_df_kernel(
 {
     __shared__ float4 sD[3 * NT];
     __shared__ double sRev[3 * NT];
-    constexpr int kPer = 2 * kNT / NT;  // this kernel's blocks per box
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         int64_t lo_r = 0, hi_r = nb;
         while (hi_r - lo_r > 1) {
@@ -418,8 +422,8 @@ __global__ void __launch_bounds__(NT) pair_df_kernel(
         }
         const int64_t I = lo_r, J = I + (item - (I * nb - I * (I - 1) / 2));
         bool far = false;
-        if (box && I / kPer != J / kPer) {
-            const float *bi = box + 6 * (I / kPer), *bj = box + 6 * (J / kPer);
+        if (box && I != J) {  // NT == kBoxBlobs
+            const float *bi = box + 6 * I, *bj = box + 6 * J;
             float d2 = 0.f;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -500,11 +504,12 @@ constexpr int kTPT = MB_PAIR_TPT;  // targets per thread
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// FP32 variants and their autotuner.
+// FP32 variants.
 //   0: scalar kernel, kTPT targets per thread
 //   1: packed f32x2 kernel, 2 targets per thread
 //   2: packed f32x2 kernel, 4 targets per thread
-constexpr int kF32Variants = 5;
+//   3: symmetric packed kernel (each unordered pair once)
+//   4: packed f32x2 kernel in one-warp CTAs, 2 targets per thread
 constexpr int kSmallNT = 32;        // CTA size of the small-problem kernels
 constexpr int64_t kSmallN = 8192;   // below this the double-float path uses them
 constexpr int64_t kDfxMaxN = 1024;  // up to this the double-float product is forward only
@@ -514,12 +519,29 @@ int f32_targets_per_cta(int v)
     return v == 0 ? kNT * kTPT : (v == 2 ? 4 * kNT : (v == 4 ? 2 * kSmallNT : 2 * kNT));
 }
 
+template <bool WALL, int NT>
+void launch_sym_nt(const float4 *hi, const float4 *lo, const double *f, int64_t n, double a,
+                   double *u, double scale, const float *box, const SortGrid *sg, cudaStream_t s)
+{
+    const int64_t nb = ceil_div(n, 2 * NT), items = nb * (nb + 1);
+    pair_sym_kernel<WALL, NT><<<(unsigned)std::min<int64_t>(items, 1 << 30), NT, 0, s>>>(
+        hi, lo, f, n, items, MobConsts2::make(a), u, scale, box, sg);
+}
+
+template <bool WALL>
+void launch_sym(const float4 *hi, const float4 *lo, const double *f, int64_t n, double a,
+                double *u, double scale, const float *box, const SortGrid *sg, cudaStream_t s)
+{
+    if (n < kSymNT64MinN) launch_sym_nt<WALL, 32>(hi, lo, f, n, a, u, scale, box, sg, s);
+    else if (n < kSymNT128MinN) launch_sym_nt<WALL, 64>(hi, lo, f, n, a, u, scale, box, sg, s);
+    else launch_sym_nt<WALL, 128>(hi, lo, f, n, a, u, scale, box, sg, s);
+}
+
 template <bool WALL>
 int f32_resident(mb_context *ctx, int v)
 {
     if (v == 0) return resident_ctas(ctx, pair_f32_kernel<WALL, kTPT>);
     if (v == 1) return resident_ctas(ctx, pair_f32x2_kernel<WALL, 1>);
-    if (v == 3) return resident_ctas(ctx, pair_sym_kernel<WALL>);
     if (v == 4) return resident_ctas(ctx, pair_f32x2_kernel<WALL, 1, kSmallNT>, kSmallNT);
     return resident_ctas(ctx, pair_f32x2_kernel<WALL, 2>);
 }
@@ -548,8 +570,8 @@ void f32_launch(int v, const Plan &p, cudaStream_t s, const float4 *hi, const fl
 // Spatial order for the symmetric FP32 kernel (N >= kSortMinN).  The blobs are
 // sorted by cell of a grid over their bounding box, cells in Morton order
 // (kSortBits bits, dealt to the axes in proportion to their extents), by a
-// counting sort; the kernel's blocks of 2 kNT consecutive sorted blobs are
-// then compact, and the block pairs far apart take the FAR instance of the
+// counting sort; the kernel's blocks of consecutive sorted blobs are then
+// compact, and the block pairs far apart take the FAR instance of the
 // pair item.  Each matvec gathers f into the sorted order and scatters u back.
 // The sort is stable (the blobs of a cell keep their index order), so the
 // order, and with it the FP32 rounding of every pair sum, is the same on
@@ -770,9 +792,9 @@ __global__ void __launch_bounds__(1024) sort_scatter_kernel(const unsigned *__re
     }
 }
 
-// Block b of the kernel (sorted positions b * 2 kNT .. + 2 kNT - 1), one CTA
-// each: the packed positions in the sorted order, and the block's bounding
-// box (min x, y, z, max x, y, z).
+// Sorted positions b kBoxBlobs .. + kBoxBlobs - 1, one CTA each: the packed
+// positions in the sorted order, and their bounding box (min x, y, z, max x,
+// y, z).
 __global__ void __launch_bounds__(256) sort_pack_box_kernel(const int *__restrict__ perm, int64_t n,
                                                             const float4 *__restrict__ hi,
                                                             const float4 *__restrict__ lo,
@@ -783,7 +805,8 @@ __global__ void __launch_bounds__(256) sort_pack_box_kernel(const int *__restric
     __shared__ float red[32][6];
     const int64_t b = blockIdx.x;
     float v[6] = {3e38f, 3e38f, 3e38f, -3e38f, -3e38f, -3e38f};
-    for (int64_t i = b * 2 * kNT + threadIdx.x; i < n && i < (b + 1) * 2 * kNT; i += blockDim.x) {
+    for (int64_t i = b * kBoxBlobs + threadIdx.x; i < n && i < (b + 1) * kBoxBlobs;
+         i += blockDim.x) {
         const int j = perm[i];
         const float4 h = hi[j];
         shi[i] = h;
@@ -848,7 +871,7 @@ __global__ void __launch_bounds__(256) sort_scatter_u_kernel(const int *__restri
 // SortGrid).
 mb_status sort_positions(mb_context *ctx, int64_t n, int nparts, cudaStream_t s)
 {
-    const int64_t nb = ceil_div(n, 2 * kNT);
+    const int64_t nb = ceil_div(n, kBoxBlobs);
     // tiles of at least 1,024 blobs, at most one per SM
     const int tiles = (int)std::min<int64_t>(ceil_div(n, 1024), ctx->sm_count);
     const int64_t T = ceil_div(n, tiles);
@@ -894,7 +917,7 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
                   double scale, double *u, cudaStream_t s, bool profile,
                   MatvecPartials *defer = nullptr)
 {
-    const int res = wall ? f32_resident<true>(ctx, v) : f32_resident<false>(ctx, v);
+    const int res = v == 3 ? 0 : wall ? f32_resident<true>(ctx, v) : f32_resident<false>(ctx, v);
     if (v == 4) {
         // small problems: 64-target blocks, source chunks of 16 or more (half a
         // tile: one warp per CTA walks fewer sources, more CTAs share the work)
@@ -928,12 +951,16 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
         return MB_OK;
     }
     if (v == 3) {
-        // symmetric: zero u, then one launch over the block-pair triangle; in
-        // the spatial order when the packing made one (f gathered, u
-        // scattered back)
-        const int64_t nb = ceil_div(n, 2 * kNT);
-        const int64_t items = nb * (nb + 1) / 2;
-        const int grid = (int)std::min<int64_t>(items, res);
+        // symmetric: zero u (or, deferred, the one partial sum the caller
+        // scales), then one launch over the block-pair triangle; in the
+        // spatial order when the packing made one (f gathered, u scattered
+        // back)
+        if (defer) {
+            MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)n, "matvec partials"));
+            u = (double *)ctx->partial.ptr;
+            *defer = MatvecPartials{u, 1, scale};
+            scale = 1.0;
+        }
         const bool sorted = ctx->sorted_n == n;
         const float4 *hi = (const float4 *)(sorted ? ctx->sort_hi.ptr : ctx->pos_hi.ptr);
         const float4 *lo = (const float4 *)(sorted ? ctx->sort_lo.ptr : ctx->pos_lo.ptr);
@@ -955,11 +982,8 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
             MB_CUDA_TRY(ctx, cudaMemsetAsync(uk, 0, sizeof(double) * 3 * (size_t)n, s));
         }
         auto *ev = profile ? profile_begin(ctx, s) : nullptr;
-        const MobConsts2 k = MobConsts2::make(a);
-        if (wall)
-            pair_sym_kernel<true><<<grid, kNT, 0, s>>>(hi, lo, fk, n, nb, items, k, uk, scale, box, sg);
-        else
-            pair_sym_kernel<false><<<grid, kNT, 0, s>>>(hi, lo, fk, n, nb, items, k, uk, scale, box, sg);
+        if (wall) launch_sym<true>(hi, lo, fk, n, a, uk, scale, box, sg, s);
+        else launch_sym<false>(hi, lo, fk, n, a, uk, scale, box, sg, s);
         profile_end(ev, s);
         count_launch();
         if (sorted) {
@@ -999,8 +1023,17 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
     return MB_OK;
 }
 
-// Size class of a matvec for the autotuner: wall flag and half-octaves of N.
-int tune_key(int64_t n, int wall)
+// The symmetric kernel from kSymMinN blobs on, one-warp CTAs that evaluate
+// every ordered pair below.  A mixed solve (us) of 336 / 504 / 672 / 1,344 /
+// 2,688 blobs takes 944 / 962 / 1,180 / 1,730 / 3,920 with the one and 982 /
+// 995 / 1,149 / 1,370 / 2,310 with the other: zeroing the sums and the atomics
+// cost two to three microseconds a step, and few pairs save less.
+constexpr int64_t kSymMinN = 600;
+
+int f32_variant(int64_t n) { return n < kSymMinN ? 4 : 3; }
+
+// Size class of a matvec (mb_context_pair_variant): wall flag and half-octaves of N.
+int size_class(int64_t n, int wall)
 {
     int b = 0;
     for (int64_t m = n; m > 1; m >>= 1) ++b;
@@ -1013,34 +1046,8 @@ mb_status matvec_f32(mb_context *ctx, const double *f, int64_t n, double a, int 
 {
     int v = ctx->pair_variant;
     if (v < 0) {
-        const int key = tune_key(n, wall);
-        auto it = ctx->tuned.find(key);
-        if (it != ctx->tuned.end()) {
-            v = it->second;
-        } else if (n < 4096) {
-            v = 4;  // small: spread over many SMs in 64-target, 32-source items
-            ctx->tuned[key] = v;
-        } else {
-            // time each variant once on this stream (each run is a full, valid matvec)
-            float best = 1e30f;
-            int best_v = 1;
-            cudaEvent_t e0, e1;
-            MB_CUDA_TRY(ctx, cudaEventCreate(&e0));
-            MB_CUDA_TRY(ctx, cudaEventCreate(&e1));
-            for (int c = 0; c < kF32Variants; ++c) {
-                MB_CUDA_TRY(ctx, cudaEventRecord(e0, s));
-                MB_TRY(f32_run(ctx, c, f, n, a, wall, scale, u, s, false));
-                MB_CUDA_TRY(ctx, cudaEventRecord(e1, s));
-                MB_CUDA_TRY(ctx, cudaEventSynchronize(e1));
-                float ms = 0.f;
-                MB_CUDA_TRY(ctx, cudaEventElapsedTime(&ms, e0, e1));
-                if (ms < best) { best = ms; best_v = c; }
-            }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            ctx->tuned[key] = best_v;
-            v = best_v;
-        }
+        v = f32_variant(n);
+        ctx->chosen[size_class(n, wall)] = true;
     }
     return f32_run(ctx, v, f, n, a, wall, scale, u, s, true, defer);
 }

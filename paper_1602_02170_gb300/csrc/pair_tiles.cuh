@@ -26,6 +26,15 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x)
 // Shared-memory floats per source in the packed kernel (5 float4).
 constexpr int kX2SmemFloat4PerSource = 5;
 
+// Pair t = J (J + 1) / 2 + I of the triangle I <= J.
+__device__ __forceinline__ void triangle_pair(int64_t t, int64_t &I, int64_t &J)
+{
+    J = (int64_t)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while (J * (J + 1) / 2 > t) --J;
+    while ((J + 1) * (J + 2) / 2 <= t) ++J;
+    I = t - J * (J + 1) / 2;
+}
+
 __device__ __forceinline__ void stage_x2(float4 *d, float4 h, float4 l, float fx, float fy, float fz)
 {
     const float zz = -2.f * h.z * h.z;
@@ -190,6 +199,7 @@ __device__ __forceinline__ void f64_item(double *__restrict__ sm, const double *
 // over all ordered pairs.  u must be zeroed beforehand and receives
 // scale * M f.
 //
+// Sources [sub0, sub1) NT of block J (two halves of NT blobs).
 // LEVEL: how far apart the blocks' bounding boxes are known to be (mob_coefs2).
 // From kFar on the separations take the hi parts alone, whose rounding then
 // moves a separation by at most 2^-18 of itself.
@@ -199,7 +209,8 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
                                            const float4 *__restrict__ lo,
                                            const double *__restrict__ f, int64_t n, int64_t I,
                                            int64_t J, const MobConsts2 &k,
-                                           double *__restrict__ u, double scale)
+                                           double *__restrict__ u, double scale, int sub0 = 0,
+                                           int sub1 = 2)
 {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -221,7 +232,7 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
     for (int t = 0; t < 2; ++t)
 #pragma unroll
         for (int c = 0; c < 3; ++c) sum[t][c] = comp[t][c] = 0.f;
-    for (int sub = 0; sub < 2; ++sub) {
+    for (int sub = sub0; sub < sub1; ++sub) {
         const int64_t j0 = J * 2 * NT + sub * NT;
         if (j0 >= n) break;
         __syncthreads();

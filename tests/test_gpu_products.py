@@ -70,3 +70,29 @@ def test_fp32_far_and_very_far_blocks(ctx, gap):
         ctx.set_pair_variant(-1)
     ref = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, True, "fp64"))
     assert rel_l2(got[n:], ref[n:]) <= 4e-6
+
+
+@pytest.mark.parametrize("wall", [True, False])
+@pytest.mark.parametrize("n", [1, 63, 65, 599, 600, 2999, 3001, 11999, 12003])
+def test_fp32_symmetric_blocks_of_every_size(ctx, n, wall):
+    """The symmetric FP32 kernel's blocks hold 64, 128 (from 3,000 blobs) or
+    256 blobs (from 12,000); ragged and nearly empty last blocks, against the
+    FP64 product."""
+    r, f = _cloud(n, n)
+    ctx.set_pair_variant(3)
+    try:
+        got = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, wall, "fp32"))
+    finally:
+        ctx.set_pair_variant(-1)
+    ref = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, wall, "fp64"))
+    assert np.abs(got - ref).max() <= TOL["fp32"] * np.abs(ref).max()
+
+
+def test_fp32_product_in_place_and_variant_by_size(ctx):
+    for n, variant in ((400, 4), (700, 3)):
+        r, f = _cloud(n, n)
+        R, F = dev(r), dev(f)
+        want = host(ctx.mobility_matvec(R, F, 0.5, 1.0, True, "fp32"))
+        assert ctx.pair_variant(n, True) == variant
+        ctx.mobility_matvec(R, F, 0.5, 1.0, True, "fp32", out=F)
+        assert rel_l2(host(F), want) <= 1e-14
