@@ -3,9 +3,7 @@
 // the FP32 pipes.  Built from the classic error-free transformations:
 // Knuth's two-sum (the exact rounding error of a + b), the fast two-sum of
 // Dekker for |a| >= |b|, and the exact product error of a * b obtained with a
-// fused multiply-add.  The reciprocal square root takes the FP32 estimate and
-// one Newton step y <- y + y (1 - x y^2) / 2, with the residual 1 - x y^2
-// formed from exact products, which doubles the number of correct bits.
+// fused multiply-add.
 //
 // GB300 runs FP64 at a small fraction of its FP32 rate; the pair kernel in
 // double-float reaches FP64-class accuracy for the refinement residuals of
@@ -15,6 +13,15 @@
 #include <cuda_runtime.h>
 
 namespace mb {
+
+// 1/sqrt(x) in FP32 for normal x: the hardware estimate without the scaling
+// of denormal arguments that rsqrtf() adds.
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 
 struct dfl {
     float hi, lo;
@@ -89,62 +96,102 @@ __device__ __forceinline__ dfl &operator+=(dfl &a, dfl b)
     return a;
 }
 
-// Products and sums with an FP32 operand c (a constant exact in FP32, or a
-// value known to have no low part): the terms of c's absent low part are
-// dropped.  a * c in 3 operations; a * 2^k exactly in 2; a + c in 7 (the
-// sloppy form above with b.lo = 0).
-__device__ __forceinline__ dfl mulf(dfl a, float c)
-{
-    const float p = a.hi * c;
-    float e = fmaf(a.hi, c, -p);
-    e = fmaf(a.lo, c, e);
-    return dfl(p, e);
-}
-
-__device__ __forceinline__ dfl mul_pow2(dfl a, float c) { return dfl(a.hi * c, a.lo * c); }
-
-__device__ __forceinline__ dfl addf(dfl a, float c)
-{
-    const dfl s = two_sum(a.hi, c);
-    return dfl(s.hi, s.lo + a.lo);
-}
-
-// y^2 of an FP32 value as an exact double-float
-__device__ __forceinline__ dfl sqf(float y)
-{
-    const float p = y * y;
-    return dfl(p, fmaf(y, y, -p));
-}
-
-__device__ __forceinline__ bool operator<(dfl a, dfl b)
-{
-    return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
-}
-
-__device__ __forceinline__ dfl mb_max(dfl a, dfl b) { return a < b ? b : a; }
-
-__device__ __forceinline__ dfl mb_rsqrt(dfl x)
-{
-    x = fast_two_sum(x.hi, x.lo);  // the FP32 estimate needs the normalised hi
-    const float y0 = rsqrtf(x.hi);
-    // r = 1 - x y0^2 (about 2^-22) to FP32 accuracy: y0^2 = s + t exactly,
-    // x_hi s = p + e exactly, and 1 - p is exact (p is within 2^-21 of 1)
-    const float s = y0 * y0, t = fmaf(y0, y0, -s);
-    const float p = x.hi * s, e = fmaf(x.hi, s, -p);
-    const float r = ((1.f - p) - e) - fmaf(x.hi, t, x.lo * s);
-    // y = y0 + y0 r / 2
-    return fast_two_sum(y0, (0.5f * y0) * r);
-}
-
-// Accumulation without renormalisation (the sloppy addition): for running
-// sums that are renormalised, or converted to double, within a few dozen
-// terms, so that lo stays within a few dozen ulp of hi.
-__device__ __forceinline__ void acc_add(dfl &a, dfl b) { a = a + b; }
-__device__ __forceinline__ void acc_add(float &a, float b) { a += b; }
-__device__ __forceinline__ void acc_add(double &a, double b) { a += b; }
-__device__ __forceinline__ void renorm(dfl &a) { a = fast_two_sum(a.hi, a.lo); }
-
 __device__ __forceinline__ double to_double(dfl a) { return (double)a.hi + (double)a.lo; }
-__device__ __forceinline__ float hi_part(dfl a) { return a.hi; }
+
+// ---------------------------------------------------------------------------
+// Two double-float values in the halves of float2s.  One paired instruction
+// does the work of two, so the FMA pipe and not the issue of instructions
+// bounds code written with these (negated operands cost nothing).
+__device__ __forceinline__ float2 splat2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+struct dfl2 {
+    float2 hi, lo;
+
+    __host__ __device__ dfl2() : hi{0.f, 0.f}, lo{0.f, 0.f} {}
+    __host__ __device__ dfl2(float2 h, float2 l) : hi(h), lo(l) {}
+    // the same value in both halves
+    __host__ __device__ dfl2(dfl a) : hi{a.hi, a.hi}, lo{a.lo, a.lo} {}
+};
+
+__device__ __forceinline__ dfl2 two_sum(float2 a, float2 b)
+{
+    const float2 s = add2(a, b), bb = sub2(s, a);
+    return dfl2(s, add2(sub2(a, sub2(s, bb)), sub2(b, bb)));
+}
+
+__device__ __forceinline__ dfl2 fast_two_sum(float2 a, float2 b)
+{
+    const float2 s = add2(a, b);
+    return dfl2(s, sub2(b, sub2(s, a)));
+}
+
+// Sums and products as for dfl: unnormalised (8 and 4 instructions);
+// subtraction renormalises (11).
+__device__ __forceinline__ dfl2 operator+(dfl2 a, dfl2 b)
+{
+    const dfl2 s = two_sum(a.hi, b.hi);
+    return dfl2(s.hi, add2(s.lo, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ dfl2 operator-(dfl2 a) { return dfl2(neg2(a.hi), neg2(a.lo)); }
+__device__ __forceinline__ dfl2 operator-(dfl2 a, dfl2 b)
+{
+    const dfl2 s = two_sum(a.hi, neg2(b.hi));
+    return fast_two_sum(s.hi, add2(s.lo, sub2(a.lo, b.lo)));
+}
+__device__ __forceinline__ dfl2 operator*(dfl2 a, dfl2 b)
+{
+    const float2 p = mul2(a.hi, b.hi);
+    return dfl2(p, fma2(a.lo, b.hi, fma2(a.hi, b.lo, fma2(a.hi, b.hi, neg2(p)))));
+}
+// a + b for |a| >= |b| (5), a c for c exact in FP32 (3), a c for c a power of
+// two (2), a + c (7)
+__device__ __forceinline__ dfl2 add_ordered(dfl2 a, dfl2 b)
+{
+    const dfl2 s = fast_two_sum(a.hi, b.hi);
+    return dfl2(s.hi, add2(s.lo, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ dfl2 mulf(dfl2 a, float c)
+{
+    const float2 c2 = splat2(c), p = mul2(a.hi, c2);
+    return dfl2(p, fma2(a.lo, c2, fma2(a.hi, c2, neg2(p))));
+}
+__device__ __forceinline__ dfl2 mul_pow2(dfl2 a, float c)
+{
+    return dfl2(mul2(a.hi, splat2(c)), mul2(a.lo, splat2(c)));
+}
+__device__ __forceinline__ dfl2 addf(dfl2 a, float c)
+{
+    const dfl2 s = two_sum(a.hi, splat2(c));
+    return dfl2(s.hi, add2(s.lo, a.lo));
+}
+// a + c for c below an ulp or so of what a is added to next: into lo (1)
+__device__ __forceinline__ dfl2 add_lo(dfl2 a, float2 c) { return dfl2(a.hi, add2(a.lo, c)); }
+__device__ __forceinline__ void renorm(dfl2 &a) { a = fast_two_sum(a.hi, a.lo); }
+
+// x^-1/2: the FP32 estimate y0 of x.hi and one step of Householder's cubic
+// iteration y0 + y0 r (1/2 + 3/8 r), r = 1 - x y0^2 formed as an FP32 number
+// from exact products (y0^2 = s + t, x_hi s = p + e; 1 - p is exact, p being
+// within 2^-20 of 1).  x may be unnormalised: its lo part enters r, and what
+// it adds to r (a few 2^-24) leaves a truncation error far below 2^-48.
+__device__ __forceinline__ dfl2 rsqrt_df(dfl2 x)
+{
+    const float2 y0 = make_float2(rsqrt_ftz(x.hi.x), rsqrt_ftz(x.hi.y));
+    const float2 s = mul2(y0, y0), t = fma2(y0, y0, neg2(s));
+    const float2 p = mul2(x.hi, s), e = fma2(x.hi, s, neg2(p));
+    const float2 q = fma2(x.hi, t, mul2(x.lo, s));
+    const float2 r = sub2(sub2(sub2(splat2(1.f), p), e), q);
+    return fast_two_sum(y0, mul2(y0, mul2(r, fma2(r, splat2(0.375f), splat2(0.5f)))));
+}
+
+// Sum of both halves in FP64.
+__device__ __forceinline__ double sum_halves(dfl2 a)
+{
+    return ((double)a.hi.x + (double)a.hi.y) + ((double)a.lo.x + (double)a.lo.y);
+}
 
 }  // namespace mb

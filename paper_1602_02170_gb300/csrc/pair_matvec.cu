@@ -351,79 +351,91 @@ __global__ void refine_blobs_kernel(const double *__restrict__ r, const double *
     }
 }
 
-// Double-float, forward only, for the smallest problems: blocks of kSmallNT
-// targets (one per thread) against source chunks of kSmallNT / 2, every
-// ordered pair evaluated (the forward half of pair_sym_rg; the reverse half
-// is dead code for the compiler), the block's sums added to u (zeroed) with
-// FP64 atomics.  Twice the pair evaluations of the symmetric kernel, in
-// several times as many one-warp CTAs: a few hundred blobs fill the GPU.
-template <bool WALL, int NT>
-__global__ void __launch_bounds__(NT) pair_dfx_kernel(
+// Double-float, forward only, for the smallest problems: 32 targets (one per
+// lane) against source chunks of 16, two sources at once in the halves of the
+// packed arithmetic, every ordered pair evaluated; the chunk's sums are added
+// to u (zeroed) with FP64 atomics.  Twice the pair evaluations of the symmetric
+// kernel, in several times as many one-warp CTAs with a quarter of the steps.
+constexpr int kDfxChunk = 16;
+
+template <bool WALL>
+__global__ void __launch_bounds__(32) pair_dfx_kernel(
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
-    int64_t n, int64_t chunk, int n_tblocks, int64_t n_items, PairConsts<dfl> k,
-    double *__restrict__ u, double scale)
+    int64_t n, MobConstsDf k, double *__restrict__ u, double scale)
 {
-    __shared__ float4 sD[3 * NT];
-    for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const int tb = (int)(item % n_tblocks);
-        const int64_t j0 = (item / n_tblocks) * chunk;
-        const int64_t j1 = j0 + chunk < n ? j0 + chunk : n;
-        const int64_t i = (int64_t)tb * NT + threadIdx.x;
-        const int64_t ic = i < n ? i : n - 1;
-        const float4 th = hi[ic], tl = lo[ic];
-        const dfl xi(th.x, tl.x), yi(th.y, tl.y), zi(th.z, tl.z);
-        __syncthreads();  // the previous item is done with sD
-        if (j0 + threadIdx.x < j1) {
-            const int64_t j = j0 + threadIdx.x;
-            const float4 h = hi[j], l = lo[j];
-            const dfl fx(f[3 * j]), fy(f[3 * j + 1]), fz(f[3 * j + 2]);
-            float4 *d = sD + 3 * threadIdx.x;
-            d[0] = make_float4(h.x, l.x, h.y, l.y);
-            d[1] = make_float4(h.z, l.z, fx.hi, fx.lo);
-            d[2] = make_float4(fy.hi, fy.lo, fz.hi, fz.lo);
+    // source pair p: x, y, z, fx, fy, fz, -2 z^2, each (hi, hi', lo, lo')
+    __shared__ float4 sD[7 * kDfxChunk / 2];
+    const int lane = threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane, ic = i < n ? i : n - 1;
+    const int64_t j0 = (int64_t)blockIdx.y * kDfxChunk;
+    const float4 th = hi[ic], tl = lo[ic];
+    const dfl2 xi(dfl(th.x, tl.x)), yi(dfl(th.y, tl.y)), zi(dfl(th.z, tl.z));
+    if (lane < kDfxChunk) {
+        const int64_t j = j0 + lane, jc = j < n ? j : n - 1;
+        const float4 h = hi[jc], l = lo[jc];
+        const double z = (double)h.z + (double)l.z;
+        const dfl v[7] = {dfl(h.x, l.x), dfl(h.y, l.y), dfl(h.z, l.z),
+                          j < n ? dfl(f[3 * jc]) : dfl(), j < n ? dfl(f[3 * jc + 1]) : dfl(),
+                          j < n ? dfl(f[3 * jc + 2]) : dfl(), dfl(-2.0 * z * z)};
+        float *d = (float *)sD + 4 * 7 * (lane >> 1) + (lane & 1);
+#pragma unroll
+        for (int c = 0; c < 7; ++c) {
+            d[4 * c] = v[c].hi;
+            d[4 * c + 2] = v[c].lo;
         }
-        __syncthreads();
-        dfl ux, uy, uz, vx, vy, vz;
-        const int cnt = (int)(j1 - j0);
-        for (int s = 0; s < cnt; ++s) {
-            const float4 A = sD[3 * s], B = sD[3 * s + 1], C = sD[3 * s + 2];
-            const dfl zj(B.x, B.y);
-            pair_sym_rg<WALL, dfl>(xi - dfl(A.x, A.y), yi - dfl(A.z, A.w), zi - zj, zi, zj,
-                                   dfl(B.z, B.w), dfl(C.x, C.y), dfl(C.z, C.w), dfl(), dfl(), dfl(),
-                                   k, ux, uy, uz, vx, vy, vz);
-        }
-        if (i < n) {
-            atomicAdd(u + 3 * i, scale * to_double(ux));
-            atomicAdd(u + 3 * i + 1, scale * to_double(uy));
-            atomicAdd(u + 3 * i + 2, scale * to_double(uz));
-        }
+    }
+    __syncwarp();
+    auto src = [&](int p, int c) {
+        const float4 q = sD[7 * p + c];
+        return dfl2(make_float2(q.x, q.y), make_float2(q.z, q.w));
+    };
+    dfl2 ux, uy, uz;
+#pragma unroll 1
+    for (int p = 0; p < kDfxChunk / 2; ++p) {
+        const dfl2 zj = src(p, 2);
+        const dfl2 dx = xi - src(p, 0), dy = yi - src(p, 1), dz = zi - zj;
+        const Mob<dfl2> m = mob_coefs_df<WALL, false>(dx, dy, dz, zi, zj, src(p, 6), k);
+        mob_apply_df<WALL>(m, dx, dy, dz, src(p, 3), src(p, 4), src(p, 5), ux, uy, uz);
+    }
+    if (i < n) {
+        atomicAdd(u + 3 * i, scale * sum_halves(ux));
+        atomicAdd(u + 3 * i + 1, scale * sum_halves(uy));
+        atomicAdd(u + 3 * i + 2, scale * sum_halves(uz));
     }
 }
 
 // Double-float kernel: symmetric over the upper-triangular pairs of blocks of
-// NT blobs (one target per thread); see dfsym_item.
-// box (optional, spatial order): the bounding boxes of the sort's blocks of
-// kBoxBlobs blobs (one block of this kernel each); block pairs whose boxes are
-// 64 a or more apart take the FAR instance of the item.
-template <bool WALL, int NT = kNT>
-__global__ void __launch_bounds__(NT) pair_df_kernel(
+// 2 NT blobs, an item being block I against half of block J (dfsym_item), one
+// CTA each as in pair_sym_kernel.  Bound by the FMA pipe (a pair takes about
+// 600 FP32 operations): packed two targets to an instruction it no longer
+// waits for the issue of instructions as the scalar form did, and twelve warps
+// an SM (168 registers a thread) are enough.
+// Times (us) of a product with the wall, forward only / NT = 32 / NT = 128,
+// and of the scalar form before:
+//    336 blobs  20 / 43 / 127, 23       9,003   - / 823 / 895, 1,222
+//    1,000      37 / 45 / 125, 39      20,011   - / 3,771 / 3,830, 5,287
+//    1,400      53 / 43 / 124, 50      65,536   - / 38,600 / 38,100, 50,050
+constexpr int64_t kDfxMaxN = 1100;       // up to this the product is forward only
+constexpr int64_t kDfNT128MinN = 24000;
+
+// box (optional, spatial order): the bounding boxes of every kBoxBlobs sorted
+// blobs; block pairs whose boxes are 64 a or more apart take the FAR instance
+// of the item.
+template <bool WALL, int NT>
+__global__ void __launch_bounds__(NT, 384 / NT) pair_df_kernel(
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
-    int64_t n, int64_t nb, int64_t n_items, PairConsts<dfl> k, double *__restrict__ u,
-    double scale, const float *__restrict__ box, float far2)
+    int64_t n, int64_t n_items, MobConstsDf k, double *__restrict__ u, double scale,
+    const float *__restrict__ box, float far2)
 {
-    __shared__ float4 sD[3 * NT];
-    __shared__ double sRev[3 * NT];
+    __shared__ float4 sD[7 * NT];
+    __shared__ double sRev[3 * NT * (NT / 32)];
+    constexpr int kPer = kBoxBlobs / (2 * NT);  // this kernel's blocks per box
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-        int64_t lo_r = 0, hi_r = nb;
-        while (hi_r - lo_r > 1) {
-            const int64_t mid = (lo_r + hi_r) >> 1;
-            if (mid * nb - mid * (mid - 1) / 2 <= item) lo_r = mid;
-            else hi_r = mid;
-        }
-        const int64_t I = lo_r, J = I + (item - (I * nb - I * (I - 1) / 2));
+        int64_t I, J;
+        triangle_pair(item >> 1, I, J);
         bool far = false;
-        if (box && I != J) {  // NT == kBoxBlobs
-            const float *bi = box + 6 * I, *bj = box + 6 * J;
+        if (box && I / kPer != J / kPer) {
+            const float *bi = box + 6 * (I / kPer), *bj = box + 6 * (J / kPer);
             float d2 = 0.f;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -432,8 +444,10 @@ __global__ void __launch_bounds__(NT) pair_df_kernel(
             }
             far = d2 > far2;  // the same in every thread
         }
-        if (far) dfsym_item<WALL, NT, true>(sD, sRev, hi, lo, f, n, I, J, k, u, scale);
-        else dfsym_item<WALL, NT, false>(sD, sRev, hi, lo, f, n, I, J, k, u, scale);
+        const int half = (int)(item & 1);
+        if (far) dfsym_item<WALL, NT, true>(sD, sRev, hi, lo, f, n, I, J, half, k, u, scale);
+        else dfsym_item<WALL, NT, false>(sD, sRev, hi, lo, f, n, I, J, half, k, u, scale);
+        __syncthreads();  // the item is done with sRev
     }
 }
 
@@ -511,8 +525,6 @@ constexpr int kTPT = MB_PAIR_TPT;  // targets per thread
 //   3: symmetric packed kernel (each unordered pair once)
 //   4: packed f32x2 kernel in one-warp CTAs, 2 targets per thread
 constexpr int kSmallNT = 32;        // CTA size of the small-problem kernels
-constexpr int64_t kSmallN = 8192;   // below this the double-float path uses them
-constexpr int64_t kDfxMaxN = 1024;  // up to this the double-float product is forward only
 
 int f32_targets_per_cta(int v)
 {
@@ -1104,6 +1116,27 @@ void launch_f64sym(mb_context *ctx, const double *r, const double *f, int64_t n,
     else launch_f64sym_c<WALL, 4>(r, f, n, pairs, a, u, scale, s);
 }
 
+template <bool WALL, int NT>
+void launch_df_nt(const float4 *hi, const float4 *lo, const double *f, int64_t n, double a,
+                  double *u, double scale, const float *box, cudaStream_t s)
+{
+    const int64_t nb = ceil_div(n, 2 * NT), items = nb * (nb + 1);
+    const float dfar = (float)(64.0 * a);
+    pair_df_kernel<WALL, NT><<<(unsigned)std::min<int64_t>(items, 1 << 30), NT, 0, s>>>(
+        hi, lo, f, n, items, MobConstsDf::make(a), u, scale, box, dfar * dfar);
+}
+
+template <bool WALL>
+void launch_df(const float4 *hi, const float4 *lo, const double *f, int64_t n, double a, double *u,
+               double scale, const float *box, cudaStream_t s)
+{
+    if (n <= kDfxMaxN)
+        pair_dfx_kernel<WALL><<<dim3((unsigned)ceil_div(n, 32), (unsigned)ceil_div(n, kDfxChunk)),
+                                32, 0, s>>>(hi, lo, f, n, MobConstsDf::make(a), u, scale);
+    else if (n < kDfNT128MinN) launch_df_nt<WALL, 32>(hi, lo, f, n, a, u, scale, box, s);
+    else launch_df_nt<WALL, 128>(hi, lo, f, n, a, u, scale, box, s);
+}
+
 mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64_t n, double a,
                         double eta, int wall, mb_precision prec, double *u, cudaStream_t s,
                         MatvecPartials *defer)
@@ -1112,24 +1145,12 @@ mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64
     if (defer) *defer = MatvecPartials{};
     if (prec == MB_FP32_KAHAN) return matvec_f32(ctx, f, n, a, wall, scale, u, s, defer);
     if (prec == MB_DF64) {
-        // symmetric double-float kernel: zero u, one launch over the block-pair
-        // triangle (32-blob blocks for small problems, so that they spread)
-        const bool small = n < kSmallN;
-        const int nt = small ? kSmallNT : kNT;
-        const int res = small ? (wall ? resident_ctas(ctx, pair_df_kernel<true, kSmallNT>, kSmallNT)
-                                      : resident_ctas(ctx, pair_df_kernel<false, kSmallNT>, kSmallNT))
-                              : (wall ? resident_ctas(ctx, pair_df_kernel<true>)
-                                      : resident_ctas(ctx, pair_df_kernel<false>));
-        const int64_t nb = ceil_div(n, nt);
-        const int64_t items = nb * (nb + 1) / 2;
-        const int grid = (int)std::min<int64_t>(items, res);
-        // in the spatial order when the packing made one (f gathered, u
-        // scattered back): far block pairs take the cheaper FAR item
-        const bool sorted = !small && ctx->sorted_n == n;
+        // zero u, then one launch; in the spatial order when the packing made
+        // one (f gathered, u scattered back)
+        const bool sorted = ctx->sorted_n == n;
         const float4 *hi = (const float4 *)(sorted ? ctx->sort_hi.ptr : ctx->pos_hi.ptr);
         const float4 *lo = (const float4 *)(sorted ? ctx->sort_lo.ptr : ctx->pos_lo.ptr);
         const float *box = sorted ? (const float *)ctx->sort_box.ptr : nullptr;
-        const float dfar = (float)(64.0 * a);
         const double *fk = f;
         double *uk = u;
         const int gv = (int)std::min<int64_t>(ceil_div(n, 256), 8 * (int64_t)ctx->sm_count);
@@ -1146,32 +1167,8 @@ mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64
             MB_CUDA_TRY(ctx, cudaMemsetAsync(u, 0, sizeof(double) * 3 * (size_t)n, s));
         }
         auto *ev = profile_begin(ctx, s);
-        const PairConsts<dfl> k = PairConsts<dfl>::make(a);
-        if (n <= kDfxMaxN) {
-            // the smallest problems: every ordered pair, many one-warp CTAs
-            const int rx = wall ? resident_ctas(ctx, pair_dfx_kernel<true, kSmallNT>, kSmallNT)
-                                : resident_ctas(ctx, pair_dfx_kernel<false, kSmallNT>, kSmallNT);
-            const Plan px = make_plan(n, kSmallNT, rx, 1024, kSmallNT / 2, kSmallNT / 2);
-            if (wall)
-                pair_dfx_kernel<true, kSmallNT><<<px.grid, kSmallNT, 0, s>>>(hi, lo, fk, n, px.chunk,
-                                                                   px.n_tblocks, px.items, k, uk,
-                                                                   scale);
-            else
-                pair_dfx_kernel<false, kSmallNT><<<px.grid, kSmallNT, 0, s>>>(hi, lo, fk, n, px.chunk,
-                                                                    px.n_tblocks, px.items, k, uk,
-                                                                    scale);
-        } else if (small && wall)
-            pair_df_kernel<true, kSmallNT><<<grid, kSmallNT, 0, s>>>(hi, lo, fk, n, nb, items, k, uk,
-                                                                    scale, nullptr, 0.f);
-        else if (small)
-            pair_df_kernel<false, kSmallNT><<<grid, kSmallNT, 0, s>>>(hi, lo, fk, n, nb, items, k,
-                                                                     uk, scale, nullptr, 0.f);
-        else if (wall)
-            pair_df_kernel<true><<<grid, kNT, 0, s>>>(hi, lo, fk, n, nb, items, k, uk, scale, box,
-                                                      dfar * dfar);
-        else
-            pair_df_kernel<false><<<grid, kNT, 0, s>>>(hi, lo, fk, n, nb, items, k, uk, scale, box,
-                                                       dfar * dfar);
+        if (wall) launch_df<true>(hi, lo, fk, n, a, uk, scale, box, s);
+        else launch_df<false>(hi, lo, fk, n, a, uk, scale, box, s);
         profile_end(ev, s);
         count_launch();
         if (sorted) {

@@ -333,192 +333,103 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
             atomicAdd(u + 3 * ib + c, scale * ((double)sum[1][c] - (double)comp[1][c]));
 }
 
-// FP64 forms of the FP32-operand operations of df32.cuh, so that the
-// regrouped pair formula below serves FP64 and double-float alike.
-__device__ __forceinline__ double mulf(double a, float c) { return a * (double)c; }
-__device__ __forceinline__ double mul_pow2(double a, float c) { return a * (double)c; }
-__device__ __forceinline__ double addf(double a, float c) { return a + (double)c; }
-
-// pair_sym (both directions of one unordered pair) for FP64 and
-// double-float operands, with the wall polynomials regrouped so that
-// constants exact in FP32 (2, 4, 6, 10, 12, 20, ...) take the cheaper
-// FP32-operand products of df32.cuh and the factors of 1/3 are applied to
-// three shared monomials once:
-//   T1 = E t2,  t4_3 = t4 / 3,  t2_3 = t2 / 3,  T2_3 = E t4 / 3,
-//   f1 = 2 (T1 - p + t4_3 - t2_3) - 10 T2_3 - 1
-//   f2 = F2 - 1,  F2 = 2 (3 p - 5 T1 + t2) + 10 (7 T2_3 - t4_3)
-//   f3 = 2 hs + e3 (20 t4_3 - 2 F2)
-//   f4 = 2 hs - 20 e3 t4_3
-//   f5 = 4 (15 T2_3 - 2 t4_3 - hs^2 - T1)
-// (the f1..f5 of rpy_wall.cuh term by term; the bracket of f3,
-// t2 (20E - 4) + t4 (40/3 - 140E/3) - 12p, equals 20 t4 / 3 - 2 (f2 + 1)),
-// and f2 / rho^2, f3 / rho, f4 / rho formed once for both directions as in
-// pair_sym2.
-//
-// FAR (double-float, block pairs whose boxes are at least 64 a apart, so
-// that t4 = (a / rho)^4 < 2^-24 and no pair overlaps): the terms carrying t4
-// are summed in FP32 and added to the double-float rest once per
-// polynomial; their rounding is then below 2^-24 t4 of the polynomial,
-// under the double-float rounding of the other terms.
-template <bool WALL, typename T, bool FAR = false>
-__device__ __forceinline__ void pair_sym_rg(T dx, T dy, T dz, T zi, T zj, T fx, T fy, T fz, T gx,
-                                            T gy, T gz, const PairConsts<T> &k, T &ux, T &uy,
-                                            T &uz, T &vx, T &vy, T &vz)
-{
-    const T dxy2 = dx * dx + dy * dy;
-    const T r2 = mb_max(dz * dz + dxy2, k.tiny);
-    const T inv = mb_rsqrt(r2);
-    const T inv2 = inv * inv;
-    T C = inv * (k.c1 + k.c2 * inv2);
-    T D = inv * inv2 * (k.c3 + k.c4 * inv2);
-    if (!FAR && r2 < k.four_a2) {
-        C = T(1) - k.k1 * (r2 * inv);
-        D = k.k2 * inv;
-    }
-    const T rf_xy = dx * fx + dy * fy;
-    const T g = D * (rf_xy + dz * fz);
-    const T rb_xy = dx * gx + dy * gy;
-    const T gb = D * (rb_xy + dz * gz);
-    if (!WALL) {
-        acc_add(ux, C * fx + g * dx);
-        acc_add(uy, C * fy + g * dy);
-        acc_add(uz, C * fz + g * dz);
-        acc_add(vx, C * gx + gb * dx);
-        acc_add(vy, C * gy + gb * dy);
-        acc_add(vz, C * gz + gb * dz);
-        return;
-    }
-    constexpr T third(1.0 / 3.0);
-    const T R3 = zi + zj;
-    const T invR = mb_rsqrt(R3 * R3 + dxy2);
-    const T invR2 = invR * invR;
-    const T hs = zj * invR;
-    const T ht = zi * invR;
-    const T e3 = hs + ht;
-    const T E = e3 * e3;
-    const T t2 = k.a2 * invR2;
-    const T p = hs * ht;
-    const T T1 = E * t2;
-    const T t2_3 = t2 * third;
-    const T hs2 = mul_pow2(hs, 2.f);
-    T f1, F2, f3, f4, f5;
-    if constexpr (FAR) {
-        // the t4 terms in FP32 (t4 / 3, E t4 / 3 from the high parts)
-        const float t4_3f = hi_part(t2) * hi_part(t2) * (1.f / 3.f);
-        const float T2_3f = hi_part(E) * t4_3f, e3t4_3f = hi_part(e3) * t4_3f;
-        f1 = addf(addf(mul_pow2(T1 + (-p) + (-t2_3), 2.f), -1.f), 2.f * t4_3f - 10.f * T2_3f);
-        F2 = addf(mul_pow2(mulf(p, 3.f) + mulf(T1, -5.f) + t2, 2.f), 10.f * (7.f * T2_3f - t4_3f));
-        f3 = addf(hs2 + e3 * mul_pow2(F2, -2.f), 20.f * e3t4_3f);
-        f4 = addf(hs2, -20.f * e3t4_3f);
-        f5 = addf(mul_pow2((-(hs * hs)) + (-T1), 4.f), 4.f * (15.f * T2_3f - 2.f * t4_3f));
-    } else {
-        const T t4 = t2 * t2;
-        const T t4_3 = t4 * third;
-        const T T2_3 = E * t4_3;
-        f1 = addf(mul_pow2(T1 + (-p) + t4_3 + (-t2_3), 2.f) + mulf(T2_3, -10.f), -1.f);
-        F2 = mul_pow2(mulf(p, 3.f) + mulf(T1, -5.f) + t2, 2.f) +
-             mulf(mulf(T2_3, 7.f) + (-t4_3), 10.f);
-        f3 = hs2 + e3 * (mulf(t4_3, 20.f) + mul_pow2(F2, -2.f));
-        f4 = hs2 + mulf(e3 * t4_3, -20.f);
-        f5 = mul_pow2(mulf(T2_3, 15.f) + mul_pow2(t4_3, -2.f) + (-(hs * hs)) + (-T1), 4.f);
-    }
-    const T f2 = addf(F2, -1.f);
-    const T s = k.sw * invR;
-    const T Cx = C + s * f1;
-    const T A2 = f2 * invR2;
-    const T A3 = f3 * invR;
-    const T A4 = f4 * invR;
-    // forward: M_ij f_j
-    const T RF = rf_xy + R3 * fz;
-    const T gw = A2 * RF + A3 * fz;
-    const T kz = A4 * RF + f5 * fz;
-    const T Gx = g + s * gw;
-    acc_add(ux, Cx * fx + Gx * dx);
-    acc_add(uy, Cx * fy + Gx * dy);
-    acc_add(uz, Cx * fz + g * dz + s * (gw * R3 + kz));
-    // reverse: M_ij^T f_i (f3 and f4 exchange roles)
-    const T RB = rb_xy + R3 * gz;
-    const T gwb = A2 * RB + A4 * gz;
-    const T kzb = A3 * RB + f5 * gz;
-    const T Gb = gb + s * gwb;
-    acc_add(vx, Cx * gx + Gb * dx);
-    acc_add(vy, Cx * gy + Gb * dy);
-    acc_add(vz, Cx * gz + gb * dz + s * (gwb * R3 + kzb));
-}
-
-// Symmetric double-float item over block pair (I, J), I <= J, blocks of NT
-// blobs, one target per thread; the rotating reverse accumulators of
-// x2sym_item in double-float.  Sources are staged as three float4 (x_hi,
-// x_lo, y_hi, y_lo), (z_hi, z_lo, fx_hi, fx_lo), (fy_hi, fy_lo, fz_hi,
-// fz_lo): a 48-byte stride, so the rotated reads stay conflict-free.
-// sRev holds NT * 3 doubles: each warp adds its per-source sums with shared-
-// memory atomics.  u must be zeroed and receives scale * M f.
+// Symmetric double-float item over half of block pair (I, J), I <= J, blocks
+// of 2 NT blobs: the scheme of x2sym_item (two targets per thread, rotating
+// reverse sums) in packed double-float.  Sources are staged as seven float4
+// (x, y, z, fx, fy, fz, -2 z^2, each hi, hi, lo, lo; the 112-byte stride keeps
+// the rotated reads conflict-free) of NT sources in sD; sRev holds
+// 3 NT (NT / 32) doubles, one sum per warp, source and component.  u must be
+// zeroed and receives scale * M f.
 template <bool WALL, int NT, bool FAR = false>
 __device__ __forceinline__ void dfsym_item(float4 *__restrict__ sD, double *__restrict__ sRev,
                                            const float4 *__restrict__ hi,
                                            const float4 *__restrict__ lo,
                                            const double *__restrict__ f, int64_t n, int64_t I,
-                                           int64_t J, const PairConsts<dfl> &k,
+                                           int64_t J, int half, const MobConstsDf &k,
                                            double *__restrict__ u, double scale)
 {
-    const int lane = threadIdx.x & 31;
+    const int64_t j0 = J * 2 * NT + half * NT;
+    if (j0 >= n) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool diag = I == J;
-    const int64_t i = I * NT + threadIdx.x;
-    const int64_t ic = i < n ? i : n - 1;
-    const float4 th = hi[ic], tl = lo[ic];
-    const dfl xi(th.x, tl.x), yi(th.y, tl.y), zi(th.z, tl.z);
-    const dfl gx = i < n ? dfl(f[3 * i]) : dfl(), gy = i < n ? dfl(f[3 * i + 1]) : dfl(),
-              gz = i < n ? dfl(f[3 * i + 2]) : dfl();
-    dfl ux, uy, uz;
-    const int64_t j0 = J * NT;
+    const int64_t ia = I * 2 * NT + threadIdx.x, ib = ia + NT;
+    dfl2 xi, yi, zi, gx, gy, gz, ux, uy, uz;
+    {
+        const int64_t ca = ia < n ? ia : n - 1, cb = ib < n ? ib : n - 1;
+        const float4 ha = hi[ca], hb = hi[cb], la = lo[ca], lb = lo[cb];
+        xi = dfl2(make_float2(ha.x, hb.x), make_float2(la.x, lb.x));
+        yi = dfl2(make_float2(ha.y, hb.y), make_float2(la.y, lb.y));
+        zi = dfl2(make_float2(ha.z, hb.z), make_float2(la.z, lb.z));
+        // padding targets carry no force, so their reverse contributions vanish
+        dfl g[2][3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            g[0][c] = ia < n ? dfl(f[3 * ia + c]) : dfl();
+            g[1][c] = ib < n ? dfl(f[3 * ib + c]) : dfl();
+        }
+        gx = dfl2(make_float2(g[0][0].hi, g[1][0].hi), make_float2(g[0][0].lo, g[1][0].lo));
+        gy = dfl2(make_float2(g[0][1].hi, g[1][1].hi), make_float2(g[0][1].lo, g[1][1].lo));
+        gz = dfl2(make_float2(g[0][2].hi, g[1][2].hi), make_float2(g[0][2].lo, g[1][2].lo));
+    }
     __syncthreads();
     {
         const int64_t j = j0 + threadIdx.x;
         const bool valid = j < n;
         const int64_t jc = valid ? j : j0;
         const float4 h = hi[jc], l = lo[jc];
-        const dfl fx = valid ? dfl(f[3 * jc]) : dfl();
-        const dfl fy = valid ? dfl(f[3 * jc + 1]) : dfl();
-        const dfl fz = valid ? dfl(f[3 * jc + 2]) : dfl();
-        float4 *d = sD + 3 * threadIdx.x;
-        d[0] = make_float4(h.x, l.x, h.y, l.y);
-        d[1] = make_float4(h.z, l.z, fx.hi, fx.lo);
-        d[2] = make_float4(fy.hi, fy.lo, fz.hi, fz.lo);
-        sRev[3 * threadIdx.x] = sRev[3 * threadIdx.x + 1] = sRev[3 * threadIdx.x + 2] = 0.0;
+        const double z = (double)h.z + (double)l.z;
+        const dfl v[7] = {dfl(h.x, l.x), dfl(h.y, l.y), dfl(h.z, l.z),
+                          valid ? dfl(f[3 * jc]) : dfl(), valid ? dfl(f[3 * jc + 1]) : dfl(),
+                          valid ? dfl(f[3 * jc + 2]) : dfl(), dfl(-2.0 * z * z)};
+#pragma unroll
+        for (int c = 0; c < 7; ++c)
+            sD[7 * threadIdx.x + c] = make_float4(v[c].hi, v[c].hi, v[c].lo, v[c].lo);
     }
     __syncthreads();
+    auto src = [&](int s, int c) {
+        const float4 q = sD[7 * s + c];
+        return dfl2(make_float2(q.x, q.y), make_float2(q.z, q.w));
+    };
     if (diag) {
 #pragma unroll 1
         for (int s = 0; s < NT; ++s) {
-            const float4 A = sD[3 * s], B = sD[3 * s + 1], C = sD[3 * s + 2];
-            const dfl zj(B.x, B.y);
-            pair_accumulate<WALL, dfl>(xi - dfl(A.x, A.y), yi - dfl(A.z, A.w), zi - zj, zi, zj,
-                                       dfl(B.z, B.w), dfl(C.x, C.y), dfl(C.z, C.w), k, ux, uy, uz);
+            const dfl2 zj = src(s, 2);
+            const dfl2 dx = xi - src(s, 0), dy = yi - src(s, 1), dz = zi - zj;
+            const Mob<dfl2> m = mob_coefs_df<WALL, false>(dx, dy, dz, zi, zj, src(s, 6), k);
+            mob_apply_df<WALL>(m, dx, dy, dz, src(s, 3), src(s, 4), src(s, 5), ux, uy, uz);
+            if ((s & 31) == 31) {
+                renorm(ux);
+                renorm(uy);
+                renorm(uz);
+            }
         }
     } else {
+        const int from = (lane + 1) & 31;
+        auto pass = [&](dfl2 &v) {
+            v.hi.x = __shfl_sync(0xffffffffu, v.hi.x, from);
+            v.hi.y = __shfl_sync(0xffffffffu, v.hi.y, from);
+            v.lo.x = __shfl_sync(0xffffffffu, v.lo.x, from);
+            v.lo.y = __shfl_sync(0xffffffffu, v.lo.y, from);
+        };
         for (int g = 0; g < NT / 32; ++g) {
-            dfl vx, vy, vz;
+            dfl2 vx, vy, vz;
 #pragma unroll 1
             for (int t = 0; t < 32; ++t) {
                 const int s = g * 32 + ((lane + t) & 31);
-                const float4 A = sD[3 * s], B = sD[3 * s + 1], C = sD[3 * s + 2];
-                const dfl zj(B.x, B.y);
-                pair_sym_rg<WALL, dfl, FAR>(xi - dfl(A.x, A.y), yi - dfl(A.z, A.w), zi - zj, zi, zj,
-                                  dfl(B.z, B.w), dfl(C.x, C.y), dfl(C.z, C.w), gx, gy, gz, k, ux,
-                                  uy, uz, vx, vy, vz);
-                const int from = (lane + 1) & 31;
-                vx.hi = __shfl_sync(0xffffffffu, vx.hi, from);
-                vx.lo = __shfl_sync(0xffffffffu, vx.lo, from);
-                vy.hi = __shfl_sync(0xffffffffu, vy.hi, from);
-                vy.lo = __shfl_sync(0xffffffffu, vy.lo, from);
-                vz.hi = __shfl_sync(0xffffffffu, vz.hi, from);
-                vz.lo = __shfl_sync(0xffffffffu, vz.lo, from);
+                const dfl2 zj = src(s, 2);
+                const dfl2 dx = xi - src(s, 0), dy = yi - src(s, 1), dz = zi - zj;
+                const Mob<dfl2> m = mob_coefs_df<WALL, FAR>(dx, dy, dz, zi, zj, src(s, 6), k);
+                mob_apply_df<WALL>(m, dx, dy, dz, src(s, 3), src(s, 4), src(s, 5), ux, uy, uz);
+                mob_apply_df<WALL, true>(m, dx, dy, dz, gx, gy, gz, vx, vy, vz);
+                pass(vx);
+                pass(vy);
+                pass(vz);
             }
-            double *o3 = sRev + 3 * (g * 32 + lane);
-            atomicAdd(o3, to_double(vx));
-            atomicAdd(o3 + 1, to_double(vy));
-            atomicAdd(o3 + 2, to_double(vz));
-            // the forward sums take sloppy additions: renormalised every 32 terms
+            double *o3 = sRev + 3 * (warp * NT + g * 32 + lane);
+            o3[0] = sum_halves(vx);
+            o3[1] = sum_halves(vy);
+            o3[2] = sum_halves(vz);
+            // the sums are unnormalised: renormalised every 32 terms
             renorm(ux);
             renorm(uy);
             renorm(uz);
@@ -527,13 +438,21 @@ __device__ __forceinline__ void dfsym_item(float4 *__restrict__ sD, double *__re
         const int64_t j = j0 + threadIdx.x;
         if (j < n) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) atomicAdd(u + 3 * j + c, scale * sRev[3 * threadIdx.x + c]);
+            for (int c = 0; c < 3; ++c) {
+                double acc = 0.0;
+#pragma unroll
+                for (int w = 0; w < NT / 32; ++w) acc += sRev[3 * (w * NT + threadIdx.x) + c];
+                atomicAdd(u + 3 * j + c, scale * acc);
+            }
         }
     }
-    if (i < n) {
-        atomicAdd(u + 3 * i, scale * to_double(ux));
-        atomicAdd(u + 3 * i + 1, scale * to_double(uy));
-        atomicAdd(u + 3 * i + 2, scale * to_double(uz));
+    const dfl2 acc[3] = {ux, uy, uz};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (ia < n)
+            atomicAdd(u + 3 * ia + c, scale * ((double)acc[c].hi.x + (double)acc[c].lo.x));
+        if (ib < n)
+            atomicAdd(u + 3 * ib + c, scale * ((double)acc[c].hi.y + (double)acc[c].lo.y));
     }
 }
 

@@ -30,90 +30,9 @@
 
 #include <type_traits>
 
+#include "df32.cuh"
+
 namespace mb {
-
-// Per-call constants of the pair interaction (units of (6 pi eta a)^-1).
-template <typename T>
-struct PairConsts {
-    T a2;       // a^2
-    T four_a2;  // 4 a^2: r^2 below this takes the overlap branch
-    T c1, c2;   // far C  = inv (c1 + c2 inv^2)
-    T c3, c4;   // far D' = inv^3 (c3 + c4 inv^2)
-    T k1, k2;   // near C = 1 - k1 r, D' = k2 inv
-    T sw;       // wall prefactor 3a/4
-    T tiny;     // floor on r^2 (coincident blobs, including i = j)
-
-    __host__ static PairConsts make(double a)
-    {
-        PairConsts k;
-        k.a2 = T(a * a);
-        k.four_a2 = T(4.0 * a * a);
-        k.c1 = T(0.75 * a);
-        k.c2 = T(0.5 * a * a * a);
-        k.c3 = T(0.75 * a);
-        k.c4 = T(-1.5 * a * a * a);
-        k.k1 = T(9.0 / (32.0 * a));
-        k.k2 = T(3.0 / (32.0 * a));
-        k.sw = T(0.75 * a);
-        k.tiny = std::is_same<T, double>::value ? T(1e-300) : T(1e-30);
-        return k;
-    }
-};
-
-__device__ __forceinline__ float mb_rsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double mb_rsqrt(double x) { return rsqrt(x); }
-__device__ __forceinline__ float mb_max(float x, float y) { return fmaxf(x, y); }
-__device__ __forceinline__ double mb_max(double x, double y) { return fmax(x, y); }
-
-// Accumulate u += M_ij f_j for one pair, given the separation d = r_i - r_j
-// (already formed by the caller, possibly from hi/lo parts), the heights
-// zi, zj and the source force f.  WALL selects the wall correction.
-template <bool WALL, typename T>
-__device__ __forceinline__ void pair_accumulate(T dx, T dy, T dz, T zi, T zj, T fx, T fy, T fz,
-                                                const PairConsts<T> &k, T &ux, T &uy, T &uz)
-{
-    const T dxy2 = dx * dx + dy * dy;
-    const T r2 = mb_max(dz * dz + dxy2, k.tiny);
-    const T inv = mb_rsqrt(r2);
-    const T inv2 = inv * inv;
-    T C = inv * (k.c1 + k.c2 * inv2);
-    T D = inv * inv2 * (k.c3 + k.c4 * inv2);
-    if (r2 < k.four_a2) {  // overlapping blobs (rare): regularised branch
-        C = T(1) - k.k1 * (r2 * inv);
-        D = k.k2 * inv;
-    }
-    const T rf_xy = dx * fx + dy * fy;
-    const T g = D * (rf_xy + dz * fz);
-    if (!WALL) {
-        ux += C * fx + g * dx;
-        uy += C * fy + g * dy;
-        uz += C * fz + g * dz;
-        return;
-    }
-    const T R3 = zi + zj;
-    const T invR = mb_rsqrt(R3 * R3 + dxy2);
-    const T hs = zj * invR;
-    const T ht = zi * invR;
-    const T e3 = hs + ht;
-    const T E = e3 * e3;
-    const T t2 = k.a2 * (invR * invR);
-    const T t4 = t2 * t2;
-    const T p = hs * ht;
-    const T f1 = T(-1) - T(2) * p + t2 * (T(2) * E - T(2.0 / 3.0)) + t4 * (T(2.0 / 3.0) - T(10.0 / 3.0) * E);
-    const T f2 = T(-1) + T(6) * p + t2 * (T(2) - T(10) * E) + t4 * (T(70.0 / 3.0) * E - T(10.0 / 3.0));
-    const T f3 = T(2) * hs + e3 * (t2 * (T(20) * E - T(4)) + t4 * (T(40.0 / 3.0) - T(140.0 / 3.0) * E) - T(12) * p);
-    const T f4 = T(2) * hs - T(20.0 / 3.0) * e3 * t4;
-    const T f5 = T(-4) * hs * hs - T(4) * E * t2 + t4 * (T(20) * E - T(8.0 / 3.0));
-    const T eF = (rf_xy + R3 * fz) * invR;
-    const T gw = (f2 * eF + f3 * fz) * invR;
-    const T kz = f4 * eF + f5 * fz;
-    const T s = k.sw * invR;
-    const T Cx = C + s * f1;
-    const T Gx = g + s * gw;
-    ux += Cx * fx + Gx * dx;
-    uy += Cx * fy + Gx * dy;
-    uz += Cx * fz + g * dz + s * (gw * R3 + kz);
-}
 
 // The regrouped form of the same interaction.  With u = 1/rho, w = u^2,
 // X = a^2 w, Q = X^2 / 3, E = R3^2 w, S = X E + Q and c = zi zj w + X / 3, the
@@ -163,15 +82,6 @@ struct MobConsts {
         return k;
     }
 };
-
-// 1/sqrt(x) in FP32 for normal x: the hardware estimate without the scaling
-// of denormal arguments that rsqrtf() adds.
-__device__ __forceinline__ float rsqrt_ftz(float x)
-{
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // 1/sqrt(x) in FP64 for x > 0.  FP64 instructions are what the FP64 kernels
 // wait for (one per ~19 cycles and SM), conversions between FP32 and FP64
@@ -348,9 +258,6 @@ struct MobConsts2 {
     }
 };
 
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 rsqrt2(float2 a)
 {
     return make_float2(rsqrt_ftz(a.x), rsqrt_ftz(a.y));
@@ -426,6 +333,121 @@ __device__ __forceinline__ Mob<float2> mob_coefs2(float2 dz, float2 dxy2, float2
     m.Bb = fma2(sw, t4, K);
     m.Z = fma2(R3, fma2(sw, add2(t3, t4), AR), fma2(dz, Dz, fma2(s, f5, m.Cx)));
     return m;
+}
+
+// Double-float, two pairs at once.
+struct MobConstsDf {
+    dfl2 a2, third, d1, s2, c2, c4, four_a2, k1, k2;
+
+    __host__ static MobConstsDf make(double a)
+    {
+        MobConstsDf k;
+        k.a2 = dfl(a * a);
+        k.third = dfl(1.0 / 3.0);
+        k.d1 = dfl(0.75 * a);
+        k.s2 = dfl(1.5 * a);
+        k.c2 = dfl(0.5 * a * a * a);
+        k.c4 = dfl(-1.5 * a * a * a);
+        k.four_a2 = dfl(4.0 * a * a);
+        k.k1 = dfl(-9.0 / (32.0 * a));
+        k.k2 = dfl(3.0 / (32.0 * a));
+        return k;
+    }
+};
+
+// The overlap branch, half by half (rare).
+__device__ __forceinline__ void overlap_df(dfl2 r2, const MobConstsDf &k, dfl2 &inv, dfl2 &C, dfl2 &D)
+{
+    dfl2 x = r2;
+    if (!(x.hi.x > 1e-30f)) { x.hi.x = 1e-30f; x.lo.x = 0.f; }
+    if (!(x.hi.y > 1e-30f)) { x.hi.y = 1e-30f; x.lo.y = 0.f; }
+    const dfl2 ir = rsqrt_df(x), Cn = addf(k.k1 * (x * ir), 1.f), Dn = k.k2 * ir;
+    const float2 g = add2(sub2(r2.hi, k.four_a2.hi), sub2(r2.lo, k.four_a2.lo));
+    if (g.x < 0.f) {
+        C.hi.x = Cn.hi.x; C.lo.x = Cn.lo.x;
+        D.hi.x = Dn.hi.x; D.lo.x = Dn.lo.x;
+        inv.hi.x = inv.lo.x = 0.f;
+    }
+    if (g.y < 0.f) {
+        C.hi.y = Cn.hi.y; C.lo.y = Cn.lo.y;
+        D.hi.y = Dn.hi.y; D.lo.y = Dn.lo.y;
+        inv.hi.y = inv.lo.y = 0.f;
+    }
+}
+
+// Coefficients in double-float, zz = -2 zj^2.  FAR (every pair 64 a or more
+// apart, so that X < 2^-12 and no pair overlaps): the terms carrying
+// X^2 = 3 Q < 2^-24 are summed in FP32 and added to the lo parts; their
+// rounding is below 2^-24 X^2 of the polynomials, under the double-float
+// rounding of the other terms.
+template <bool WALL, bool FAR>
+__device__ __forceinline__ Mob<dfl2> mob_coefs_df(dfl2 dx, dfl2 dy, dfl2 dz, dfl2 zi, dfl2 zj,
+                                                  dfl2 zz, const MobConstsDf &k)
+{
+    Mob<dfl2> m;
+    const dfl2 dxy2 = dx * dx + dy * dy;
+    const dfl2 r2 = dz * dz + dxy2;
+    dfl2 inv = rsqrt_df(r2);
+    const dfl2 inv2 = inv * inv;
+    dfl2 inv3 = inv * inv2;
+    renorm(inv3);  // inv3, w and f2 enter most products: their lo parts kept short
+    // 3a/4 exceeds (3a^3/2) / r^2 wherever this is used (r > 2a)
+    dfl2 C = k.c2 * inv3, D = inv3 * add_ordered(k.d1, k.c4 * inv2);
+    if (!FAR) {
+        const float2 g = add2(sub2(r2.hi, k.four_a2.hi), sub2(r2.lo, k.four_a2.lo));
+        if (g.x < 0.f || g.y < 0.f) overlap_df(r2, k, inv, C, D);
+    }
+    if (!WALL) {
+        m.Cx = k.d1 * inv + C;
+        m.H = D;
+        return m;
+    }
+    const dfl2 R3 = zi + zj, H2 = R3 * R3;
+    const dfl2 u = rsqrt_df(H2 + dxy2);
+    dfl2 w = u * u;
+    renorm(w);
+    const dfl2 X = k.a2 * w, E = H2 * w, X3 = X * k.third, V = X * E;
+    const dfl2 c = (zi * zj) * w + X3, zw = zz * w;
+    dfl2 d1, f2, br, t4, f5;
+    if (FAR) {
+        const float2 Q = mul2(X3.hi, X.hi), EQ = mul2(E.hi, Q);
+        d1 = add_lo(V + (-c), fma2(splat2(-5.f), EQ, Q));
+        f2 = add_lo(addf(mulf(c, 3.f), -0.5f) + mulf(V, -5.f),
+                    fma2(splat2(35.f), EQ, mul2(splat2(-5.f), Q)));
+        br = add_lo(addf(mul_pow2(f2, -2.f), -1.f), mul2(splat2(10.f), Q));
+        t4 = add_lo(zj, mul2(mul2(splat2(-10.f), Q), R3.hi));
+        f5 = add_lo(zw + mul_pow2(V, -2.f), fma2(splat2(30.f), EQ, mul2(splat2(-4.f), Q)));
+    } else {
+        const dfl2 Q = X3 * X, EQ = E * Q, S = V + Q;
+        d1 = (S + mulf(EQ, -5.f)) + (-c);
+        f2 = (addf(mulf(c, 3.f), -0.5f) + mulf(S, -5.f)) + mulf(EQ, 35.f);
+        br = addf(mul_pow2(f2, -2.f), -1.f) + mulf(Q, 10.f);
+        t4 = zj + mulf(R3 * Q, -10.f);
+        f5 = (zw + mul_pow2(S + Q, -2.f)) + mulf(EQ, 30.f);
+    }
+    renorm(f2);
+    const dfl2 t3 = R3 * br + zj;
+    const dfl2 s = k.s2 * u, sw = s * w;
+    m.Cx = (k.d1 * (inv + (-u)) + s * d1) + C;
+    const dfl2 A2 = sw * f2, AR = A2 * R3, Dz = D * dz, K = Dz + AR;
+    m.H = D + A2;
+    m.Bf = sw * t3 + K;
+    m.Bb = sw * t4 + K;
+    m.Z = ((sw * (t3 + t4) + AR) * R3 + Dz * dz) + (s * f5 + m.Cx);
+    return m;
+}
+
+// u += M f (TRANS: M^T f), unnormalised sums.
+template <bool WALL, bool TRANS = false>
+__device__ __forceinline__ void mob_apply_df(const Mob<dfl2> &m, dfl2 dx, dfl2 dy, dfl2 dz,
+                                             dfl2 fx, dfl2 fy, dfl2 fz, dfl2 &ux, dfl2 &uy,
+                                             dfl2 &uz)
+{
+    const dfl2 rf = dx * fx + dy * fy;
+    const dfl2 G = WALL ? m.H * rf + (TRANS ? m.Bb : m.Bf) * fz : m.H * (rf + dz * fz);
+    ux = ux + (m.Cx * fx + G * dx);
+    uy = uy + (m.Cx * fy + G * dy);
+    uz = uz + (WALL ? m.Z * fz + (TRANS ? m.Bf : m.Bb) * rf : m.Cx * fz + G * dz);
 }
 
 // u += M f (TRANS: M^T f) for the two targets in the halves.

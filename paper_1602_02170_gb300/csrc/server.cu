@@ -316,14 +316,16 @@ __global__ void eng_zero_kernel(const Work *__restrict__ W, const RSeg *__restri
 // Symmetric double-float kernel over every listed request's block-pair
 // triangle (blocks of kNT blobs); y zeroed beforehand; n_tblocks holds the
 // request's block count.
+constexpr int kDfNT = kNT / 2;  // threads: blocks of kNT blobs, two per thread
+
 template <bool WALL>
-__global__ void __launch_bounds__(kNT) eng_df_kernel(const Work *__restrict__ W,
+__global__ void __launch_bounds__(kDfNT, 3) eng_df_kernel(const Work *__restrict__ W,
                                                      const int64_t *__restrict__ item_off, int nw,
                                                      int64_t n_items, const int *__restrict__ mask,
-                                                     PairConsts<dfl> k, double scale)
+                                                     MobConstsDf k, double scale)
 {
-    __shared__ float4 sD[3 * kNT];
-    __shared__ double sRev[3 * kNT];
+    __shared__ float4 sD[7 * kDfNT];
+    __shared__ double sRev[3 * kDfNT * (kDfNT / 32)];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const Work P = W[find_owner(item_off, nw, item)];
         if (!mask[P.slot]) continue;
@@ -336,7 +338,10 @@ __global__ void __launch_bounds__(kNT) eng_df_kernel(const Work *__restrict__ W,
             else hi_r = mid;
         }
         const int64_t I = lo_r, J = I + (local - (I * nb - I * (I - 1) / 2));
-        dfsym_item<WALL, kNT>(sD, sRev, P.hi, P.lo, P.f, P.n, I, J, k, P.y, scale);
+        for (int half = 0; half < 2; ++half) {
+            dfsym_item<WALL, kDfNT>(sD, sRev, P.hi, P.lo, P.f, P.n, I, J, half, k, P.y, scale);
+            __syncthreads();  // this half is done with sRev
+        }
     }
 }
 
@@ -1028,13 +1033,13 @@ struct Engine {
         const int tpc = x2 ? 2 * (np_variant == 3 ? 1 : np_variant) * kNT : kNT;
         int occ = 1;
         if (dfs)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_df_kernel<true>, kNT, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_df_kernel<true>, kDfNT, 0);
         else if (sym)
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_sym_kernel<true>, kNT, 0);
         else if (prec == MB_FP32_KAHAN)
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_x2_kernel<true, 1>, kNT, 0);
         else if (prec == MB_DF64)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_df_kernel<true>, kNT, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_df_kernel<true>, kDfNT, 0);
         else
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_f64_kernel<true>, kNT, 0);
         const int res = std::max(1, occ) * ctx->sm_count;
@@ -1107,9 +1112,9 @@ struct Engine {
             count_launch();
         }
         if (dfs) {
-            const PairConsts<dfl> k = PairConsts<dfl>::make(prm.a);
-            if (wall) eng_df_kernel<true><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
-            else eng_df_kernel<false><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
+            const MobConstsDf k = MobConstsDf::make(prm.a);
+            if (wall) eng_df_kernel<true><<<grid, kDfNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
+            else eng_df_kernel<false><<<grid, kDfNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
         } else if (sym) {
             const MobConsts2 k = MobConsts2::make(prm.a);
             if (wall) eng_sym_kernel<true><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);

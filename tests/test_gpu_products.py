@@ -96,3 +96,36 @@ def test_fp32_product_in_place_and_variant_by_size(ctx):
         assert ctx.pair_variant(n, True) == variant
         ctx.mobility_matvec(R, F, 0.5, 1.0, True, "fp32", out=F)
         assert rel_l2(host(F), want) <= 1e-14
+
+
+@pytest.mark.parametrize("wall", [True, False])
+@pytest.mark.parametrize("n", [1, 15, 33, 1100, 1101, 1153, 23999, 24001])
+def test_df64_blocks_of_every_size(ctx, n, wall):
+    """Double-float: forward only up to 1,100 blobs, blocks of 64 blobs above
+    and of 256 from 24,000, ragged and nearly empty last blocks, in a narrow
+    strip (so that the largest sizes have far and near block pairs), against
+    the FP64 product.  Positions are carried to 2^-49 of coordinates up to 30
+    at separations of 0.1 and more, the arithmetic to about 2^-45: 1e-12."""
+    r, f = I.blob_cloud(n, n, 0.1, 30.0, 0.1, 0.5)
+    r[:, 1] *= 0.2
+    got = host(ctx.mobility_matvec(dev(r), dev(f), 0.1, 1.0, wall, "df64"))
+    ref = host(ctx.mobility_matvec(dev(r), dev(f), 0.1, 1.0, wall, "fp64"))
+    assert rel_l2(got, ref) <= 1e-12
+
+
+def test_df64_overlaps_in_both_halves(ctx):
+    """Coincident, overlapping and touching blobs 32 and 64 places apart, the
+    halves of one packed pair and its neighbours, above the forward-only
+    size."""
+    rng = np.random.default_rng(3)
+    r = np.stack([np.arange(1300) * 3.0, np.full(1300, 1.0), rng.uniform(0.5, 2.0, 1300)], axis=1)
+    for p in range(0, 1200, 97):
+        r[p + 1] = r[p]
+        r[p + 32] = r[p] + [0.3, 0.0, 0.0]
+        r[p + 64] = r[p] + [0.0, 1.0, 0.0]
+    f = rng.standard_normal(r.shape)
+    ref = O.matvec(r, f, 0.5, 1.0, True)
+    got = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, True, "df64"))
+    # coordinates up to 3,900 carried to 2^-49, separations from 0.3 on: 1e-10
+    assert np.isfinite(got).all()
+    assert rel_l2(got, ref) <= 1e-10
