@@ -1,0 +1,48 @@
+"""Blob build, K and K^T where their tiles and lane groups change: bodies of
+one blob, empty bodies, more bodies in a tile of 256 blobs than it keeps in
+shared memory (64), and enough bodies for half a warp each (2,048).
+
+Sums of up to 700 terms of size 1 with coordinates up to 60: 1e-12."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from tests.gpu_common import ctx, dev, host  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(counts, seed):
+    rng = np.random.default_rng(seed)
+    counts = np.asarray(counts)
+    start = np.concatenate([[0], np.cumsum(counts)]).astype(np.int64)
+    nb, n = len(counts), int(start[-1])
+    return (rng.uniform(0, 60, (nb, 3)), rng.standard_normal((nb, 4)), start,
+            rng.standard_normal((n, 3)), rng)
+
+
+COUNTS = {
+    "one blob": [1],
+    "ones": [1] * 700,
+    "ragged": [255, 1, 257, 0, 3, 700, 42],
+    "empty": [5] + [0] * 90 + [7] + [0] * 90 + [300],
+    "many": [3, 15, 42] * 700,
+    "tiles of two rounds": [162] * 1650,
+}
+
+
+@pytest.mark.parametrize("name", COUNTS)
+def test_kinematics_by_body_sizes(ctx, name):
+    q, theta, start, rho, rng = _case(COUNTS[name], len(name))
+    nb, n = len(q), len(rho)
+    S = torch.as_tensor(start, device="cuda")
+    r = host(ctx.blob_positions(dev(q), dev(theta), S, dev(rho)))
+    unit = theta / np.linalg.norm(theta, axis=1, keepdims=True)
+    assert np.abs(r - O.blob_positions(q, unit, start, rho)).max() <= 1e-12
+    UO, lam = rng.standard_normal((nb, 6)), rng.standard_normal((n, 3))
+    v = host(ctx.K_apply(dev(r), dev(q), S, dev(UO)))
+    assert np.abs(v - O.K_apply(UO[:, :3], UO[:, 3:], r, q, start)).max() <= 1e-12
+    FT = host(ctx.KT_apply(dev(r), dev(q), S, dev(lam)))
+    F, T = O.KT_apply(lam, r, q, start)
+    assert np.abs(FT - np.concatenate([F, T], 1)).max() <= 1e-11
