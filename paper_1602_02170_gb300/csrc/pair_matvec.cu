@@ -293,42 +293,48 @@ __global__ void __launch_bounds__(32) pair_f64sym_kernel(
     }
 }
 
-// Flow evaluation at points other than the blobs (targets != sources):
-// packed FP32 and FP64 items over (target block, source chunk), partials
-// reduced like the matvec's.  The targets are tracers of the blob radius a
-// (Appendix B renders flows with small blobs of radius a').
-template <bool WALL>
-__global__ void __launch_bounds__(kNT, 3) eval_f32x2_kernel(
+// Flow evaluation at points other than the blobs (targets != sources): one
+// packed FP32 (2 NT targets) or FP64 (32 targets, one warp) item of a target
+// block against a source chunk per CTA, partials reduced like the matvec's.
+// The targets are tracers of the blob radius a (Appendix B renders flows with
+// small blobs of radius a').  Bound by the FMA or the FP64 pipe; the chunks
+// (eval_plan) give every SM several items whatever the number of points, where
+// chunks of 512 sources and blocks of 512 or 256 points left most idle.
+// With the wall (us): 3,072 points and 6,720 blobs 135 -> 78 in FP32 and 6,360
+// -> 2,890 in FP64, 100 points 133 -> 26 and 3,180 -> 145, 65,536 points and
+// blobs 11,200 -> 10,270 in FP32.
+template <bool WALL, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) eval_f32x2_kernel(
     const float4 *__restrict__ thi, const float4 *__restrict__ tlo, int64_t nt,
     const float4 *__restrict__ hi, const float4 *__restrict__ lo, const double *__restrict__ f,
     int64_t ns, int64_t chunk, int n_tblocks, int64_t n_items, MobConsts2 k,
     double *__restrict__ out, double scale, int direct)
 {
-    __shared__ float4 sP[kX2SmemFloat4PerSource * kNT];
+    __shared__ float4 sP[kX2SmemFloat4PerSource * NT];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int tb = (int)(item % n_tblocks);
         const int64_t sc = item / n_tblocks;
         const int64_t j_begin = sc * chunk;
         const int64_t j_end = j_begin + chunk < ns ? j_begin + chunk : ns;
-        x2_item<WALL, 1, kNT>(sP, thi, tlo, nt, hi, lo, f, tb, j_begin, j_end, k,
-                              direct ? out : out + 3 * sc * nt, direct ? scale : 1.0);
+        x2_item<WALL, 1, NT>(sP, thi, tlo, nt, hi, lo, f, tb, j_begin, j_end, k,
+                             direct ? out : out + 3 * sc * nt, direct ? scale : 1.0);
     }
 }
 
 template <bool WALL>
-__global__ void __launch_bounds__(kNT) eval_f64_kernel(
+__global__ void __launch_bounds__(32) eval_f64_kernel(
     const double *__restrict__ x, int64_t nt, const double *__restrict__ r,
     const double *__restrict__ f, int64_t ns, int64_t chunk, int n_tblocks, int64_t n_items,
     MobConsts<double> k, double *__restrict__ out, double scale, int direct)
 {
-    __shared__ double sm[6 * kNT];
+    __shared__ double sm[6 * 32];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int tb = (int)(item % n_tblocks);
         const int64_t sc = item / n_tblocks;
         const int64_t j_begin = sc * chunk;
         const int64_t j_end = j_begin + chunk < ns ? j_begin + chunk : ns;
-        f64_item<WALL, kNT>(sm, x, nt, r, f, tb, j_begin, j_end, k,
-                            direct ? out : out + 3 * sc * nt, direct ? scale : 1.0);
+        f64_item<WALL, 32>(sm, x, nt, r, f, tb, j_begin, j_end, k,
+                           direct ? out : out + 3 * sc * nt, direct ? scale : 1.0);
     }
 }
 
@@ -451,17 +457,39 @@ __global__ void __launch_bounds__(NT, 384 / NT) pair_df_kernel(
     }
 }
 
-// u_i = scale * sum_s partial[s][i]  (fixed order)
-__global__ void reduce_partials_kernel(const double *__restrict__ partial, int64_t n, int S,
-                                       double scale, double *__restrict__ u)
+// u_i = scale * sum_s partial[s][i] in a fixed order: 32 entries a CTA, eight
+// warps summing every eighth chunk of them, then one adding the eight sums (a
+// thread that walked all chunks by itself would wait for each load in turn).
+constexpr int kReduceWarps = 8;
+
+__global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(
+    const double *__restrict__ partial, int64_t n, int S, double scale, double *__restrict__ u)
 {
+    __shared__ double sum[kReduceWarps][32];
     const int64_t m = 3 * n;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t e0 = blockIdx.x * (int64_t)32; e0 < m; e0 += (int64_t)gridDim.x * 32) {
         double acc = 0.0;
-        for (int s = 0; s < S; ++s) acc += partial[s * m + e];
-        u[e] = scale * acc;
+        if (e0 + lane < m)
+#pragma unroll 4
+            for (int s = warp; s < S; s += kReduceWarps) acc += partial[s * m + e0 + lane];
+        sum[warp][lane] = acc;
+        __syncthreads();
+        if (warp == 0 && e0 + lane < m) {
+#pragma unroll
+            for (int w = 1; w < kReduceWarps; ++w) acc += sum[w][lane];
+            u[e0 + lane] = scale * acc;
+        }
+        __syncthreads();
     }
+}
+
+void launch_reduce_partials(const double *partial, int64_t n, int S, double scale, double *u,
+                            cudaStream_t s)
+{
+    reduce_partials_kernel<<<(int)std::min<int64_t>(ceil_div(3 * n, 32), 65535), 32 * kReduceWarps, 0,
+                             s>>>(partial, n, S, scale, u);
+    count_launch();
 }
 
 struct Plan {
@@ -475,10 +503,9 @@ struct Plan {
 // Split sources into S chunks so that the items fill whole waves of the
 // resident grid as evenly as possible, with chunks of at least two tiles.
 Plan make_plan(int64_t n, int targets_per_cta, int resident, int64_t s_cap = 64, int tile = kNT,
-               int64_t min_chunk = 2 * kNT, int64_t n_src = -1)
+               int64_t min_chunk = 2 * kNT)
 {
-    // n targets; n_src sources (the same blobs unless given)
-    const int64_t ns = n_src < 0 ? n : n_src;
+    const int64_t ns = n;
     Plan p;
     p.n_tblocks = (int)ceil_div(n, targets_per_cta);
     const int64_t max_s = std::max<int64_t>(1, std::min<int64_t>(s_cap, ceil_div(ns, min_chunk)));
@@ -955,9 +982,7 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
                 *defer = MatvecPartials{out, p.S, scale};
                 return MB_OK;
             }
-            const int grid = (int)std::min<int64_t>(ceil_div(3 * n, 256), 8 * (int64_t)ctx->sm_count);
-            reduce_partials_kernel<<<grid, 256, 0, s>>>(out, n, p.S, scale, u);
-            count_launch();
+            launch_reduce_partials(out, n, p.S, scale, u, s);
             MB_CUDA_TRY(ctx, cudaGetLastError());
         }
         return MB_OK;
@@ -1027,9 +1052,7 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
         return MB_OK;
     }
     if (!direct) {
-        const int grid = (int)std::min<int64_t>(ceil_div(3 * n, 256), 8 * (int64_t)ctx->sm_count);
-        reduce_partials_kernel<<<grid, 256, 0, s>>>(out, n, p.S, scale, u);
-        count_launch();
+        launch_reduce_partials(out, n, p.S, scale, u, s);
         MB_CUDA_TRY(ctx, cudaGetLastError());
     }
     return MB_OK;
@@ -1223,74 +1246,91 @@ mb_status matvec_device(mb_context *ctx, const double *r, const double *f, int64
     return matvec_packed(ctx, r, f, n, a, eta, wall, prec, u, s);
 }
 
+// Target blocks of `block` points against source chunks (whole tiles of
+// `tile` sources, or a single chunk of 16 or more below one tile) so that there
+// are about `want` items.  Splitting costs a reduction launch and 24 B a point
+// and chunk, so chunks are shorter than 64 sources only as far as every
+// scheduler needs an item at all.  The context's budget has to hold the chunks'
+// partial sums, else there are fewer, down to one.
+Plan eval_plan(const mb_context *ctx, int64_t nt, int64_t ns, int block, int64_t want, int tile,
+               int64_t shortest)
+{
+    Plan p;
+    p.n_tblocks = (int)ceil_div(nt, block);
+    const size_t room = ctx->budget > ctx->held ? ctx->budget - ctx->held : 0;
+    const int64_t fits = (int64_t)(std::max(room, ctx->partial.bytes) / (sizeof(double) * 3)) / nt;
+    const int64_t need = std::min<int64_t>(4 * ctx->sm_count / p.n_tblocks, ceil_div(ns, shortest));
+    const int64_t good = std::min(ceil_div(want, p.n_tblocks), ceil_div(ns, 4 * shortest));
+    const int64_t s = std::max<int64_t>(1, std::min(std::max(need, good), fits));
+    p.chunk = ceil_div(ns, s);
+    if (p.chunk > tile / 2) p.chunk = ceil_div(p.chunk, tile) * tile;
+    p.S = (int)ceil_div(ns, p.chunk);
+    p.items = (int64_t)p.n_tblocks * p.S;
+    p.grid = (int)std::min<int64_t>(p.items, 1 << 30);
+    return p;
+}
+
+template <bool WALL, int NT>
+void launch_eval_f32(const Plan &p, const float4 *thi, const float4 *tlo, int64_t nt,
+                     const float4 *hi, const float4 *lo, const double *f, int64_t ns, double a,
+                     double *out, double scale, int direct, cudaStream_t s)
+{
+    eval_f32x2_kernel<WALL, NT><<<p.grid, NT, 0, s>>>(thi, tlo, nt, hi, lo, f, ns, p.chunk,
+                                                      p.n_tblocks, p.items, MobConsts2::make(a),
+                                                      out, scale, direct);
+}
+
 mb_status matvec_eval(mb_context *ctx, const double *x, int64_t nt, const double *r,
                       const double *f, int64_t ns, double a, double eta, int wall,
                       mb_precision prec, double *u, cudaStream_t s)
 {
     const double scale = 1.0 / (6.0 * kPi * eta * a);
-    if (prec == MB_FP64) {
-        const int res = wall ? resident_ctas(ctx, eval_f64_kernel<true>)
-                             : resident_ctas(ctx, eval_f64_kernel<false>);
-        const Plan p = make_plan(nt, kNT, res, 64, kNT, 2 * kNT, ns);
-        double *out = u;
-        const int direct = p.S == 1;
-        if (!direct) {
-            MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)nt * p.S, "eval partials"));
-            out = (double *)ctx->partial.ptr;
-        }
-        const MobConsts<double> k = MobConsts<double>::make(a);
-        if (wall)
-            eval_f64_kernel<true><<<p.grid, kNT, 0, s>>>(x, nt, r, f, ns, p.chunk, p.n_tblocks,
-                                                         p.items, k, out, scale, direct);
-        else
-            eval_f64_kernel<false><<<p.grid, kNT, 0, s>>>(x, nt, r, f, ns, p.chunk, p.n_tblocks,
-                                                          p.items, k, out, scale, direct);
-        count_launch();
-        MB_CUDA_TRY(ctx, cudaGetLastError());
-        if (!direct) {
-            const int grid = (int)std::min<int64_t>(ceil_div(3 * nt, 256), 8 * (int64_t)ctx->sm_count);
-            reduce_partials_kernel<<<grid, 256, 0, s>>>(out, nt, p.S, scale, u);
-            count_launch();
-            MB_CUDA_TRY(ctx, cudaGetLastError());
-        }
-        return MB_OK;
-    }
-    if (prec != MB_FP32_KAHAN)
+    if (prec != MB_FP64 && prec != MB_FP32_KAHAN)
         return set_err(ctx, MB_EINVAL, "flow evaluation supports MB_FP32_KAHAN and MB_FP64");
-    // sources packed into the context's position buffers, targets into the eval ones
-    MB_TRY(matvec_pack_positions(ctx, r, ns, s, false));
-    MB_TRY(ensure(ctx, ctx->eval_hi, sizeof(float4) * (size_t)nt, "packed targets"));
-    MB_TRY(ensure(ctx, ctx->eval_lo, sizeof(float4) * (size_t)nt, "packed targets"));
-    {
+    if (prec == MB_FP32_KAHAN) {
+        // sources packed into the context's position buffers, targets into the eval ones
+        MB_TRY(matvec_pack_positions(ctx, r, ns, s, false));
+        MB_TRY(ensure(ctx, ctx->eval_hi, sizeof(float4) * (size_t)nt, "packed targets"));
+        MB_TRY(ensure(ctx, ctx->eval_lo, sizeof(float4) * (size_t)nt, "packed targets"));
         const int grid = (int)std::min<int64_t>(ceil_div(nt, 256), 8 * (int64_t)ctx->sm_count);
         pack_hilo_kernel<false><<<grid, 256, 0, s>>>(x, nt, (float4 *)ctx->eval_hi.ptr,
                                                      (float4 *)ctx->eval_lo.ptr, nullptr);
         count_launch();
     }
-    const int res = wall ? resident_ctas(ctx, eval_f32x2_kernel<true>)
-                         : resident_ctas(ctx, eval_f32x2_kernel<false>);
-    const Plan p = make_plan(nt, 2 * kNT, res, 64, kNT, 2 * kNT, ns);
+    // FP32: kEvalItems items a resident warp slot, in one-warp CTAs unless
+    // blocks of 256 points give as many; FP64 as the product's items
+    constexpr int kEvalItems = 4;
+    const int64_t slots = 16 * (int64_t)ctx->sm_count;
+    const bool wide = ceil_div(nt, 256) * ceil_div(ns, 128) >= kEvalItems * slots / 4;
+    const Plan p = prec == MB_FP64
+                       ? eval_plan(ctx, nt, ns, 32, (int64_t)kF64ItemsPerWarp * 4 * ctx->sm_count, 4, 4)
+                   : wide ? eval_plan(ctx, nt, ns, 256, kEvalItems * slots / 4, 128, 128)
+                          : eval_plan(ctx, nt, ns, 64, kEvalItems * slots, 32, 16);
     double *out = u;
     const int direct = p.S == 1;
     if (!direct) {
         MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)nt * p.S, "eval partials"));
         out = (double *)ctx->partial.ptr;
     }
-    const MobConsts2 k = MobConsts2::make(a);
-    const float4 *thi = (const float4 *)ctx->eval_hi.ptr, *tlo = (const float4 *)ctx->eval_lo.ptr;
-    const float4 *hi = (const float4 *)ctx->pos_hi.ptr, *lo = (const float4 *)ctx->pos_lo.ptr;
-    if (wall)
-        eval_f32x2_kernel<true><<<p.grid, kNT, 0, s>>>(thi, tlo, nt, hi, lo, f, ns, p.chunk,
-                                                       p.n_tblocks, p.items, k, out, scale, direct);
-    else
-        eval_f32x2_kernel<false><<<p.grid, kNT, 0, s>>>(thi, tlo, nt, hi, lo, f, ns, p.chunk,
-                                                        p.n_tblocks, p.items, k, out, scale, direct);
+    if (prec == MB_FP64) {
+        const MobConsts<double> k = MobConsts<double>::make(a);
+        if (wall)
+            eval_f64_kernel<true><<<p.grid, 32, 0, s>>>(x, nt, r, f, ns, p.chunk, p.n_tblocks,
+                                                        p.items, k, out, scale, direct);
+        else
+            eval_f64_kernel<false><<<p.grid, 32, 0, s>>>(x, nt, r, f, ns, p.chunk, p.n_tblocks,
+                                                         p.items, k, out, scale, direct);
+    } else {
+        const float4 *thi = (const float4 *)ctx->eval_hi.ptr, *tlo = (const float4 *)ctx->eval_lo.ptr;
+        const float4 *hi = (const float4 *)ctx->pos_hi.ptr, *lo = (const float4 *)ctx->pos_lo.ptr;
+        const auto launch = wide ? (wall ? launch_eval_f32<true, 128> : launch_eval_f32<false, 128>)
+                                 : (wall ? launch_eval_f32<true, 32> : launch_eval_f32<false, 32>);
+        launch(p, thi, tlo, nt, hi, lo, f, ns, a, out, scale, direct, s);
+    }
     count_launch();
     MB_CUDA_TRY(ctx, cudaGetLastError());
     if (!direct) {
-        const int grid = (int)std::min<int64_t>(ceil_div(3 * nt, 256), 8 * (int64_t)ctx->sm_count);
-        reduce_partials_kernel<<<grid, 256, 0, s>>>(out, nt, p.S, scale, u);
-        count_launch();
+        launch_reduce_partials(out, nt, p.S, scale, u, s);
         MB_CUDA_TRY(ctx, cudaGetLastError());
     }
     return MB_OK;
@@ -1448,9 +1488,7 @@ extern "C" mb_status mb_mobility_matvec_noalloc(const double *r, const double *f
                                                             p.items, k, out, scale, direct);
     count_launch();
     if (!direct) {
-        const int grid = (int)std::min<int64_t>(ceil_div(3 * n, 256), 1024);
-        reduce_partials_kernel<<<grid, 256, 0, s>>>(partial, n, p.S, scale, u);
-        count_launch();
+        launch_reduce_partials(partial, n, p.S, scale, u, s);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {

@@ -129,3 +129,30 @@ def test_df64_overlaps_in_both_halves(ctx):
     # coordinates up to 3,900 carried to 2^-49, separations from 0.3 on: 1e-10
     assert np.isfinite(got).all()
     assert rel_l2(got, ref) <= 1e-10
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("nt,ns", [(1, 1), (31, 3), (63, 15), (65, 17), (257, 129), (20000, 50), (70, 6000), (3000, 2500)])
+def test_eval_splits(ctx, prec, nt, ns):
+    """Flow evaluation from one item to chunks of every length, against the
+    oracle's matvec over blobs and force-free points (FP32: of the unbounded
+    flow's norm, as its terms nearly cancel near the wall)."""
+    r, f = _cloud(nt + ns, ns)
+    x, _ = _cloud(nt, nt)
+    got = host(ctx.mobility_eval(dev(x), dev(r), dev(f), 0.5, 1.0, True, prec))
+    ref = O.eval_points(x, r, f, 0.5, 1.0, True)
+    free = O.eval_points(x, r, f, 0.5, 1.0, False)
+    assert np.linalg.norm(got - ref) <= TOL[prec] * np.linalg.norm(free)
+
+
+def test_eval_within_a_small_budget():
+    """A context whose budget holds no partial sums evaluates in one chunk."""
+    import paper_1602_02170_gb300 as mb
+
+    r, f = _cloud(1, 3000)
+    x, _ = _cloud(2, 2000)
+    with mb.Context(0) as big, mb.Context(0, 200_000) as small:
+        want = host(big.mobility_eval(dev(x), dev(r), dev(f), 0.5, 1.0, True, "fp32"))
+        got = host(small.mobility_eval(dev(x), dev(r), dev(f), 0.5, 1.0, True, "fp32"))
+        assert small.workspace_bytes() <= 200_000 < big.workspace_bytes()
+    assert rel_l2(got, want) <= TOL["fp32"]
