@@ -230,9 +230,9 @@ mb_status mb_context_pair_variant(const mb_context *ctx, int64_t n, int wall, in
  * that cannot take cudaMalloc's implicit device synchronisation.
  *
  * It takes no context and allocates nothing (no cudaMalloc, no cudaFree, no
- * allocating library routine).  Its scratch — packed FP32 hi/lo positions
- * and per-chunk partial sums, about 14 MiB — is one file-scope device array
- * of the library, sized for at most MB_NOALLOC_MAX_BLOBS blobs; every GPU
+ * allocating library routine).  Its scratch — packed FP32 hi/lo positions,
+ * their spatial order, sorted forces and sums, about 10 MiB — is one
+ * file-scope device array of the library, sized for at most MB_NOALLOC_MAX_BLOBS blobs; every GPU
  * that loads the library holds it until the process exits.  Larger N is
  * rejected with MB_EINVAL before anything is queued.
  *
@@ -246,8 +246,9 @@ mb_status mb_context_pair_variant(const mb_context *ctx, int64_t n, int wall, in
  *
  * r, f, u: N x 3 device pointers on the device current on the calling
  * thread (host pointers and memory of another GPU are MB_EINVAL); the
- * result is the same product as mb_mobility_matvec (up to FP32 rounding
- * order).
+ * result is the same product as mb_mobility_matvec, by the same kernels (from
+ * 600 blobs on FP64 atomics add the FP32 sums, so results may differ between
+ * calls in the last FP64 bits).  u may be f or r.
  * Errors are reported through mb_last_error(NULL).
  */
 #define MB_NOALLOC_MAX_BLOBS 65536

@@ -576,6 +576,13 @@ void launch_sym(const float4 *hi, const float4 *lo, const double *f, int64_t n, 
     else launch_sym_nt<WALL, 128>(hi, lo, f, n, a, u, scale, box, sg, s);
 }
 
+// Variant 4: 64-target blocks, source chunks of 16 or more (half a tile: one
+// warp per CTA walks fewer sources, more CTAs share the work).
+Plan small_plan(int64_t n, int resident)
+{
+    return make_plan(n, f32_targets_per_cta(4), resident, 1024, kSmallNT / 2, kSmallNT / 2);
+}
+
 template <bool WALL>
 int f32_resident(mb_context *ctx, int v)
 {
@@ -905,48 +912,69 @@ __global__ void __launch_bounds__(256) sort_scatter_u_kernel(const int *__restri
     }
 }
 
+// Arrays of a spatial order of n blobs.
+struct SortBufs {
+    const float4 *hi, *lo;  // packed positions
+    SortGrid *grid;         // followed by pack_hilo_kernel's bounding-box partials
+    unsigned *key;          // n
+    int *perm;              // n
+    int *H;                 // 2^sort_bits(n) (sort_tiles(n) + 1)
+    float4 *shi, *slo;      // n, sorted
+    float *box;             // 6 per kBoxBlobs
+};
+
+// Tiles of at least 1,024 blobs, at most one per SM.
+int sort_tiles(int64_t n, int sms) { return (int)std::min<int64_t>(ceil_div(n, 1024), sms); }
+
+unsigned *sort_parts(SortGrid *grid) { return (unsigned *)((char *)grid + sizeof(SortGrid)); }
+
 // The order of the packed positions, for N >= kSortMinN: pack_hilo_kernel
-// has left nparts bounding-box partials in the sort_grid buffer (after the
-// SortGrid).
-mb_status sort_positions(mb_context *ctx, int64_t n, int nparts, cudaStream_t s)
+// has left nparts bounding-box partials after the SortGrid.
+cudaError_t sort_launch(const SortBufs &b, int64_t n, int nparts, int sms, cudaStream_t s)
 {
-    const int64_t nb = ceil_div(n, kBoxBlobs);
-    // tiles of at least 1,024 blobs, at most one per SM
-    const int tiles = (int)std::min<int64_t>(ceil_div(n, 1024), ctx->sm_count);
+    const int tiles = sort_tiles(n, sms);
     const int64_t T = ceil_div(n, tiles);
-    MB_TRY(ensure(ctx, ctx->sort_perm, sizeof(int) * (size_t)n, "spatial order"));
-    MB_TRY(ensure(ctx, ctx->sort_key, sizeof(unsigned) * (size_t)n, "spatial order"));
     const int nbits = sort_bits(n), B = 1 << nbits;
     const size_t hist_smem = sizeof(int) * (size_t)B;
     const size_t scan_smem = sizeof(int) * (size_t)(B + B / 32);
     const size_t scatter_smem = hist_smem + sizeof(unsigned) * kSortKeysSmem;
-    MB_TRY(ensure(ctx, ctx->sort_count, hist_smem * (size_t)(tiles + 1), "spatial order"));
+    cudaError_t e = cudaFuncSetAttribute(sort_hist_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist_smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(sort_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)scan_smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(sort_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)scatter_smem);
+    if (e != cudaSuccess) return e;
+    sort_hist_kernel<<<tiles, 1024, hist_smem, s>>>(b.hi, n, T, sort_parts(b.grid), nparts, nbits,
+                                                    b.grid, b.key, b.H);
+    sort_tile_scan_kernel<<<(B + 255) / 256, 256, 0, s>>>(b.H, tiles, B);
+    sort_scan_kernel<<<1, 1024, scan_smem, s>>>(b.H + tiles * (int64_t)B, B);
+    sort_scatter_kernel<<<tiles, 1024, scatter_smem, s>>>(b.key, n, T, b.H, tiles, B, b.perm);
+    sort_pack_box_kernel<<<(int)ceil_div(n, kBoxBlobs), 256, 0, s>>>(b.perm, n, b.hi, b.lo, b.shi,
+                                                                     b.slo, b.box);
+    count_launch(5);
+    return cudaGetLastError();
+}
+
+mb_status sort_positions(mb_context *ctx, int64_t n, int nparts, cudaStream_t s)
+{
+    const int64_t nb = ceil_div(n, kBoxBlobs);
+    MB_TRY(ensure(ctx, ctx->sort_perm, sizeof(int) * (size_t)n, "spatial order"));
+    MB_TRY(ensure(ctx, ctx->sort_key, sizeof(unsigned) * (size_t)n, "spatial order"));
+    MB_TRY(ensure(ctx, ctx->sort_count,
+                  (sizeof(int) << sort_bits(n)) * (size_t)(sort_tiles(n, ctx->sm_count) + 1),
+                  "spatial order"));
     MB_TRY(ensure(ctx, ctx->sort_hi, sizeof(float4) * (size_t)n, "spatial order"));
     MB_TRY(ensure(ctx, ctx->sort_lo, sizeof(float4) * (size_t)n, "spatial order"));
     MB_TRY(ensure(ctx, ctx->sort_box, sizeof(float) * 6 * (size_t)nb, "spatial order"));
-    MB_CUDA_TRY(ctx, cudaFuncSetAttribute(sort_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)hist_smem));
-    MB_CUDA_TRY(ctx, cudaFuncSetAttribute(sort_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)scan_smem));
-    MB_CUDA_TRY(ctx, cudaFuncSetAttribute(sort_scatter_kernel,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)scatter_smem));
-    SortGrid *grid = (SortGrid *)ctx->sort_grid.ptr;
-    const unsigned *part = (const unsigned *)((char *)ctx->sort_grid.ptr + sizeof(SortGrid));
-    const float4 *hi = (const float4 *)ctx->pos_hi.ptr, *lo = (const float4 *)ctx->pos_lo.ptr;
-    int *H = (int *)ctx->sort_count.ptr;
-    unsigned *key = (unsigned *)ctx->sort_key.ptr;
-    sort_hist_kernel<<<tiles, 1024, hist_smem, s>>>(hi, n, T, part, nparts, nbits, grid, key, H);
-    sort_tile_scan_kernel<<<(B + 255) / 256, 256, 0, s>>>(H, tiles, B);
-    sort_scan_kernel<<<1, 1024, scan_smem, s>>>(H + tiles * (int64_t)B, B);
-    sort_scatter_kernel<<<tiles, 1024, scatter_smem, s>>>(key, n, T, H, tiles, B,
-                                                          (int *)ctx->sort_perm.ptr);
-    sort_pack_box_kernel<<<(int)nb, 256, 0, s>>>((const int *)ctx->sort_perm.ptr, n, hi, lo,
-                                                 (float4 *)ctx->sort_hi.ptr,
-                                                 (float4 *)ctx->sort_lo.ptr,
-                                                 (float *)ctx->sort_box.ptr);
-    count_launch(5);
-    MB_CUDA_TRY(ctx, cudaGetLastError());
+    const SortBufs b{(const float4 *)ctx->pos_hi.ptr, (const float4 *)ctx->pos_lo.ptr,
+                     (SortGrid *)ctx->sort_grid.ptr,  (unsigned *)ctx->sort_key.ptr,
+                     (int *)ctx->sort_perm.ptr,       (int *)ctx->sort_count.ptr,
+                     (float4 *)ctx->sort_hi.ptr,      (float4 *)ctx->sort_lo.ptr,
+                     (float *)ctx->sort_box.ptr};
+    MB_CUDA_TRY(ctx, sort_launch(b, n, nparts, ctx->sm_count, s));
     ctx->sorted_n = n;
     return MB_OK;
 }
@@ -958,9 +986,7 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
 {
     const int res = v == 3 ? 0 : wall ? f32_resident<true>(ctx, v) : f32_resident<false>(ctx, v);
     if (v == 4) {
-        // small problems: 64-target blocks, source chunks of 16 or more (half a
-        // tile: one warp per CTA walks fewer sources, more CTAs share the work)
-        const Plan p = make_plan(n, f32_targets_per_cta(4), res, 1024, kSmallNT / 2, kSmallNT / 2);
+        const Plan p = small_plan(n, res);
         double *out = u;
         const int direct = p.S == 1;
         if (!direct) {
@@ -1100,7 +1126,7 @@ mb_status matvec_pack_positions(mb_context *ctx, const double *r, int64_t n, cud
                       "spatial order"));
         pack_hilo_kernel<true><<<grid, 256, 0, s>>>(
             r, n, (float4 *)ctx->pos_hi.ptr, (float4 *)ctx->pos_lo.ptr,
-            (unsigned *)((char *)ctx->sort_grid.ptr + sizeof(SortGrid)));
+            sort_parts((SortGrid *)ctx->sort_grid.ptr));
     } else {
         pack_hilo_kernel<false><<<grid, 256, 0, s>>>(r, n, (float4 *)ctx->pos_hi.ptr,
                                                      (float4 *)ctx->pos_lo.ptr, nullptr);
@@ -1360,26 +1386,51 @@ mb_status render_flow(mb_context *ctx, const double *x, int64_t nt, const double
 // reserved it, so a cudaMalloc would fail or fragment it) and code on
 // latency-critical paths that cannot take cudaMalloc's implicit device
 // synchronisation.  The scratch that mb_mobility_matvec keeps in its context
-// (packed hi/lo positions and per-chunk partial sums) lives here in one
-// file-scope device array instead, sized for MB_NOALLOC_MAX_BLOBS blobs and at
-// most kNoallocMaxChunks source chunks.  Every GPU that loads the library
-// holds the array until the process exits.  All calls share it: calls whose
-// work overlaps on the GPU race on it.  Each call writes every element it
-// later reads, so nothing needs clearing between calls.
+// lives here in one file-scope device array instead, laid out for
+// MB_NOALLOC_MAX_BLOBS blobs.  Every GPU that loads the library holds the
+// array until the process exits.  All calls share it: calls whose work
+// overlaps on the GPU race on it.  Each call writes every element it later
+// reads, so nothing needs clearing between calls.
+//
+// The kernels and the rule by size are mb_mobility_matvec's: one-warp CTAs
+// and a reduction below kSymMinN, the symmetric kernel above, in the spatial
+// order from kSortMinN on.  A scalar kernel for every ordered pair ran at every
+// size: 5,003 blobs 121 -> 64 us, 65,536 13.1 -> 5.2 ms with the wall, 20,011
+// 705 -> 339 us and 65,536 6.0 -> 2.9 ms without (all against the first form).
 namespace {
 
 constexpr int64_t kNoallocMaxBlobs = MB_NOALLOC_MAX_BLOBS;
-constexpr int kNoallocMaxChunks = 8;
-constexpr size_t kNoallocPosBytes = sizeof(float4) * kNoallocMaxBlobs;
-constexpr size_t kNoallocBytes =
-    2 * kNoallocPosBytes + sizeof(double) * 3 * kNoallocMaxChunks * kNoallocMaxBlobs;
+constexpr int kNoallocPackCtas = 256;
+constexpr int kNoallocBits = 13;      // sort_bits(kNoallocMaxBlobs)
+constexpr int kNoallocMaxTiles = 64;  // sort_tiles(kNoallocMaxBlobs, any)
+static_assert(kNoallocMaxBlobs <= ((int64_t)8 << kNoallocBits) &&
+                  kNoallocMaxBlobs <= 1024 * (int64_t)kNoallocMaxTiles &&
+                  kNoallocMaxBlobs <= 256 * (int64_t)kNoallocPackCtas,
+              "the scratch holds the largest order");
+static_assert(kSymMinN * (kSymMinN / (kSmallNT / 2) + 1) <= kNoallocMaxBlobs,
+              "u holds the partial sums of the small problems");
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
+struct NoallocScratch {
+    float4 hi[kNoallocMaxBlobs], lo[kNoallocMaxBlobs];
+    float4 shi[kNoallocMaxBlobs], slo[kNoallocMaxBlobs];
+    double f[3 * kNoallocMaxBlobs], u[3 * kNoallocMaxBlobs];  // sorted; below kSymMinN u holds
+                                                              // the chunks' partial sums
+    unsigned key[kNoallocMaxBlobs];
+    int perm[kNoallocMaxBlobs];
+    int H[(kNoallocMaxTiles + 1) << kNoallocBits];
+    float box[6 * ((kNoallocMaxBlobs + kBoxBlobs - 1) / kBoxBlobs)];
+    struct {
+        SortGrid grid;
+        unsigned parts[6 * kNoallocPackCtas];
+    } sort;
+};
+
+static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoallocScratch)];
 
 struct NoallocDevice {
     bool ready = false;
-    unsigned char *scratch = nullptr;  // device address of g_noalloc_scratch
-    int resident_wall = 0, resident_free = 0;
+    NoallocScratch *scratch = nullptr;  // device address of g_noalloc_scratch
+    int sms = 0, resident_wall = 0, resident_free = 0;
 };
 constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mu;
@@ -1401,21 +1452,75 @@ mb_status noalloc_setup(int dev, NoallocDevice **out)
         }
         int sms = 0, occ_w = 0, occ_f = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_w, pair_f32_kernel<true, kTPT>,
-                                                          kNT, 0) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_f, pair_f32_kernel<false, kTPT>,
-                                                          kNT, 0) != cudaSuccess) {
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &occ_w, pair_f32x2_kernel<true, 1, kSmallNT>, kSmallNT, 0) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &occ_f, pair_f32x2_kernel<false, 1, kSmallNT>, kSmallNT, 0) != cudaSuccess) {
             cudaGetLastError();
             set_thread_err("device query failed in the allocation-free matvec set-up");
             return MB_ECUDA;
         }
-        d.scratch = (unsigned char *)ptr;
+        d.scratch = (NoallocScratch *)ptr;
+        d.sms = sms;
         d.resident_wall = std::max(1, occ_w) * sms;
         d.resident_free = std::max(1, occ_f) * sms;
         d.ready = true;
     }
     *out = &d;
     return MB_OK;
+}
+
+cudaError_t noalloc_run(const NoallocDevice &d, const double *r, const double *f, int64_t n,
+                        double a, double eta, int wall, double *u, cudaStream_t s)
+{
+    NoallocScratch *w = d.scratch;
+    const double scale = 1.0 / (6.0 * kPi * eta * a);
+    const int pack = (int)std::min<int64_t>(ceil_div(n, 256), kNoallocPackCtas);
+    const bool sorted = n >= kSortMinN;
+    if (sorted) pack_hilo_kernel<true><<<pack, 256, 0, s>>>(r, n, w->hi, w->lo, w->sort.parts);
+    else pack_hilo_kernel<false><<<pack, 256, 0, s>>>(r, n, w->hi, w->lo, nullptr);
+    count_launch();
+    if (n < kSymMinN) {
+        const Plan p = small_plan(n, wall ? d.resident_wall : d.resident_free);
+        const int direct = p.S == 1;
+        double *out = direct ? u : w->u;
+        if (wall) f32_launch<true>(4, p, s, w->hi, w->lo, f, n, a, out, scale, direct);
+        else f32_launch<false>(4, p, s, w->hi, w->lo, f, n, a, out, scale, direct);
+        count_launch();
+        if (!direct) launch_reduce_partials(out, n, p.S, scale, u, s);
+        return cudaGetLastError();
+    }
+    cudaError_t e = cudaSuccess;
+    double *us = u;
+    const SortGrid *sg = nullptr;
+    if (sorted) {
+        const SortBufs b{w->hi, w->lo, &w->sort.grid, w->key, w->perm, w->H, w->shi, w->slo, w->box};
+        e = sort_launch(b, n, pack, d.sms, s);
+        if (e != cudaSuccess) return e;
+        us = w->u;
+        sg = b.grid;
+        sort_gather_kernel<<<pack, 256, 0, s>>>(w->perm, n, f, w->f, us);
+        count_launch();
+        f = w->f;
+    } else {
+        if (overlap(u, f, n)) {  // u is zeroed and added to while f is read
+            e = cudaMemcpyAsync(w->f, f, sizeof(double) * 3 * (size_t)n, cudaMemcpyDeviceToDevice, s);
+            if (e != cudaSuccess) return e;
+            f = w->f;
+        }
+        e = cudaMemsetAsync(u, 0, sizeof(double) * 3 * (size_t)n, s);
+        if (e != cudaSuccess) return e;
+    }
+    const float4 *hi = sorted ? w->shi : w->hi, *lo = sorted ? w->slo : w->lo;
+    const float *box = sorted ? w->box : nullptr;
+    if (wall) launch_sym<true>(hi, lo, f, n, a, us, scale, box, sg, s);
+    else launch_sym<false>(hi, lo, f, n, a, us, scale, box, sg, s);
+    count_launch();
+    if (sorted) {
+        sort_scatter_u_kernel<<<pack, 256, 0, s>>>(w->perm, n, us, u);
+        count_launch();
+    }
+    return cudaGetLastError();
 }
 
 // Device memory of device `dev` (the one whose scratch array the call uses),
@@ -1467,31 +1572,9 @@ extern "C" mb_status mb_mobility_matvec_noalloc(const double *r, const double *f
     NoallocDevice *d = nullptr;
     mb_status st = noalloc_setup(dev, &d);
     if (st != MB_OK) return st;
-    cudaStream_t s = (cudaStream_t)stream;
-    float4 *hi = (float4 *)d->scratch;
-    float4 *lo = (float4 *)(d->scratch + kNoallocPosBytes);
-    double *partial = (double *)(d->scratch + 2 * kNoallocPosBytes);
-    const double scale = 1.0 / (6.0 * kPi * eta * a);
-    const int grid_pack = (int)std::min<int64_t>(ceil_div(n, 256), 1024);
-    pack_hilo_kernel<false><<<grid_pack, 256, 0, s>>>(r, n, hi, lo, nullptr);
-    count_launch();
-    const Plan p = make_plan(n, kNT * kTPT, wall ? d->resident_wall : d->resident_free,
-                             kNoallocMaxChunks);
-    const int direct = p.S == 1;
-    double *out = direct ? u : partial;
-    const MobConsts<float> k = MobConsts<float>::make(a);
-    if (wall)
-        pair_f32_kernel<true, kTPT><<<p.grid, kNT, 0, s>>>(hi, lo, f, n, p.chunk, p.n_tblocks,
-                                                           p.items, k, out, scale, direct);
-    else
-        pair_f32_kernel<false, kTPT><<<p.grid, kNT, 0, s>>>(hi, lo, f, n, p.chunk, p.n_tblocks,
-                                                            p.items, k, out, scale, direct);
-    count_launch();
-    if (!direct) {
-        launch_reduce_partials(partial, n, p.S, scale, u, s);
-    }
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = noalloc_run(*d, r, f, n, a, eta, wall, u, (cudaStream_t)stream);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         set_thread_err(cudaGetErrorString(e));
         return MB_ECUDA;
     }

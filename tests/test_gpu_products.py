@@ -156,3 +156,20 @@ def test_eval_within_a_small_budget():
         got = host(small.mobility_eval(dev(x), dev(r), dev(f), 0.5, 1.0, True, "fp32"))
         assert small.workspace_bytes() <= 200_000 < big.workspace_bytes()
     assert rel_l2(got, want) <= TOL["fp32"]
+
+
+@pytest.mark.parametrize("wall", [True, False])
+@pytest.mark.parametrize("n", [1, 33, 599, 600, 3001, 16383, 16384, 20011])
+def test_noalloc_every_size_and_in_place(ctx, n, wall):
+    """The allocation-free product takes the one-warp kernel below 600 blobs,
+    the symmetric one above and the spatial order from 16,384 on, and may
+    overwrite its forces; against the FP64 product."""
+    import paper_1602_02170_gb300 as mb
+
+    r, f = _cloud(n, n)
+    R, F = dev(r), dev(f)
+    ref = host(ctx.mobility_matvec(R, F, 0.5, 1.0, wall, "fp64"))
+    got = host(mb.mobility_matvec_noalloc(R, F, 0.5, 1.0, wall))
+    assert np.abs(got - ref).max() <= TOL["fp32"] * np.abs(ref).max()
+    mb.mobility_matvec_noalloc(R, F, 0.5, 1.0, wall, out=F)
+    assert np.abs(host(F) - got).max() <= 1e-14 * np.abs(ref).max()
