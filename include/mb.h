@@ -447,14 +447,12 @@ typedef struct {
  * together, on the serving engine below with every problem admitted at once.  All problems share `params` (a, eta, wall, tolerance,
  * iteration limits, precision).  The blob build, K, K^T and the block-
  * diagonal preconditioner of Section 2.2.2 run over all bodies of all
- * problems in one launch each; the pair kernel runs as one persistent launch
- * over all problems' (target block, source chunk) work items, so problems of
- * very different sizes share the GPU; each problem keeps its own GMRES
- * state and stops consuming pair-kernel work once converged.  The first
- * FP32 matvec times the packed kernel with 2 and 4 targets per thread and
- * the symmetric kernel (each unordered pair once for both blobs) and keeps
- * the fastest (autotuned tile shape).  The arena is sized exactly for
- * the batch.
+ * problems in one launch each; the pair kernel runs as one launch
+ * over all problems' pairs of blob blocks (each unordered pair once for both
+ * blobs; block sizes by the pairs of the batch), so problems of very
+ * different sizes share the GPU; each problem keeps its own GMRES
+ * state and stops consuming pair-kernel work once converged.  The arena
+ * is sized exactly for the batch.
  *
  * problems: host array of n_problems descriptors (pointing to device data);
  * infos: host array of n_problems (may be NULL), filled per problem

@@ -48,7 +48,7 @@ namespace {
 #endif
 constexpr int kNT = MB_PAIR_NT;
 constexpr double kPi = 3.14159265358979323846;
-constexpr int64_t kSeg = 4096;   // elements per vector chunk item
+constexpr int64_t kMaxSeg = 4096;  // elements per vector chunk item, at most
 constexpr int kRT = 256;         // threads of reduction kernels
 
 using clk = std::chrono::steady_clock;
@@ -274,30 +274,26 @@ __global__ void __launch_bounds__(kNT, NP == 1 ? 3 : 2) eng_x2_kernel(
     }
 }
 
-// Symmetric packed pair kernel over every listed request's block-pair
-// triangle (blocks of 2*kNT blobs); item -> request -> (I, J); results are
-// added to y with FP64 atomics (y zeroed beforehand).  n_tblocks holds the
-// request's block count.
-template <bool WALL>
-__global__ void __launch_bounds__(kNT, 2) eng_sym_kernel(
+// Symmetric packed pair kernel over every listed request's block pairs (blocks
+// of 2 NT blobs, an item being block I against half of block J as in
+// pair_sym_kernel); results are added to y with FP64 atomics (y zeroed
+// beforehand).  Bound by the FMA pipe once every SM has work: Engine::matvec
+// picks NT by the pairs of the tick.
+template <bool WALL, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) eng_sym_kernel(
     const Work *__restrict__ W, const int64_t *__restrict__ item_off, int nw, int64_t n_items,
     const int *__restrict__ mask, MobConsts2 k, double scale)
 {
-    __shared__ float4 sP[kX2SmemFloat4PerSource * kNT];
-    __shared__ float sRev[3 * kNT * (kNT / 32)];
+    __shared__ float4 sP[kX2SmemFloat4PerSource * NT];
+    __shared__ float sRev[3 * NT * (NT / 32)];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const Work P = W[find_owner(item_off, nw, item)];
         if (!mask[P.slot]) continue;
         const int64_t local = item - P.item_off + P.tri_lo;
-        const int64_t nb = P.n_tblocks;
-        int64_t lo_r = 0, hi_r = nb;
-        while (hi_r - lo_r > 1) {
-            const int64_t mid = (lo_r + hi_r) >> 1;
-            if (mid * nb - mid * (mid - 1) / 2 <= local) lo_r = mid;
-            else hi_r = mid;
-        }
-        const int64_t I = lo_r, J = I + (local - (I * nb - I * (I - 1) / 2));
-        x2sym_item<WALL, kNT>(sP, sRev, P.hi, P.lo, P.f, P.n, I, J, k, P.y, scale);
+        const int half = (int)(local & 1);
+        int64_t I, J;
+        triangle_pair(local >> 1, I, J);
+        x2sym_item<WALL, NT>(sP, sRev, P.hi, P.lo, P.f, P.n, I, J, k, P.y, scale, half, half + 1);
     }
 }
 
@@ -313,55 +309,53 @@ __global__ void eng_zero_kernel(const Work *__restrict__ W, const RSeg *__restri
     }
 }
 
-// Symmetric double-float kernel over every listed request's block-pair
-// triangle (blocks of kNT blobs); y zeroed beforehand; n_tblocks holds the
-// request's block count.
-constexpr int kDfNT = kNT / 2;  // threads: blocks of kNT blobs, two per thread
-
-template <bool WALL>
-__global__ void __launch_bounds__(kDfNT, 3) eng_df_kernel(const Work *__restrict__ W,
-                                                     const int64_t *__restrict__ item_off, int nw,
-                                                     int64_t n_items, const int *__restrict__ mask,
-                                                     MobConstsDf k, double scale)
+// The same in double-float (items as in pair_df_kernel).
+template <bool WALL, int NT>
+__global__ void __launch_bounds__(NT, 384 / NT) eng_df_kernel(
+    const Work *__restrict__ W, const int64_t *__restrict__ item_off, int nw, int64_t n_items,
+    const int *__restrict__ mask, MobConstsDf k, double scale)
 {
-    __shared__ float4 sD[7 * kDfNT];
-    __shared__ double sRev[3 * kDfNT * (kDfNT / 32)];
+    __shared__ float4 sD[7 * NT];
+    __shared__ double sRev[3 * NT * (NT / 32)];
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const Work P = W[find_owner(item_off, nw, item)];
         if (!mask[P.slot]) continue;
         const int64_t local = item - P.item_off;
-        const int64_t nb = P.n_tblocks;
-        int64_t lo_r = 0, hi_r = nb;
-        while (hi_r - lo_r > 1) {
-            const int64_t mid = (lo_r + hi_r) >> 1;
-            if (mid * nb - mid * (mid - 1) / 2 <= local) lo_r = mid;
-            else hi_r = mid;
-        }
-        const int64_t I = lo_r, J = I + (local - (I * nb - I * (I - 1) / 2));
-        for (int half = 0; half < 2; ++half) {
-            dfsym_item<WALL, kDfNT>(sD, sRev, P.hi, P.lo, P.f, P.n, I, J, half, k, P.y, scale);
-            __syncthreads();  // this half is done with sRev
-        }
+        int64_t I, J;
+        triangle_pair(local >> 1, I, J);
+        dfsym_item<WALL, NT>(sD, sRev, P.hi, P.lo, P.f, P.n, I, J, (int)(local & 1), k, P.y, scale);
+        __syncthreads();  // the item is done with sRev
     }
 }
 
-template <bool WALL>
-__global__ void __launch_bounds__(kNT) eng_f64_kernel(const Work *__restrict__ W,
-                                                      const int64_t *__restrict__ item_off, int nw,
-                                                      int64_t n_items, const int *__restrict__ mask,
-                                                      MobConsts<double> k, double scale)
+// The same in FP64: one-warp items of 32 targets and C sources (as in
+// pair_f64sym_kernel).
+template <bool WALL, int C>
+__global__ void __launch_bounds__(32) eng_f64sym_kernel(
+    const Work *__restrict__ W, const int64_t *__restrict__ item_off, int nw, int64_t n_items,
+    const int *__restrict__ mask, MobConsts<double> k, double scale)
 {
-    __shared__ double sm[6 * kNT];
+    __shared__ double sm[6 * C];
+    constexpr int kParts = 32 / C;
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const Work P = W[find_owner(item_off, nw, item)];
         if (!mask[P.slot]) continue;
-        const int64_t local = item - P.item_off;
-        const int tb = (int)(local % P.n_tblocks);
-        const int64_t sc = local / P.n_tblocks;
-        const int64_t j0 = sc * P.chunk, j1 = j0 + P.chunk < P.n ? j0 + P.chunk : P.n;
-        f64_item<WALL, kNT>(sm, P.r, P.n, P.r, P.f, tb, j0, j1, k,
-                            P.S == 1 ? P.y : P.part + 3 * sc * P.n, P.S == 1 ? scale : 1.0);
+        const int64_t local = item - P.item_off, t = local / kParts;
+        int64_t I, J;
+        triangle_pair(t, I, J);
+        const int64_t j0 = J * 32 + (local - t * kParts) * C;
+        if (j0 < P.n) f64sym_item<WALL, C>(sm, P.r, P.f, P.n, I, j0, I == J, k, P.y, scale);
+        __syncwarp();  // the item is done with sm
     }
+}
+
+// One launch over every item of the list.
+template <typename K, typename C>
+void eng_launch(K kernel, int threads, const Work *W, const int64_t *off, int nw, int64_t items,
+                const int *mask, const C &k, double scale, cudaStream_t s)
+{
+    kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(items, 1 << 30)), threads, 0, s>>>(
+        W, off, nw, items, mask, k, scale);
 }
 
 // y = scale * sum_s partial[s] for work entries with S > 1
@@ -825,9 +819,10 @@ struct Engine {
     bool mixed = false;
     double tick_pairs = -1;  // per-request pair budget of one tick's Arnoldi matvec (< 0: none)
     int max_bypass = 64;     // admissions that may overtake a queued request (< 0: none)
-    int np_variant = 1;     // FP32 tile shape: 1, 2 = packed with 2 or 4 targets per
-                            // thread, 3 = symmetric (autotuned)
-    std::map<int, int> tuned_by_class;  // autotuned tile shape per size class of a tick's pairs
+    int np_variant = 3;      // FP32 tile shape: 1, 2 = packed with 2 or 4 targets per
+                             // thread, 3 = symmetric
+    int sym_nt = 128;        // threads of the symmetric FP32 items
+    int64_t seg_len = kMaxSeg;  // elements per vector chunk item of this tick
 
     struct Req {
         int64_t ticket = 0;
@@ -986,6 +981,13 @@ struct Engine {
         return MB_OK;
     }
 
+    // Items of a symmetric product of n blobs: pairs of blocks of 2 nt blobs, two each.
+    static int64_t sym_items(int64_t n, int nt)
+    {
+        const int64_t nb = ceil_div(n, 2 * (int64_t)nt);
+        return nb * (nb + 1);
+    }
+
     // ------------------------------------------------------------ tick helpers
     void segs_of(const Req *rq, std::vector<Seg> &out, bool blobs_part = true, bool bodies_part = true)
     {
@@ -994,8 +996,8 @@ struct Engine {
                                        3 * n_cap + 6 * (rq->body_off + rq->prob.n_bodies)}};
         for (int k = 0; k < 2; ++k) {
             if ((k == 0 && !blobs_part) || (k == 1 && !bodies_part)) continue;
-            for (int64_t a = ranges[k][0]; a < ranges[k][1]; a += kSeg)
-                out.push_back(Seg{a, std::min(ranges[k][1], a + kSeg), rq->slot, 0});
+            for (int64_t a = ranges[k][0]; a < ranges[k][1]; a += seg_len)
+                out.push_back(Seg{a, std::min(ranges[k][1], a + seg_len), rq->slot, 0});
         }
     }
 
@@ -1027,24 +1029,25 @@ struct Engine {
     {
         if (list.empty()) return MB_OK;
         const double scale = 1.0 / (6.0 * kPi * prm.eta * prm.a);
-        const bool x2 = prec == MB_FP32_KAHAN;
-        const bool dfs = prec == MB_DF64;          // symmetric double-float
-        const bool sym = (x2 && np_variant == 3) || dfs;
-        const int tpc = x2 ? 2 * (np_variant == 3 ? 1 : np_variant) * kNT : kNT;
-        int occ = 1;
-        if (dfs)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_df_kernel<true>, kDfNT, 0);
-        else if (sym)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_sym_kernel<true>, kNT, 0);
-        else if (prec == MB_FP32_KAHAN)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_x2_kernel<true, 1>, kNT, 0);
-        else if (prec == MB_DF64)
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_df_kernel<true>, kDfNT, 0);
-        else
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_f64_kernel<true>, kNT, 0);
-        const int res = std::max(1, occ) * ctx->sm_count;
+        const bool x2 = prec == MB_FP32_KAHAN && np_variant != 3;  // a pinned packed variant
         double pairs = 0;
-        for (int sl : list) pairs += (double)running[sl]->prob.n_blobs * running[sl]->prob.n_blobs;
+        int64_t pairs32 = 0;  // pairs of 32-blob blocks
+        for (int sl : list) {
+            const int64_t n = running[sl]->prob.n_blobs, nb = ceil_div(n, 32);
+            pairs += (double)n * n;
+            pairs32 += nb * (nb + 1) / 2;
+        }
+        // Symmetric items of the whole list: blocks small enough that every SM
+        // has work, by the bounds measured for single products (pair_matvec.cu;
+        // FP32: sym_nt).
+        const int64_t want = 16 * 4 * (int64_t)ctx->sm_count;
+        const int df_nt = pairs < 24000.0 * 24000.0 ? 32 : 128;
+        const int fc = pairs32 >= want ? 32 : 2 * pairs32 >= want ? 16 : 4 * pairs32 >= want ? 8 : 4;
+        // packed items: targets per CTA, source chunk
+        const int tpc = 2 * np_variant * kNT;
+        int occ = 1;
+        if (x2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, eng_x2_kernel<true, 1>, kNT, 0);
+        const int res = std::max(1, occ) * ctx->sm_count;
         int64_t chunk = (int64_t)std::ceil(pairs / (8.0 * res) / tpc / kNT) * kNT;
         chunk = std::max<int64_t>(chunk, 2 * kNT);
         std::vector<Work> W;
@@ -1063,20 +1066,22 @@ struct Engine {
             wk.slot = rq->slot;
             wk.item_off = items;
             ioff.push_back(items);
-            if (sym) {
-                const int64_t nb = ceil_div(wk.n, tpc);
-                wk.n_tblocks = (int)nb;
+            if (!x2) {
                 wk.S = 1;
                 wk.chunk = wk.n;
-                wk.tri_lo = 0;
-                int64_t cnt = nb * (nb + 1) / 2;
-                if (tri && x2) {
+                if (prec == MB_FP64) {
+                    const int64_t nb = ceil_div(wk.n, 32);
+                    items += nb * (nb + 1) / 2 * (32 / fc);
+                } else if (prec == MB_DF64) {
+                    items += sym_items(wk.n, df_nt);
+                } else if (tri) {
                     wk.tri_lo = (int)(*tri)[li].first;
-                    cnt = (*tri)[li].second - (*tri)[li].first;
+                    items += (*tri)[li].second - (*tri)[li].first;
+                } else {
+                    items += sym_items(wk.n, sym_nt);
                 }
-                items += cnt;
-                for (int64_t a = 0; a < 3 * wk.n; a += kSeg)
-                    rs.push_back(RSeg{a, std::min<int64_t>(3 * wk.n, a + kSeg), (int)li, 0});
+                for (int64_t a = 0; a < 3 * wk.n; a += seg_len)
+                    rs.push_back(RSeg{a, std::min<int64_t>(3 * wk.n, a + seg_len), (int)li, 0});
                 W.push_back(wk);
                 continue;
             }
@@ -1087,8 +1092,8 @@ struct Engine {
             items += (int64_t)wk.n_tblocks * wk.S;
             if (wk.S > 1) {
                 wk.part = (double *)0 + part;  // offset, fixed up below
-                for (int64_t a = 0; a < 3 * wk.n; a += kSeg)
-                    rs.push_back(RSeg{a, std::min<int64_t>(3 * wk.n, a + kSeg), (int)li, 0});
+                for (int64_t a = 0; a < 3 * wk.n; a += seg_len)
+                    rs.push_back(RSeg{a, std::min<int64_t>(3 * wk.n, a + seg_len), (int)li, 0});
                 part += 3 * wk.n * wk.S;
             }
             W.push_back(wk);
@@ -1103,24 +1108,33 @@ struct Engine {
         RSeg *dR = upload(rs, toff, s, &stt);
         MB_TRY(stt);
         const int nw = (int)W.size();
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(items, res));
         const bool wall = prm.wall != 0;
         auto *ev = profile_begin(ctx, s);
-        if (sym) {
+        if (!x2) {
             eng_zero_kernel<<<grid_for((int64_t)rs.size(), 1), 256, 0, s>>>(
                 dW, dR, (int)rs.size(), zero_mask ? zero_mask : mask);
             count_launch();
         }
-        if (dfs) {
-            const MobConstsDf k = MobConstsDf::make(prm.a);
-            if (wall) eng_df_kernel<true><<<grid, kDfNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
-            else eng_df_kernel<false><<<grid, kDfNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
-        } else if (sym) {
+        if (prec == MB_DF64) {
+            const auto kern = df_nt == 32 ? (wall ? eng_df_kernel<true, 32> : eng_df_kernel<false, 32>)
+                                          : (wall ? eng_df_kernel<true, 128> : eng_df_kernel<false, 128>);
+            eng_launch(kern, df_nt, dW, dI, nw, items, mask, MobConstsDf::make(prm.a), scale, s);
+        } else if (prec == MB_FP64) {
+            const auto kern =
+                fc == 32   ? (wall ? eng_f64sym_kernel<true, 32> : eng_f64sym_kernel<false, 32>)
+                : fc == 16 ? (wall ? eng_f64sym_kernel<true, 16> : eng_f64sym_kernel<false, 16>)
+                : fc == 8  ? (wall ? eng_f64sym_kernel<true, 8> : eng_f64sym_kernel<false, 8>)
+                           : (wall ? eng_f64sym_kernel<true, 4> : eng_f64sym_kernel<false, 4>);
+            eng_launch(kern, 32, dW, dI, nw, items, mask, MobConsts<double>::make(prm.a), scale, s);
+        } else if (!x2) {
+            const auto kern =
+                sym_nt == 32   ? (wall ? eng_sym_kernel<true, 32> : eng_sym_kernel<false, 32>)
+                : sym_nt == 64 ? (wall ? eng_sym_kernel<true, 64> : eng_sym_kernel<false, 64>)
+                               : (wall ? eng_sym_kernel<true, 128> : eng_sym_kernel<false, 128>);
+            eng_launch(kern, sym_nt, dW, dI, nw, items, mask, MobConsts2::make(prm.a), scale, s);
+        } else {
             const MobConsts2 k = MobConsts2::make(prm.a);
-            if (wall) eng_sym_kernel<true><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
-            else eng_sym_kernel<false><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
-        } else if (prec == MB_FP32_KAHAN) {
-            const MobConsts2 k = MobConsts2::make(prm.a);
+            const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(items, res));
             if (np_variant == 1) {
                 if (wall) eng_x2_kernel<true, 1><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
                 else eng_x2_kernel<false, 1><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
@@ -1128,14 +1142,10 @@ struct Engine {
                 if (wall) eng_x2_kernel<true, 2><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
                 else eng_x2_kernel<false, 2><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
             }
-        } else {
-            const MobConsts<double> k = MobConsts<double>::make(prm.a);
-            if (wall) eng_f64_kernel<true><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
-            else eng_f64_kernel<false><<<grid, kNT, 0, s>>>(dW, dI, nw, items, mask, k, scale);
         }
         profile_end(ev, s);
         count_launch();
-        if (!rs.empty() && !sym) {
+        if (!rs.empty() && x2) {
             eng_reduce_kernel<<<grid_for((int64_t)rs.size(), 1), 256, 0, s>>>(dW, dR, (int)rs.size(),
                                                                            mask, scale);
             count_launch();
@@ -1237,6 +1247,13 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
         running[rq->slot] = rq;
         admitted.push_back(rq);
     }
+    // vector chunks: two or more for every SM, of 512 elements at least
+    {
+        int64_t len = 0;
+        for (const Req *rq : running)
+            if (rq) len += 3 * rq->prob.n_blobs + 6 * rq->prob.n_bodies;
+        seg_len = std::min(kMaxSeg, std::max<int64_t>(512, ceil_div(len, 2 * 256 * (int64_t)ctx->sm_count) * 256));
+    }
     if (!admitted.empty()) {
         std::vector<SlotIn> in;
         std::vector<int> slots;
@@ -1335,57 +1352,23 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
         *n_queued = (int)queue.size();
         return MB_OK;
     }
-    // tile shape: the context's pinned pair variant if any (the scalar
-    // variant maps to packed x2), else autotuned once per size class of the
-    // tick's pair work (powers of 4): small ticks favour the packed shapes,
-    // large ones the symmetric shape.  It stays fixed while a split matvec is
-    // in progress, since only the symmetric shape splits.
-    bool mid_split = false, tune = false;
+    // FP32 tile shape: the context's pinned pair variant if any (the scalar
+    // variant maps to packed x2), else the symmetric items, in blocks by the
+    // pairs of the tick: the bounds of launch_sym for one problem of as many
+    // pairs.  They stay fixed while a split matvec is in progress.  Measured on
+    // 12 problems of 228 to 2,850 blobs, the batch: 10.8 -> 7.9 ms against
+    // 256-thread packed items (63 to 111 CTAs, 109-191 us a product), which a
+    // trial of three shapes on each batch's first ticks had picked.
+    bool mid_split = false;
     double tick_pair_sum = 0;
     for (int sl : arn) {
         const Req *rq = running[sl];
         tick_pair_sum += (double)rq->prob.n_blobs * rq->prob.n_blobs;
         mid_split = mid_split || (rq->phase == 3 && rq->mv_next > 0);
     }
-    const int size_class = (int)(std::log2(std::max(1.0, tick_pair_sum)) / 2);
-    if (inner == MB_FP32_KAHAN && ctx->pair_variant >= 0) {
-        np_variant = std::min(3, std::max(1, ctx->pair_variant));
-    } else if (inner == MB_FP32_KAHAN && !mid_split) {
-        auto it = tuned_by_class.find(size_class);
-        if (it != tuned_by_class.end()) np_variant = it->second;
-        else tune = true;
-    }
-    if (tune) {
-        float best = 1e30f;
-        int best_v = 1;
-        cudaEvent_t e0, e1;
-        MB_CUDA_TRY(ctx, cudaEventCreate(&e0));
-        MB_CUDA_TRY(ctx, cudaEventCreate(&e1));
-        // time the candidates on every 8th active request (the size mix of
-        // the whole list at an eighth of its pair work), all of them when few
-        std::vector<int> sample;
-        for (size_t i = 0; i < arn.size(); i += (arn.size() >= 16 ? 8 : 1)) sample.push_back(arn[i]);
-        std::vector<int64_t> zk(sample.size(), 0);
-        std::vector<int> ones(s_cap, 0);
-        for (int sl : sample) ones[sl] = 1;
-        for (int cand = 1; cand <= 3; ++cand) {
-            np_variant = cand;
-            size_t off2 = 0;
-            int *dm = upload(ones, off2, s, &stt);
-            MB_TRY(stt);
-            MB_CUDA_TRY(ctx, cudaEventRecord(e0, s));
-            MB_TRY(matvec(sample, b, zk, t, zk, MB_FP32_KAHAN, dm, s, off2));
-            MB_CUDA_TRY(ctx, cudaEventRecord(e1, s));
-            MB_CUDA_TRY(ctx, cudaEventSynchronize(e1));
-            float ms = 0.f;
-            MB_CUDA_TRY(ctx, cudaEventElapsedTime(&ms, e0, e1));
-            if (ms < best) { best = ms; best_v = cand; }
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        np_variant = best_v;
-        tuned_by_class[size_class] = best_v;
-        toff = 0;
+    if (!mid_split) {
+        np_variant = ctx->pair_variant >= 0 ? std::min(3, std::max(1, ctx->pair_variant)) : 3;
+        sym_nt = tick_pair_sum < 3000.0 * 3000.0 ? 32 : tick_pair_sum < 12000.0 * 12000.0 ? 64 : 128;
     }
 
     // ---- 2. true residuals and cycle starts
@@ -1478,8 +1461,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
         std::vector<std::pair<int64_t, int64_t>> tri;
         for (int sl : arn) {
             Req *rq = running[sl];
-            const int64_t nblk = ceil_div(rq->prob.n_blobs, 2 * (int64_t)kNT);
-            const int64_t items = nblk * (nblk + 1) / 2;
+            const int64_t items = sym_items(rq->prob.n_blobs, sym_nt);
             if (rq->phase != 3 || rq->mv_next == 0) {
                 const double pairs = 0.5 * (double)rq->prob.n_blobs * rq->prob.n_blobs;
                 rq->mv_chunks = can_split
