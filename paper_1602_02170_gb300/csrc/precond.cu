@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kSetupThreads) precond_setup_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, MobConsts<double> k,
     double scale, double *__restrict__ P, double *__restrict__ scratch, int64_t scratch_stride,
-    int *__restrict__ flag, int flag_slot, int schur, const double *__restrict__ shift)
+    int *__restrict__ flag, const int *__restrict__ flag_slot, int schur, const double *__restrict__ shift)
 {
     extern __shared__ double sm[];
     for (int64_t p = blockIdx.x; p < nb; p += gridDim.x) {
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kSetupThreads) precond_setup_kernel(
         }
         if (bad) {
             if (threadIdx.x == 0) {
-                if (flag_slot >= 0) flag[flag_slot] = 2;
+                if (flag_slot) flag[flag_slot[p]] = 2;
                 else atomicMin(flag, (int)p);
             }
             __syncthreads();
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kSetupThreads) precond_setup_kernel(
         __syncthreads();
         if (bad) {
             if (threadIdx.x == 0) {
-                if (flag_slot >= 0) flag[flag_slot] = 2;
+                if (flag_slot) flag[flag_slot[p]] = 2;
                 else atomicMin(flag, (int)p);
             }
             __syncthreads();
@@ -511,7 +511,7 @@ template <bool L_SMEM>
 __global__ void __launch_bounds__(256) pc_factor_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
-    SplitScratch scr, int *__restrict__ flag, int flag_slot, int64_t p_base, int schur)
+    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base, int schur)
 {
     extern __shared__ double sm[];
     __shared__ int bad, pfail;
@@ -664,7 +664,7 @@ __global__ void __launch_bounds__(256) pc_factor_kernel(
         __syncthreads();
         if (fail) {  // uniform: a pivot was not positive
             if (threadIdx.x == 0) {
-                if (flag_slot >= 0) flag[flag_slot] = 2;
+                if (flag_slot) flag[flag_slot[p_base + p]] = 2;
                 else atomicMin(flag, (int)(p_base + p));
             }
             continue;
@@ -698,7 +698,7 @@ __global__ void __launch_bounds__(256) pc_factor_kernel(
         __syncthreads();
         if (bad) {
             if (threadIdx.x == 0) {
-                if (flag_slot >= 0) flag[flag_slot] = 2;
+                if (flag_slot) flag[flag_slot[p_base + p]] = 2;
                 else atomicMin(flag, (int)(p_base + p));
             }
             continue;
@@ -771,7 +771,7 @@ template <bool SROWS>
 __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc_factor_cluster_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
-    SplitScratch scr, int *__restrict__ flag, int flag_slot, int64_t p_base, int schur)
+    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base, int schur)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -1038,7 +1038,7 @@ __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc
         }
         if (fail) {
             if (rank == 0 && threadIdx.x == 0) {
-                if (flag_slot >= 0) flag[flag_slot] = 2;
+                if (flag_slot) flag[flag_slot[p_base + p]] = 2;
                 else atomicMin(flag, (int)(p_base + p));
             }
             continue;
@@ -1085,7 +1085,7 @@ __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc
             __syncthreads();
             if (bad) {
                 if (threadIdx.x == 0) {
-                    if (flag_slot >= 0) flag[flag_slot] = 2;
+                    if (flag_slot) flag[flag_slot[p_base + p]] = 2;
                     else atomicMin(flag, (int)(p_base + p));
                 }
             } else if (threadIdx.x < 36) {
@@ -1680,7 +1680,7 @@ __global__ void __launch_bounds__(256) pc_keep_factor_kernel(
 // with `factored`).
 mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double *q,
                       const int64_t *start, const int64_t *poff, double *P, int max_np, double a,
-                      double eta, int wall, int *flag, int flag_slot, int schur, cudaStream_t s,
+                      double eta, int wall, int *flag, const int *flag_slot, int schur, cudaStream_t s,
                       const double *shift, bool factored = false)
 {
     const int nmax = 3 * max_np;
@@ -1739,7 +1739,7 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
                                                   (int)tsm));
             pc_trinv_smem_kernel<<<gt, 32 * kTrinvSmemWarps, tsm, s>>>(ng, st, po, P, scr,
                                                                       col_groups);
-        } else if (nmax <= 4 * kTile) {
+        } else if (nmax <= kSetupSmallRows) {
             // double-float S3 and S4 (see pc_to_df_kernel)
             const int gc = (int)std::min<int64_t>(ceil_div(ng * nmax, 8), 8 * (int64_t)ctx->sm_count);
             pc_to_df_kernel<<<gc, 256, 0, s>>>(ng, st, po, P, scr);
@@ -1901,13 +1901,13 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
         if (nmax <= kSplitMaxRowsSmem)
             return setup_split(ctx, nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,
                                (const int64_t *)ctx->pinv_off.ptr, (double *)ctx->pinv.ptr, max_np,
-                               a, eta, wall, (int *)ctx->flag.ptr, -1, schur, s, shift, factored);
+                               a, eta, wall, (int *)ctx->flag.ptr, nullptr, schur, s, shift, factored);
         MB_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
         kern<<<grid, kSetupThreads, smem, s>>>(nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,
                                                (const int64_t *)ctx->pinv_off.ptr, k, scale,
                                                (double *)ctx->pinv.ptr, scratch, stride,
-                                               (int *)ctx->flag.ptr, -1, schur, shift);
+                                               (int *)ctx->flag.ptr, nullptr, schur, shift);
         count_launch();
         MB_CUDA_TRY(ctx, cudaGetLastError());
         return MB_OK;
@@ -1941,9 +1941,15 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
     return MB_OK;
 }
 
+size_t precond_scratch_bytes(int64_t nb, int max_np)
+{
+    return std::min<size_t>(sizeof(double) * (size_t)nb * split_stride(3 * max_np),
+                            (size_t)MB_SETUP_SCRATCH_MB << 20);
+}
+
 mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, const double *q,
                               const int64_t *start, const int64_t *poff, double *P, int max_np,
-                              double a, double eta, int wall, int *flags, int flag_slot,
+                              double a, double eta, int wall, int *flags, const int *flag_slot,
                               cudaStream_t s, int schur)
 {
     const int nmax = 3 * max_np;
@@ -2076,7 +2082,7 @@ mb_status precond_setup_shared(mb_context *ctx, int64_t nb, int64_t n, const dou
         max_ref_np = std::max<int>(max_ref_np, (int)(rstart[t + 1] - rstart[t]));
     MB_TRY(precond_setup_range(ctx, ns, dref, dref + 3 * rstart[ns], dstart, doff,
                                (double *)ctx->pinv.ptr, max_ref_np, a, eta, 0,
-                               (int *)ctx->flag.ptr, -1, s, schur));
+                               (int *)ctx->flag.ptr, nullptr, s, schur));
     int first_bad = big;
     MB_CUDA_TRY(ctx, cudaMemcpyAsync(&first_bad, ctx->flag.ptr, sizeof(int),
                                      cudaMemcpyDeviceToHost, s));

@@ -1271,29 +1271,63 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
                                                           q, theta, F, T, bstart, body_b0, body_b1,
                                                           blob_slot, body_slot, blob_body, st.bad);
         count_launch();
-        for (Req *rq : admitted) {
-            const int64_t b0 = rq->blob_off, b1 = rq->blob_off + rq->prob.n_blobs;
+        // Blob build and preconditioner of each run of requests that lie next
+        // to each other in the arena (all of a batch): a request's bodies alone
+        // are too few for the setup's kernels, and one after the other each
+        // waits for the last one's longest body.  Runs hold small bodies only
+        // (the setup's kernels follow the largest one), and no more of them
+        // than a quarter of the budget left holds scratch for.
+        // 12 problems of 8 to 100 bodies, the batch: 7.9 -> 5.6 ms.
+        for (size_t i = 0; i < admitted.size();) {
+            const Req *first = admitted[i], *prev = first;
+            int64_t nb = first->prob.n_bodies, nblob = first->prob.n_blobs;
+            int max_np = first->max_np;
+            size_t end = i + 1;
+            const size_t room = ctx->budget > ctx->held ? ctx->budget - ctx->held : 0;
+            for (; end < admitted.size(); ++end) {
+                const Req *rq = admitted[end];
+                const int np = std::max(max_np, rq->max_np);
+                if (rq->blob_off != prev->blob_off + prev->prob.n_blobs ||
+                    rq->body_off != prev->body_off + prev->prob.n_bodies ||
+                    rq->start_off != prev->start_off + prev->prob.n_bodies + 1 ||
+                    3 * np > kSetupSmallRows ||
+                    precond_scratch_bytes(nb + rq->prob.n_bodies, np) > std::max(room / 4, ctx->sol_dots.bytes))
+                    break;
+                nb += rq->prob.n_bodies;
+                nblob += rq->prob.n_blobs;
+                max_np = np;
+                prev = rq;
+            }
+            const int64_t b0 = first->blob_off, b1 = b0 + nblob;
             eng_blob_kernel<<<grid_for(b1 - b0, 256), 256, 0, s>>>(blob_body, b0, b1, q, theta, rho, r);
             eng_pack_kernel<<<grid_for(b1 - b0, 256), 256, 0, s>>>(r, b0, b1, hi, lo);
             count_launch(2);
-            // preconditioner offsets of this request's bodies in the P range
-            std::vector<int64_t> po(rq->prob.n_bodies);
-            int64_t acc = rq->pc_off;
-            for (int64_t p = 0; p < rq->prob.n_bodies; ++p) {
-                po[p] = acc;
-                const int64_t np = rq->hstart[p + 1] - rq->hstart[p];
-                acc += (3 * np + 6) * (3 * np + 6);
+            // the run's blob ranges (over its requests' own, which hold one
+            // entry more each) and preconditioner offsets
+            std::vector<int64_t> po, bs;
+            po.reserve(nb);
+            bs.reserve(nb + 1);
+            for (; i < end; ++i) {
+                const Req *rq = admitted[i];
+                int64_t acc = rq->pc_off;
+                for (int64_t p = 0; p < rq->prob.n_bodies; ++p) {
+                    po.push_back(acc);
+                    bs.push_back(rq->blob_off + rq->hstart[p]);
+                    const int64_t np = rq->hstart[p + 1] - rq->hstart[p];
+                    acc += (3 * np + 6) * (3 * np + 6);
+                }
             }
-            MB_CUDA_TRY(ctx, cudaMemcpyAsync(poff + rq->body_off, po.data(),
+            bs.push_back(b1);
+            MB_CUDA_TRY(ctx, cudaMemcpyAsync(poff + first->body_off, po.data(),
                                              sizeof(int64_t) * po.size(), cudaMemcpyHostToDevice, s));
-            // the copy reads a host vector: make it complete before it goes out of scope
+            MB_CUDA_TRY(ctx, cudaMemcpyAsync(bstart + first->start_off, bs.data(),
+                                             sizeof(int64_t) * bs.size(), cudaMemcpyHostToDevice, s));
+            // the copies read host vectors: make them complete before these go out of scope
             MB_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-            int max_np = 0;
-            for (int64_t p = 0; p < rq->prob.n_bodies; ++p)
-                max_np = std::max<int>(max_np, (int)(rq->hstart[p + 1] - rq->hstart[p]));
-            MB_TRY(precond_setup_range(ctx, rq->prob.n_bodies, r, q + 3 * rq->body_off,
-                                       bstart + rq->start_off, poff + rq->body_off, P, max_np,
-                                       prm.a, prm.eta, prm.wall, st.bad, rq->slot, s));
+            MB_TRY(precond_setup_range(ctx, nb, r, q + 3 * first->body_off,
+                                       bstart + first->start_off, poff + first->body_off, P, max_np,
+                                       prm.a, prm.eta, prm.wall, st.bad,
+                                       body_slot + first->body_off, s));
         }
         std::vector<Seg> segs;
         std::vector<int> seg_off, list;

@@ -144,3 +144,33 @@ def test_batch_with_a_zero_force_problem(ctx):
     assert torch.count_nonzero(U1) == 0 and torch.count_nonzero(lam1) == 0
     alone = ctx.solve_batch([P0], s0.a, tol=1e-10, prec="mixed")[0]
     assert rel_l2(host(res[0][0]), host(alone[0])) <= 1e-9
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64", "df64"])
+@pytest.mark.parametrize("bodies", [[1, 2, 1], [20, 1, 33], [90, 70]])
+def test_batch_block_sizes(ctx, bodies, prec):
+    """The engine's symmetric items take blocks by the pairs of a tick (the
+    first set stays below 3,000^2, the last above) and the FP64 ones 4 to 32
+    sources, for problems of one block and of many; every request's bodies
+    are set up together.  Against the same problems solved alone."""
+    susp = [I.mixed_suspension(70 + k, nb) for k, nb in enumerate(bodies)]
+    res = ctx.solve_batch([_prob(s) for s in susp], A, 1.0, True, tol=1e-10, prec=prec)
+    for s, (U, W, lam, info) in zip(susp, res):
+        p = _prob(s)
+        Ua, Wa, la, _ = ctx.solve_mobility(p["q"], p["theta"], p["blob_start"], p["rho"], p["F"],
+                                           p["T"], A, 1.0, True, tol=1e-10, prec=prec)
+        assert info["converged"] == 1
+        assert rel_l2(host(U), host(Ua)) <= 1e-6
+        assert rel_l2(host(W), host(Wa)) <= 1e-6
+        assert rel_l2(host(lam), host(la)) <= 1e-5
+
+
+def test_batch_singular_request_among_joint_setups(ctx):
+    """A blob at a / 2 fails its own request only, and the batch names it."""
+    susp = [I.mixed_suspension(80 + k, 5) for k in range(3)]
+    r = O.blob_positions(susp[1].q, susp[1].theta, susp[1].blob_start, susp[1].rho)
+    lo, hi = susp[1].blob_start[3], susp[1].blob_start[4]
+    susp[1].q[3, 2] -= r[lo:hi, 2].min() - 0.5 * A
+    with pytest.raises(mb.MBError) as ei:
+        ctx.solve_batch([_prob(s) for s in susp], A, 1.0, True, tol=1e-10, prec="mixed")
+    assert ei.value.name == "MB_ESINGULAR" and "problem 1" in str(ei.value)
