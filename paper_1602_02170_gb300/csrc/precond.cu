@@ -500,87 +500,123 @@ __device__ __forceinline__ double k_entry(const double *__restrict__ rb, double 
          : e3 == 6 ? dy : e3 == 7 ? -dx : 0.0;
 }
 
-// S2: one CTA per body.  Right-looking Cholesky on the lower triangle with
-// the six columns B = K_p appended (so that B ends as G = L^-1 K_p): step c
-// scales column c by 1/sqrt(d_c), then subtracts its outer product from the
-// trailing triangle and its multiples of row c from the rows of B below,
-// one FP64 FMA per entry (FP64 issue is the bound on this chip).  Blocks in
-// shared memory take the steps in panels of kPanel columns; blocks in global
-// memory use the left-looking order.
-template <bool L_SMEM>
-__global__ void __launch_bounds__(256) pc_factor_kernel(
+// A double as stored for S3: packed double-float (DF) or FP64.
+__device__ __forceinline__ double df_pack(dfl v)
+{
+    return __hiloint2double(__float_as_int(v.hi), __float_as_int(v.lo));
+}
+
+__device__ __forceinline__ dfl df_unpack(double d)
+{
+    return dfl(__int_as_float(__double2hiint(d)), __int_as_float(__double2loint(d)));
+}
+
+__device__ __forceinline__ dfl df_of(double d)
+{
+    const float h = (float)d;
+    return dfl(h, (float)(d - (double)h));
+}
+
+template <bool DF>
+__device__ __forceinline__ double s3_input(double v)
+{
+    return DF ? df_pack(df_of(v)) : v;
+}
+
+// The Cholesky factor of an 8 x 8 block (w <= 8 rows) by one warp: lane l + 8 g
+// holds entries (l, g) and (l, g + 4) in v0, v1, so that a pivot costs two FMAs
+// per lane rather than one per later column; the column loop unrolled, the
+// other lanes' entries by shuffles.  Entries above a row's diagonal may take
+// finite junk and are never read.  il[c] = 1 / L_cc.  Returns 1 in every lane
+// if a pivot is not positive.
+__device__ __forceinline__ int panel_cholesky8(double &v0, double &v1, int w, int lane,
+                                               double *__restrict__ ils)
+{
+    const int l = lane & 7, g = lane >> 3;
+    int f = 0;
+#pragma unroll
+    for (int c = 0; c < kPanel; ++c) {
+        if (c < w && !f) {
+            const int sc = 8 * (c & 3);  // lanes of column c: sc .. sc + 7
+            double &vc = c < 4 ? v0 : v1;
+            const double d = __shfl_sync(0xffffffffu, vc, c + sc);
+            if (!pivot_ok(d)) {
+                f = 1;  // the same value in every lane
+            } else {
+                const double il = pivot_rsqrt(d);
+                if (lane == 0) ils[c] = il;
+                vc *= g == (c & 3) && l >= c ? il : 1.0;  // lane (c, .): sqrt(d)
+                double lac = __shfl_sync(0xffffffffu, vc, l + sc);  // L[l][c]
+                lac = l > c && l < w ? lac : 0.0;
+                if (c < 4) {
+                    const double x0 = __shfl_sync(0xffffffffu, vc, g + sc);  // L[g][c]
+                    v0 -= (g > c ? lac : 0.0) * x0;
+                }
+                const double x1 = __shfl_sync(0xffffffffu, vc, g + 4 + sc);  // L[g+4][c]
+                v1 -= (g + 4 > c ? lac : 0.0) * x1;
+            }
+        }
+    }
+    return f;
+}
+
+// S2, 3 n_p <= kSmemMaxRows: one CTA per body, for more bodies than clusters
+// fit at once.  Right-looking Cholesky in shared memory with the six columns
+// B = K_p appended (so that B ends as G = L^-1 K_p), in panels of kPanel
+// columns: warp 0 factors the diagonal block, then the rows below it and the
+// panel's six B columns solve against it (one row a thread), then every thread
+// takes entries of the trailing triangle and of B, eight FMAs each.
+//
+// Bound by the issue of FP64 instructions (one per ~76 cycles and sub-partition,
+// whatever the lanes do), so what counts is that every lane of each has work:
+// the triangle is dealt out entry by entry and not row by row (a third of the
+// lanes of 32-column pieces of rows are idle), and the rows of the lower
+// triangle lie back to back, so that two CTAs fit an SM and one's serial
+// diagonal blocks run beside the other's updates.  300 bodies of 126 and 45
+// rows in turn, setup and application: 1,260 -> 851 us against a square block, a
+// panel of all rows on one warp and rows dealt to warps (672 us in that kernel
+// and 34 in the conversion of its outputs, which is now done here).
+template <bool DF>
+__global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
-    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base, int schur)
+    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base,
+    int schur)
 {
     extern __shared__ double sm[];
     __shared__ int bad, pfail;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nmax = scr.nmax;
+    double *L = sm;                                       // rows of the lower triangle
+    double *B = L + (size_t)nmax * (nmax + 1) / 2;        // n x 6
+    double *pT = B + 6 * nmax;                            // the panel's columns, kPanel x nmax
+    double *ils = pT + (size_t)kPanel * nmax;             // 1 / L_cc
+    double *S = ils + nmax, *Nm = S + 36;
+    auto row = [&](int i) { return L + i * (i + 1) / 2; };
     for (int64_t p = blockIdx.x; p < nb; p += gridDim.x) {
         const int64_t b0 = start[p];
         const int np = (int)(start[p + 1] - b0);
         const int n = 3 * np, m = n + 6;
         double *Pp = P + poff[p];
-        double *L = L_SMEM ? sm : Pp;
-        const int ld = L_SMEM ? n : m;
-        double *B = L_SMEM ? sm + (size_t)n * n : scr.G(p);
-        double *ils = L_SMEM ? B + 6 * n : sm;  // 1 / sqrt(d_c)
-        double *S = ils + n;
-        double *Nm = S + 36;
-        double *col = Nm + 36;  // pivot row (global blocks) / kPanel scaled columns (shared)
         const double qx = q[3 * p], qy = q[3 * p + 1], qz = q[3 * p + 2];
-        __syncthreads();
+        __syncthreads();  // done with the previous body
         if (threadIdx.x == 0) bad = 0;
-        if (L_SMEM)
-            for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-                const int i = e / n, j = e % n;
-                if (j <= i) L[e] = Pp[(size_t)i * m + j];
-            }
-        // B = K_p: rows of blob i are [I, -[d_i]x]
+        for (int i = warp; i < n; i += nw)
+            for (int j = lane; j <= i; j += 32) row(i)[j] = Pp[(size_t)i * m + j];
         for (int e = threadIdx.x; e < 6 * n; e += blockDim.x)
             B[e] = k_entry(r + 3 * b0, qx, qy, qz, e / 6, e % 6);
         int fail = 0;
-        if constexpr (L_SMEM) {
-        // Blocked order: warp 0 factors a panel of kPanel columns (rows c0..n-1)
-        // warp-synchronously, keeping the scaled columns transposed in pT
-        // (rows read without bank conflicts); then every warp subtracts the
-        // panel's rank-kPanel product from the trailing triangle and from
-        // the rows of B below the panel.  The same FMAs as column by column,
-        // with two CTA barriers per panel instead of two per column.
-        double *pT = col;
         for (int c0 = 0; c0 < n; c0 += kPanel) {
-            const int w = n - c0 < kPanel ? n - c0 : kPanel;
-            __syncthreads();  // the previous trailing update is complete
+            const int w = n - c0 < kPanel ? n - c0 : kPanel, t0 = c0 + w, nr = n - t0;
+            __syncthreads();  // the previous update is complete
             if (warp == 0) {
-                int f = 0;
-                for (int c = c0; c < c0 + w; ++c) {
-                    const double d = L[(size_t)c * ld + c];
-                    if (!pivot_ok(d)) {  // the same value in every lane
-                        f = 1;
-                        break;
-                    }
-                    const double il = pivot_rsqrt(d);
-                    if (lane == 0) ils[c] = il;
-                    double *pc = pT + (size_t)(c - c0) * n;
-                    for (int i = c + lane; i < n; i += 32) {
-                        const double v = L[(size_t)i * ld + c] * il;
-                        L[(size_t)i * ld + c] = v;
-                        pc[i] = v;
-                    }
-                    if (lane < 6) B[6 * c + lane] *= il;
-                    __syncwarp();
-                    // the panel's later columns, and the rows of B inside the panel
-                    const int ce = c0 + w - 1;
-                    for (int i = c + 1 + lane; i < n; i += 32) {
-                        const double lic = pc[i];
-                        const int top = i < ce ? i : ce;
-                        for (int cc = c + 1; cc <= top; ++cc) L[(size_t)i * ld + cc] -= lic * pc[cc];
-                    }
-                    for (int e = lane; e < 6 * (ce - c); e += 32) {
-                        const int i = c + 1 + e / 6, b = e % 6;
-                        B[6 * i + b] -= pc[i] * B[6 * c + b];
-                    }
-                    __syncwarp();
+                const int l = lane & 7, g = lane >> 3;
+                double v0 = l < w && g <= l ? row(c0 + l)[c0 + g] : 0.0;
+                double v1 = l < w && g + 4 <= l ? row(c0 + l)[c0 + g + 4] : 0.0;
+                const int f = panel_cholesky8(v0, v1, w, lane, ils + c0);
+                if (l < w) {
+                    if (g <= l) row(c0 + l)[c0 + g] = v0;
+                    if (g + 4 <= l) row(c0 + l)[c0 + g + 4] = v1;
                 }
                 if (lane == 0) pfail = f;
             }
@@ -589,30 +625,140 @@ __global__ void __launch_bounds__(256) pc_factor_kernel(
                 fail = 1;
                 break;
             }
-            const int t0 = c0 + w;
-            for (int i = t0 + warp; i < n; i += nw) {
-                double li[kPanel];
+            for (int e = threadIdx.x; e < nr + 6; e += blockDim.x) {
+                // a row below the block (w = kPanel then) or a column of B
+                double y[kPanel];
 #pragma unroll
-                for (int kk = 0; kk < kPanel; ++kk) li[kk] = kk < w ? pT[(size_t)kk * n + i] : 0.0;
-                double *Li = L + (size_t)i * ld;
-                for (int j = t0 + lane; j <= i; j += 32) {
-                    double acc = Li[j];
+                for (int k = 0; k < kPanel; ++k)
+                    y[k] = k >= w ? 0.0 : e < nr ? row(t0 + e)[c0 + k] : B[6 * (c0 + k) + e - nr];
 #pragma unroll
-                    for (int kk = 0; kk < kPanel; ++kk)
-                        if (kk < w) acc -= li[kk] * pT[(size_t)kk * n + j];
-                    Li[j] = acc;
+                for (int k = 0; k < kPanel; ++k) {
+                    if (k >= w) break;
+                    y[k] *= ils[c0 + k];
+#pragma unroll
+                    for (int j = k + 1; j < kPanel; ++j)
+                        if (j < w) y[j] -= y[k] * row(c0 + j)[c0 + k];
                 }
-                if (lane < 6) {
-                    double acc = B[6 * i + lane];
 #pragma unroll
-                    for (int kk = 0; kk < kPanel; ++kk)
-                        if (kk < w) acc -= li[kk] * B[6 * (c0 + kk) + lane];
-                    B[6 * i + lane] = acc;
+                for (int k = 0; k < kPanel; ++k) {
+                    if (k >= w) break;
+                    if (e < nr) {
+                        row(t0 + e)[c0 + k] = y[k];
+                        pT[(size_t)k * nmax + t0 + e] = y[k];
+                    } else {
+                        B[6 * (c0 + k) + e - nr] = y[k];
+                    }
                 }
             }
+            __syncthreads();
+            const int tri = nr * (nr + 1) / 2;
+            for (int e = threadIdx.x; e < tri + 6 * nr; e += blockDim.x) {
+                int i, j;
+                const double *other;  // the second factors, `step` apart
+                int step;
+                double *dst;
+                if (e < tri) {
+                    tri_index(e, i, j);
+                    i += t0;
+                    j += t0;
+                    dst = row(i) + j;
+                    other = pT + j;
+                    step = nmax;
+                } else {
+                    i = t0 + (e - tri) / 6;
+                    j = (e - tri) % 6;
+                    dst = B + 6 * i + j;
+                    other = B + 6 * c0 + j;
+                    step = 6;
+                }
+                double acc = *dst;
+#pragma unroll
+                for (int k = 0; k < kPanel; ++k) acc -= pT[(size_t)k * nmax + i] * other[k * step];
+                *dst = acc;
+            }
         }
-        } else {
-        // Block in global memory: left-looking (Crout) order.  Column j is
+        __syncthreads();
+        if (fail) {  // uniform: a pivot was not positive
+            if (threadIdx.x == 0) {
+                if (flag_slot) flag[flag_slot[p_base + p]] = 2;
+                else atomicMin(flag, (int)(p_base + p));
+            }
+            continue;
+        }
+        // dW, G to scratch; L^T into P_p's upper triangle (row k holds column k of L)
+        double *dW = scr.dW(p), *G = scr.G(p);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) dW[i] = s3_input<DF>(ils[i]);
+        for (int e = threadIdx.x; e < 6 * n; e += blockDim.x) G[e] = s3_input<DF>(B[e]);
+        for (int k = warp; k < n; k += nw)
+            for (int i = k + lane; i < n; i += 32)
+                Pp[(size_t)k * m + i] = i == k ? row(i)[k] : s3_input<DF>(row(i)[k]);
+        // S = G^T G (symmetric 6 x 6), one warp per entry of its lower triangle
+        for (int e = warp; e < 21; e += nw) {
+            int a, bb;
+            tri_index(e, a, bb);
+            double acc = 0.0;
+            for (int i = lane; i < n; i += 32) acc += B[6 * i + a] * B[6 * i + bb];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) S[6 * a + bb] = S[6 * bb + a] = acc;
+        }
+        __syncthreads();
+        // N = S^-1 (warp 0)
+        if (warp == 0) {
+            const int f = inverse6_warp(S, Nm, lane);
+            if (lane == 0 && f) bad = schur;
+        }
+        __syncthreads();
+        if (bad) {
+            if (threadIdx.x == 0) {
+                if (flag_slot) flag[flag_slot[p_base + p]] = 2;
+                else atomicMin(flag, (int)(p_base + p));
+            }
+            continue;
+        }
+        if (threadIdx.x < 36) {
+            scr.N(p)[threadIdx.x] = s3_input<DF>(Nm[threadIdx.x]);
+            Pp[(size_t)(n + threadIdx.x / 6) * m + n + threadIdx.x % 6] = -Nm[threadIdx.x];
+        }
+    }
+}
+
+size_t factor_small_smem(int nmax)
+{
+    return sizeof(double) * ((size_t)nmax * (nmax + 1) / 2 + (7 + kPanel) * (size_t)nmax + 72);
+}
+
+// S2 for larger blocks: one CTA per body, factored in place in global memory
+// with the six columns B = K_p appended in the scratch.
+__global__ void __launch_bounds__(256) pc_factor_kernel(
+    int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
+    const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
+    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base,
+    int schur)
+{
+    extern __shared__ double sm[];
+    __shared__ int bad;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int64_t p = blockIdx.x; p < nb; p += gridDim.x) {
+        const int64_t b0 = start[p];
+        const int np = (int)(start[p + 1] - b0);
+        const int n = 3 * np, m = n + 6;
+        double *Pp = P + poff[p];
+        double *L = Pp;
+        const int ld = m;
+        double *B = scr.G(p);
+        double *ils = sm;  // 1 / sqrt(d_c)
+        double *S = ils + n;
+        double *Nm = S + 36;
+        double *col = Nm + 36;  // pivot row
+        const double qx = q[3 * p], qy = q[3 * p + 1], qz = q[3 * p + 2];
+        __syncthreads();
+        if (threadIdx.x == 0) bad = 0;
+        // B = K_p: rows of blob i are [I, -[d_i]x]
+        for (int e = threadIdx.x; e < 6 * n; e += blockDim.x)
+            B[e] = k_entry(r + 3 * b0, qx, qy, qz, e / 6, e % 6);
+        int fail = 0;
+        // Left-looking (Crout) order.  Column j is
         // L[i][j] = (A[i][j] - L[i][0:j] . L[j][0:j]) / L[j][j], one coalesced
         // dot product per row with the pivot row L[j][0:j] in shared memory
         // (`col`); every entry is written once, so the inner loop only loads
@@ -660,7 +806,6 @@ __global__ void __launch_bounds__(256) pc_factor_kernel(
                 }
             }
         }
-        }
         __syncthreads();
         if (fail) {  // uniform: a pivot was not positive
             if (threadIdx.x == 0) {
@@ -669,15 +814,12 @@ __global__ void __launch_bounds__(256) pc_factor_kernel(
             }
             continue;
         }
-        // dW, G to scratch; L^T into P_p's upper triangle (row k holds column k of L)
-        double *dW = scr.dW(p), *G = scr.G(p);
+        // dW to scratch; L^T into P_p's upper triangle (row k holds column k of L)
+        double *dW = scr.dW(p);
         for (int i = threadIdx.x; i < n; i += blockDim.x) dW[i] = ils[i];
-        if (L_SMEM)
-            for (int e = threadIdx.x; e < 6 * n; e += blockDim.x) G[e] = B[e];
         for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
             const int kk = e / n, i = e % n;
             if (i > kk) Pp[(size_t)kk * m + i] = L[(size_t)i * ld + kk];
-            else if (L_SMEM && i == kk) Pp[(size_t)kk * m + kk] = L[(size_t)kk * ld + kk];
         }
         __syncthreads();
         // S = G^T G (symmetric 6 x 6), one warp per entry
@@ -767,7 +909,7 @@ __device__ __forceinline__ double panel_solve8(double y, const double (&dk)[kPan
 // memory, each CTA updating its own rows and reading the others' rows
 // through L2 (ld.global.cg) after the cluster barriers, which order global
 // memory at cluster scope as well.
-template <bool SROWS>
+template <bool SROWS, bool DF>
 __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc_factor_cluster_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
@@ -856,39 +998,11 @@ __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc
             const int li0 = t0 > rank ? (t0 - rank + kFacCluster - 1) / kFacCluster : 0;
             const int nr = nown > li0 ? nown - li0 : 0;
             if (warp == 0) {
-                // (A) the block's Cholesky on registers: lane l + 8 g holds
-                // entries (l, g) and (l, g + 4) (v0, v1), so that a pivot
-                // costs two FMAs per lane rather than one per later column;
-                // the column loop unrolled, the other lanes' entries by
-                // shuffles.  Entries above a row's diagonal may take finite
-                // junk and are never read.
+                // (A) the block's Cholesky on registers
                 const int l = lane & 7, g = lane >> 3;
                 double v0 = l < w && g <= l ? D[l * kPanel + g] : 0.0;
                 double v1 = l < w && g + 4 <= l ? D[l * kPanel + g + 4] : 0.0;
-                int f = 0;
-#pragma unroll
-                for (int c = 0; c < kPanel; ++c) {
-                    if (c < w && !f) {
-                        const int sc = 8 * (c & 3);  // lanes of column c: sc .. sc + 7
-                        double &vc = c < 4 ? v0 : v1;
-                        const double d = __shfl_sync(0xffffffffu, vc, c + sc);
-                        if (!pivot_ok(d)) {
-                            f = 1;  // the same value in every lane
-                        } else {
-                            const double il = pivot_rsqrt(d);
-                            if (lane == 0) ils[c0 + c] = il;
-                            vc *= g == (c & 3) && l >= c ? il : 1.0;  // lane (c, .): sqrt(d)
-                            double lac = __shfl_sync(0xffffffffu, vc, l + sc);  // L[l][c]
-                            lac = l > c && l < w ? lac : 0.0;
-                            if (c < 4) {
-                                const double x0 = __shfl_sync(0xffffffffu, vc, g + sc);  // L[g][c]
-                                v0 -= (g > c ? lac : 0.0) * x0;
-                            }
-                            const double x1 = __shfl_sync(0xffffffffu, vc, g + 4 + sc);  // L[g+4][c]
-                            v1 -= (g + 4 > c ? lac : 0.0) * x1;
-                        }
-                    }
-                }
+                const int f = panel_cholesky8(v0, v1, w, lane, ils + c0);
                 if (l < w) {
                     if (g <= l) D[l * kPanel + g] = v0;
                     if (g + 4 <= l) D[l * kPanel + g + 4] = v1;
@@ -1049,15 +1163,15 @@ __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc
         double *dW = scr.dW(p), *G = scr.G(p);
         for (int e = threadIdx.x; e < nown * n; e += blockDim.x) {
             const int li = e / n, k = e % n, i = rank + kFacCluster * li;
-            if (k <= i) Pp[(size_t)k * m + i] = own(li)[k];
+            if (k <= i) Pp[(size_t)k * m + i] = k == i ? own(li)[k] : s3_input<DF>(own(li)[k]);
         }
         for (int li = threadIdx.x; li < nown; li += blockDim.x) {
             const int i = rank + kFacCluster * li;
-            dW[i] = ils[i];
+            dW[i] = s3_input<DF>(ils[i]);
         }
         for (int e = threadIdx.x; e < 6 * nown; e += blockDim.x) {
             const int li = e / 6, i = rank + kFacCluster * li;
-            G[6 * i + e % 6] = Br[e];
+            G[6 * i + e % 6] = s3_input<DF>(Br[e]);
         }
         // partial S = G^T G over own rows, one warp per entry
         for (int ab = warp; ab < 36; ab += nw) {
@@ -1089,7 +1203,7 @@ __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc
                     else atomicMin(flag, (int)(p_base + p));
                 }
             } else if (threadIdx.x < 36) {
-                scr.N(p)[threadIdx.x] = Nm[threadIdx.x];
+                scr.N(p)[threadIdx.x] = s3_input<DF>(Nm[threadIdx.x]);
                 Pp[(size_t)(n + threadIdx.x / 6) * m + n + threadIdx.x % 6] = -Nm[threadIdx.x];
             }
         }
@@ -1173,48 +1287,9 @@ __global__ void __launch_bounds__(256) pc_trinv_kernel(
 // preconditioner changes the iteration count, not the solution, which the
 // flexible GMRES takes from true residuals.
 //
-// S2' converts, in place, the FP64 inputs of S3 to double-float pairs packed
-// in the same 8 bytes: the rows of L^T in P_p's upper triangle, and dW, G and
-// N in the scratch.
-__device__ __forceinline__ double df_pack(dfl v)
-{
-    return __hiloint2double(__float_as_int(v.hi), __float_as_int(v.lo));
-}
-
-__device__ __forceinline__ dfl df_unpack(double d)
-{
-    return dfl(__int_as_float(__double2hiint(d)), __int_as_float(__double2loint(d)));
-}
-
-__device__ __forceinline__ dfl df_of(double d)
-{
-    const float h = (float)d;
-    return dfl(h, (float)(d - (double)h));
-}
-
-__global__ void __launch_bounds__(256) pc_to_df_kernel(int64_t nb,
-                                                       const int64_t *__restrict__ start,
-                                                       const int64_t *__restrict__ poff,
-                                                       double *__restrict__ P, SplitScratch scr)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t rows = nb * scr.nmax;
-    for (int64_t it = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); it < rows;
-         it += warps) {
-        const int64_t p = it / scr.nmax;
-        const int k = (int)(it % scr.nmax);
-        const int n = 3 * (int)(start[p + 1] - start[p]), m = n + 6;
-        if (k >= n) continue;
-        double *Lk = P + poff[p] + (size_t)k * m;
-        for (int i = k + 1 + lane; i < n; i += 32) Lk[i] = df_pack(df_of(Lk[i]));
-        if (lane == 0) scr.dW(p)[k] = df_pack(df_of(scr.dW(p)[k]));
-        if (lane < 6) scr.G(p)[6 * k + lane] = df_pack(df_of(scr.G(p)[6 * k + lane]));
-        if (k == 0)
-            for (int e = lane; e < 36; e += 32) scr.N(p)[e] = df_pack(df_of(scr.N(p)[e]));
-    }
-}
-
+// S2 leaves the inputs of S3 (the rows of L^T in P_p's upper triangle, and dW,
+// G and N in the scratch) as double-float pairs packed in the 8 bytes of an
+// FP64 number.
 __device__ __forceinline__ void cp_async8(double *smem, const double *gmem)
 {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -1692,9 +1767,6 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
     const MobConsts<double> k = MobConsts<double>::make(a);
     const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
     const bool lsmem = nmax <= kSmemMaxRows;
-    const size_t fsmem =
-        sizeof(double) * (lsmem ? (size_t)nmax * nmax + (7 + kPanel) * (size_t)nmax + 72
-                                : 2 * (size_t)nmax + 72);
     const int col_groups = (int)ceil_div(nmax, 8);
     const int T = (int)ceil_div(nmax, kTile);
     const int tiles = T * (T + 1) / 2;
@@ -1708,17 +1780,25 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
             pc_assemble_kernel<true><<<ga, 64, 0, s>>>(ng, r, st, po, k, scale, P, shift);
         else
             pc_assemble_kernel<false><<<ga, 64, 0, s>>>(ng, r, st, po, k, scale, P, shift);
-        if (ng < ctx->sm_count) {
-            // fewer bodies than SMs: a cluster of CTAs per body, the rows in
-            // shared memory or in place in global memory
+        // A cluster of CTAs per body while all clusters (two CTAs an SM) run at
+        // once, or, for blocks in global memory, with fewer bodies than SMs; one
+        // CTA per body otherwise.  42-blob bodies, clusters: 97 us for 8, 118
+        // for 32, 148 for 40, 264 for 100.
+        const bool df = nmax <= kSetupSmallRows;  // double-float S3 and S4
+        if (lsmem ? ng * kFacCluster <= 2 * (int64_t)ctx->sm_count : ng < ctx->sm_count) {
             const size_t csm = factor_cluster_smem(nmax, lsmem);
-            auto fk = lsmem ? pc_factor_cluster_kernel<true> : pc_factor_cluster_kernel<false>;
+            auto fk = df ? pc_factor_cluster_kernel<true, true>
+                         : lsmem ? pc_factor_cluster_kernel<true, false>
+                                 : pc_factor_cluster_kernel<false, false>;
             MB_CUDA_TRY(ctx, cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)csm));
             fk<<<(int)ng * kFacCluster, 256, csm, s>>>(ng, r, q + 3 * g0, st, po, P, scr, flag,
                                                        flag_slot, g0, schur);
         } else {
-            auto factor = lsmem ? pc_factor_kernel<true> : pc_factor_kernel<false>;
+            const size_t fsmem = lsmem ? factor_small_smem(nmax)
+                                       : sizeof(double) * (2 * (size_t)nmax + 72);
+            auto factor = df ? pc_factor_small_kernel<true>
+                             : lsmem ? pc_factor_small_kernel<false> : pc_factor_kernel;
             MB_CUDA_TRY(ctx, cudaFuncSetAttribute(factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)fsmem));
             factor<<<(int)std::min<int64_t>(ng, 4 * (int64_t)ctx->sm_count), 256, fsmem, s>>>(
@@ -1739,10 +1819,8 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
                                                   (int)tsm));
             pc_trinv_smem_kernel<<<gt, 32 * kTrinvSmemWarps, tsm, s>>>(ng, st, po, P, scr,
                                                                       col_groups);
-        } else if (nmax <= kSetupSmallRows) {
-            // double-float S3 and S4 (see pc_to_df_kernel)
-            const int gc = (int)std::min<int64_t>(ceil_div(ng * nmax, 8), 8 * (int64_t)ctx->sm_count);
-            pc_to_df_kernel<<<gc, 256, 0, s>>>(ng, st, po, P, scr);
+        } else if (df) {
+            // double-float S3 and S4
             if (ng < ctx->sm_count) {
                 // four columns per CTA, a warp pair each; the staged triangle
                 // of L^T, G and the pairs' exchange
@@ -1762,7 +1840,7 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
                 const int gp = (int)std::min<int64_t>(ng * tiles, 16 * (int64_t)ctx->sm_count);
                 pc_product_df_kernel<kTile><<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles, schur);
             }
-            count_launch(5);
+            count_launch(4);
             MB_CUDA_TRY(ctx, cudaGetLastError());
             continue;
         } else if (nmax <= 256)
