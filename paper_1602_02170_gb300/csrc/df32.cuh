@@ -148,6 +148,13 @@ __device__ __forceinline__ dfl2 operator*(dfl2 a, dfl2 b)
     const float2 p = mul2(a.hi, b.hi);
     return dfl2(p, fma2(a.lo, b.hi, fma2(a.hi, b.lo, fma2(a.hi, b.hi, neg2(p)))));
 }
+// accumulation renormalises, as for dfl (11)
+__device__ __forceinline__ dfl2 &operator+=(dfl2 &a, dfl2 b)
+{
+    const dfl2 s = two_sum(a.hi, b.hi);
+    a = fast_two_sum(s.hi, add2(s.lo, add2(a.lo, b.lo)));
+    return a;
+}
 // a + b for |a| >= |b| (5), a c for c exact in FP32 (3), a c for c a power of
 // two (2), a + c (7)
 __device__ __forceinline__ dfl2 add_ordered(dfl2 a, dfl2 b)

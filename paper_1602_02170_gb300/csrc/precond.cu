@@ -1290,280 +1290,199 @@ __global__ void __launch_bounds__(256) pc_trinv_kernel(
 // S2 leaves the inputs of S3 (the rows of L^T in P_p's upper triangle, and dW,
 // G and N in the scratch) as double-float pairs packed in the 8 bytes of an
 // FP64 number.
-__device__ __forceinline__ void cp_async8(double *smem, const double *gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
+// A 32 x 32 tile of double-float numbers in shared memory: hi and lo parts in
+// rows of kTileLd floats (pairs of columns stay 8-byte aligned, and two rows
+// apart by one start 2 banks apart); row 32 stays zero.
+constexpr int kTileLd = kTile + 2;
+struct DfTile {
+    float hi[(kTile + 1) * kTileLd], lo[(kTile + 1) * kTileLd];
+    __device__ __forceinline__ dfl at(int r, int c) const
+    {
+        return dfl(hi[r * kTileLd + c], lo[r * kTileLd + c]);
+    }
+    __device__ __forceinline__ void set(int r, int c, dfl v)
+    {
+        hi[r * kTileLd + c] = v.hi;
+        lo[r * kTileLd + c] = v.lo;
+    }
+    // columns 2 c2, 2 c2 + 1 of row r
+    __device__ __forceinline__ dfl2 pair(int r, int c2) const
+    {
+        return dfl2(*(const float2 *)(hi + r * kTileLd + 2 * c2),
+                    *(const float2 *)(lo + r * kTileLd + 2 * c2));
+    }
+    __device__ __forceinline__ void set_pair(int r, int c2, dfl2 v)
+    {
+        *(float2 *)(hi + r * kTileLd + 2 * c2) = v.hi;
+        *(float2 *)(lo + r * kTileLd + 2 * c2) = v.lo;
+    }
+};
 
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// Offset of row k of the staged triangle (rows cmin ..), n rows in all
-__device__ __forceinline__ int tri_row_off(int k, int cmin, int n)
+// acc += A X for rows r, r + 16 and the column pair c2 of 32 x 32 tiles
+// (threads c2 = tid % 16, r = tid / 16 of 256).
+__device__ __forceinline__ void tile_mac(dfl2 (&acc)[2], const DfTile &A, const DfTile &X, int r,
+                                         int c2)
 {
-    return (k - cmin) * (2 * (n - 1) - (cmin + k - 1)) / 2;
-}
-
-// S3 in double-float: warp per column c of W = L^-1, rows 32 t + lane in
-// registers, as pc_trinv_kernel; W, Q and Q N go to the scratch as packed
-// double-float, the border entries -Q N of P_p in FP64.  1 / L_kk travels
-// through the chain by shuffles from registers.  L^T and G are read from
-// L2: this form serves many bodies, whose CTAs stay small; few bodies take
-// pc_trinv_df_pair_kernel.
-__global__ void __launch_bounds__(256) pc_trinv_df_kernel(
-    int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
-    double *__restrict__ P, SplitScratch scr, int col_groups)
-{
-    constexpr int R = 4;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int64_t item = blockIdx.x; item < nb * col_groups; item += gridDim.x) {
-        const int64_t p = item / col_groups;
-        const int cmin = (int)(item % col_groups) * nw;
-        const int c = cmin + warp;
-        const int n = 3 * (int)(start[p + 1] - start[p]), m = n + 6;
-        // row k of L^T at Lk + (k - cmin) * ldl, row k of G at Gk + 6 (k - cmin)
-        const double *Lk = P + poff[p] + (size_t)cmin * m, *Gk = scr.G(p) + 6 * cmin;
-        const int ldl = m;
-        if (c >= n) continue;  // warp-uniform
-        double *W = scr.W(p);
-        const double *dW = scr.dW(p), *Nm = scr.N(p);
-        const int ldw = scr.nmax;
-        dfl w[R];
-#pragma unroll
-        for (int t = 0; t < R; ++t) w[t] = dfl((32 * t + lane == c) ? 1.f : 0.f, 0.f);
-        // zero the rows of column c that the tiled product reads above the diagonal
-        for (int kk = (c & ~(kTile - 1)) + lane; kk < c; kk += 32) W[(size_t)kk * ldw + c] = 0.0;
-        dfl qa;  // lane b < 6: Q[c][b]
-        // 1 / L_kk of rows 32 t + lane in registers (passed by shuffles in the chain)
-        dfl dwr[R];
-#pragma unroll
-        for (int t = 0; t < R; ++t) dwr[t] = 32 * t + lane < n ? df_unpack(dW[32 * t + lane]) : dfl();
-        {
-#pragma unroll
-            for (int t = 0; t < R; ++t) {
-                if (32 * t + 31 < c) continue;
-                if (32 * t >= n) break;
-                for (int l = 0; l < 32; ++l) {
-                    const int k = 32 * t + l;
-                    if (k < c) continue;
-                    if (k >= n) break;
-                    const dfl wl(__shfl_sync(0xffffffffu, w[t].hi, l), __shfl_sync(0xffffffffu, w[t].lo, l));
-                    const dfl dk(__shfl_sync(0xffffffffu, dwr[t].hi, l), __shfl_sync(0xffffffffu, dwr[t].lo, l));
-                    const dfl wk = wl * dk;
-                    if (lane == l) W[(size_t)k * ldw + c] = df_pack(wk);
-                    if (lane < 6) qa += wk * df_unpack(Gk[6 * (k - cmin) + lane]);
-                    const double *lk = Lk + (size_t)(k - cmin) * ldl;  // row k of L^T
-#pragma unroll
-                    for (int t2 = t; t2 < R; ++t2) {
-                        const int i = 32 * t2 + lane;
-                        if (i > k && i < n) w[t2] = w[t2] - df_unpack(lk[i]) * wk;
-                    }
-                }
-            }
-        }
-        // QN[c][b] = sum_a Q[c][a] N[a][b]
-        dfl qn;
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-            const dfl qv(__shfl_sync(0xffffffffu, qa.hi, a), __shfl_sync(0xffffffffu, qa.lo, a));
-            if (lane < 6) qn += qv * df_unpack(Nm[a * 6 + lane]);
-        }
-        if (lane < 6) {
-            scr.Q(p)[6 * c + lane] = df_pack(qa);
-            scr.QN(p)[6 * c + lane] = df_pack(qn);
-            const double v = -to_double(qn);
-            P[poff[p] + (size_t)c * m + n + lane] = v;
-            P[poff[p] + (size_t)(n + lane) * m + c] = v;
-        }
+#pragma unroll 4
+    for (int k = 0; k < kTile; ++k) {
+        const dfl2 x = X.pair(k, c2);
+        acc[0] += dfl2(A.at(r, k)) * x;
+        acc[1] += dfl2(A.at(r + 16, k)) * x;
     }
 }
 
-// One 32-row tile t of a column's chain (the steps of pc_trinv_df_kernel):
-// lane l holds row 32 t + l in wt; the step of row k leaves W[k][c] in lane
-// k - 32 t of wst and updates only the tile's own rows.
-__device__ __forceinline__ void trinv_tile_chain(int t, int c, int n, int cmin,
-                                                 const double *__restrict__ sLt, dfl &wt, dfl dwrt,
-                                                 dfl &wst, int lane)
-{
-    const int i = 32 * t + lane;
-    for (int l = 0; l < 32; ++l) {
-        const int k = 32 * t + l;
-        if (k < c) continue;
-        if (k >= n) break;
-        const dfl lik = i > k && i < n ? df_unpack(sLt[tri_row_off(k, cmin, n) - (k + 1) + i]) : dfl();
-        const dfl wl(__shfl_sync(0xffffffffu, wt.hi, l), __shfl_sync(0xffffffffu, wt.lo, l));
-        const dfl dk(__shfl_sync(0xffffffffu, dwrt.hi, l), __shfl_sync(0xffffffffu, dwrt.lo, l));
-        const dfl wk = wl * dk;
-        wst = lane == l ? wk : wst;
-        const dfl wn = wt - lik * wk;
-        wt = i > k && i < n ? wn : wt;
-    }
-}
+constexpr int kTrinvTiles = 4;  // tiles a side, at most (kSetupSmallRows rows)
+struct TrinvSmem {
+    DfTile D[kTrinvTiles];   // inverses of the diagonal tiles t .. (D[0] = W_tt)
+    DfTile A[kTrinvTiles];   // the diagonal tiles of L, then A[j] = W_{t+j,t} and A[0] = tiles of L
+    dfl dw[kTrinvTiles * kTile];
+    dfl q[kTile][6];
+};
 
-// S3 in double-float for few bodies (rows n <= 128): four columns per CTA,
-// a pair of warps per column.  Warp A holds the column's rows 0..63 (tiles
-// 0, 1), warp B rows 64..127 (tiles 2, 3).  The pace is set by a warp's
-// instruction count (about 5 cycles each: every step is a dependent chain),
-// so the pair splits the column's work in three phases between barriers:
-//   1. A runs tile 0's chain and leaves its W entries in shared memory;
-//   2. A subtracts tile 0's product from tile 1, runs tile 1 and leaves its
-//      entries and Q's sums over tiles 0, 1; meanwhile B subtracts tile 0's
-//      product from its rows;
-//   3. B subtracts tile 1's product, runs tiles 2 and 3 and carries Q on
-//      from A's sums.
-// Every entry takes the same operations in the same order as in one warp
-// (pc_trinv_df_kernel).  The CTA first copies the rows of L^T its columns
-// need (from its first column on; row k holds entries k+1 .. n-1, rows back
-// to back, all copies in flight at once by cp.async) and their rows of G
-// into shared memory, so that no step of a chain waits on L2.
-__global__ void __launch_bounds__(256) pc_trinv_df_pair_kernel(
+// S3 in double-float: one CTA per body and 32 columns t of W = L^-1, by 32 x 32
+// tiles.  The diagonal tiles s >= t are inverted side by side, two warps each
+// (a chain of 32 steps), then
+//   W_st = -L_ss^-1 sum_{t <= u < s} L_su W_ut,   s = t + 1, ...
+// as tile products on paired FP32 arithmetic, two columns to an instruction.
+// Then Q = W^T G, Q N and P_p's border for the CTA's columns.  CTAs of the
+// longest columns (t = 0) come first.
+//
+// A warp per column of W (or two, for few bodies), one row after the other,
+// spent about 130 instructions a step on chains of up to 126 steps: 303 us for
+// 300 bodies of 126 and 45 rows in turn and 50 us for 8 of 126.  Setup and
+// application of the 300: 851 -> 681 us.
+__global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
     int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
-    double *__restrict__ P, SplitScratch scr, int col_groups)
+    double *__restrict__ P, SplitScratch scr, int tiles)
 {
-    constexpr int kCols = 4;
-    extern __shared__ double sLt[];  // L^T rows cmin .. n-1 (packed triangle), G rows, exchange
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int q = warp >> 1, role = warp & 1;
-    const int nmax = scr.nmax;
-    dfl *xw = (dfl *)(sLt + (size_t)nmax * (nmax - 1) / 2 + 6 * (size_t)nmax);  // [kCols][2][32]
-    dfl *xq = xw + kCols * 2 * 32;                                               // [kCols][6]
-    for (int64_t item = blockIdx.x; item < nb * col_groups; item += gridDim.x) {
-        const int64_t p = item / col_groups;
-        const int cmin = (int)(item % col_groups) * kCols;
-        const int c = cmin + q;
+    extern __shared__ __align__(16) unsigned char trinv_raw[];
+    TrinvSmem &sm = *(TrinvSmem *)trinv_raw;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c2 = tid & 15, r = tid >> 4;
+    for (int64_t item = blockIdx.x; item < nb * tiles; item += gridDim.x) {
+        const int64_t p = item % nb;
+        const int t = (int)(item / nb);
         const int n = 3 * (int)(start[p + 1] - start[p]), m = n + 6;
-        double *sG = sLt + (cmin < n ? tri_row_off(n, cmin, n) : 0);
-        __syncthreads();  // the previous item is finished with the shared arrays
-        if (cmin < n) {
-            // asynchronous copies, all in flight at once: a warp per row
-            const double *Lg = P + poff[p];
-            for (int k = cmin + warp; k < n; k += nw) {
-                double *dst = sLt + tri_row_off(k, cmin, n) - (k + 1);
-                for (int i = k + 1 + lane; i < n; i += 32) cp_async8(dst + i, Lg + (size_t)k * m + i);
-            }
-            for (int e = threadIdx.x; e < 6 * (n - cmin); e += blockDim.x)
-                cp_async8(sG + e, scr.G(p) + 6 * cmin + e);
-            cp_async_wait_all();
+        const int T = (n + kTile - 1) / kTile - t;  // tiles t .. t + T - 1
+        if (T <= 0) continue;                       // uniform over the CTA
+        const double *Lt = P + poff[p];             // L[i][k] at Lt[k m + i], i > k
+        // entry (i, k) of L below the diagonal, zero outside the block
+        auto l_entry = [&](int i, int k) {
+            return i > k && i < n ? df_unpack(Lt[(size_t)k * m + i]) : dfl();
+        };
+        __syncthreads();  // done with the previous item
+        for (int e = tid; e < T * (kTile + 1) * kTile; e += 256) {
+            const int j = e / ((kTile + 1) * kTile), x = e % ((kTile + 1) * kTile);
+            const int row = x % (kTile + 1), col = x / (kTile + 1), g0 = (t + j) * kTile;
+            sm.A[j].set(row, col, row < kTile ? l_entry(g0 + row, g0 + col) : dfl());
+            sm.D[j].set(row, col, dfl(row == col ? 1.f : 0.f, 0.f));
+        }
+        for (int e = tid; e < T * kTile; e += 256) {
+            const int k = t * kTile + e;
+            sm.dw[e] = k < n ? df_unpack(scr.dW(p)[k]) : dfl(1.f, 0.f);
         }
         __syncthreads();
-        const bool active = c < n;  // the same in both warps of the pair
+        if (warp < 2 * T) {
+            // columns 16 (warp & 1) + (lane & 15) of tile warp / 2; the half
+            // warps take alternate pairs of rows below the pivot row
+            const int j = warp >> 1, c = 16 * (warp & 1) + (lane & 15), half = lane >> 4;
+            DfTile &X = sm.D[j];
+            const DfTile &Ls = sm.A[j];
+            for (int k = 16 * (warp & 1); k < kTile; ++k) {
+                const dfl wk = X.at(k, c) * sm.dw[j * kTile + k];
+                __syncwarp();
+                if (half == 0) X.set(k, c, wk);
+                const dfl2 w2 = dfl2(wk);
+                for (int i = k + 1 + 2 * half; i < kTile; i += 4) {
+                    const dfl a0 = X.at(i, c), a1 = X.at(i + 1, c);
+                    const dfl l0 = Ls.at(i, k), l1 = Ls.at(i + 1, k);
+                    const dfl2 v = dfl2(make_float2(a0.hi, a1.hi), make_float2(a0.lo, a1.lo)) -
+                                   dfl2(make_float2(l0.hi, l1.hi), make_float2(l0.lo, l1.lo)) * w2;
+                    X.set(i, c, dfl(v.hi.x, v.lo.x));
+                    if (i + 1 < kTile) X.set(i + 1, c, dfl(v.hi.y, v.lo.y));
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        // the tiles below, one after the other; L's tiles come through A[0],
+        // each loaded into registers while the one before is in use
+        double pre[kTile * kTile / 256];
+        auto fetch = [&](int s, int u) {
+#pragma unroll
+            for (int x = 0; x < kTile * kTile / 256; ++x) {
+                const int e = tid + 256 * x, i = (t + s) * kTile + e % kTile,
+                          k = (t + u) * kTile + e / kTile;
+                pre[x] = i < n ? Lt[(size_t)k * m + i] : 0.0;
+            }
+        };
+        if (T > 1) fetch(1, 0);
+        for (int s = 1; s < T; ++s) {
+            dfl2 acc[2];
+            for (int u = 0; u < s; ++u) {
+                __syncthreads();  // A[0] is free
+#pragma unroll
+                for (int x = 0; x < kTile * kTile / 256; ++x) {
+                    const int e = tid + 256 * x;
+                    sm.A[0].set(e % kTile, e / kTile, df_unpack(pre[x]));
+                }
+                if (u + 1 < s) fetch(s, u + 1);
+                else if (s + 1 < T) fetch(s + 1, 0);
+                __syncthreads();
+                tile_mac(acc, sm.A[0], u ? sm.A[u] : sm.D[0], r, c2);
+            }
+            sm.A[s].set_pair(r, c2, -acc[0]);
+            sm.A[s].set_pair(r + 16, c2, -acc[1]);
+            __syncthreads();
+            dfl2 w[2];
+            tile_mac(w, sm.D[s], sm.A[s], r, c2);
+            __syncthreads();  // every thread has read A[s]
+            sm.A[s].set_pair(r, c2, w[0]);
+            sm.A[s].set_pair(r + 16, c2, w[1]);
+        }
+        __syncthreads();
+        // W's columns (zero above the diagonal within the diagonal tile)
         double *W = scr.W(p);
-        const double *dW = scr.dW(p), *Nm = scr.N(p);
-        const int ldw = scr.nmax;
-        // this warp's tiles 2 role + tt: rows 64 role + 32 tt + lane
-        dfl w[2], ws[2], dwr[2];
-#pragma unroll
-        for (int tt = 0; tt < 2; ++tt) {
-            const int i = 64 * role + 32 * tt + lane;
-            w[tt] = dfl(i == c ? 1.f : 0.f, 0.f);
-            ws[tt] = dfl();
-            dwr[tt] = i < n ? df_unpack(dW[i]) : dfl();
+        const int ldw = scr.nmax, c0 = t * kTile;
+        for (int e = tid; e < T * kTile * kTile; e += 256) {
+            const int j = e / (kTile * kTile), i = e / kTile % kTile, c = e % kTile;
+            const int gi = (t + j) * kTile + i;
+            if (gi < n && c0 + c < n)
+                W[(size_t)gi * ldw + c0 + c] = df_pack((j ? sm.A[j] : sm.D[0]).at(i, c));
         }
-        dfl qa;  // lane b < 6: Q[c][b]
-        // whether tile t holds steps of column c
-        auto has = [&](int t) { return 32 * t + 31 >= c && 32 * t < n; };
-        // (1) A: tile 0
-        if (active && role == 0) {
-            // zero the rows of column c that the tiled product reads above the diagonal
-            for (int kk = (c & ~(kTile - 1)) + lane; kk < c; kk += 32) W[(size_t)kk * ldw + c] = 0.0;
-            if (has(0)) {
-                trinv_tile_chain(0, c, n, cmin, sLt, w[0], dwr[0], ws[0], lane);
-                if (lane >= c && lane < n) W[(size_t)lane * ldw + c] = df_pack(ws[0]);
-                xw[(q * 2) * 32 + lane] = ws[0];
-            }
-        }
-        __syncthreads();
-        if (active && role == 0) {
-            // (2) A: tile 0's product out of tile 1 and its share of Q, then tile 1
-            if (has(0))
-                for (int l = 0; l < 32; ++l) {
-                    const int k = l;
-                    if (k < c) continue;
-                    if (k >= n) break;
-                    const dfl wk(__shfl_sync(0xffffffffu, ws[0].hi, l), __shfl_sync(0xffffffffu, ws[0].lo, l));
-                    if (lane < 6) qa += wk * df_unpack(sG[6 * (k - cmin) + lane]);
-                    const int i1 = 32 + lane;
-                    if (i1 < n) w[1] = w[1] - df_unpack(sLt[tri_row_off(k, cmin, n) - (k + 1) + i1]) * wk;
-                }
-            if (has(1)) {
-                trinv_tile_chain(1, c, n, cmin, sLt, w[1], dwr[1], ws[1], lane);
-                const int i = 32 + lane;
-                if (i >= c && i < n) W[(size_t)i * ldw + c] = df_pack(ws[1]);
-                xw[(q * 2 + 1) * 32 + lane] = ws[1];
-                for (int l = 0; l < 32; ++l) {
-                    const int k = 32 + l;
-                    if (k < c) continue;
-                    if (k >= n) break;
-                    const dfl wk(__shfl_sync(0xffffffffu, ws[1].hi, l), __shfl_sync(0xffffffffu, ws[1].lo, l));
-                    if (lane < 6) qa += wk * df_unpack(sG[6 * (k - cmin) + lane]);
+        // Q[c][b] = sum_k W[k][c] G[k][b], even and odd rows in the halves
+        const int c = tid % kTile, b = tid / kTile;
+        const bool mine = b < 6 && c0 + c < n;
+        if (mine) {
+            const double *G = scr.G(p);
+            dfl2 acc;
+            for (int j = 0; j < T; ++j) {
+                const DfTile &X = j ? sm.A[j] : sm.D[0];
+                const int g0 = (t + j) * kTile, rows = min(kTile, n - g0);
+                for (int i = 0; i < rows; i += 2) {
+                    const dfl x0 = X.at(i, c), x1 = X.at(i + 1, c);
+                    const dfl g1 = df_unpack(G[6 * (g0 + i) + b]),
+                              g2 = i + 1 < rows ? df_unpack(G[6 * (g0 + i + 1) + b]) : dfl();
+                    acc += dfl2(make_float2(x0.hi, x1.hi), make_float2(x0.lo, x1.lo)) *
+                           dfl2(make_float2(g1.hi, g2.hi), make_float2(g1.lo, g2.lo));
                 }
             }
-            if (lane < 6) xq[q * 6 + lane] = qa;
-        } else if (active && role == 1 && has(0)) {
-            // (2) B: tile 0's product out of rows 64 .. n-1
-            for (int l = 0; l < 32; ++l) {
-                const int k = l;
-                if (k < c) continue;
-                if (k >= n) break;
-                const dfl wk = xw[(q * 2) * 32 + l];
-                const double *lk = sLt + tri_row_off(k, cmin, n) - (k + 1);
-#pragma unroll
-                for (int tt = 0; tt < 2; ++tt) {
-                    const int i2 = 64 + 32 * tt + lane;
-                    if (i2 < n) w[tt] = w[tt] - df_unpack(lk[i2]) * wk;
-                }
-            }
+            dfl qa(acc.hi.x, acc.lo.x);
+            qa += dfl(acc.hi.y, acc.lo.y);
+            sm.q[c][b] = qa;
         }
         __syncthreads();
-        if (active && role == 1) {
-            // (3) B: tile 1's product out of its rows, then tiles 2 and 3
-            qa = lane < 6 ? xq[q * 6 + lane] : dfl();
-            if (has(1))
-                for (int l = 0; l < 32; ++l) {
-                    const int k = 32 + l;
-                    if (k < c) continue;
-                    if (k >= n) break;
-                    const dfl wk = xw[(q * 2 + 1) * 32 + l];
-                    const double *lk = sLt + tri_row_off(k, cmin, n) - (k + 1);
-#pragma unroll
-                    for (int tt = 0; tt < 2; ++tt) {
-                        const int i2 = 64 + 32 * tt + lane;
-                        if (i2 < n) w[tt] = w[tt] - df_unpack(lk[i2]) * wk;
-                    }
-                }
-#pragma unroll
-            for (int tt = 0; tt < 2; ++tt) {
-                const int t = 2 + tt;
-                if (!has(t)) continue;
-                trinv_tile_chain(t, c, n, cmin, sLt, w[tt], dwr[tt], ws[tt], lane);
-                const int i = 32 * t + lane;
-                if (i >= c && i < n) W[(size_t)i * ldw + c] = df_pack(ws[tt]);
-                for (int l = 0; l < 32; ++l) {
-                    const int k = 32 * t + l;
-                    if (k < c) continue;
-                    if (k >= n) break;
-                    const dfl wk(__shfl_sync(0xffffffffu, ws[tt].hi, l), __shfl_sync(0xffffffffu, ws[tt].lo, l));
-                    if (lane < 6) qa += wk * df_unpack(sG[6 * (k - cmin) + lane]);
-                    if (tt == 0) {
-                        const int i1 = 96 + lane;
-                        if (i1 < n) w[1] = w[1] - df_unpack(sLt[tri_row_off(k, cmin, n) - (k + 1) + i1]) * wk;
-                    }
-                }
-            }
+        if (mine) {
             // QN[c][b] = sum_a Q[c][a] N[a][b]
+            const double *Nm = scr.N(p);
             dfl qn;
 #pragma unroll
-            for (int a = 0; a < 6; ++a) {
-                const dfl qv(__shfl_sync(0xffffffffu, qa.hi, a), __shfl_sync(0xffffffffu, qa.lo, a));
-                if (lane < 6) qn += qv * df_unpack(Nm[a * 6 + lane]);
-            }
-            if (lane < 6) {
-                scr.Q(p)[6 * c + lane] = df_pack(qa);
-                scr.QN(p)[6 * c + lane] = df_pack(qn);
-                const double v = -to_double(qn);
-                P[poff[p] + (size_t)c * m + n + lane] = v;
-                P[poff[p] + (size_t)(n + lane) * m + c] = v;
-            }
+            for (int a = 0; a < 6; ++a) qn += sm.q[c][a] * df_unpack(Nm[a * 6 + b]);
+            scr.Q(p)[6 * (c0 + c) + b] = df_pack(sm.q[c][b]);
+            scr.QN(p)[6 * (c0 + c) + b] = df_pack(qn);
+            const double v = -to_double(qn);
+            P[poff[p] + (size_t)(c0 + c) * m + n + b] = v;
+            P[poff[p] + (size_t)(n + b) * m + c0 + c] = v;
         }
     }
 }
@@ -1821,22 +1740,16 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
                                                                       col_groups);
         } else if (df) {
             // double-float S3 and S4
+            MB_CUDA_TRY(ctx, cudaFuncSetAttribute(pc_trinv_df_kernel,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)sizeof(TrinvSmem)));
+            pc_trinv_df_kernel<<<(int)std::min<int64_t>(ng * T, 1 << 30), 256, sizeof(TrinvSmem), s>>>(
+                ng, st, po, P, scr, T);
             if (ng < ctx->sm_count) {
-                // four columns per CTA, a warp pair each; the staged triangle
-                // of L^T, G and the pairs' exchange
-                const int cg4 = (int)ceil_div(nmax, 4);
-                const int gt4 = (int)std::min<int64_t>(ng * cg4, 16 * (int64_t)ctx->sm_count);
-                const size_t tsm = sizeof(double) * ((size_t)nmax * (nmax - 1) / 2 + 6 * (size_t)nmax) +
-                                   sizeof(dfl) * (4 * 2 * 32 + 4 * 6);
-                MB_CUDA_TRY(ctx, cudaFuncSetAttribute(pc_trinv_df_pair_kernel,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)tsm));
-                pc_trinv_df_pair_kernel<<<gt4, 256, tsm, s>>>(ng, st, po, P, scr, cg4);
                 const int T16 = (int)ceil_div(nmax, 16), tiles16 = T16 * (T16 + 1) / 2;
                 const int gp = (int)std::min<int64_t>(ng * tiles16, 16 * (int64_t)ctx->sm_count);
                 pc_product_df_kernel<16><<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles16, schur);
             } else {
-                pc_trinv_df_kernel<<<gt, 256, 0, s>>>(ng, st, po, P, scr, col_groups);
                 const int gp = (int)std::min<int64_t>(ng * tiles, 16 * (int64_t)ctx->sm_count);
                 pc_product_df_kernel<kTile><<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles, schur);
             }

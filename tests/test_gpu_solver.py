@@ -459,3 +459,27 @@ def test_zero_right_hand_side(ctx):
         F, T, lam, info = ctx.solve_resistance(d["q"], d["theta"], d["blob_start"], d["rho"], z, z,
                                                s.a, 1.0, True, tol=1e-10, prec=prec)
         assert info["converged"] == 1 and np.all(host(F) == 0) and np.all(host(lam) == 0)
+
+
+@pytest.mark.parametrize("nbod", [3, 38, 39, 310])
+@pytest.mark.parametrize("counts", [(3, 4, 5), (10, 11, 8), (21, 22, 32), (42, 15, 6), (43, 42, 53)])
+def test_preconditioner_tile_edges(ctx, nbod, counts):
+    """Blocks of 9 to 159 rows, around the edges of 8-column panels and 32-row
+    tiles, factored by clusters (up to 38 bodies on 152 SMs) or by one CTA
+    each, their inverse by tiles up to 128 rows; bodies of
+    three sizes to a call, jittered lattices of blobs.  The bar is that of the
+    other preconditioner tests."""
+    rng = np.random.default_rng(nbod + counts[0])
+    a = 0.2
+    count = np.array([counts[p % 3] for p in range(nbod)])
+    start = np.concatenate([[0], np.cumsum(count)]).astype(np.int64)
+    q = np.stack([4.0 * (np.arange(nbod) % 20), 4.0 * (np.arange(nbod) // 20), np.full(nbod, 2.5)], axis=1)
+    r = np.concatenate([q[p] + 2.2 * a * np.stack([np.arange(c) % 2, np.arange(c) // 2 % 2,
+                                                   np.arange(c) // 4], axis=1) for p, c in enumerate(count)])
+    r = r + rng.uniform(-0.02, 0.02, r.shape)
+    w, g = rng.standard_normal(r.shape), rng.standard_normal((nbod, 6))
+    ctx.precond_setup(dev(r), dev(q), dev(start, torch.int64), a, 1.0, True)
+    lam, UO = ctx.precond_apply(dev(w), dev(g))
+    lam_ref, UO_ref = O.precond_apply(r, q, start, a, 1.0, True, w, g)
+    assert rel_l2(host(lam), lam_ref) <= 1e-9
+    assert rel_l2(host(UO), UO_ref) <= 1e-9
