@@ -19,6 +19,8 @@
 #include <algorithm>
 #include <mutex>
 
+#include <cooperative_groups.h>
+
 #include "mb_internal.cuh"
 #include "pair_tiles.cuh"
 #include "rpy_wall.cuh"
@@ -223,8 +225,11 @@ __global__ void __launch_bounds__(NT, NT == kNT ? (NP == 1 ? 3 : 2) : 16) pair_f
 // z, max x, y, z), and grid->far2, the squared distance beyond which a block
 // pair is far (see x2sym_item); such pairs take the kFar instance, and the
 // kVeryFar one from kVeryFarRadii radii on.
+// The smallest blocks round each sum once (mob_apply2), which keeps the error of
+// products below 4,096 blobs at that of sums over 16 sources (2,000 blobs without
+// the wall: 1.6e-7 -> 1.5e-7).
 constexpr int kBoxBlobs = 256;
-constexpr int64_t kSymNT64MinN = 3000, kSymNT128MinN = 12000;
+constexpr int64_t kSymNT64MinN = 4096, kSymNT128MinN = 12000;
 
 struct SortGrid {
     float lo[3], inv_h[3];  // cell of x: (x - lo) * inv_h per axis
@@ -264,6 +269,97 @@ __global__ void __launch_bounds__(NT, 512 / NT) pair_sym_kernel(
             x2sym_item<WALL, NT, kFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
         else x2sym_item<WALL, NT, kNear>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
     }
+}
+
+// A whole FP32 product of a few hundred blobs in one launch: a cluster of
+// kSmallCluster CTAs per block of 64 targets, each of its warps taking a share
+// of the sources (at most 32) straight from the caller's FP64 arrays, and the
+// warps' sums meeting in distributed shared memory.  Such a product is bound by
+// its launches, not by arithmetic: packed positions, one-warp CTAs and a
+// reduction were three (336 blobs, a pass: 32.6 -> 29.4 us).  u must not
+// overlap r or f.
+constexpr int kSmallCluster = 8, kSmallWarps = 4;
+constexpr int64_t kSmallMaxN = 32 * kSmallCluster * kSmallWarps;
+
+template <bool WALL>
+__global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(32 * kSmallWarps)
+    pair_small_kernel(const double *__restrict__ r, const double *__restrict__ f, int n, MobConsts2 k,
+                      double *__restrict__ u, double scale)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ float4 sP[kSmallWarps][kX2SmemFloat4PerSource * 32];
+    __shared__ float part[kSmallWarps][3 * 64];
+    __shared__ double tot[3 * 64];
+    const int rank = (int)cluster.block_rank(), tb = blockIdx.x / kSmallCluster;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int chunk = (n + kSmallCluster * kSmallWarps - 1) / (kSmallCluster * kSmallWarps);
+    const int j0 = (rank * kSmallWarps + warp) * chunk, cnt = max(0, min(chunk, n - j0));
+    auto split = [&](int i, float4 &h, float4 &l) {
+        const double x = r[3 * i], y = r[3 * i + 1], z = r[3 * i + 2];
+        h = make_float4((float)x, (float)y, (float)z, 0.f);
+        l = make_float4((float)(x - (double)h.x), (float)(y - (double)h.y), (float)(z - (double)h.z), 0.f);
+    };
+    float4 h[2], l[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) split(min(64 * tb + 32 * t + lane, n - 1), h[t], l[t]);
+    if (lane < cnt) {
+        float4 hj, lj;
+        const int j = j0 + lane;
+        split(j, hj, lj);
+        stage_x2(sP[warp] + kX2SmemFloat4PerSource * lane, hj, lj, (float)f[3 * j],
+                 (float)f[3 * j + 1], (float)f[3 * j + 2]);
+    }
+    __syncwarp();
+    const float2 xh = make_float2(h[0].x, h[1].x), xl = make_float2(l[0].x, l[1].x);
+    const float2 yh = make_float2(h[0].y, h[1].y), yl = make_float2(l[0].y, l[1].y);
+    const float2 zh = make_float2(h[0].z, h[1].z), zl = make_float2(l[0].z, l[1].z);
+    float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
+#pragma unroll 2
+    for (int s = 0; s < cnt; ++s) {
+        const float4 *Q = sP[warp] + kX2SmemFloat4PerSource * s;
+        const float4 P0 = Q[0], P1 = Q[1], P2 = Q[2], P3 = Q[3], P4 = Q[4];
+        const float2 zj = make_float2(P1.x, P1.y);
+        const float2 dx = add2(add2(xh, make_float2(P0.x, P0.y)), add2(xl, make_float2(P2.x, P2.y)));
+        const float2 dy = add2(add2(yh, make_float2(P0.z, P0.w)), add2(yl, make_float2(P2.z, P2.w)));
+        const float2 dz = add2(fma2(zj, k.m1, zh), add2(zl, make_float2(P3.x, P3.y)));
+        const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
+        const Mob<float2> m = mob_coefs2<WALL, kNear>(dz, dxy2, zh, zj, make_float2(P1.z, P1.w), k);
+        mob_apply2<WALL, false, true>(m, dx, dy, dz, make_float2(P3.z, P3.w),
+                                      make_float2(P4.x, P4.y), make_float2(P4.z, P4.w), ax, ay, az);
+    }
+    const float2 a[3] = {ax, ay, az};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        part[warp][3 * lane + c] = a[c].x;
+        part[warp][3 * (32 + lane) + c] = a[c].y;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 3 * 64; e += blockDim.x) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < kSmallWarps; ++w) v += (double)part[w][e];
+        tot[e] = v;
+    }
+    cluster.sync();
+    constexpr int kShare = 3 * 64 / kSmallCluster;
+    const int e = rank * kShare + threadIdx.x;
+    if (threadIdx.x < kShare && 64 * tb + e / 3 < n) {
+        double v = 0.0;
+#pragma unroll
+        for (int b = 0; b < kSmallCluster; ++b) v += cluster.map_shared_rank(tot, b)[e];
+        u[3 * 64 * (int64_t)tb + e] = scale * v;
+    }
+    cluster.sync();  // no CTA ends while another reads its sums
+}
+
+template <bool WALL>
+void launch_small(const double *r, const double *f, int64_t n, double a, double *u, double scale,
+                  cudaStream_t s)
+{
+    pair_small_kernel<WALL><<<(unsigned)(kSmallCluster * ceil_div(n, 64)), 32 * kSmallWarps, 0, s>>>(
+        r, f, (int)n, MobConsts2::make(a), u, scale);
+    count_launch();
 }
 
 // FP64 kernel: one warp per CTA and item, an item being a block of 32
@@ -1090,6 +1186,7 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
 // 995 / 1,149 / 1,370 / 2,310 with the other: zeroing the sums and the atomics
 // cost two to three microseconds a step, and few pairs save less.
 constexpr int64_t kSymMinN = 600;
+static_assert(kSymMinN <= kSmallMaxN, "a product below kSymMinN takes the one-launch kernel");
 
 int f32_variant(int64_t n) { return n < kSymMinN ? 4 : 3; }
 
@@ -1256,17 +1353,28 @@ mb_status matvec_device(mb_context *ctx, const double *r, const double *f, int64
                         double eta, int wall, mb_precision prec, double *u, cudaStream_t s)
 {
     // The symmetric kernels zero u and add to it while they read f (FP64: and
-    // r), so a product in place works on copies.
+    // r), and the small one writes it, so a product in place works on copies.
+    const bool small = prec == MB_FP32_KAHAN && ctx->pair_variant < 0 && n < kSymMinN;
     const size_t bytes = sizeof(double) * 3 * (size_t)n;
     if (overlap(u, f, n)) {
         MB_TRY(ensure(ctx, ctx->stage_f, bytes, "in-place product"));
         MB_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->stage_f.ptr, f, bytes, cudaMemcpyDeviceToDevice, s));
         f = (const double *)ctx->stage_f.ptr;
     }
-    if (prec == MB_FP64 && overlap(u, r, n)) {
+    if ((prec == MB_FP64 || small) && overlap(u, r, n)) {
         MB_TRY(ensure(ctx, ctx->stage_r, bytes, "in-place product"));
         MB_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->stage_r.ptr, r, bytes, cudaMemcpyDeviceToDevice, s));
         r = (const double *)ctx->stage_r.ptr;
+    }
+    if (small) {
+        const double scale = 1.0 / (6.0 * kPi * eta * a);
+        ctx->chosen[size_class(n, wall)] = true;
+        auto *ev = profile_begin(ctx, s);
+        if (wall) launch_small<true>(r, f, n, a, u, scale, s);
+        else launch_small<false>(r, f, n, a, u, scale, s);
+        profile_end(ev, s);
+        MB_CUDA_TRY(ctx, cudaGetLastError());
+        return MB_OK;
     }
     if (prec != MB_FP64) MB_TRY(matvec_pack_positions(ctx, r, n, s));
     return matvec_packed(ctx, r, f, n, a, eta, wall, prec, u, s);
@@ -1392,8 +1500,8 @@ mb_status render_flow(mb_context *ctx, const double *x, int64_t nt, const double
 // overlaps on the GPU race on it.  Each call writes every element it later
 // reads, so nothing needs clearing between calls.
 //
-// The kernels and the rule by size are mb_mobility_matvec's: one-warp CTAs
-// and a reduction below kSymMinN, the symmetric kernel above, in the spatial
+// The kernels and the rule by size are mb_mobility_matvec's: the one-launch
+// kernel below kSymMinN, the symmetric kernel above, in the spatial
 // order from kSortMinN on.  A scalar kernel for every ordered pair ran at every
 // size: 5,003 blobs 121 -> 64 us, 65,536 13.1 -> 5.2 ms with the wall, 20,011
 // 705 -> 339 us and 65,536 6.0 -> 2.9 ms without (all against the first form).
@@ -1407,14 +1515,12 @@ static_assert(kNoallocMaxBlobs <= ((int64_t)8 << kNoallocBits) &&
                   kNoallocMaxBlobs <= 1024 * (int64_t)kNoallocMaxTiles &&
                   kNoallocMaxBlobs <= 256 * (int64_t)kNoallocPackCtas,
               "the scratch holds the largest order");
-static_assert(kSymMinN * (kSymMinN / (kSmallNT / 2) + 1) <= kNoallocMaxBlobs,
-              "u holds the partial sums of the small problems");
 
 struct NoallocScratch {
     float4 hi[kNoallocMaxBlobs], lo[kNoallocMaxBlobs];
     float4 shi[kNoallocMaxBlobs], slo[kNoallocMaxBlobs];
-    double f[3 * kNoallocMaxBlobs], u[3 * kNoallocMaxBlobs];  // sorted; below kSymMinN u holds
-                                                              // the chunks' partial sums
+    double f[3 * kNoallocMaxBlobs], u[3 * kNoallocMaxBlobs];  // sorted, or copies for a product
+                                                              // in place
     unsigned key[kNoallocMaxBlobs];
     int perm[kNoallocMaxBlobs];
     int H[(kNoallocMaxTiles + 1) << kNoallocBits];
@@ -1430,14 +1536,14 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoallocS
 struct NoallocDevice {
     bool ready = false;
     NoallocScratch *scratch = nullptr;  // device address of g_noalloc_scratch
-    int sms = 0, resident_wall = 0, resident_free = 0;
+    int sms = 0;
 };
 constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 NoallocDevice g_noalloc_dev[kNoallocMaxDevices];
 
 // First call on a device: look up the array's device address (host code may
-// not use the symbol itself) and the resident-grid sizes.  No allocation.
+// not use the symbol itself) and the SM count.  No allocation.
 mb_status noalloc_setup(int dev, NoallocDevice **out)
 {
     if (dev < 0 || dev >= kNoallocMaxDevices) return MB_EINVAL;
@@ -1450,20 +1556,14 @@ mb_status noalloc_setup(int dev, NoallocDevice **out)
             set_thread_err("cudaGetSymbolAddress of the allocation-free scratch failed");
             return MB_ECUDA;
         }
-        int sms = 0, occ_w = 0, occ_f = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &occ_w, pair_f32x2_kernel<true, 1, kSmallNT>, kSmallNT, 0) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &occ_f, pair_f32x2_kernel<false, 1, kSmallNT>, kSmallNT, 0) != cudaSuccess) {
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
             set_thread_err("device query failed in the allocation-free matvec set-up");
             return MB_ECUDA;
         }
         d.scratch = (NoallocScratch *)ptr;
         d.sms = sms;
-        d.resident_wall = std::max(1, occ_w) * sms;
-        d.resident_free = std::max(1, occ_f) * sms;
         d.ready = true;
     }
     *out = &d;
@@ -1475,21 +1575,27 @@ cudaError_t noalloc_run(const NoallocDevice &d, const double *r, const double *f
 {
     NoallocScratch *w = d.scratch;
     const double scale = 1.0 / (6.0 * kPi * eta * a);
+    if (n < kSymMinN) {
+        const size_t bytes = sizeof(double) * 3 * (size_t)n;
+        cudaError_t e = cudaSuccess;
+        if (overlap(u, f, n)) {
+            e = cudaMemcpyAsync(w->f, f, bytes, cudaMemcpyDeviceToDevice, s);
+            f = w->f;
+        }
+        if (e == cudaSuccess && overlap(u, r, n)) {
+            e = cudaMemcpyAsync(w->u, r, bytes, cudaMemcpyDeviceToDevice, s);
+            r = w->u;
+        }
+        if (e != cudaSuccess) return e;
+        if (wall) launch_small<true>(r, f, n, a, u, scale, s);
+        else launch_small<false>(r, f, n, a, u, scale, s);
+        return cudaGetLastError();
+    }
     const int pack = (int)std::min<int64_t>(ceil_div(n, 256), kNoallocPackCtas);
     const bool sorted = n >= kSortMinN;
     if (sorted) pack_hilo_kernel<true><<<pack, 256, 0, s>>>(r, n, w->hi, w->lo, w->sort.parts);
     else pack_hilo_kernel<false><<<pack, 256, 0, s>>>(r, n, w->hi, w->lo, nullptr);
     count_launch();
-    if (n < kSymMinN) {
-        const Plan p = small_plan(n, wall ? d.resident_wall : d.resident_free);
-        const int direct = p.S == 1;
-        double *out = direct ? u : w->u;
-        if (wall) f32_launch<true>(4, p, s, w->hi, w->lo, f, n, a, out, scale, direct);
-        else f32_launch<false>(4, p, s, w->hi, w->lo, f, n, a, out, scale, direct);
-        count_launch();
-        if (!direct) launch_reduce_partials(out, n, p.S, scale, u, s);
-        return cudaGetLastError();
-    }
     cudaError_t e = cudaSuccess;
     double *us = u;
     const SortGrid *sg = nullptr;

@@ -213,6 +213,7 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
                                            int sub1 = 2)
 {
     constexpr int NW = NT / 32;
+    constexpr bool ONCE = NT == 32;  // the smallest blocks' sums (mob_apply2)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool diag = I == J;
     const int64_t ia = I * 2 * NT + threadIdx.x, ib = ia + NT;
@@ -260,8 +261,9 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
                 const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
                 const Mob<float2> m =
                     mob_coefs2<WALL, kNear>(dz, dxy2, zh, zj, make_float2(P1.z, P1.w), k);
-                mob_apply2<WALL>(m, dx, dy, dz, make_float2(P3.z, P3.w), make_float2(P4.x, P4.y),
-                                 make_float2(P4.z, P4.w), ax, ay, az);
+                mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, make_float2(P3.z, P3.w),
+                                              make_float2(P4.x, P4.y), make_float2(P4.z, P4.w),
+                                              ax, ay, az);
             }
         } else {
             for (int g = 0; g < NT / 32; ++g) {
@@ -285,9 +287,10 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
                                                                     : mul2(dx, dx));
                     const Mob<float2> m =
                         mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, zj, make_float2(P1.z, P1.w), k);
-                    mob_apply2<WALL>(m, dx, dy, dz, make_float2(P3.z, P3.w),
-                                     make_float2(P4.x, P4.y), make_float2(P4.z, P4.w), ax, ay, az);
-                    mob_apply2<WALL, true>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
+                    mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, make_float2(P3.z, P3.w),
+                                                  make_float2(P4.x, P4.y),
+                                                  make_float2(P4.z, P4.w), ax, ay, az);
+                    mob_apply2<WALL, true, ONCE>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
                     // hand the accumulator to lane - 1, which meets this source next step
                     const int from = (lane + 1) & 31;
                     rx.x = __shfl_sync(0xffffffffu, rx.x, from);

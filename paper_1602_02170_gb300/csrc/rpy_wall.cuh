@@ -458,8 +458,11 @@ __device__ __forceinline__ void mob_apply_df(const Mob<dfl2> &m, dfl2 dx, dfl2 d
     uz = uz + (WALL ? m.Z * fz + (TRANS ? m.Bf : m.Bb) * rf : m.Cx * fz + G * dz);
 }
 
-// u += M f (TRANS: M^T f) for the two targets in the halves.
-template <bool WALL, bool TRANS = false>
+// u += M f (TRANS: M^T f) for the two targets in the halves.  ONCE: one
+// rounding at the size of the sum instead of two (six instructions more for
+// both directions), where there is nothing else to round: sums of a few terms
+// that go on in FP64.
+template <bool WALL, bool TRANS = false, bool ONCE = false>
 __device__ __forceinline__ void mob_apply2(const Mob<float2> &m, float2 dx, float2 dy, float2 dz,
                                            float2 fx, float2 fy, float2 fz, float2 &ux, float2 &uy,
                                            float2 &uz)
@@ -467,6 +470,13 @@ __device__ __forceinline__ void mob_apply2(const Mob<float2> &m, float2 dx, floa
     const float2 rf = fma2(dx, fx, mul2(dy, fy));
     const float2 G = WALL ? fma2(m.H, rf, mul2(TRANS ? m.Bb : m.Bf, fz))
                           : mul2(m.H, fma2(dz, fz, rf));
+    if (ONCE) {
+        ux = add2(ux, fma2(m.Cx, fx, mul2(G, dx)));
+        uy = add2(uy, fma2(m.Cx, fy, mul2(G, dy)));
+        uz = add2(uz, WALL ? fma2(m.Z, fz, mul2(TRANS ? m.Bf : m.Bb, rf))
+                           : fma2(m.Cx, fz, mul2(G, dz)));
+        return;
+    }
     ux = fma2(m.Cx, fx, fma2(G, dx, ux));
     uy = fma2(m.Cx, fy, fma2(G, dy, uy));
     uz = WALL ? fma2(m.Z, fz, fma2(TRANS ? m.Bf : m.Bb, rf, uz))

@@ -854,6 +854,7 @@ struct Engine {
         release(ctx, scratch);
         release(ctx, tick);
         release(ctx, work_buf);
+        release(ctx, dpart_buf);
         if (hstate) cudaFreeHost(hstate);
     }
 
@@ -1402,7 +1403,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
     }
     if (!mid_split) {
         np_variant = ctx->pair_variant >= 0 ? std::min(3, std::max(1, ctx->pair_variant)) : 3;
-        sym_nt = tick_pair_sum < 3000.0 * 3000.0 ? 32 : tick_pair_sum < 12000.0 * 12000.0 ? 64 : 128;
+        sym_nt = tick_pair_sum < 4096.0 * 4096.0 ? 32 : tick_pair_sum < 12000.0 * 12000.0 ? 64 : 128;
     }
 
     // ---- 2. true residuals and cycle starts

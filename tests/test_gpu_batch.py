@@ -150,7 +150,7 @@ def test_batch_with_a_zero_force_problem(ctx):
 @pytest.mark.parametrize("bodies", [[1, 2, 1], [20, 1, 33], [90, 70]])
 def test_batch_block_sizes(ctx, bodies, prec):
     """The engine's symmetric items take blocks by the pairs of a tick (the
-    first set stays below 3,000^2, the last above) and the FP64 ones 4 to 32
+    first set stays below 4,096^2, the last above) and the FP64 ones 4 to 32
     sources, for problems of one block and of many; every request's bodies
     are set up together.  Against the same problems solved alone."""
     susp = [I.mixed_suspension(70 + k, nb) for k, nb in enumerate(bodies)]
