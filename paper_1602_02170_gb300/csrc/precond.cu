@@ -424,18 +424,6 @@ constexpr int kSplitMaxRows = 512;
 constexpr int kTile = 32;
 constexpr int kPanel = 8;  // columns per panel of the shared-memory Cholesky
 
-__device__ __forceinline__ int64_t owner_body(const int64_t *__restrict__ start, int64_t nb,
-                                              int64_t b)
-{
-    int64_t lo = 0, hi = nb;
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (start[mid] <= b) lo = mid;
-        else hi = mid;
-    }
-    return lo;
-}
-
 struct SplitScratch {
     double *base;
     int64_t stride;  // doubles per body
@@ -452,37 +440,37 @@ int64_t split_stride(int nmax) { return (int64_t)nmax * nmax + 19 * (int64_t)nma
 
 // S1: M_p (scaled) into P_p[0:n, 0:n], row stride m = n + 6: the blocks on
 // and below the diagonal (bj <= bi), the only ones the factorisations read
-// (M_p is symmetric), one warp per blob row and 32 columns (blockIdx.y).
-// Launched with small CTAs so that the rows of a few bodies still reach
-// every SM: the blocks' dependent FP64 arithmetic is the cost.
+// (M_p is symmetric), one per thread in the order of the triangle.  FP64
+// instructions are the cost whatever the lanes do, so the lanes are filled: a
+// warp per blob row and 32 columns left half of them idle for 42 blobs and
+// three quarters for 15 (300 of them in turn: 68 us).  Launched with small CTAs
+// so that the blocks of a few bodies still reach every SM.
+constexpr int kAssembleThreads = 64;
+
 template <bool WALL>
-__global__ void __launch_bounds__(256) pc_assemble_kernel(
+__global__ void __launch_bounds__(kAssembleThreads) pc_assemble_kernel(
     int64_t nb, const double *__restrict__ r, const int64_t *__restrict__ start,
     const int64_t *__restrict__ poff, MobConsts<double> k, double scale, double *__restrict__ P,
-    const double *__restrict__ shift)
+    const double *__restrict__ shift, int parts)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t s0 = start[0], rows = start[nb] - s0;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t it = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); it < rows;
-         it += warps) {
-        const int64_t b = s0 + it;
-        const int64_t p = owner_body(start, nb, b);
-        const int64_t b0 = start[p];
-        const int np = (int)(start[p + 1] - b0), bi = (int)(b - b0);
-        const int m = 3 * np + 6;
-        double *Pp = P + poff[p];
-        const int bj = 32 * (int)blockIdx.y + lane;
-        if (bj <= bi) {
-            double blk[9];
-            block_f64<WALL>(r + 3 * b, r + 3 * (b0 + bj), k, blk);
+    for (int64_t item = blockIdx.x; item < nb * parts; item += gridDim.x) {
+        const int64_t p = item / parts, b0 = start[p];
+        const int np = (int)(start[p + 1] - b0), m = 3 * np + 6;
+        const int e = (int)(item % parts) * kAssembleThreads + threadIdx.x;
+        if (e >= np * (np + 1) / 2) continue;
+        int bi, bj;
+        tri_index(e, bi, bj);
+        double blk[9];
+        block_f64<WALL>(r + 3 * (b0 + bi), r + 3 * (b0 + bj), k, blk);
+        double *out = P + poff[p] + (size_t)(3 * bi) * m + 3 * bj;
 #pragma unroll
-            for (int al = 0; al < 3; ++al)
+        for (int al = 0; al < 3; ++al)
 #pragma unroll
-                for (int be = 0; be < 3; ++be)
-                    Pp[(size_t)(3 * bi + al) * m + 3 * bj + be] =
-                        scale * blk[3 * al + be] + (shift && bi == bj && al == be ? shift[b] : 0.0);
-        }
+            for (int be = 0; be < 3; ++be) {
+                double v = scale * blk[3 * al + be];
+                if (al == be && shift && bi == bj) v += shift[b0 + bi];
+                out[(size_t)al * m + be] = v;
+            }
     }
 }
 
@@ -1487,17 +1475,77 @@ __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
     }
 }
 
-// S4 in double-float: P_p's n x n block = W^T W - (Q N) Q^T in TILE x TILE
-// tiles (as pc_product_kernel; 16 x 16 when there are few bodies, so that the
-// tiles reach more SMs), the tiles of W staged in shared memory as
-// double-float, the result stored in FP64.  256 threads: thread (ty, tx)
-// forms rows ty + (256 / TILE) rr of the tile's column tx.
-template <int TILE>
-__global__ void __launch_bounds__(256) pc_product_df_kernel(
+// S4 in double-float: P_p's n x n block = W^T W - (Q N) Q^T in tiles (as
+// pc_product_kernel), the result stored in FP64.  Many bodies: 32 x 32 tiles
+// on paired arithmetic, two columns to an instruction (300 bodies of 126 and
+// 45 rows in turn: 106 -> 97 us).  Few bodies: 16 x 16
+// tiles, so that they reach more SMs.
+//
+// Entry (i, j) and its mirror from W^T W's.
+__device__ __forceinline__ void product_store(dfl v, int i, int j, int n, int m, int schur,
+                                              const double *__restrict__ QN,
+                                              const double *__restrict__ Qs, double *__restrict__ Pp)
+{
+    if (i >= n || j > i) return;
+    if (schur)
+#pragma unroll
+        for (int bb = 0; bb < 6; ++bb)
+            v = v - df_unpack(QN[6 * i + bb]) * df_unpack(Qs[6 * j + bb]);
+    const double vd = to_double(v);
+    Pp[(size_t)i * m + j] = vd;
+    Pp[(size_t)j * m + i] = vd;
+}
+
+__global__ void __launch_bounds__(256, 3) pc_product_df_kernel(
     int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
     double *__restrict__ P, SplitScratch scr, int tiles_per_body, int schur)
 {
-    constexpr int kRows = 256 / TILE, kRR = TILE / kRows;
+    __shared__ DfTile Wi, Wj;
+    const int tid = threadIdx.x, c2 = tid & 15, r = tid >> 4;
+    const int ldw = scr.nmax;
+    for (int64_t item = blockIdx.x; item < nb * tiles_per_body; item += gridDim.x) {
+        const int64_t p = item / tiles_per_body;
+        int I, J;
+        tri_index((int)(item % tiles_per_body), I, J);
+        const int n = 3 * (int)(start[p + 1] - start[p]), m = n + 6;
+        const int i0 = I * kTile, j0 = J * kTile;
+        if (i0 >= n) continue;  // CTA-uniform
+        const double *W = scr.W(p);
+        const DfTile &X = I == J ? Wi : Wj;
+        dfl2 acc[2];
+        for (int k0 = i0; k0 < n; k0 += kTile) {
+            __syncthreads();
+#pragma unroll
+            for (int x = 0; x < kTile * kTile / 256; ++x) {
+                const int e = tid + 256 * x, kk = e / kTile, cc = e % kTile;
+                const double *row = W + (size_t)(k0 + kk) * ldw;
+                Wi.set(kk, cc, k0 + kk < n && i0 + cc < n ? df_unpack(row[i0 + cc]) : dfl());
+                if (I != J) Wj.set(kk, cc, k0 + kk < n ? df_unpack(row[j0 + cc]) : dfl());
+            }
+            __syncthreads();
+#pragma unroll 4
+            for (int k = 0; k < kTile; ++k) {
+                const dfl2 x = X.pair(k, c2);
+                acc[0] += dfl2(Wi.at(k, r)) * x;
+                acc[1] += dfl2(Wi.at(k, r + 16)) * x;
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = i0 + r + 16 * h, j = j0 + 2 * c2;
+            double *Pp = P + poff[p];
+            product_store(dfl(acc[h].hi.x, acc[h].lo.x), i, j, n, m, schur, scr.QN(p), scr.Q(p), Pp);
+            product_store(dfl(acc[h].hi.y, acc[h].lo.y), i, j + 1, n, m, schur, scr.QN(p), scr.Q(p),
+                          Pp);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) pc_product_df16_kernel(
+    int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
+    double *__restrict__ P, SplitScratch scr, int tiles_per_body, int schur)
+{
+    constexpr int TILE = 16;
     __shared__ dfl Wi[TILE][TILE + 1], Wj[TILE][TILE + 1];
     const int tx = threadIdx.x % TILE, ty = threadIdx.x / TILE;
     for (int64_t item = blockIdx.x; item < nb * tiles_per_body; item += gridDim.x) {
@@ -1509,7 +1557,7 @@ __global__ void __launch_bounds__(256) pc_product_df_kernel(
         if (i0 >= n) continue;  // CTA-uniform
         const double *W = scr.W(p);
         const int ldw = scr.nmax;
-        dfl acc[kRR];
+        dfl acc;
         for (int k0 = i0; k0 < n; k0 += TILE) {
             __syncthreads();
             for (int e = threadIdx.x; e < TILE * TILE; e += blockDim.x) {
@@ -1520,28 +1568,9 @@ __global__ void __launch_bounds__(256) pc_product_df_kernel(
             }
             __syncthreads();
 #pragma unroll 4
-            for (int kk = 0; kk < TILE; ++kk) {
-                const dfl wj = Wj[kk][tx];
-#pragma unroll
-                for (int rr = 0; rr < kRR; ++rr) acc[rr] += Wi[kk][ty + kRows * rr] * wj;
-            }
+            for (int kk = 0; kk < TILE; ++kk) acc += Wi[kk][ty] * Wj[kk][tx];
         }
-        const double *Qs = scr.Q(p), *QN = scr.QN(p);
-        double *Pp = P + poff[p];
-        const int j = j0 + tx;
-#pragma unroll
-        for (int rr = 0; rr < kRR; ++rr) {
-            const int i = i0 + ty + kRows * rr;
-            if (i >= n || j >= n || (I == J && j > i)) continue;
-            dfl v = acc[rr];
-            if (schur)
-#pragma unroll
-                for (int bb = 0; bb < 6; ++bb)
-                    v = v - df_unpack(QN[6 * i + bb]) * df_unpack(Qs[6 * j + bb]);
-            const double vd = to_double(v);
-            Pp[(size_t)i * m + j] = vd;
-            Pp[(size_t)j * m + i] = vd;
-        }
+        product_store(acc, i0 + ty, j0 + tx, n, m, schur, scr.QN(p), scr.Q(p), P + poff[p]);
     }
 }
 
@@ -1693,12 +1722,10 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
         const int64_t ng = std::min(group, nb - g0);
         const int64_t *st = start + g0;
         const int64_t *po = poff + g0;
-        const dim3 ga((unsigned)std::min<int64_t>(ceil_div(ng * max_np, 2), 32 * (int64_t)ctx->sm_count),
-                      (unsigned)ceil_div(max_np, 32));
-        if (wall)
-            pc_assemble_kernel<true><<<ga, 64, 0, s>>>(ng, r, st, po, k, scale, P, shift);
-        else
-            pc_assemble_kernel<false><<<ga, 64, 0, s>>>(ng, r, st, po, k, scale, P, shift);
+        const int parts = (int)ceil_div((int64_t)max_np * (max_np + 1) / 2, kAssembleThreads);
+        const auto assemble = wall ? pc_assemble_kernel<true> : pc_assemble_kernel<false>;
+        assemble<<<(unsigned)std::min<int64_t>(ng * parts, 1 << 30), kAssembleThreads, 0, s>>>(
+            ng, r, st, po, k, scale, P, shift, parts);
         // A cluster of CTAs per body while all clusters (two CTAs an SM) run at
         // once, or, for blocks in global memory, with fewer bodies than SMs; one
         // CTA per body otherwise.  42-blob bodies, clusters: 97 us for 8, 118
@@ -1748,10 +1775,10 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
             if (ng < ctx->sm_count) {
                 const int T16 = (int)ceil_div(nmax, 16), tiles16 = T16 * (T16 + 1) / 2;
                 const int gp = (int)std::min<int64_t>(ng * tiles16, 16 * (int64_t)ctx->sm_count);
-                pc_product_df_kernel<16><<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles16, schur);
+                pc_product_df16_kernel<<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles16, schur);
             } else {
-                const int gp = (int)std::min<int64_t>(ng * tiles, 16 * (int64_t)ctx->sm_count);
-                pc_product_df_kernel<kTile><<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles, schur);
+                const int gp = (int)std::min<int64_t>(ng * tiles, 1 << 30);
+                pc_product_df_kernel<<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles, schur);
             }
             count_launch(4);
             MB_CUDA_TRY(ctx, cudaGetLastError());
