@@ -363,8 +363,9 @@ __global__ void pc_to_f32_kernel(const double *__restrict__ a, int64_t count, fl
 
 // TP: the blocks' type, FP64, or FP32 (an FP32 copy of the explicit blocks
 // for the FP32 inner iterations of mixed precision; products and sums in
-// FP32 too).
-template <typename TP>
+// FP32 too).  SYMV (FP64, 32 rows or more to a CTA): by symv_rows, else a warp
+// per row.
+template <typename TP, bool SYMV>
 __global__ void __launch_bounds__(256) precond_apply_kernel(
     int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
     const TP *__restrict__ P, const double *__restrict__ w, const double *__restrict__ g,
@@ -388,6 +389,14 @@ __global__ void __launch_bounds__(256) precond_apply_kernel(
             xs[e] = TP(e < n ? w[3 * b0 + e] : g[6 * p + (e - n)]);
         __syncthreads();
         const TP *Pp = P + poff[p];
+        if constexpr (SYMV) {
+            __shared__ double red[8 * kSymvRows];
+            symv_rows(Pp, m, xs, me, r0, r1, red, [&](int row, double y) {
+                if (row < n) lam[3 * b0 + row] = y;
+                else UO[6 * p + (row - n)] = y;
+            });
+            continue;
+        }
         for (int row = r0 + warp; row < r1; row += nw) {
             const TP *pr = Pp + (size_t)row * m;
             TP acc = TP(0);
@@ -2290,15 +2299,20 @@ static void precond_apply_impl(mb_context *ctx, const double *w, const double *g
     }
     const int rows = (int)ceil_div(m, chunks);
     if (f32)
-        precond_apply_kernel<float><<<grid, 256, sizeof(float) * m, s>>>(
+        precond_apply_kernel<float, false><<<grid, 256, sizeof(float) * m, s>>>(
             ctx->pc_nb, (const int64_t *)ctx->blob_start_copy.ptr,
             (const int64_t *)ctx->pinv_off.ptr, (const float *)ctx->pinv32.ptr, w, g, lam, UO,
             chunks, rows, body_rows);
-    else
-        precond_apply_kernel<double><<<grid, 256, sizeof(double) * m, s>>>(
+    else {
+        // 32 rows or more to a CTA fill the lanes of symv_rows; with fewer a
+        // warp per row keeps all eight warps at work
+        const auto kern = rows >= 32 ? precond_apply_kernel<double, true>
+                                     : precond_apply_kernel<double, false>;
+        kern<<<grid, 256, sizeof(double) * m, s>>>(
             ctx->pc_nb, (const int64_t *)ctx->blob_start_copy.ptr,
             (const int64_t *)ctx->pinv_off.ptr, (const double *)ctx->pinv.ptr, w, g, lam, UO,
             chunks, rows, body_rows);
+    }
     count_launch();
 }
 

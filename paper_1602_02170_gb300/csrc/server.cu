@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(256) eng_precond_apply_kernel(
     const int *__restrict__ jidx, int64_t ld, int64_t n_cap, const int *__restrict__ mask)
 {
     extern __shared__ double xs[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __shared__ double red[8 * kSymvRows];
     for (int64_t p = p_lo + blockIdx.x; p < p_hi; p += gridDim.x) {
         const int s = body_slot[p];
         if (s < 0 || !mask[s]) continue;  // uniform across the CTA
@@ -464,18 +464,10 @@ __global__ void __launch_bounds__(256) eng_precond_apply_kernel(
         for (int e = threadIdx.x; e < m; e += blockDim.x)
             xs[e] = e < n ? v[3 * b0 + e] : v[3 * n_cap + 6 * p + (e - n)];
         __syncthreads();
-        const double *Pp = P + poff[p];
-        for (int row = warp; row < m; row += nw) {
-            const double *pr = Pp + (size_t)row * m;
-            double acc = 0.0;
-            for (int c = lane; c < m; c += 32) acc += pr[c] * xs[c];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) {
-                if (row < n) z[3 * b0 + row] = acc;
-                else z[3 * n_cap + 6 * p + (row - n)] = acc;
-            }
-        }
+        symv_rows(P + poff[p], m, xs, m, 0, m, red, [&](int row, double y) {
+            if (row < n) z[3 * b0 + row] = y;
+            else z[3 * n_cap + 6 * p + (row - n)] = y;
+        });
     }
 }
 
