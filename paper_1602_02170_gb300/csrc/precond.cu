@@ -569,7 +569,10 @@ __device__ __forceinline__ int panel_cholesky8(double &v0, double &v1, int w, in
 // the triangle is dealt out entry by entry and not row by row (a third of the
 // lanes of 32-column pieces of rows are idle), and the rows of the lower
 // triangle lie back to back, so that two CTAs fit an SM and one's serial
-// diagonal blocks run beside the other's updates.  300 bodies of 126 and 45
+// diagonal blocks run beside the other's updates.  Bodies of several sizes come
+// in pc_order_kernel's order: dealt out as they come, two long ones share an SM
+// beside two short ones on the next (306 us in this kernel for the 300, 221 in
+// order).  300 bodies of 126 and 45
 // rows in turn, setup and application: 1,260 -> 851 us against a square block, a
 // panel of all rows on one warp and rows dealt to warps (672 us in that kernel
 // and 34 in the conversion of its outputs, which is now done here).
@@ -578,7 +581,7 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
     SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base,
-    int schur)
+    int schur, const int *__restrict__ order)
 {
     extern __shared__ double sm[];
     __shared__ int bad, pfail;
@@ -590,7 +593,8 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
     double *ils = pT + (size_t)kPanel * nmax;             // 1 / L_cc
     double *S = ils + nmax, *Nm = S + 36;
     auto row = [&](int i) { return L + i * (i + 1) / 2; };
-    for (int64_t p = blockIdx.x; p < nb; p += gridDim.x) {
+    for (int64_t it = blockIdx.x; it < nb; it += gridDim.x) {
+        const int64_t p = order ? order[it] : it;
         const int64_t b0 = start[p];
         const int np = (int)(start[p + 1] - b0);
         const int n = 3 * np, m = n + 6;
@@ -718,6 +722,30 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
             Pp[(size_t)(n + threadIdx.x / 6) * m + n + threadIdx.x % 6] = -Nm[threadIdx.x];
         }
     }
+}
+
+// Bodies from the largest to the smallest (a counting sort by blobs, at most
+// kSmemMaxRows / 3): CTAs start in this order, so that the long ones spread over
+// the SMs and the short ones fill in beside them.
+__global__ void __launch_bounds__(1024) pc_order_kernel(int64_t nb, const int64_t *__restrict__ start,
+                                                        int *__restrict__ order)
+{
+    constexpr int kMax = kSmemMaxRows / 3;
+    __shared__ int count[kMax + 2];
+    for (int b = threadIdx.x; b < kMax + 2; b += blockDim.x) count[b] = 0;
+    __syncthreads();
+    for (int64_t p = threadIdx.x; p < nb; p += blockDim.x)
+        atomicAdd(count + (int)(start[p + 1] - start[p]), 1);
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int b = kMax, at = 0; b >= 0; --b) {
+            const int c = count[b];
+            count[b] = at;
+            at += c;
+        }
+    __syncthreads();
+    for (int64_t p = threadIdx.x; p < nb; p += blockDim.x)
+        order[atomicAdd(count + (int)(start[p + 1] - start[p]), 1)] = (int)p;
 }
 
 size_t factor_small_smem(int nmax)
@@ -1335,6 +1363,7 @@ struct TrinvSmem {
     dfl dw[kTrinvTiles * kTile];
     dfl q[kTile][6];
 };
+static_assert(sizeof(dfl) * 6 * kTrinvTiles * kTile <= sizeof(DfTile), "G fits one tile");
 
 // S3 in double-float: one CTA per body and 32 columns t of W = L^-1, by 32 x 32
 // tiles.  The diagonal tiles s >= t are inverted side by side, two warps each
@@ -1347,7 +1376,7 @@ struct TrinvSmem {
 // A warp per column of W (or two, for few bodies), one row after the other,
 // spent about 130 instructions a step on chains of up to 126 steps: 303 us for
 // 300 bodies of 126 and 45 rows in turn and 50 us for 8 of 126.  Setup and
-// application of the 300: 851 -> 681 us.
+// application of the 300: 851 -> 681 us (this kernel 112 us now, 49 for 8 bodies).
 __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
     int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
     double *__restrict__ P, SplitScratch scr, int tiles)
@@ -1368,6 +1397,7 @@ __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
             return i > k && i < n ? df_unpack(Lt[(size_t)k * m + i]) : dfl();
         };
         __syncthreads();  // done with the previous item
+#pragma unroll 4
         for (int e = tid; e < T * (kTile + 1) * kTile; e += 256) {
             const int j = e / ((kTile + 1) * kTile), x = e % ((kTile + 1) * kTile);
             const int row = x % (kTile + 1), col = x / (kTile + 1), g0 = (t + j) * kTile;
@@ -1390,6 +1420,7 @@ __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
                 __syncwarp();
                 if (half == 0) X.set(k, c, wk);
                 const dfl2 w2 = dfl2(wk);
+#pragma unroll 2
                 for (int i = k + 1 + 2 * half; i < kTile; i += 4) {
                     const dfl a0 = X.at(i, c), a1 = X.at(i + 1, c);
                     const dfl l0 = Ls.at(i, k), l1 = Ls.at(i + 1, k);
@@ -1438,6 +1469,11 @@ __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
             sm.A[s].set_pair(r + 16, c2, w[1]);
         }
         __syncthreads();
+        // G's rows into A[0], free by now
+        dfl *Gs = (dfl *)&sm.A[0];
+        const int rows = n - t * kTile;
+#pragma unroll 3
+        for (int e = tid; e < 6 * rows; e += 256) Gs[e] = df_unpack(scr.G(p)[6 * t * kTile + e]);
         // W's columns (zero above the diagonal within the diagonal tile)
         double *W = scr.W(p);
         const int ldw = scr.nmax, c0 = t * kTile;
@@ -1447,19 +1483,19 @@ __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
             if (gi < n && c0 + c < n)
                 W[(size_t)gi * ldw + c0 + c] = df_pack((j ? sm.A[j] : sm.D[0]).at(i, c));
         }
+        __syncthreads();
         // Q[c][b] = sum_k W[k][c] G[k][b], even and odd rows in the halves
         const int c = tid % kTile, b = tid / kTile;
         const bool mine = b < 6 && c0 + c < n;
         if (mine) {
-            const double *G = scr.G(p);
             dfl2 acc;
             for (int j = 0; j < T; ++j) {
                 const DfTile &X = j ? sm.A[j] : sm.D[0];
-                const int g0 = (t + j) * kTile, rows = min(kTile, n - g0);
-                for (int i = 0; i < rows; i += 2) {
+#pragma unroll 4
+                for (int i = 0; i < min(kTile, rows - j * kTile); i += 2) {
+                    const int k = j * kTile + i;
                     const dfl x0 = X.at(i, c), x1 = X.at(i + 1, c);
-                    const dfl g1 = df_unpack(G[6 * (g0 + i) + b]),
-                              g2 = i + 1 < rows ? df_unpack(G[6 * (g0 + i + 1) + b]) : dfl();
+                    const dfl g1 = Gs[6 * k + b], g2 = k + 1 < rows ? Gs[6 * (k + 1) + b] : dfl();
                     acc += dfl2(make_float2(x0.hi, x1.hi), make_float2(x0.lo, x1.lo)) *
                            dfl2(make_float2(g1.hi, g2.hi), make_float2(g1.lo, g2.lo));
                 }
@@ -1487,7 +1523,7 @@ __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
 // S4 in double-float: P_p's n x n block = W^T W - (Q N) Q^T in tiles (as
 // pc_product_kernel), the result stored in FP64.  Many bodies: 32 x 32 tiles
 // on paired arithmetic, two columns to an instruction (300 bodies of 126 and
-// 45 rows in turn: 106 -> 97 us).  Few bodies: 16 x 16
+// 45 rows in turn: 106 -> 86 us).  Few bodies: 16 x 16
 // tiles, so that they reach more SMs.
 //
 // Entry (i, j) and its mirror from W^T W's.
@@ -1521,16 +1557,29 @@ __global__ void __launch_bounds__(256, 3) pc_product_df_kernel(
         if (i0 >= n) continue;  // CTA-uniform
         const double *W = scr.W(p);
         const DfTile &X = I == J ? Wi : Wj;
+        // tiles pass through registers, loaded while the ones before are in use
+        constexpr int kLoads = kTile * kTile / 256;
+        double wi[kLoads], wj[kLoads];
+        auto fetch = [&](int k0) {
+#pragma unroll
+            for (int x = 0; x < kLoads; ++x) {
+                const int e = tid + 256 * x, k = k0 + e / kTile, cc = e % kTile;
+                const double *row = W + (size_t)k * ldw;
+                wi[x] = k < n && i0 + cc < n ? row[i0 + cc] : 0.0;
+                wj[x] = k < n && I != J ? row[j0 + cc] : 0.0;
+            }
+        };
+        fetch(i0);
         dfl2 acc[2];
         for (int k0 = i0; k0 < n; k0 += kTile) {
             __syncthreads();
 #pragma unroll
-            for (int x = 0; x < kTile * kTile / 256; ++x) {
-                const int e = tid + 256 * x, kk = e / kTile, cc = e % kTile;
-                const double *row = W + (size_t)(k0 + kk) * ldw;
-                Wi.set(kk, cc, k0 + kk < n && i0 + cc < n ? df_unpack(row[i0 + cc]) : dfl());
-                if (I != J) Wj.set(kk, cc, k0 + kk < n ? df_unpack(row[j0 + cc]) : dfl());
+            for (int x = 0; x < kLoads; ++x) {
+                const int e = tid + 256 * x;
+                Wi.set(e / kTile, e % kTile, df_unpack(wi[x]));
+                if (I != J) Wj.set(e / kTile, e % kTile, df_unpack(wj[x]));
             }
+            if (k0 + kTile < n) fetch(k0 + kTile);
             __syncthreads();
 #pragma unroll 4
             for (int k = 0; k < kTile; ++k) {
@@ -1708,18 +1757,20 @@ __global__ void __launch_bounds__(256) pc_keep_factor_kernel(
     }
 }
 
+// sizes: the bodies are not all of one size.
 // Runs S1..S4 over groups of bodies whose scratch fits the cap (S1, S2, S3'
 // with `factored`).
 mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double *q,
                       const int64_t *start, const int64_t *poff, double *P, int max_np, double a,
                       double eta, int wall, int *flag, const int *flag_slot, int schur, cudaStream_t s,
-                      const double *shift, bool factored = false)
+                      const double *shift, bool sizes, bool factored = false)
 {
     const int nmax = 3 * max_np;
     const int64_t stride = split_stride(nmax);
     const int64_t cap_bytes = (int64_t)MB_SETUP_SCRATCH_MB << 20;
     const int64_t group = std::max<int64_t>(1, std::min<int64_t>(nb, cap_bytes / (8 * stride)));
-    MB_TRY(ensure(ctx, ctx->sol_dots, sizeof(double) * stride * group, "preconditioner scratch"));
+    MB_TRY(ensure(ctx, ctx->sol_dots, (sizeof(double) * stride + sizeof(int)) * group,
+                  "preconditioner scratch"));
     SplitScratch scr{(double *)ctx->sol_dots.ptr, stride, nmax};
     const MobConsts<double> k = MobConsts<double>::make(a);
     const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
@@ -1750,14 +1801,27 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
             fk<<<(int)ng * kFacCluster, 256, csm, s>>>(ng, r, q + 3 * g0, st, po, P, scr, flag,
                                                        flag_slot, g0, schur);
         } else {
-            const size_t fsmem = lsmem ? factor_small_smem(nmax)
-                                       : sizeof(double) * (2 * (size_t)nmax + 72);
-            auto factor = df ? pc_factor_small_kernel<true>
-                             : lsmem ? pc_factor_small_kernel<false> : pc_factor_kernel;
-            MB_CUDA_TRY(ctx, cudaFuncSetAttribute(factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)fsmem));
-            factor<<<(int)std::min<int64_t>(ng, 4 * (int64_t)ctx->sm_count), 256, fsmem, s>>>(
-                ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur);
+            if (lsmem) {
+                const size_t fsmem = factor_small_smem(nmax);
+                auto factor = df ? pc_factor_small_kernel<true> : pc_factor_small_kernel<false>;
+                MB_CUDA_TRY(ctx, cudaFuncSetAttribute(factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      (int)fsmem));
+                int *order = nullptr;
+                if (sizes && ng > ctx->sm_count) {
+                    order = (int *)(scr.base + stride * group);
+                    pc_order_kernel<<<1, 1024, 0, s>>>(ng, st, order);
+                    count_launch();
+                }
+                factor<<<(unsigned)std::min<int64_t>(ng, 1 << 30), 256, fsmem, s>>>(
+                    ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur, order);
+            } else {
+                const size_t fsmem = sizeof(double) * (2 * (size_t)nmax + 72);
+                MB_CUDA_TRY(ctx, cudaFuncSetAttribute(pc_factor_kernel,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      (int)fsmem));
+                pc_factor_kernel<<<(int)std::min<int64_t>(ng, 4 * (int64_t)ctx->sm_count), 256, fsmem, s>>>(
+                    ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur);
+            }
         }
         if (factored) {
             pc_keep_factor_kernel<<<(int)std::min<int64_t>(ceil_div(ng, 8), 8 * (int64_t)ctx->sm_count),
@@ -1886,11 +1950,12 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
         return set_err(ctx, MB_EINVAL, "blob_start[0] must be 0 and blob_start[n_b] = N");
     std::vector<int64_t> off(nb + 1);
     off[0] = 0;
-    int max_np = 0;
+    int max_np = 0, min_np = 0x7fffffff;
     for (int64_t p = 0; p < nb; ++p) {
         const int64_t np = hstart[p + 1] - hstart[p];
         if (np < 1) return set_err(ctx, MB_EINVAL, "body %lld has no blobs", (long long)p);
         max_np = std::max<int>(max_np, (int)np);
+        min_np = std::min<int>(min_np, (int)np);
         off[p + 1] = off[p] + (3 * np + 6) * (3 * np + 6);
     }
     MB_TRY(ensure(ctx, ctx->pinv, sizeof(double) * off[nb], "preconditioner"));
@@ -1928,7 +1993,7 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
         if (nmax <= kSplitMaxRowsSmem)
             return setup_split(ctx, nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,
                                (const int64_t *)ctx->pinv_off.ptr, (double *)ctx->pinv.ptr, max_np,
-                               a, eta, wall, (int *)ctx->flag.ptr, nullptr, schur, s, shift, factored);
+                               a, eta, wall, (int *)ctx->flag.ptr, nullptr, schur, s, shift, min_np < max_np, factored);
         MB_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
         kern<<<grid, kSetupThreads, smem, s>>>(nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,
@@ -1977,7 +2042,7 @@ size_t precond_scratch_bytes(int64_t nb, int max_np)
 mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, const double *q,
                               const int64_t *start, const int64_t *poff, double *P, int max_np,
                               double a, double eta, int wall, int *flags, const int *flag_slot,
-                              cudaStream_t s, int schur)
+                              cudaStream_t s, bool sizes, int schur)
 {
     const int nmax = 3 * max_np;
     const bool lsmem = nmax <= kSmemMaxRows;
@@ -1997,7 +2062,7 @@ mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, cons
     auto launch = [&](auto kern) -> mb_status {
         if (nmax <= kSplitMaxRowsSmem)
             return setup_split(ctx, nb, r, q, start, poff, P, max_np, a, eta, wall, flags,
-                               flag_slot, schur, s, nullptr);
+                               flag_slot, schur, s, nullptr, sizes);
         MB_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
         kern<<<grid, kSetupThreads, smem, s>>>(nb, r, q, start, poff, k, scale, P, scratch, stride,
@@ -2109,7 +2174,7 @@ mb_status precond_setup_shared(mb_context *ctx, int64_t nb, int64_t n, const dou
         max_ref_np = std::max<int>(max_ref_np, (int)(rstart[t + 1] - rstart[t]));
     MB_TRY(precond_setup_range(ctx, ns, dref, dref + 3 * rstart[ns], dstart, doff,
                                (double *)ctx->pinv.ptr, max_ref_np, a, eta, 0,
-                               (int *)ctx->flag.ptr, nullptr, s, schur));
+                               (int *)ctx->flag.ptr, nullptr, s, true, schur));
     int first_bad = big;
     MB_CUDA_TRY(ctx, cudaMemcpyAsync(&first_bad, ctx->flag.ptr, sizeof(int),
                                      cudaMemcpyDeviceToHost, s));

@@ -1274,7 +1274,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
         for (size_t i = 0; i < admitted.size();) {
             const Req *first = admitted[i], *prev = first;
             int64_t nb = first->prob.n_bodies, nblob = first->prob.n_blobs;
-            int max_np = first->max_np;
+            int max_np = first->max_np, min_np = max_np;
             size_t end = i + 1;
             const size_t room = ctx->budget > ctx->held ? ctx->budget - ctx->held : 0;
             for (; end < admitted.size(); ++end) {
@@ -1308,6 +1308,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
                     bs.push_back(rq->blob_off + rq->hstart[p]);
                     const int64_t np = rq->hstart[p + 1] - rq->hstart[p];
                     acc += (3 * np + 6) * (3 * np + 6);
+                    min_np = std::min(min_np, (int)np);
                 }
             }
             bs.push_back(b1);
@@ -1320,7 +1321,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
             MB_TRY(precond_setup_range(ctx, nb, r, q + 3 * first->body_off,
                                        bstart + first->start_off, poff + first->body_off, P, max_np,
                                        prm.a, prm.eta, prm.wall, st.bad,
-                                       body_slot + first->body_off, s));
+                                       body_slot + first->body_off, s, min_np < max_np));
         }
         std::vector<Seg> segs;
         std::vector<int> seg_off, list;
