@@ -437,15 +437,16 @@ struct SplitScratch {
     double *base;
     int64_t stride;  // doubles per body
     int nmax;
+    int64_t wsize;   // doubles of W (0: none, the factored form)
     __device__ double *W(int64_t p) const { return base + p * stride; }
-    __device__ double *G(int64_t p) const { return W(p) + (int64_t)nmax * nmax; }
+    __device__ double *G(int64_t p) const { return W(p) + wsize; }
     __device__ double *Q(int64_t p) const { return G(p) + 6 * nmax; }
     __device__ double *QN(int64_t p) const { return Q(p) + 6 * nmax; }
     __device__ double *dW(int64_t p) const { return QN(p) + 6 * nmax; }
     __device__ double *N(int64_t p) const { return dW(p) + nmax; }
 };
 
-int64_t split_stride(int nmax) { return (int64_t)nmax * nmax + 19 * (int64_t)nmax + 36; }
+int64_t split_stride(int nmax, int64_t wsize) { return wsize + 19 * (int64_t)nmax + 36; }
 
 // S1: M_p (scaled) into P_p[0:n, 0:n], row stride m = n + 6: the blocks on
 // and below the diagonal (bj <= bi), the only ones the factorisations read
@@ -753,134 +754,9 @@ size_t factor_small_smem(int nmax)
     return sizeof(double) * ((size_t)nmax * (nmax + 1) / 2 + (7 + kPanel) * (size_t)nmax + 72);
 }
 
-// S2 for larger blocks: one CTA per body, factored in place in global memory
-// with the six columns B = K_p appended in the scratch.
-__global__ void __launch_bounds__(256) pc_factor_kernel(
-    int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
-    const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
-    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base,
-    int schur)
-{
-    extern __shared__ double sm[];
-    __shared__ int bad;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int64_t p = blockIdx.x; p < nb; p += gridDim.x) {
-        const int64_t b0 = start[p];
-        const int np = (int)(start[p + 1] - b0);
-        const int n = 3 * np, m = n + 6;
-        double *Pp = P + poff[p];
-        double *L = Pp;
-        const int ld = m;
-        double *B = scr.G(p);
-        double *ils = sm;  // 1 / sqrt(d_c)
-        double *S = ils + n;
-        double *Nm = S + 36;
-        double *col = Nm + 36;  // pivot row
-        const double qx = q[3 * p], qy = q[3 * p + 1], qz = q[3 * p + 2];
-        __syncthreads();
-        if (threadIdx.x == 0) bad = 0;
-        // B = K_p: rows of blob i are [I, -[d_i]x]
-        for (int e = threadIdx.x; e < 6 * n; e += blockDim.x)
-            B[e] = k_entry(r + 3 * b0, qx, qy, qz, e / 6, e % 6);
-        int fail = 0;
-        // Left-looking (Crout) order.  Column j is
-        // L[i][j] = (A[i][j] - L[i][0:j] . L[j][0:j]) / L[j][j], one coalesced
-        // dot product per row with the pivot row L[j][0:j] in shared memory
-        // (`col`); every entry is written once, so the inner loop only loads
-        // and the many independent loads in flight hide the memory latency
-        // that the right-looking update's read-modify-writes exposed.  Row j
-        // of G = L^-1 K follows from the same pivot row.
-        for (int c = 0; c < n; ++c) {
-            __syncthreads();  // step c - 1 finished with col
-            // the pivot row with its diagonal entry: every warp reads A[c][c]
-            // from here, since thread 0 overwrites it in L below
-            for (int k = threadIdx.x; k <= c; k += blockDim.x) col[k] = L[(size_t)c * ld + k];
-            __syncthreads();
-            // pivot d = A[c][c] - |L[c][0:c]|^2, computed by every warp alike
-            double acc = 0.0;
-            for (int k = lane; k < c; k += 32) acc += col[k] * col[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            const double d = col[c] - acc;
-            if (!pivot_ok(d)) {  // the same value in every thread
-                fail = 1;
-                break;
-            }
-            const double il = pivot_rsqrt(d);
-            if (threadIdx.x == 0) {
-                ils[c] = il;
-                L[(size_t)c * ld + c] = d * il;  // sqrt(d)
-            }
-            for (int i = c + 1 + warp; i < n; i += nw) {
-                const double *Li = L + (size_t)i * ld;
-                double dot = 0.0;
-                for (int k = lane; k < c; k += 32) dot += Li[k] * col[k];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                if (lane == 0) L[(size_t)i * ld + c] = (Li[c] - dot) * il;
-            }
-            if (warp == nw - 1) {
-                // G[c][b] = (K[c][b] - L[c][0:c] . G[0:c][b]) / L[c][c]
-#pragma unroll
-                for (int b = 0; b < 6; ++b) {
-                    double g = 0.0;
-                    for (int k = lane; k < c; k += 32) g += col[k] * B[6 * k + b];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-                    if (lane == 0) B[6 * c + b] = (B[6 * c + b] - g) * il;
-                }
-            }
-        }
-        __syncthreads();
-        if (fail) {  // uniform: a pivot was not positive
-            if (threadIdx.x == 0) {
-                if (flag_slot) flag[flag_slot[p_base + p]] = 2;
-                else atomicMin(flag, (int)(p_base + p));
-            }
-            continue;
-        }
-        // dW to scratch; L^T into P_p's upper triangle (row k holds column k of L)
-        double *dW = scr.dW(p);
-        for (int i = threadIdx.x; i < n; i += blockDim.x) dW[i] = ils[i];
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            const int kk = e / n, i = e % n;
-            if (i > kk) Pp[(size_t)kk * m + i] = L[(size_t)i * ld + kk];
-        }
-        __syncthreads();
-        // S = G^T G (symmetric 6 x 6), one warp per entry
-        for (int ab = warp; ab < 36; ab += nw) {
-            const int a = ab / 6, bb = ab % 6;
-            double acc = 0.0;
-            for (int i = lane; i < n; i += 32) acc += B[6 * i + a] * B[6 * i + bb];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) S[ab] = acc;
-        }
-        __syncthreads();
-        // N = S^-1 (warp 0)
-        if (warp == 0) {
-            const int f = inverse6_warp(S, Nm, lane);
-            if (lane == 0 && f) bad = schur;
-        }
-        __syncthreads();
-        if (bad) {
-            if (threadIdx.x == 0) {
-                if (flag_slot) flag[flag_slot[p_base + p]] = 2;
-                else atomicMin(flag, (int)(p_base + p));
-            }
-            continue;
-        }
-        double *Ns = scr.N(p);
-        if (threadIdx.x < 36) {
-            Ns[threadIdx.x] = Nm[threadIdx.x];
-            Pp[(size_t)(n + threadIdx.x / 6) * m + n + threadIdx.x % 6] = -Nm[threadIdx.x];
-        }
-    }
-}
-
-// S2 on a cluster of kFacCluster CTAs per body, for problems with fewer
-// bodies than SMs (one SM per body would leave most of the chip idle, and
-// one SM sustains only about 1.7 FP64 FMA per clock).  Rows are dealt cyclically:
+// S2 on a cluster of kFacCluster CTAs per body, for few bodies (one SM per body
+// would leave most of the chip idle, and one SM sustains only about 1.7 FP64
+// FMA per clock) and for blocks beyond one CTA's shared memory.  Rows are dealt cyclically:
 // CTA r holds rows i = r + kFacCluster t of M_p (and of B = K_p).  Panel q
 // (columns c0 .. c0 + w - 1, t0 = c0 + w) runs in three stages:
 //   (A) warp 0 factors the panel's diagonal block, which every CTA holds in
@@ -1736,23 +1612,49 @@ __global__ void __launch_bounds__(256) pc_product_kernel(
 
 // S3' for the factored form (instead of S3 and S4): P_p keeps L^T in its
 // upper triangle (written by S2) and receives G = L^-1 K_p in the border
-// columns n..n+5 of rows 0..n-1 and 1 / L_kk in the border row n; the corner
-// already holds -N.  precond_apply_factored_kernel applies it.
-__global__ void __launch_bounds__(256) pc_keep_factor_kernel(
+// columns n..n+5 of rows 0..n-1, 1 / L_kk in the border row n, and the inverses
+// of the kFacPanel-row diagonal blocks of L below the diagonal; the corner
+// already holds -N.  precond_apply_factored_kernel applies it.  A warp per
+// diagonal block, lane c its column c (a forward substitution on registers).
+constexpr int kFacPanel = 32;
+constexpr int kFactoredMinBodies = 64;
+constexpr int kKeepWarps = 4;
+
+__global__ void __launch_bounds__(32 * kKeepWarps) pc_keep_factor_kernel(
     int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
-    double *__restrict__ P, SplitScratch scr)
+    double *__restrict__ P, SplitScratch scr, int panels)
 {
-    const int warps = (int)(gridDim.x * (blockDim.x >> 5));
-    const int lane = threadIdx.x & 31;
-    for (int64_t p = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); p < nb;
-         p += warps) {
+    __shared__ double Ls[kKeepWarps][kFacPanel][kFacPanel];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t it = blockIdx.x * (int64_t)kKeepWarps + warp; it < nb * panels;
+         it += gridDim.x * (int64_t)kKeepWarps) {
+        const int64_t p = it / panels;
+        const int c0 = (int)(it % panels) * kFacPanel;
         const int n = 3 * (int)(start[p + 1] - start[p]), m = n + 6;
+        if (c0 >= n) continue;
+        const int pw = min(kFacPanel, n - c0);
         double *Pp = P + poff[p];
-        const double *G = scr.G(p), *dW = scr.dW(p);
-        for (int i = lane; i < n; i += 32) {
+        const double *G = scr.G(p) + 6 * c0, *dW = scr.dW(p) + c0;
+        if (lane < pw) {
 #pragma unroll
-            for (int b = 0; b < 6; ++b) Pp[(size_t)i * m + n + b] = G[6 * i + b];
-            Pp[(size_t)n * m + i] = dW[i];
+            for (int b = 0; b < 6; ++b) Pp[(size_t)(c0 + lane) * m + n + b] = G[6 * lane + b];
+            Pp[(size_t)n * m + c0 + lane] = dW[lane];
+        }
+        __syncwarp();
+        for (int k = 0; k < kFacPanel; ++k)  // L[i][k], i = lane
+            Ls[warp][k][lane] = k < lane && lane < pw ? Pp[(size_t)(c0 + k) * m + c0 + lane] : 0.0;
+        __syncwarp();
+        double acc[kFacPanel];
+#pragma unroll
+        for (int i = 0; i < kFacPanel; ++i) acc[i] = i == lane ? 1.0 : 0.0;
+#pragma unroll
+        for (int k = 0; k < kFacPanel; ++k) {
+            if (k < pw) {
+                acc[k] *= dW[k];
+#pragma unroll
+                for (int i = k + 1; i < kFacPanel; ++i) acc[i] -= Ls[warp][k][i] * acc[k];
+                if (lane < k) Pp[(size_t)(c0 + k) * m + c0 + lane] = acc[k];
+            }
         }
     }
 }
@@ -1766,12 +1668,12 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
                       const double *shift, bool sizes, bool factored = false)
 {
     const int nmax = 3 * max_np;
-    const int64_t stride = split_stride(nmax);
+    const int64_t wsize = factored ? 0 : (int64_t)nmax * nmax, stride = split_stride(nmax, wsize);
     const int64_t cap_bytes = (int64_t)MB_SETUP_SCRATCH_MB << 20;
     const int64_t group = std::max<int64_t>(1, std::min<int64_t>(nb, cap_bytes / (8 * stride)));
     MB_TRY(ensure(ctx, ctx->sol_dots, (sizeof(double) * stride + sizeof(int)) * group,
                   "preconditioner scratch"));
-    SplitScratch scr{(double *)ctx->sol_dots.ptr, stride, nmax};
+    SplitScratch scr{(double *)ctx->sol_dots.ptr, stride, nmax, wsize};
     const MobConsts<double> k = MobConsts<double>::make(a);
     const double scale = 1.0 / (6.0 * 3.14159265358979323846 * eta * a);
     const bool lsmem = nmax <= kSmemMaxRows;
@@ -1786,12 +1688,14 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
         const auto assemble = wall ? pc_assemble_kernel<true> : pc_assemble_kernel<false>;
         assemble<<<(unsigned)std::min<int64_t>(ng * parts, 1 << 30), kAssembleThreads, 0, s>>>(
             ng, r, st, po, k, scale, P, shift, parts);
-        // A cluster of CTAs per body while all clusters (two CTAs an SM) run at
-        // once, or, for blocks in global memory, with fewer bodies than SMs; one
-        // CTA per body otherwise.  42-blob bodies, clusters: 97 us for 8, 118
-        // for 32, 148 for 40, 264 for 100.
+        // A cluster of CTAs per body for blocks in global memory, and for smaller
+        // ones while all clusters (two CTAs an SM) run at once; one CTA per body
+        // otherwise.  42-blob bodies, clusters: 97 us for 8, 118 for 32, 148 for
+        // 40, 264 for 100.  A CTA per body in global memory, column by column,
+        // took the whole setup of 300 bodies of 54, 80 and 100 blobs from 1.8, 3.6
+        // and 5.7 ms to 3.3, 7.2 and 11.6.
         const bool df = nmax <= kSetupSmallRows;  // double-float S3 and S4
-        if (lsmem ? ng * kFacCluster <= 2 * (int64_t)ctx->sm_count : ng < ctx->sm_count) {
+        if (!lsmem || ng * kFacCluster <= 2 * (int64_t)ctx->sm_count) {
             const size_t csm = factor_cluster_smem(nmax, lsmem);
             auto fk = df ? pc_factor_cluster_kernel<true, true>
                          : lsmem ? pc_factor_cluster_kernel<true, false>
@@ -1801,31 +1705,23 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
             fk<<<(int)ng * kFacCluster, 256, csm, s>>>(ng, r, q + 3 * g0, st, po, P, scr, flag,
                                                        flag_slot, g0, schur);
         } else {
-            if (lsmem) {
-                const size_t fsmem = factor_small_smem(nmax);
-                auto factor = df ? pc_factor_small_kernel<true> : pc_factor_small_kernel<false>;
-                MB_CUDA_TRY(ctx, cudaFuncSetAttribute(factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)fsmem));
-                int *order = nullptr;
-                if (sizes && ng > ctx->sm_count) {
-                    order = (int *)(scr.base + stride * group);
-                    pc_order_kernel<<<1, 1024, 0, s>>>(ng, st, order);
-                    count_launch();
-                }
-                factor<<<(unsigned)std::min<int64_t>(ng, 1 << 30), 256, fsmem, s>>>(
-                    ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur, order);
-            } else {
-                const size_t fsmem = sizeof(double) * (2 * (size_t)nmax + 72);
-                MB_CUDA_TRY(ctx, cudaFuncSetAttribute(pc_factor_kernel,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)fsmem));
-                pc_factor_kernel<<<(int)std::min<int64_t>(ng, 4 * (int64_t)ctx->sm_count), 256, fsmem, s>>>(
-                    ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur);
+            const size_t fsmem = factor_small_smem(nmax);
+            auto factor = df ? pc_factor_small_kernel<true> : pc_factor_small_kernel<false>;
+            MB_CUDA_TRY(ctx, cudaFuncSetAttribute(factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)fsmem));
+            int *order = nullptr;
+            if (sizes && ng > ctx->sm_count) {
+                order = (int *)(scr.base + stride * group);
+                pc_order_kernel<<<1, 1024, 0, s>>>(ng, st, order);
+                count_launch();
             }
+            factor<<<(unsigned)std::min<int64_t>(ng, 1 << 30), 256, fsmem, s>>>(
+                ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur, order);
         }
         if (factored) {
-            pc_keep_factor_kernel<<<(int)std::min<int64_t>(ceil_div(ng, 8), 8 * (int64_t)ctx->sm_count),
-                                    256, 0, s>>>(ng, st, po, P, scr);
+            const int panels = (int)ceil_div(nmax, kFacPanel);
+            pc_keep_factor_kernel<<<(unsigned)std::min<int64_t>(ceil_div(ng * panels, kKeepWarps), 1 << 30),
+                                    32 * kKeepWarps, 0, s>>>(ng, st, po, P, scr, panels);
             count_launch(3);
             MB_CUDA_TRY(ctx, cudaGetLastError());
             continue;
@@ -1984,11 +1880,18 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
         MB_TRY(ensure(ctx, ctx->sol_dots, sizeof(double) * stride * grid, "Cholesky scratch"));
         scratch = (double *)ctx->sol_dots.ptr;
     }
-    // Many bodies with large blocks keep the factored form: its application
-    // costs the FP64 FMAs of the explicit inverse's GEMV and its setup a third
-    // of the explicit inverse's (no L^-1, no W^T W).  Few or small bodies keep
-    // the explicit inverse, whose application spreads over many CTAs.
-    const bool factored = !lsmem && nmax <= kSplitMaxRowsSmem && nb >= ctx->sm_count;
+    // Bodies with large blocks keep the factored form: its application costs the
+    // FP64 FMAs of the explicit inverse's GEMV and its setup a third of the
+    // explicit inverse's (no L^-1, no W^T W).  Few or small bodies keep the
+    // explicit inverse, whose application spreads over many CTAs.  162-blob
+    // shells, setup / application / mixed solve (ms), explicit and factored: 32
+    // bodies 5.9 / 0.05 / 9.4 and 2.0 / 0.15 / 8.2, 80 bodies 14.6 / 0.12 / 27.7
+    // and 5.7 / 0.15 / 21.7, 151 bodies 25.8 / 0.16 / 65.8 and 9.3 / 0.23 / 53.9; the
+    // line lies where an application costs half as much again.  The resistance
+    // problem takes three times the iterations, so there the inverse pays up to
+    // one body an SM.
+    const bool factored = !lsmem && nmax <= kSplitMaxRowsSmem &&
+                          nb >= (schur ? std::min(kFactoredMinBodies, ctx->sm_count) : ctx->sm_count);
     auto launch = [&](auto kern) -> mb_status {
         if (nmax <= kSplitMaxRowsSmem)
             return setup_split(ctx, nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,
@@ -2035,7 +1938,7 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
 
 size_t precond_scratch_bytes(int64_t nb, int max_np)
 {
-    return std::min<size_t>(sizeof(double) * (size_t)nb * split_stride(3 * max_np),
+    return std::min<size_t>(sizeof(double) * (size_t)nb * split_stride(3 * max_np, 9 * (int64_t)max_np * max_np),
                             (size_t)MB_SETUP_SCRATCH_MB << 20);
 }
 
@@ -2199,29 +2102,32 @@ mb_status precond_setup_shared(mb_context *ctx, int64_t nb, int64_t n, const dou
 
 // Application of the factored form (see pc_keep_factor_kernel), one CTA per
 // body, x = the body's rows in shared memory:
-//   y = L^-1 w                  forward substitution by panels of kFacPanel
-//                               rows: warp 0 solves the panel's triangle,
-//                               then all threads subtract the panel's columns
-//                               from the rows below (rows of L^T, coalesced);
+//   y = L^-1 w                  forward by panels of kFacPanel rows: the panel's
+//                               rows are multiplied by the inverse of their
+//                               diagonal block (an eighth of the columns to a
+//                               warp, no chain), then all threads subtract the
+//                               panel's columns from the rows below (rows of
+//                               L^T, coalesced);
 //   U = -N (g + G^T y)          the body rows (skipped for the blob block alone);
-//   lambda = L^-T (y + G U)     backward substitution by panels from the
-//                               bottom: the panel's rows first lose their dot
-//                               products with the solved rows (a warp per
-//                               row), then warp 0 solves the panel's triangle.
-// The panel's triangle is staged in shared memory with its columns scaled by
-// 1 / L_kk, so that each step of warp 0's dependent chain is one shuffle and
-// one FMA.  The same FMAs as the explicit inverse's GEMV (n^2 per body).
-constexpr int kFacPanel = 32;
-
+//   lambda = L^-T (y + G U)     backward by panels from the bottom: the panel's
+//                               rows first lose their dot products with the
+//                               solved rows (four rows to a warp, whose sums
+//                               share one butterfly), then the same product
+//                               with the transposed inverse.
+// The same FMAs as the explicit inverse's GEMV (n^2 per body).  A panel's
+// inverse is staged while the panel before is subtracted.  Solving each panel's
+// triangle by a chain of 32 steps on one warp, and a butterfly to every row,
+// took 415 us for 256 bodies of 486 rows, and this takes 283.
 __global__ void __launch_bounds__(256) precond_apply_factored_kernel(
     int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
     const double *__restrict__ P, const double *__restrict__ w, const double *__restrict__ g,
     double *__restrict__ lam, double *__restrict__ UO, int body_rows)
 {
-    extern __shared__ double x[];              // n: the body's vector
-    __shared__ double T[kFacPanel * kFacPanel];  // scaled panel triangle
+    extern __shared__ double x[];  // n: the body's vector
+    __shared__ double T[2][kFacPanel][kFacPanel + 1];  // T[k][l] = (block's inverse)[l][k]
+    __shared__ double part[8][kFacPanel];
     __shared__ double red[8 * 6];
-    __shared__ double hU[12];                   // h = g + G^T y, then U
+    __shared__ double hU[12];  // h = g + G^T y, then U
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const unsigned full = 0xffffffffu;
     for (int64_t p = blockIdx.x; p < nb; p += gridDim.x) {
@@ -2229,38 +2135,53 @@ __global__ void __launch_bounds__(256) precond_apply_factored_kernel(
         const int n = 3 * (int)(start[p + 1] - b0), m = n + 6;
         const double *Pp = P + poff[p];
         const double *dW = Pp + (size_t)n * m;  // border row n: 1 / L_kk
-        __syncthreads();  // the previous body is finished with x, T, hU
-        for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = w[3 * b0 + i];
-        // ---- forward: y = L^-1 w; L[i][k] = Lt[k][i] = Pp[k m + i]
-        for (int c0 = 0; c0 < n; c0 += kFacPanel) {
+        // the inverse of the diagonal block at c0, zero outside the block
+        auto stage = [&](int c0, int buf) {
             const int pw = min(kFacPanel, n - c0);
-            // T[k][l] = L[c0 + l][c0 + k] / L_kk for k < l (row k of L^T, scaled)
-            for (int e = threadIdx.x; e < pw * pw; e += blockDim.x) {
-                const int k = e / pw, l = e % pw;
-                T[k * kFacPanel + l] = l > k ? Pp[(size_t)(c0 + k) * m + c0 + l] * dW[c0 + k] : 0.0;
+            for (int e = threadIdx.x; e < kFacPanel * kFacPanel; e += blockDim.x) {
+                const int l = e / kFacPanel, k = e % kFacPanel;
+                T[buf][k][l] = l >= pw || k > l ? 0.0
+                               : k < l          ? Pp[(size_t)(c0 + l) * m + c0 + k]
+                                                : dW[c0 + k];
             }
+        };
+        // rows c0 .. of x times the staged inverse (TRANS: transposed)
+        auto panel = [&](int c0, int buf, bool trans) {
+            double v = 0.0;
+#pragma unroll
+            for (int u = 0; u < kFacPanel / 8; ++u) {
+                const int k = kFacPanel / 8 * warp + u;
+                const double t = trans ? T[buf][lane][k] : T[buf][k][lane];
+                v += t * (c0 + k < n ? x[c0 + k] : 0.0);
+            }
+            part[warp][lane] = v;
             __syncthreads();
             if (warp == 0) {
-                // lane l: a = x[c0 + l] minus the panel's earlier columns;
-                // y_k = a_k / L_kk at the end
-                double a = lane < pw ? x[c0 + lane] : 0.0;
-                for (int k = 0; k < pw - 1; ++k) {
-                    const double ak = __shfl_sync(full, a, k);
-                    if (lane > k) a -= T[k * kFacPanel + lane] * ak;
-                }
-                if (lane < pw) x[c0 + lane] = a * dW[c0 + lane];
+#pragma unroll
+                for (int u = 1; u < 8; ++u) v += part[u][lane];
+                if (c0 + lane < n) x[c0 + lane] = v;
             }
             __syncthreads();
+        };
+        __syncthreads();  // the previous body is finished with x, T, hU
+        for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = w[3 * b0 + i];
+        stage(0, 0);
+        __syncthreads();
+        // ---- forward: y = L^-1 w; L[i][k] = Lt[k][i] = Pp[k m + i]
+        int buf = 0;
+        for (int c0 = 0; c0 < n; c0 += kFacPanel, buf ^= 1) {
+            const int pw = min(kFacPanel, n - c0);
+            panel(c0, buf, false);
+            if (c0 + kFacPanel < n) stage(c0 + kFacPanel, buf ^ 1);
             for (int i = c0 + pw + threadIdx.x; i < n; i += blockDim.x) {
                 double s0 = x[i], s1 = 0.0, s2 = 0.0, s3 = 0.0;
-                int k = 0;
-                for (; k + 4 <= pw; k += 4) {
+#pragma unroll
+                for (int k = 0; k < kFacPanel; k += 4) {  // rows below: the panel is full
                     s0 -= Pp[(size_t)(c0 + k) * m + i] * x[c0 + k];
                     s1 -= Pp[(size_t)(c0 + k + 1) * m + i] * x[c0 + k + 1];
                     s2 -= Pp[(size_t)(c0 + k + 2) * m + i] * x[c0 + k + 2];
                     s3 -= Pp[(size_t)(c0 + k + 3) * m + i] * x[c0 + k + 3];
                 }
-                for (; k < pw; ++k) s0 -= Pp[(size_t)(c0 + k) * m + i] * x[c0 + k];
                 x[i] = (s0 + s1) + (s2 + s3);
             }
             __syncthreads();
@@ -2305,32 +2226,32 @@ __global__ void __launch_bounds__(256) precond_apply_factored_kernel(
             __syncthreads();
         }
         // ---- backward: lambda = L^-T x; row k of L^T is Pp[k m + k ..]
-        for (int c1 = n; c1 > 0; c1 -= kFacPanel) {
-            const int c0 = c1 > kFacPanel ? c1 - kFacPanel : 0, pw = c1 - c0;
-            // the panel's rows lose their products with the solved rows
-            for (int k = warp; k < pw; k += nw) {
-                const double *lr = Pp + (size_t)(c0 + k) * m;
-                double sacc = 0.0;
-                for (int i = c1 + lane; i < n; i += 32) sacc += lr[i] * x[i];
+        const int last = (n - 1) / kFacPanel * kFacPanel;
+        buf = (last / kFacPanel) & 1;  // still holds the last panel's inverse
+        for (int c0 = last; c0 >= 0; c0 -= kFacPanel, buf ^= 1) {
+            const int c1 = c0 + kFacPanel;
+            if (c0 > 0) stage(c0 - kFacPanel, buf ^ 1);
+            if (c1 < n) {
+                // rows 4 warp .. 4 warp + 3 of the panel lose their products
+                // with the solved rows
+                const double *lr = Pp + (size_t)(c0 + 4 * warp) * m;
+                double s[4] = {0.0, 0.0, 0.0, 0.0};
+                for (int i = c1 + lane; i < n; i += 32) {
+                    const double xi = x[i];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) sacc += __shfl_xor_sync(full, sacc, o);
-                if (lane == 0) x[c0 + k] -= sacc;
-            }
-            // T[l][k] = Lt[c0 + l][c0 + k] / L_kk for l < k
-            for (int e = threadIdx.x; e < pw * pw; e += blockDim.x) {
-                const int l = e / pw, k = e % pw;
-                T[l * kFacPanel + k] = l < k ? Pp[(size_t)(c0 + l) * m + c0 + k] * dW[c0 + k] : 0.0;
-            }
-            __syncthreads();
-            if (warp == 0) {
-                double a = lane < pw ? x[c0 + lane] : 0.0;
-                for (int k = pw - 1; k > 0; --k) {
-                    const double ak = __shfl_sync(full, a, k);
-                    if (lane < k) a -= T[lane * kFacPanel + k] * ak;
+                    for (int u = 0; u < 4; ++u) s[u] += lr[(size_t)u * m + i] * xi;
                 }
-                if (lane < pw) x[c0 + lane] = a * dW[c0 + lane];
+                // halves exchanged: after two steps a lane holds one row's sum
+                const bool h16 = lane & 16, h8 = lane & 8;
+                const double a = (h16 ? s[2] : s[0]) + __shfl_xor_sync(full, h16 ? s[0] : s[2], 16);
+                const double b = (h16 ? s[3] : s[1]) + __shfl_xor_sync(full, h16 ? s[1] : s[3], 16);
+                double v = (h8 ? b : a) + __shfl_xor_sync(full, h8 ? a : b, 8);
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
+                if ((lane & 7) == 0) x[c0 + 4 * warp + (h16 ? 2 : 0) + (h8 ? 1 : 0)] -= v;
+                __syncthreads();
             }
-            __syncthreads();
+            panel(c0, buf, true);
         }
         for (int i = threadIdx.x; i < n; i += blockDim.x) lam[3 * b0 + i] = x[i];
     }

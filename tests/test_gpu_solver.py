@@ -461,13 +461,13 @@ def test_zero_right_hand_side(ctx):
         assert info["converged"] == 1 and np.all(host(F) == 0) and np.all(host(lam) == 0)
 
 
-@pytest.mark.parametrize("nbod", [3, 38, 39, 310])
-@pytest.mark.parametrize("counts", [(3, 4, 5), (10, 11, 8), (21, 22, 32), (42, 15, 6), (43, 42, 53)])
+@pytest.mark.parametrize("nbod", [3, 38, 39, 64, 310])
+@pytest.mark.parametrize("counts", [(3, 4, 5), (10, 11, 8), (21, 22, 32), (42, 15, 6), (43, 42, 53), (54, 64, 75)])
 def test_preconditioner_tile_edges(ctx, nbod, counts):
-    """Blocks of 9 to 159 rows, around the edges of 8-column panels and 32-row
-    tiles, factored by clusters (up to 38 bodies on 152 SMs) or by one CTA
-    each, their inverse by tiles up to 128 rows; bodies of
-    three sizes to a call, jittered lattices of blobs.  The bar is that of the
+    """Blocks of 9 to 225 rows, around the edges of 8-column panels and 32-row
+    tiles, factored by clusters (up to 38 bodies on 152 SMs, or above 160 rows)
+    or by one CTA each, their inverse by tiles up to 128 rows, in the factored
+    form from 64 bodies on above 160 rows; bodies of three sizes to a call, jittered lattices of blobs.  The bar is that of the
     other preconditioner tests."""
     rng = np.random.default_rng(nbod + counts[0])
     a = 0.2
