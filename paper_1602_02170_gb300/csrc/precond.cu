@@ -561,9 +561,10 @@ __device__ __forceinline__ int panel_cholesky8(double &v0, double &v1, int w, in
 // S2, 3 n_p <= kSmemMaxRows: one CTA per body, for more bodies than clusters
 // fit at once.  Right-looking Cholesky in shared memory with the six columns
 // B = K_p appended (so that B ends as G = L^-1 K_p), in panels of kPanel
-// columns: warp 0 factors the diagonal block, then the rows below it and the
-// panel's six B columns solve against it (one row a thread), then every thread
-// takes entries of the trailing triangle and of B, eight FMAs each.
+// columns: the rows below the diagonal block and the panel's six B columns solve
+// against it (one row a thread), then every thread takes entries of the trailing
+// triangle and of B, eight FMAs each, while warp 0 factors the next diagonal
+// block.
 //
 // Bound by the issue of FP64 instructions (one per ~76 cycles and sub-partition,
 // whatever the lanes do), so what counts is that every lane of each has work:
@@ -573,7 +574,7 @@ __device__ __forceinline__ int panel_cholesky8(double &v0, double &v1, int w, in
 // diagonal blocks run beside the other's updates.  Bodies of several sizes come
 // in pc_order_kernel's order: dealt out as they come, two long ones share an SM
 // beside two short ones on the next (306 us in this kernel for the 300, 221 in
-// order).  300 bodies of 126 and 45
+// order, 203 with the next diagonal block beside the update).  300 bodies of 126 and 45
 // rows in turn, setup and application: 1,260 -> 851 us against a square block, a
 // panel of all rows on one warp and rows dealt to warps (672 us in that kernel
 // and 34 in the conversion of its outputs, which is now done here).
@@ -607,23 +608,34 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
             for (int j = lane; j <= i; j += 32) row(i)[j] = Pp[(size_t)i * m + j];
         for (int e = threadIdx.x; e < 6 * n; e += blockDim.x)
             B[e] = k_entry(r + 3 * b0, qx, qy, qz, e / 6, e % 6);
+        // warp 0: the diagonal block at t0 less the product of the panel before
+        // (prev), factored in place
+        auto diagonal = [&](int t0, bool prev) {
+            const int w = min(kPanel, n - t0), l = lane & 7, g = lane >> 3;
+            double v0 = l < w && g <= l ? row(t0 + l)[t0 + g] : 0.0;
+            double v1 = l < w && g + 4 <= l ? row(t0 + l)[t0 + g + 4] : 0.0;
+            if (prev && l < w) {
+#pragma unroll
+                for (int k = 0; k < kPanel; ++k) {
+                    const double *pk = pT + (size_t)k * nmax + t0;
+                    if (g < w) v0 -= pk[l] * pk[g];
+                    if (g + 4 < w) v1 -= pk[l] * pk[g + 4];
+                }
+            }
+            const int f = panel_cholesky8(v0, v1, w, lane, ils + t0);
+            if (l < w) {
+                if (g <= l) row(t0 + l)[t0 + g] = v0;
+                if (g + 4 <= l) row(t0 + l)[t0 + g + 4] = v1;
+            }
+            if (lane == 0) pfail = f;
+        };
+        __syncthreads();
+        if (warp == 0) diagonal(0, false);
         int fail = 0;
         for (int c0 = 0; c0 < n; c0 += kPanel) {
             const int w = n - c0 < kPanel ? n - c0 : kPanel, t0 = c0 + w, nr = n - t0;
-            __syncthreads();  // the previous update is complete
-            if (warp == 0) {
-                const int l = lane & 7, g = lane >> 3;
-                double v0 = l < w && g <= l ? row(c0 + l)[c0 + g] : 0.0;
-                double v1 = l < w && g + 4 <= l ? row(c0 + l)[c0 + g + 4] : 0.0;
-                const int f = panel_cholesky8(v0, v1, w, lane, ils + c0);
-                if (l < w) {
-                    if (g <= l) row(c0 + l)[c0 + g] = v0;
-                    if (g + 4 <= l) row(c0 + l)[c0 + g + 4] = v1;
-                }
-                if (lane == 0) pfail = f;
-            }
-            __syncthreads();
-            if (pfail) {  // uniform
+            __syncthreads();  // the block is factored and the update before complete
+            if (pfail) {      // uniform
                 fail = 1;
                 break;
             }
@@ -653,8 +665,15 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
                 }
             }
             __syncthreads();
-            const int tri = nr * (nr + 1) / 2;
-            for (int e = threadIdx.x; e < tri + 6 * nr; e += blockDim.x) {
+            if (nr == 0) break;
+            // warp 0 factors the next diagonal block (the first w2 rows of the
+            // triangle) while the others take the rest
+            if (warp == 0) {
+                diagonal(t0, true);
+                continue;
+            }
+            const int tri = nr * (nr + 1) / 2, w2 = min(kPanel, nr);
+            for (int e = w2 * (w2 + 1) / 2 + threadIdx.x - 32; e < tri + 6 * nr; e += blockDim.x - 32) {
                 int i, j;
                 const double *other;  // the second factors, `step` apart
                 int step;
