@@ -452,7 +452,8 @@ typedef struct {
  * blobs; block sizes by the pairs of the batch), so problems of very
  * different sizes share the GPU; each problem keeps its own GMRES
  * state and stops consuming pair-kernel work once converged.  The arena
- * is sized exactly for the batch.
+ * is sized exactly for the batch; up to 256 MiB of it stay with the context
+ * for the next batch, until other workspace needs the room.
  *
  * problems: host array of n_problems descriptors (pointing to device data);
  * infos: host array of n_problems (may be NULL), filled per problem

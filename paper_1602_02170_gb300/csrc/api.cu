@@ -56,6 +56,7 @@ mb_status ensure(mb_context *ctx, DevBuf &buf, size_t bytes, const char *what)
     if (bytes == 0) bytes = 16;
     if (buf.bytes >= bytes) return MB_OK;
     const size_t grow = bytes + bytes / 8;  // headroom against repeated growth
+    if (ctx->held - buf.bytes + grow > ctx->budget) release_batch(ctx);
     if (ctx->held - buf.bytes + grow > ctx->budget)
         return set_err(ctx, MB_ENOMEM, "%s: %zu bytes would exceed the HBM budget (%zu held of %zu)",
                        what, grow, ctx->held - buf.bytes, ctx->budget);
@@ -67,6 +68,10 @@ mb_status ensure(mb_context *ctx, DevBuf &buf, size_t bytes, const char *what)
         buf.bytes = 0;
     }
     cudaError_t e = cudaMalloc(&buf.ptr, grow);
+    if (e != cudaSuccess && release_batch(ctx)) {
+        cudaGetLastError();
+        e = cudaMalloc(&buf.ptr, grow);
+    }
     if (e != cudaSuccess) {
         buf.ptr = nullptr;
         return cuda_err(ctx, e, what);
@@ -74,6 +79,17 @@ mb_status ensure(mb_context *ctx, DevBuf &buf, size_t bytes, const char *what)
     buf.bytes = grow;
     ctx->held += grow;
     return MB_OK;
+}
+
+bool release_batch(mb_context *ctx)
+{
+    bool any = false;
+    for (DevBuf &b : ctx->batch_keep)
+        if (b.ptr) {
+            release(ctx, b);
+            any = true;
+        }
+    return any;
 }
 
 void release(mb_context *ctx, DevBuf &buf)
@@ -221,6 +237,8 @@ mb_status mb_context_destroy(mb_context *ctx)
         if (g.exec) cudaGraphExecDestroy(g.exec);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     for (DevBuf *b : bufs) release(ctx, *b);
+    release_batch(ctx);
+    if (ctx->batch_host) cudaFreeHost(ctx->batch_host);
     if (ctx->host_small) cudaFreeHost(ctx->host_small);
     if (ctx->host_post) cudaFreeHost(ctx->host_post);
     if (ctx->post_seq_dev) cudaFree(ctx->post_seq_dev);

@@ -22,8 +22,8 @@
 //      tolerance, as in the single-problem solver);
 //   3. runs one Arnoldi step of right-preconditioned flexible GMRES for every
 //      active request, whatever its step index: one batched preconditioner
-//      apply, one batched pair-kernel launch over all requests' (target
-//      block, source chunk) items, segmented CGS2 reductions and Givens
+//      apply, one batched pair-kernel launch over all requests' pairs of
+//      blob blocks, segmented CGS2 reductions and Givens
 //      rotations per request.
 // Requests therefore join and leave between iterations while others are in
 // flight, and all of them share the same kernel launches.  mb_solve_batch is
@@ -795,7 +795,7 @@ struct Engine {
     int64_t n_cap = 0, b_cap = 0, pc_cap = 0, start_cap = 0;
     int s_cap = 0;
     int64_t ld = 0;  // vector length 3 n_cap + 6 b_cap
-    mb::DevBuf arena, partial, scratch, tick, work_buf;
+    mb::DevBuf arena, partial, scratch, tick, work_buf, dpart_buf;
     // device arrays carved from the arena
     double *rho, *r, *slip, *q, *theta, *F, *T, *P;
     float4 *hi, *lo;
@@ -806,6 +806,7 @@ struct Engine {
     SlotState st{};
     int *flag = nullptr;
     int *hstate = nullptr;  // pinned mirror of per-slot ints (kSlotInts arrays)
+    size_t hstate_bytes = 0;
     RangeAlloc blobs, bodies, pcs, starts;
     std::vector<int> free_slots;
     bool mixed = false;
@@ -848,6 +849,28 @@ struct Engine {
         release(ctx, work_buf);
         release(ctx, dpart_buf);
         if (hstate) cudaFreeHost(hstate);
+    }
+
+    // Takes over the buffers that the context keeps of the last batch (create
+    // grows them as needed), and leaves this engine's to the next one.
+    void take_kept(mb_context *c)
+    {
+        ctx = c;
+        DevBuf *own[4] = {&arena, &partial, &tick, &dpart_buf};
+        for (int k = 0; k < 4; ++k) std::swap(*own[k], c->batch_keep[k]);
+        hstate = (int *)c->batch_host;
+        hstate_bytes = c->batch_host_bytes;
+        c->batch_host = nullptr;
+        c->batch_host_bytes = 0;
+    }
+    void leave_kept()
+    {
+        if (arena.bytes + partial.bytes + tick.bytes + dpart_buf.bytes > kBatchKeepBytes) return;
+        DevBuf *own[4] = {&arena, &partial, &tick, &dpart_buf};
+        for (int k = 0; k < 4; ++k) std::swap(*own[k], ctx->batch_keep[k]);
+        ctx->batch_host = hstate;
+        ctx->batch_host_bytes = hstate_bytes;
+        hstate = nullptr;
     }
 
     mb_status create(mb_context *c, const mb_params *p, int64_t max_blobs, int64_t max_bodies,
@@ -924,7 +947,14 @@ struct Engine {
         MB_CUDA_TRY(ctx, cudaMemset(body_slot, 0xff, sizeof(int) * b_cap));
         MB_CUDA_TRY(ctx, cudaMemset(blob_body, 0xff, sizeof(int64_t) * n_cap));
         MB_CUDA_TRY(ctx, cudaMemset(ints, 0, sizeof(int) * kSlotInts * s_cap));
-        MB_CUDA_TRY(ctx, cudaMallocHost(&hstate, sizeof(int) * kSlotInts * s_cap + 64));
+        const size_t host_bytes = sizeof(int) * kSlotInts * s_cap + 64;
+        if (hstate_bytes < host_bytes) {
+            if (hstate) cudaFreeHost(hstate);
+            hstate = nullptr;
+            hstate_bytes = 0;
+            MB_CUDA_TRY(ctx, cudaMallocHost(&hstate, host_bytes));
+            hstate_bytes = host_bytes;
+        }
         blobs.init(n_cap);
         bodies.init(b_cap);
         pcs.init(pc_cap);
@@ -1171,7 +1201,6 @@ struct Engine {
         MB_CUDA_TRY(ctx, cudaGetLastError());
         return MB_OK;
     }
-    mb::DevBuf dpart_buf;
     mb_status ensure_dpart(int64_t n)
     {
         MB_TRY(ensure(ctx, dpart_buf, sizeof(double) * std::max<int64_t>(1, n), "server dot partials"));
@@ -1661,6 +1690,7 @@ mb_status solve_batch(mb_context *ctx, int np, const mb_problem *probs, const mb
     }
     Engine *E = new (std::nothrow) Engine();
     if (!E) return MB_ENOMEM;
+    E->take_kept(ctx);
     mb_status st = E->create(ctx, prm, nt, bt, std::max<int64_t>(1, pct), np);
     std::vector<int64_t> tickets(np, 0);
     for (int p = 0; p < np && st == MB_OK; ++p) {
@@ -1693,6 +1723,7 @@ mb_status solve_batch(mb_context *ctx, int np, const mb_problem *probs, const mb
             result = set_err(ctx, MB_ENOTCONVERGED, "%d of %d problems did not converge within maxit",
                              n_bad, np);
     }
+    if (st == MB_OK) E->leave_kept();  // the last tick has ended
     delete E;
     return result;
 }
