@@ -363,8 +363,7 @@ __global__ void pc_to_f32_kernel(const double *__restrict__ a, int64_t count, fl
 
 // TP: the blocks' type, FP64, or FP32 (an FP32 copy of the explicit blocks
 // for the FP32 inner iterations of mixed precision; products and sums in
-// FP32 too).  SYMV (FP64, 32 rows or more to a CTA): by symv_rows, else a warp
-// per row.
+// FP32 too).  SYMV (FP64): by symv_rows, else a warp per row.
 template <typename TP, bool SYMV>
 __global__ void __launch_bounds__(256) precond_apply_kernel(
     int64_t nb, const int64_t *__restrict__ start, const int64_t *__restrict__ poff,
@@ -1905,8 +1904,9 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
     // explicit inverse, whose application spreads over many CTAs.  162-blob
     // shells, setup / application / mixed solve (ms), explicit and factored: 32
     // bodies 5.9 / 0.05 / 9.4 and 2.0 / 0.15 / 8.2, 80 bodies 14.6 / 0.12 / 27.7
-    // and 5.7 / 0.15 / 21.7, 151 bodies 25.8 / 0.16 / 65.8 and 9.3 / 0.23 / 53.9; the
-    // line lies where an application costs half as much again.  The resistance
+    // and 5.7 / 0.15 / 21.7, 151 bodies 25.8 / 0.16 / 65.8 and 9.3 / 0.23 / 53.9 (120 of
+    // 200 blobs, setup / application: 37.0 / 0.13 and 13.1 / 0.32); the line lies
+    // where an application of 162-blob bodies costs half as much again.  The resistance
     // problem takes three times the iterations, so there the inverse pays up to
     // one body an SM.
     const bool factored = !lsmem && nmax <= kSplitMaxRowsSmem &&
@@ -2309,10 +2309,12 @@ static void precond_apply_impl(mb_context *ctx, const double *w, const double *g
             (const int64_t *)ctx->pinv_off.ptr, (const float *)ctx->pinv32.ptr, w, g, lam, UO,
             chunks, rows, body_rows);
     else {
-        // 32 rows or more to a CTA fill the lanes of symv_rows; with fewer a
-        // warp per row keeps all eight warps at work
-        const auto kern = rows >= 32 ? precond_apply_kernel<double, true>
-                                     : precond_apply_kernel<double, false>;
+        // symv_rows for whole or half blocks (one body an SM or more).  Shorter
+        // pieces of rows walked column by column read DRAM in short strips: 60
+        // bodies of 154 blobs 77 us against 49 by a warp per row, 40 of 300 blobs
+        // 227 against 105.
+        const auto kern = chunks <= 2 ? precond_apply_kernel<double, true>
+                                      : precond_apply_kernel<double, false>;
         kern<<<grid, 256, sizeof(double) * m, s>>>(
             ctx->pc_nb, (const int64_t *)ctx->blob_start_copy.ptr,
             (const int64_t *)ctx->pinv_off.ptr, (const double *)ctx->pinv.ptr, w, g, lam, UO,
