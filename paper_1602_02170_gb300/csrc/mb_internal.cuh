@@ -319,7 +319,7 @@ __device__ __forceinline__ void symv_rows(const double *__restrict__ P, int m,
     constexpr int kT = kSymvRows / 32;
     for (int b = r0; b < r1; b += kSymvRows) {
         double acc[kT] = {};
-        const int nt = min(kT, (r1 - b + 31) >> 5);  // 32-row pieces of this round
+        const int nt = min(kT, (r1 - b + 31) >> 5);  // 32-row pieces of this pass
         for (int c = warp; c < cols; c += 8) {
             const double *pc = P + (size_t)c * m + b + lane;
             const double x = xs[c];

@@ -1504,7 +1504,7 @@ mb_status render_flow(mb_context *ctx, const double *x, int64_t nt, const double
 // kernel below kSymMinN, the symmetric kernel above, in the spatial
 // order from kSortMinN on.  A scalar kernel for every ordered pair ran at every
 // size: 5,003 blobs 121 -> 64 us, 65,536 13.1 -> 5.2 ms with the wall, 20,011
-// 705 -> 339 us and 65,536 6.0 -> 2.9 ms without (all against the first form).
+// 705 -> 323 us and 65,536 6.0 -> 2.8 ms without.
 namespace {
 
 constexpr int64_t kNoallocMaxBlobs = MB_NOALLOC_MAX_BLOBS;

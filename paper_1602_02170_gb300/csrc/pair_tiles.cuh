@@ -186,6 +186,75 @@ __device__ __forceinline__ void f64_item(double *__restrict__ sm, const double *
     }
 }
 
+// A source of the symmetric item, every operand in both halves of a float2.
+struct SrcX2 {
+    float2 nx, ny, z, fx, fy, fz;  // -x, -y, z (hi parts), force
+    float2 nxl, nyl, nzl;          // - lo parts (kNear only)
+    float2 zz;                     // -2 z^2 (wall only)
+};
+
+// With the wall the sources are staged duplicated, as in x2_item: the FMA pipe
+// bounds the item and every register move would add to the issue.  Without it
+// an item does less than half the arithmetic, and its rotated shared-memory
+// reads (four wavefronts per float4, all warps of the SM in turn) and shuffles
+// bound it instead: three float4 a source,
+//   (-x_hi, -y_hi, z_hi, f_x)  (f_y, f_z, -, -)  (-x_lo, -y_lo, -z_lo, -),
+// of which a far item reads one and a half, and moves to duplicate them.
+// Without the wall: 20,011 blobs 338 -> 323 us, 65,536 2.93 -> 2.77 ms.
+template <bool WALL>
+__device__ __forceinline__ void stage_sym(float4 *sP, int slot, float4 h, float4 l, float fx, float fy,
+                                          float fz)
+{
+    if (WALL) {
+        stage_x2(sP + kX2SmemFloat4PerSource * slot, h, l, fx, fy, fz);
+        return;
+    }
+    float4 *d = sP + 3 * slot;
+    d[0] = make_float4(-h.x, -h.y, h.z, fx);
+    d[1] = make_float4(fy, fz, 0.f, 0.f);
+    d[2] = make_float4(-l.x, -l.y, -l.z, 0.f);
+}
+
+template <bool WALL, bool LO>
+__device__ __forceinline__ SrcX2 load_sym(const float4 *sP, int slot)
+{
+    SrcX2 q;
+    if (WALL) {
+        const float4 *P = sP + kX2SmemFloat4PerSource * slot;
+        const float4 P0 = P[0], P1 = P[1], P3 = P[3], P4 = P[4];
+        q.nx = make_float2(P0.x, P0.y);
+        q.ny = make_float2(P0.z, P0.w);
+        q.z = make_float2(P1.x, P1.y);
+        q.zz = make_float2(P1.z, P1.w);
+        q.fx = make_float2(P3.z, P3.w);
+        q.fy = make_float2(P4.x, P4.y);
+        q.fz = make_float2(P4.z, P4.w);
+        if (LO) {
+            const float4 P2 = P[2];
+            q.nxl = make_float2(P2.x, P2.y);
+            q.nyl = make_float2(P2.z, P2.w);
+            q.nzl = make_float2(P3.x, P3.y);
+        }
+    } else {
+        const float4 *P = sP + 3 * slot;
+        const float4 A = P[0];
+        const float2 B = *(const float2 *)(P + 1);
+        q.nx = splat2(A.x);
+        q.ny = splat2(A.y);
+        q.z = splat2(A.z);
+        q.fx = splat2(A.w);
+        q.fy = splat2(B.x);
+        q.fz = splat2(B.y);
+        if (LO) {
+            const float4 D = P[2];
+            q.nxl = splat2(D.x);
+            q.nyl = splat2(D.y);
+            q.nzl = splat2(D.z);
+        }
+    }
+    return q;
+}
+
 // Symmetric packed item over block pair (I, J), I <= J, blocks of 2*NT blobs
 // (two targets per thread, as in x2_item with NP = 1).  Each unordered pair
 // is evaluated once.  Forward contributions accumulate in the thread's
@@ -245,25 +314,20 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
             const float fx = valid ? (float)f[3 * jc] : 0.f;
             const float fy = valid ? (float)f[3 * jc + 1] : 0.f;
             const float fz = valid ? (float)f[3 * jc + 2] : 0.f;
-            stage_x2(sP + kX2SmemFloat4PerSource * threadIdx.x, h, l, fx, fy, fz);
+            stage_sym<WALL>(sP, threadIdx.x, h, l, fx, fy, fz);
         }
         __syncthreads();
         float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
         if (diag) {
 #pragma unroll 2
             for (int s = 0; s < NT; ++s) {
-                const float4 *P = sP + kX2SmemFloat4PerSource * s;
-                const float4 P0 = P[0], P1 = P[1], P2 = P[2], P3 = P[3], P4 = P[4];
-                const float2 zj = make_float2(P1.x, P1.y);
-                const float2 dx = add2(add2(xh, make_float2(P0.x, P0.y)), add2(xl, make_float2(P2.x, P2.y)));
-                const float2 dy = add2(add2(yh, make_float2(P0.z, P0.w)), add2(yl, make_float2(P2.z, P2.w)));
-                const float2 dz = add2(fma2(zj, k.m1, zh), add2(zl, make_float2(P3.x, P3.y)));
+                const SrcX2 q = load_sym<WALL, true>(sP, s);
+                const float2 dx = add2(add2(xh, q.nx), add2(xl, q.nxl));
+                const float2 dy = add2(add2(yh, q.ny), add2(yl, q.nyl));
+                const float2 dz = add2(fma2(q.z, k.m1, zh), add2(zl, q.nzl));
                 const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
-                const Mob<float2> m =
-                    mob_coefs2<WALL, kNear>(dz, dxy2, zh, zj, make_float2(P1.z, P1.w), k);
-                mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, make_float2(P3.z, P3.w),
-                                              make_float2(P4.x, P4.y), make_float2(P4.z, P4.w),
-                                              ax, ay, az);
+                const Mob<float2> m = mob_coefs2<WALL, kNear>(dz, dxy2, zh, q.z, q.zz, k);
+                mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
             }
         } else {
             for (int g = 0; g < NT / 32; ++g) {
@@ -271,25 +335,19 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
 #pragma unroll 2
                 for (int t = 0; t < 32; ++t) {
                     const int s = g * 32 + ((lane + t) & 31);
-                    const float4 *P = sP + kX2SmemFloat4PerSource * s;
-                    const float4 P0 = P[0], P1 = P[1], P3 = P[3], P4 = P[4];
-                    const float2 zj = make_float2(P1.x, P1.y);
-                    float2 dx = add2(xh, make_float2(P0.x, P0.y));
-                    float2 dy = add2(yh, make_float2(P0.z, P0.w));
-                    float2 dz = fma2(zj, k.m1, zh);
+                    const SrcX2 q = load_sym<WALL, LEVEL == kNear>(sP, s);
+                    float2 dx = add2(xh, q.nx);
+                    float2 dy = add2(yh, q.ny);
+                    float2 dz = fma2(q.z, k.m1, zh);
                     if (LEVEL == kNear) {
-                        const float4 P2 = P[2];
-                        dx = add2(dx, add2(xl, make_float2(P2.x, P2.y)));
-                        dy = add2(dy, add2(yl, make_float2(P2.z, P2.w)));
-                        dz = add2(dz, add2(zl, make_float2(P3.x, P3.y)));
+                        dx = add2(dx, add2(xl, q.nxl));
+                        dy = add2(dy, add2(yl, q.nyl));
+                        dz = add2(dz, add2(zl, q.nzl));
                     }
                     const float2 dxy2 = fma2(dy, dy, LEVEL == kNear ? fma2(dx, dx, k.tiny)
                                                                     : mul2(dx, dx));
-                    const Mob<float2> m =
-                        mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, zj, make_float2(P1.z, P1.w), k);
-                    mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, make_float2(P3.z, P3.w),
-                                                  make_float2(P4.x, P4.y),
-                                                  make_float2(P4.z, P4.w), ax, ay, az);
+                    const Mob<float2> m = mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, q.z, q.zz, k);
+                    mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
                     mob_apply2<WALL, true, ONCE>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
                     // hand the accumulator to lane - 1, which meets this source next step
                     const int from = (lane + 1) & 31;
