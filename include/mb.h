@@ -449,7 +449,8 @@ typedef struct {
  * diagonal preconditioner of Section 2.2.2 run over all bodies of all
  * problems in one launch each; the pair kernel runs as one launch
  * over all problems' pairs of blob blocks (each unordered pair once for both
- * blobs; block sizes by the pairs of the batch), so problems of very
+ * blobs, added with FP64 atomics, so results may differ between calls in
+ * the last bits; block sizes by the pairs of the batch), so problems of very
  * different sizes share the GPU; each problem keeps its own GMRES
  * state and stops consuming pair-kernel work once converged.  The arena
  * is sized exactly for the batch; up to 256 MiB of it stay with the context
