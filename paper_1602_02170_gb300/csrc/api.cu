@@ -81,6 +81,14 @@ mb_status ensure(mb_context *ctx, DevBuf &buf, size_t bytes, const char *what)
     return MB_OK;
 }
 
+size_t ensure_room(const mb_context *ctx, const DevBuf &buf)
+{
+    size_t held = ctx->held - buf.bytes;
+    for (const DevBuf &b : ctx->batch_keep) held -= b.bytes;
+    const size_t room = ctx->budget > held ? ctx->budget - held : 0;
+    return std::max(buf.bytes, room / 9 * 8);  // ensure() adds an eighth
+}
+
 bool release_batch(mb_context *ctx)
 {
     bool any = false;

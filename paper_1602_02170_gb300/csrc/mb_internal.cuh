@@ -153,6 +153,8 @@ mb_status cuda_err(mb_context *ctx, cudaError_t e, const char *what);
 mb_status wait_stream(mb_context *ctx, cudaStream_t s, const char *what);
 // Make `buf` hold at least `bytes`; respects the context budget.
 mb_status ensure(mb_context *ctx, DevBuf &buf, size_t bytes, const char *what);
+// Most bytes that the budget lets ensure() give to `buf`.
+size_t ensure_room(const mb_context *ctx, const DevBuf &buf);
 void release(mb_context *ctx, DevBuf &buf);
 constexpr size_t kBatchKeepBytes = (size_t)256 << 20;
 // Frees what the context keeps of the last batch; false if there was nothing.

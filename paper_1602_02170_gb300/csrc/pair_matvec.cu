@@ -1391,8 +1391,7 @@ Plan eval_plan(const mb_context *ctx, int64_t nt, int64_t ns, int block, int64_t
 {
     Plan p;
     p.n_tblocks = (int)ceil_div(nt, block);
-    const size_t room = ctx->budget > ctx->held ? ctx->budget - ctx->held : 0;
-    const int64_t fits = (int64_t)(std::max(room, ctx->partial.bytes) / (sizeof(double) * 3)) / nt;
+    const int64_t fits = (int64_t)(ensure_room(ctx, ctx->partial) / (sizeof(double) * 3)) / nt;
     const int64_t need = std::min<int64_t>(4 * ctx->sm_count / p.n_tblocks, ceil_div(ns, shortest));
     const int64_t good = std::min(ceil_div(want, p.n_tblocks), ceil_div(ns, 4 * shortest));
     const int64_t s = std::max<int64_t>(1, std::min(std::max(need, good), fits));

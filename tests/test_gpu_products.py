@@ -158,6 +158,25 @@ def test_eval_within_a_small_budget():
     assert rel_l2(got, want) <= TOL["fp32"]
 
 
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("chunks", [0.9, 1.0, 1.2, 2.0, 3.5, 6.8, 9.0, 10.1, 16.0, 40.0])
+def test_eval_at_every_budget(ctx, prec, chunks):
+    """Whatever the budget beyond the packed positions, the evaluation takes the
+    chunks whose partial sums it holds, headroom of the allocation included."""
+    import paper_1602_02170_gb300 as mb
+
+    nt, ns = 2000, 3000
+    r, f = _cloud(1, ns)
+    x, _ = _cloud(2, nt)
+    packed = 2 * 18 * (ns + nt) if prec == "fp32" else 0  # 16 bytes and an eighth
+    want = host(ctx.mobility_eval(dev(x), dev(r), dev(f), 0.5, 1.0, True, prec))
+    budget = packed + int(24 * nt * chunks)
+    with mb.Context(0, max(1, budget)) as c:
+        got = host(c.mobility_eval(dev(x), dev(r), dev(f), 0.5, 1.0, True, prec))
+        assert c.workspace_bytes() <= budget
+    assert rel_l2(got, want) <= TOL[prec]
+
+
 @pytest.mark.parametrize("wall", [True, False])
 @pytest.mark.parametrize("n", [1, 33, 599, 600, 3001, 16383, 16384, 20011])
 def test_noalloc_every_size_and_in_place(ctx, n, wall):
