@@ -166,6 +166,8 @@ mb_status matvec_device(mb_context *ctx, const double *r, const double *f, int64
                         double eta, int wall, mb_precision prec, double *u, cudaStream_t s);
 // FP32 variant chosen for N blobs, and the size class of a matvec (pair_matvec.cu).
 int f32_variant(int64_t n);
+// Arrays that the sums of an FP64 product of n blobs are spread over (pair_matvec.cu).
+int f64_sums(int64_t n);
 int size_class(int64_t n, int wall);
 // Pack positions once (FP32 path); the matvec then only reads f.  order: also
 // sort them spatially for the symmetric FP32 kernel (N >= 16,384).

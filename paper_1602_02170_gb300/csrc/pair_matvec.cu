@@ -372,10 +372,12 @@ void launch_small(const double *r, const double *f, int64_t n, double a, double 
 // pair once in one-warp CTAs; 16,384 blobs: 28.3 -> 21.3 ms against 256-thread
 // symmetric items of the ungrouped formula (1.36 TFLOP/s in the method's 108
 // flop per ordered pair, of 1.06 measured: each pair is evaluated once).
+// u: S arrays of 3 n (f64_sums), block J's items adding to the targets in array
+// J mod S and block I's to the sources in array I mod S.
 template <bool WALL, int C>
 __global__ void __launch_bounds__(32) pair_f64sym_kernel(
     const double *__restrict__ r, const double *__restrict__ f, int64_t n, int64_t n_items,
-    MobConsts<double> k, double *__restrict__ u, double scale)
+    MobConsts<double> k, double *u, int S, double scale)
 {
     __shared__ double sm[6 * C];
     constexpr int kParts = 32 / C;
@@ -384,7 +386,9 @@ __global__ void __launch_bounds__(32) pair_f64sym_kernel(
         int64_t I, J;
         triangle_pair(t, I, J);
         const int64_t j0 = J * 32 + (item - t * kParts) * C;
-        if (j0 < n) f64sym_item<WALL, C>(sm, r, f, n, I, j0, I == J, k, u, scale);
+        if (j0 < n)
+            f64sym_item<WALL, C>(sm, r, f, n, I, j0, I == J, k, u + 3 * n * (J % S),
+                                 u + 3 * n * (I % S), scale);
         __syncwarp();  // the item is done with sm
     }
 }
@@ -1241,25 +1245,49 @@ mb_status matvec_pack_positions(mb_context *ctx, const double *r, int64_t n, cud
 // reductions and atomics (C = 4: 12% of the FP64 instructions).
 constexpr int kF64ItemsPerWarp = 16;
 
+// Arrays that the sums of an FP64 product are spread over.  Every addition to
+// an array is rounded at the size that the array's sum has by then, and a blob
+// takes n / 32 + n / C of them, so the error grows with the square root of
+// n / S.  Relative L2 error of the product against 113-bit values, S = 1, 8 and
+// 16, and of chunk sums in a fixed order or blocks of 256 blobs (with the wall, in
+// 1e-16): 336 blobs 3.3, 2.8, 2.7, 3.3; 1,000 6.2, 3.7, 3.5, 5.4; 8,191 6.7,
+// 4.6, 4.4, 8.4; 16,384 8.5, 4.9, 4.7, 6.2; 65,536 16.7, 7.3, 5.9, 8.4.  Adding
+// the arrays is a launch more: 336 blobs 21.6 -> 25.8 us, 2,730 614 -> 620.
+constexpr int64_t kF64SumsMinN = 400;
+
+int f64_sums(int64_t n) { return n < kF64SumsMinN ? 1 : n < 32768 ? 8 : 16; }
+
+// One where the arrays don't fit the budget, or would have to be allocated
+// within a stream capture.
+int f64_sums_held(mb_context *ctx, int64_t n, cudaStream_t s)
+{
+    const int S = f64_sums(n);
+    const size_t bytes = sizeof(double) * 3 * (size_t)n * S;
+    if (ctx->partial.bytes >= bytes) return S;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    return st == cudaStreamCaptureStatusNone && ensure_room(ctx, ctx->partial) >= bytes ? S : 1;
+}
+
 template <bool WALL, int C>
 void launch_f64sym_c(const double *r, const double *f, int64_t n, int64_t pairs, double a,
-                     double *u, double scale, cudaStream_t s)
+                     double *u, int S, double scale, cudaStream_t s)
 {
     const int64_t items = pairs * (32 / C);
     pair_f64sym_kernel<WALL, C><<<(unsigned)std::min<int64_t>(items, 1 << 30), 32, 0, s>>>(
-        r, f, n, items, MobConsts<double>::make(a), u, scale);
+        r, f, n, items, MobConsts<double>::make(a), u, S, scale);
 }
 
 template <bool WALL>
 void launch_f64sym(mb_context *ctx, const double *r, const double *f, int64_t n, double a,
-                   double *u, double scale, cudaStream_t s)
+                   double *u, int S, double scale, cudaStream_t s)
 {
     const int64_t nb = ceil_div(n, 32), pairs = nb * (nb + 1) / 2;
     const int64_t want = (int64_t)kF64ItemsPerWarp * 4 * ctx->sm_count;
-    if (pairs >= want) launch_f64sym_c<WALL, 32>(r, f, n, pairs, a, u, scale, s);
-    else if (2 * pairs >= want) launch_f64sym_c<WALL, 16>(r, f, n, pairs, a, u, scale, s);
-    else if (4 * pairs >= want) launch_f64sym_c<WALL, 8>(r, f, n, pairs, a, u, scale, s);
-    else launch_f64sym_c<WALL, 4>(r, f, n, pairs, a, u, scale, s);
+    if (pairs >= want) launch_f64sym_c<WALL, 32>(r, f, n, pairs, a, u, S, scale, s);
+    else if (2 * pairs >= want) launch_f64sym_c<WALL, 16>(r, f, n, pairs, a, u, S, scale, s);
+    else if (4 * pairs >= want) launch_f64sym_c<WALL, 8>(r, f, n, pairs, a, u, S, scale, s);
+    else launch_f64sym_c<WALL, 4>(r, f, n, pairs, a, u, S, scale, s);
 }
 
 template <bool WALL, int NT>
@@ -1324,21 +1352,22 @@ mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64
         MB_CUDA_TRY(ctx, cudaGetLastError());
         return MB_OK;
     }
-    // FP64: u (or, deferred, the one partial sum the caller scales) zeroed,
-    // then one launch over the block-pair triangle
-    double *uk = u, sk = scale;
-    if (defer) {
-        MB_TRY(ensure(ctx, ctx->partial, sizeof(double) * 3 * (size_t)n, "matvec partials"));
-        uk = (double *)ctx->partial.ptr;
-        *defer = MatvecPartials{uk, 1, sk};
-        sk = 1.0;
-    }
-    MB_CUDA_TRY(ctx, cudaMemsetAsync(uk, 0, sizeof(double) * 3 * (size_t)n, s));
+    // FP64: u (or, of several sums or deferred, the sums that a launch or the
+    // caller adds and scales) zeroed, then one launch over the block-pair triangle
+    const int S = f64_sums_held(ctx, n, s);
+    const bool sums = defer || S > 1;
+    const size_t bytes = sizeof(double) * 3 * (size_t)n * S;
+    if (sums) MB_TRY(ensure(ctx, ctx->partial, bytes, "matvec partials"));
+    double *uk = sums ? (double *)ctx->partial.ptr : u;
+    const double sk = sums ? 1.0 : scale;
+    MB_CUDA_TRY(ctx, cudaMemsetAsync(uk, 0, bytes, s));
     auto *ev = profile_begin(ctx, s);
-    if (wall) launch_f64sym<true>(ctx, r, f, n, a, uk, sk, s);
-    else launch_f64sym<false>(ctx, r, f, n, a, uk, sk, s);
+    if (wall) launch_f64sym<true>(ctx, r, f, n, a, uk, S, sk, s);
+    else launch_f64sym<false>(ctx, r, f, n, a, uk, S, sk, s);
     profile_end(ev, s);
     count_launch();
+    if (defer) *defer = MatvecPartials{uk, S, scale};
+    else if (sums) launch_reduce_partials(uk, n, S, scale, u, s);
     MB_CUDA_TRY(ctx, cudaGetLastError());
     return MB_OK;
 }

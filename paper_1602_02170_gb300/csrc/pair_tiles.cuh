@@ -523,14 +523,15 @@ __device__ __forceinline__ void dfsym_item(float4 *__restrict__ sD, double *__re
 // evaluated once for both blobs: at step t lane l meets source (l + t) mod C,
 // and the reverse sums move to lane l - 1 within the groups of C lanes after
 // each step, so that after C steps lane l holds source (l mod C)'s sum over
-// its group's targets; the groups are then added.  All sums reach u with FP64
-// atomics, so u must be zeroed beforehand.  A diagonal item (I == J) runs
-// forward only over all ordered pairs.
+// its group's targets; the groups are then added.  The targets' sums are added
+// to u and the sources' to v with FP64 atomics; both must be zeroed beforehand,
+// and may be the same array.  A diagonal item (I == J) runs forward only over
+// all ordered pairs.
 template <bool WALL, int C>
 __device__ __forceinline__ void f64sym_item(double *__restrict__ sm, const double *__restrict__ r,
                                             const double *__restrict__ f, int64_t n, int64_t I,
                                             int64_t j0, bool diag, const MobConsts<double> &k,
-                                            double *__restrict__ u, double scale)
+                                            double *u, double *v, double scale)
 {
     const int lane = threadIdx.x & 31;
     const int64_t i = I * 32 + lane, ic = i < n ? i : n - 1;
@@ -577,9 +578,9 @@ __device__ __forceinline__ void f64sym_item(double *__restrict__ sm, const doubl
         }
         const int64_t j = j0 + lane;
         if (lane < C && j < n) {
-            atomicAdd(u + 3 * j, scale * vx);
-            atomicAdd(u + 3 * j + 1, scale * vy);
-            atomicAdd(u + 3 * j + 2, scale * vz);
+            atomicAdd(v + 3 * j, scale * vx);
+            atomicAdd(v + 3 * j + 1, scale * vy);
+            atomicAdd(v + 3 * j + 2, scale * vz);
         }
     }
     if (i < n) {

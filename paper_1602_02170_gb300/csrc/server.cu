@@ -297,7 +297,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) eng_sym_kernel(
     }
 }
 
-// y = 0 on the listed rows (RSeg work index -> that entry's y)
+// y = 0 on the listed rows (RSeg work index -> that entry's y), or with S > 1
+// its S sums
 __global__ void eng_zero_kernel(const Work *__restrict__ W, const RSeg *__restrict__ rs, int nrs,
                                 const int *__restrict__ mask)
 {
@@ -305,7 +306,11 @@ __global__ void eng_zero_kernel(const Work *__restrict__ W, const RSeg *__restri
         const RSeg R = rs[it];
         const Work P = W[R.work];
         if (!mask[P.slot]) continue;
-        for (int64_t e = R.start + threadIdx.x; e < R.end; e += blockDim.x) P.y[e] = 0.0;
+        for (int64_t e = R.start + threadIdx.x; e < R.end; e += blockDim.x) {
+            if (P.S == 1) P.y[e] = 0.0;
+            else
+                for (int s = 0; s < P.S; ++s) P.part[3 * s * P.n + e] = 0.0;
+        }
     }
 }
 
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(NT, 384 / NT) eng_df_kernel(
 }
 
 // The same in FP64: one-warp items of 32 targets and C sources (as in
-// pair_f64sym_kernel).
+// pair_f64sym_kernel), added to y or, with S > 1, spread over the S sums.
 template <bool WALL, int C>
 __global__ void __launch_bounds__(32) eng_f64sym_kernel(
     const Work *__restrict__ W, const int64_t *__restrict__ item_off, int nw, int64_t n_items,
@@ -344,7 +349,10 @@ __global__ void __launch_bounds__(32) eng_f64sym_kernel(
         int64_t I, J;
         triangle_pair(t, I, J);
         const int64_t j0 = J * 32 + (local - t * kParts) * C;
-        if (j0 < P.n) f64sym_item<WALL, C>(sm, P.r, P.f, P.n, I, j0, I == J, k, P.y, scale);
+        double *u = P.S == 1 ? P.y : P.part + 3 * P.n * (J % P.S);
+        double *v = P.S == 1 ? P.y : P.part + 3 * P.n * (I % P.S);
+        if (j0 < P.n)
+            f64sym_item<WALL, C>(sm, P.r, P.f, P.n, I, j0, I == J, k, u, v, P.S == 1 ? scale : 1.0);
         __syncwarp();  // the item is done with sm
     }
 }
@@ -1055,11 +1063,14 @@ struct Engine {
         const bool x2 = prec == MB_FP32_KAHAN && np_variant != 3;  // a pinned packed variant
         double pairs = 0;
         int64_t pairs32 = 0;  // pairs of 32-blob blocks
+        size_t sums = 0;      // entries of the FP64 items' sums
         for (int sl : list) {
             const int64_t n = running[sl]->prob.n_blobs, nb = ceil_div(n, 32);
             pairs += (double)n * n;
             pairs32 += nb * (nb + 1) / 2;
+            if (f64_sums(n) > 1) sums += 3 * (size_t)n * f64_sums(n);
         }
+        const bool spread = prec == MB_FP64 && sizeof(double) * sums <= ensure_room(ctx, partial);
         // Symmetric items of the whole list: blocks small enough that every SM
         // has work, by the bounds measured for single products (pair_matvec.cu;
         // FP32: sym_nt).
@@ -1093,6 +1104,11 @@ struct Engine {
                 wk.S = 1;
                 wk.chunk = wk.n;
                 if (prec == MB_FP64) {
+                    if (spread && f64_sums(wk.n) > 1) {
+                        wk.S = f64_sums(wk.n);
+                        wk.part = (double *)0 + part;  // offset, fixed up below
+                        part += 3 * wk.n * wk.S;
+                    }
                     const int64_t nb = ceil_div(wk.n, 32);
                     items += nb * (nb + 1) / 2 * (32 / fc);
                 } else if (prec == MB_DF64) {
@@ -1168,7 +1184,7 @@ struct Engine {
         }
         profile_end(ev, s);
         count_launch();
-        if (!rs.empty() && x2) {
+        if (!rs.empty() && (x2 || (spread && sums > 0))) {
             eng_reduce_kernel<<<grid_for((int64_t)rs.size(), 1), 256, 0, s>>>(dW, dR, (int)rs.size(),
                                                                            mask, scale);
             count_launch();

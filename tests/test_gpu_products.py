@@ -38,6 +38,32 @@ def test_fp64_length_scale_outside_fp32_range(ctx):
     assert rel_l2(got * 1e-25, ref) <= TOL["fp64"]
 
 
+def test_fp64_sums_of_many_blobs(ctx):
+    """65,536 blobs without the wall, a few targets in extended precision.  A
+    target takes 4,096 additions of items' sums, spread over 16 arrays: 256
+    roundings of 0.29 ulp (rms) each at half of the array's final size, 2.5e-16
+    of the whole, beside about 4e-16 of the pairs' and the items' own: 9e-16
+    (in one array the additions alone are four times as much)."""
+    n, a = 65536, 0.5
+    r, f = I.blob_cloud(9, n, a, 400.0, a, 3 * a)
+    got = host(ctx.mobility_matvec(dev(r), dev(f), a, 1.0, False, "fp64"))
+    X = np.longdouble
+    R, F, a = r.astype(X), f.astype(X), X(a)
+    at = np.random.default_rng(9).permutation(n)[:24]
+    ref = np.empty((len(at), 3), X)
+    for k, i in enumerate(at):
+        d = R[i] - R
+        r2 = np.maximum((d * d).sum(1), X(1e-30))
+        q = np.sqrt(r2)
+        near = r2 < 4 * a * a
+        C = np.where(near, 1 - 9 * q / (32 * a), 3 * a / (4 * q) + a ** 3 / (2 * q * r2))
+        D = np.where(near, 3 / (32 * a * q), (3 * a / 4 - 3 * a ** 3 / (2 * r2)) / (q * r2))
+        ref[k] = (C[:, None] * F + (D * (d * F).sum(1))[:, None] * d).sum(0)
+    ref /= 6 * X("3.14159265358979323846264338327950288") * a
+    err = np.sqrt((((got[at] - ref) ** 2).sum() / (ref ** 2).sum()).astype(np.float64))
+    assert err <= 9e-16
+
+
 @pytest.mark.parametrize("target", ["f", "r"])
 def test_fp64_product_in_place(ctx, target):
     """The velocities may overwrite the forces or the positions."""
