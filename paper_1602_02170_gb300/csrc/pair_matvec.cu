@@ -225,9 +225,13 @@ __global__ void __launch_bounds__(NT, NT == kNT ? (NP == 1 ? 3 : 2) : 16) pair_f
 // z, max x, y, z), and grid->far2, the squared distance beyond which a block
 // pair is far (see x2sym_item); such pairs take the kFar instance, and the
 // kVeryFar one from kVeryFarRadii radii on.
-// The smallest blocks round each sum once (mob_apply2), which keeps the error of
-// products below 4,096 blobs at that of sums over 16 sources (2,000 blobs without
-// the wall: 1.6e-7 -> 1.5e-7).
+// Blocks of 64 and 128 blobs fold their FP32 sums every 16 steps, and all but those
+// of 128 with the wall round each term once (x2sym_item): they stand where packed
+// kernels summed chunks of 16 to 32 sources, and whole blocks' sums were up to 1.6
+// times as far off.  Relative L2 error of 6,480 blobs in shells of 162, whole /
+// folded (the packed kernel): 2.4e-7 / 1.8e-7 (1.9e-7) with the wall, 2.3e-7 /
+// 1.3e-7 (1.4e-7) without; 2,100 blobs in shells of 42 without 1.35e-7 / 1.15e-7
+// (1.25e-7).  9,003 blobs 134 -> 136 us with the wall, 76 -> 87 without.
 constexpr int kBoxBlobs = 256;
 constexpr int64_t kSymNT64MinN = 4096, kSymNT128MinN = 12000;
 

@@ -282,7 +282,11 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
                                            int sub1 = 2)
 {
     constexpr int NW = NT / 32;
-    constexpr bool ONCE = NT == 32;  // the smallest blocks' sums (mob_apply2)
+    // Blocks of 64 and 128 blobs: FP32 sums over 16 steps instead of 32 to 64,
+    // and but for blocks of 128 with the wall one rounding a term
+    // (mob_apply2).  These sizes replace kernels whose sums held 16 to 32 terms.
+    constexpr bool FINE = NT <= 64, ONCE = NT == 32 || (NT == 64 && !WALL);
+    constexpr int kRun = FINE ? 16 : 32;  // steps between folds within a group
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool diag = I == J;
     const int64_t ia = I * 2 * NT + threadIdx.x, ib = ia + NT;
@@ -318,58 +322,79 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
         }
         __syncthreads();
         float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
+        auto fold = [&]() {
+            kahan_add(sum[0][0], comp[0][0], ax.x);
+            kahan_add(sum[0][1], comp[0][1], ay.x);
+            kahan_add(sum[0][2], comp[0][2], az.x);
+            kahan_add(sum[1][0], comp[1][0], ax.y);
+            kahan_add(sum[1][1], comp[1][1], ay.y);
+            kahan_add(sum[1][2], comp[1][2], az.y);
+            ax = ay = az = make_float2(0.f, 0.f);
+        };
         if (diag) {
+            for (int s0 = 0; s0 < NT; s0 += FINE ? kRun : NT) {
 #pragma unroll 2
-            for (int s = 0; s < NT; ++s) {
-                const SrcX2 q = load_sym<WALL, true>(sP, s);
-                const float2 dx = add2(add2(xh, q.nx), add2(xl, q.nxl));
-                const float2 dy = add2(add2(yh, q.ny), add2(yl, q.nyl));
-                const float2 dz = add2(fma2(q.z, k.m1, zh), add2(zl, q.nzl));
-                const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
-                const Mob<float2> m = mob_coefs2<WALL, kNear>(dz, dxy2, zh, q.z, q.zz, k);
-                mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
+                for (int s = s0; s < s0 + (FINE ? kRun : NT); ++s) {
+                    const SrcX2 q = load_sym<WALL, true>(sP, s);
+                    const float2 dx = add2(add2(xh, q.nx), add2(xl, q.nxl));
+                    const float2 dy = add2(add2(yh, q.ny), add2(yl, q.nyl));
+                    const float2 dz = add2(fma2(q.z, k.m1, zh), add2(zl, q.nzl));
+                    const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
+                    const Mob<float2> m = mob_coefs2<WALL, kNear>(dz, dxy2, zh, q.z, q.zz, k);
+                    mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
+                }
+                if (FINE) fold();
             }
         } else {
             for (int g = 0; g < NT / 32; ++g) {
                 float2 rx = make_float2(0.f, 0.f), ry = rx, rz = rx;
+                float half[3] = {0.f, 0.f, 0.f};  // FINE: sums of the first run of steps
+                for (int t0 = 0; t0 < 32; t0 += kRun) {
 #pragma unroll 2
-                for (int t = 0; t < 32; ++t) {
-                    const int s = g * 32 + ((lane + t) & 31);
-                    const SrcX2 q = load_sym<WALL, LEVEL == kNear>(sP, s);
-                    float2 dx = add2(xh, q.nx);
-                    float2 dy = add2(yh, q.ny);
-                    float2 dz = fma2(q.z, k.m1, zh);
-                    if (LEVEL == kNear) {
-                        dx = add2(dx, add2(xl, q.nxl));
-                        dy = add2(dy, add2(yl, q.nyl));
-                        dz = add2(dz, add2(zl, q.nzl));
+                    for (int t = t0; t < t0 + kRun; ++t) {
+                        const int s = g * 32 + ((lane + t) & 31);
+                        const SrcX2 q = load_sym<WALL, LEVEL == kNear>(sP, s);
+                        float2 dx = add2(xh, q.nx);
+                        float2 dy = add2(yh, q.ny);
+                        float2 dz = fma2(q.z, k.m1, zh);
+                        if (LEVEL == kNear) {
+                            dx = add2(dx, add2(xl, q.nxl));
+                            dy = add2(dy, add2(yl, q.nyl));
+                            dz = add2(dz, add2(zl, q.nzl));
+                        }
+                        const float2 dxy2 = fma2(dy, dy, LEVEL == kNear ? fma2(dx, dx, k.tiny)
+                                                                        : mul2(dx, dx));
+                        const Mob<float2> m = mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, q.z, q.zz, k);
+                        mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
+                        mob_apply2<WALL, true, ONCE>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
+                        // hand the accumulator to lane - 1, which meets this source next step
+                        const int from = (lane + 1) & 31;
+                        rx.x = __shfl_sync(0xffffffffu, rx.x, from);
+                        rx.y = __shfl_sync(0xffffffffu, rx.y, from);
+                        ry.x = __shfl_sync(0xffffffffu, ry.x, from);
+                        ry.y = __shfl_sync(0xffffffffu, ry.y, from);
+                        rz.x = __shfl_sync(0xffffffffu, rz.x, from);
+                        rz.y = __shfl_sync(0xffffffffu, rz.y, from);
                     }
-                    const float2 dxy2 = fma2(dy, dy, LEVEL == kNear ? fma2(dx, dx, k.tiny)
-                                                                    : mul2(dx, dx));
-                    const Mob<float2> m = mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, q.z, q.zz, k);
-                    mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
-                    mob_apply2<WALL, true, ONCE>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
-                    // hand the accumulator to lane - 1, which meets this source next step
-                    const int from = (lane + 1) & 31;
-                    rx.x = __shfl_sync(0xffffffffu, rx.x, from);
-                    rx.y = __shfl_sync(0xffffffffu, rx.y, from);
-                    ry.x = __shfl_sync(0xffffffffu, ry.x, from);
-                    ry.y = __shfl_sync(0xffffffffu, ry.y, from);
-                    rz.x = __shfl_sync(0xffffffffu, rz.x, from);
-                    rz.y = __shfl_sync(0xffffffffu, rz.y, from);
+                    if (FINE) fold();
+                    if (FINE && t0 == 0) {
+                        half[0] = rx.x + rx.y;
+                        half[1] = ry.x + ry.y;
+                        half[2] = rz.x + rz.y;
+                        rx = ry = rz = make_float2(0.f, 0.f);
+                    }
                 }
                 float *o3 = sRev + 3 * (warp * NT + g * 32 + lane);
-                o3[0] = rx.x + rx.y;
-                o3[1] = ry.x + ry.y;
-                o3[2] = rz.x + rz.y;
+                const float2 rev[3] = {rx, ry, rz};
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    o3[c] = rev[c].x + rev[c].y;
+                    // after half a round lane l held the sums of source l + 16
+                    if (FINE) o3[c] += __shfl_xor_sync(0xffffffffu, half[c], 16);
+                }
             }
         }
-        kahan_add(sum[0][0], comp[0][0], ax.x);
-        kahan_add(sum[0][1], comp[0][1], ay.x);
-        kahan_add(sum[0][2], comp[0][2], az.x);
-        kahan_add(sum[1][0], comp[1][0], ax.y);
-        kahan_add(sum[1][1], comp[1][1], ay.y);
-        kahan_add(sum[1][2], comp[1][2], az.y);
+        if (!FINE) fold();
         if (!diag) {
             __syncthreads();
             const int64_t j = j0 + threadIdx.x;

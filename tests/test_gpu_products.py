@@ -114,6 +114,26 @@ def test_fp32_symmetric_blocks_of_every_size(ctx, n, wall):
     assert np.abs(got - ref).max() <= TOL["fp32"] * np.abs(ref).max()
 
 
+@pytest.mark.parametrize("wall,bar", [(True, 2.1e-7), (False, 1.7e-7)])
+def test_fp32_sums_of_the_middle_sizes(ctx, wall, bar):
+    """40 shells of 162 blobs (blocks of 128 blobs): pair terms good to about
+    1.1e-7, or 1.5e-7 where the wall's parts nearly cancel, in FP32 sums of 16
+    terms (0.4 x 2^-24 sqrt(16 / 2) = 0.7e-7 for one rounding a term, 1e-7 for
+    two): 1.3e-7 and 1.8e-7, a sixth more allowed.  Sums over 64 terms have
+    twice the rounding, 1.8e-7 and 2.5e-7."""
+    rng = np.random.default_rng(11)
+    nb, a = 40, 0.12
+    p = np.arange(nb)
+    q = np.stack([p % 7 * 3.125, p // 7 * 3.125, rng.uniform(1.05 + a, 1.45 + a, nb)], axis=1)
+    th = I.random_unit_quaternions(rng, nb)
+    start = 162 * np.arange(nb + 1)
+    r = O.blob_positions(q, th, start, np.tile(I.shell(162), (nb, 1)))
+    f = rng.standard_normal(r.shape)
+    got = host(ctx.mobility_matvec(dev(r), dev(f), a, 1.0, wall, "fp32"))
+    ref = host(ctx.mobility_matvec(dev(r), dev(f), a, 1.0, wall, "fp64"))
+    assert rel_l2(got, ref) <= bar
+
+
 def test_fp32_product_in_place_and_variant_by_size(ctx):
     for n, variant in ((400, 4), (700, 3)):
         r, f = _cloud(n, n)
