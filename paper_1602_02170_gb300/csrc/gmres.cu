@@ -990,7 +990,7 @@ static mb_status solve_rigid(mb_context *ctx, int resist, int64_t nb, int64_t n,
     if (p->precond == MB_PRECOND_FREE_SHARED)
         MB_TRY(precond_setup_shared(ctx, nb, n, theta, blob_start, rho, p->a, p->eta, s, !resist));
     else
-        MB_TRY(precond_setup(ctx, nb, n, r, q, blob_start, p->a, p->eta, p->wall, s, !resist,
+        MB_TRY(precond_setup(ctx, nb, n, r, q, blob_start, p->a, p->eta, p->wall, s, true, !resist,
                              shift));
     if (p->prec != MB_FP64) MB_TRY(matvec_pack_positions(ctx, r, n, s));
     MB_TRY(wait_stream(ctx, s, "solver setup"));

@@ -237,10 +237,12 @@ void launch_saddle_rows(const MatvecPartials &mp, int64_t n, int64_t nb, const d
 // Preconditioner (precond.cu)
 // schur = 0 keeps only the blob blocks M_pp^-1 (resistance problem).
 // shift (N per-blob values or null) is added to the diagonal of each M_pp
-// (permeable bodies, Appendix C).
+// (permeable bodies, Appendix C).  solve: for the few dozen applications of one
+// solve, which a cheaper setup may make up for with dearer ones.
 mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
                         const double *q, const int64_t *blob_start, double a, double eta,
-                        int wall, cudaStream_t s, int schur = 1, const double *shift = nullptr);
+                        int wall, cudaStream_t s, bool solve = false, int schur = 1,
+                        const double *shift = nullptr);
 // Asynchronous setup of the blocks of nb bodies: start (nb+1, global blob
 // indices), poff (nb offsets into P).  A failing body p sets flags[flag_slot[p]]
 // = 2, or, without flag_slot, lowers flags[0] to p.  sizes: the bodies may be of

@@ -1853,7 +1853,7 @@ __global__ void __launch_bounds__(256) precond_apply_shared_kernel(
 
 mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
                         const double *q, const int64_t *blob_start, double a, double eta,
-                        int wall, cudaStream_t s, int schur, const double *shift)
+                        int wall, cudaStream_t s, bool solve, int schur, const double *shift)
 {
     // body sizes on the host
     std::vector<int64_t> hstart(nb + 1);
@@ -1898,19 +1898,19 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
         MB_TRY(ensure(ctx, ctx->sol_dots, sizeof(double) * stride * grid, "Cholesky scratch"));
         scratch = (double *)ctx->sol_dots.ptr;
     }
-    // Bodies with large blocks keep the factored form: its application costs the
-    // FP64 FMAs of the explicit inverse's GEMV and its setup a third of the
-    // explicit inverse's (no L^-1, no W^T W).  Few or small bodies keep the
-    // explicit inverse, whose application spreads over many CTAs.  162-blob
-    // shells, setup / application / mixed solve (ms), explicit and factored: 32
-    // bodies 5.9 / 0.05 / 9.4 and 2.0 / 0.15 / 8.2, 80 bodies 14.6 / 0.12 / 27.7
-    // and 5.7 / 0.15 / 21.7, 151 bodies 25.8 / 0.16 / 65.8 and 9.3 / 0.23 / 53.9 (120 of
-    // 200 blobs, setup / application: 37.0 / 0.13 and 13.1 / 0.32); the line lies
-    // where an application of 162-blob bodies costs half as much again.  The resistance
-    // problem takes three times the iterations, so there the inverse pays up to
-    // one body an SM.
-    const bool factored = !lsmem && nmax <= kSplitMaxRowsSmem &&
-                          nb >= (schur ? std::min(kFactoredMinBodies, ctx->sm_count) : ctx->sm_count);
+    // From as many bodies as SMs on, large blocks keep the factored form: its
+    // application costs the FP64 FMAs of the explicit inverse's GEMV and its setup a
+    // third of the explicit inverse's (no L^-1, no W^T W).  Fewer or small bodies
+    // keep the explicit inverse, whose application spreads over many CTAs.  A
+    // mobility solve applies it some 15 to 50 times, so there the line lies at
+    // kFactoredMinBodies: with 64, 100 and 151 bodies of 54 to 300 blobs, setups of
+    // 1.0-68 ms explicit against 0.5-20 factored, applications of 16-161 us against
+    // 39-625, mixed solves of 15 to 46 steps 5.2-381 ms against 2.8-245 (fewer
+    // bodies: 32 of 162 blobs 9.4 against 8.2).  Those who set up and apply by
+    // themselves may apply more often, and the resistance problem takes three
+    // times the iterations.
+    const int64_t line = solve && schur ? std::min(kFactoredMinBodies, ctx->sm_count) : ctx->sm_count;
+    const bool factored = !lsmem && nmax <= kSplitMaxRowsSmem && nb >= line;
     auto launch = [&](auto kern) -> mb_status {
         if (nmax <= kSplitMaxRowsSmem)
             return setup_split(ctx, nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,

@@ -483,3 +483,30 @@ def test_preconditioner_tile_edges(ctx, nbod, counts):
     lam_ref, UO_ref = O.precond_apply(r, q, start, a, 1.0, True, w, g)
     assert rel_l2(host(lam), lam_ref) <= 1e-9
     assert rel_l2(host(UO), UO_ref) <= 1e-9
+
+
+def test_preconditioner_form_by_use(ctx):
+    """70 bodies of 54 blobs, fewer than SMs: a setup by itself keeps the explicit
+    inverses (the blocks and the scratch of their triangular inverses), whose
+    applications cost less; a solve takes the factored form, and its solution
+    satisfies both rows of the saddle system."""
+    a, nbod, per = 0.2, 70, 54
+    rng = np.random.default_rng(1)
+    q = np.stack([4.0 * (np.arange(nbod) % 10), 4.0 * (np.arange(nbod) // 10), np.full(nbod, 2.5)], axis=1)
+    k = np.arange(per)
+    rho = np.tile(2.2 * a * np.stack([k % 3 - 1, k // 3 % 3 - 1, k // 9 - 2.5], axis=1), (nbod, 1))
+    rho = rho + rng.uniform(-0.02, 0.02, rho.shape)
+    start = dev(per * np.arange(nbod + 1), torch.int64)
+    r = dev(np.repeat(q, per, axis=0) + rho)
+    with mb.Context(0) as c:
+        c.precond_setup(r, dev(q), start, a, 1.0, True)
+        assert c.workspace_bytes() >= 8 * nbod * ((3 * per + 6) ** 2 + (3 * per) ** 2)
+    F, T = rng.standard_normal((nbod, 3)), rng.standard_normal((nbod, 3))
+    theta = dev(np.tile([1.0, 0.0, 0.0, 0.0], (nbod, 1)))
+    for prec in ("fp64", "mixed"):
+        U, W, lam, info = ctx.solve_mobility(dev(q), theta, start, dev(rho), dev(F), dev(T), a, 1.0,
+                                             True, tol=1e-11, prec=prec)
+        assert info["converged"] == 1
+        u = host(ctx.mobility_matvec(r, lam, a, 1.0, True, "fp64"))
+        assert rel_l2(u, host(ctx.K_apply(r, dev(q), start, torch.cat([U, W], dim=1)))) <= 1e-8
+        assert rel_l2(host(ctx.KT_apply(r, dev(q), start, lam)), np.concatenate([F, T], axis=1)) <= 1e-8
