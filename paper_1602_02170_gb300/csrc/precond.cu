@@ -1309,13 +1309,14 @@ __global__ void __launch_bounds__(256, 3) pc_trinv_df_kernel(
             const int j = warp >> 1, c = 16 * (warp & 1) + (lane & 15), half = lane >> 4;
             DfTile &X = sm.D[j];
             const DfTile &Ls = sm.A[j];
-            for (int k = 16 * (warp & 1); k < kTile; ++k) {
+            const int last = min(kTile, n - (t + j) * kTile);  // the tile's rows
+            for (int k = 16 * (warp & 1); k < last; ++k) {
                 const dfl wk = X.at(k, c) * sm.dw[j * kTile + k];
                 __syncwarp();
                 if (half == 0) X.set(k, c, wk);
                 const dfl2 w2 = dfl2(wk);
 #pragma unroll 2
-                for (int i = k + 1 + 2 * half; i < kTile; i += 4) {
+                for (int i = k + 1 + 2 * half; i < last; i += 4) {
                     const dfl a0 = X.at(i, c), a1 = X.at(i + 1, c);
                     const dfl l0 = Ls.at(i, k), l1 = Ls.at(i + 1, k);
                     const dfl2 v = dfl2(make_float2(a0.hi, a1.hi), make_float2(a0.lo, a1.lo)) -
@@ -1475,8 +1476,9 @@ __global__ void __launch_bounds__(256, 3) pc_product_df_kernel(
             }
             if (k0 + kTile < n) fetch(k0 + kTile);
             __syncthreads();
+            const int last = min(kTile, n - k0);
 #pragma unroll 4
-            for (int k = 0; k < kTile; ++k) {
+            for (int k = 0; k < last; ++k) {
                 const dfl2 x = X.pair(k, c2);
                 acc[0] += dfl2(Wi.at(k, r)) * x;
                 acc[1] += dfl2(Wi.at(k, r + 16)) * x;
