@@ -243,14 +243,19 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
                         const double *q, const int64_t *blob_start, double a, double eta,
                         int wall, cudaStream_t s, bool solve = false, int schur = 1,
                         const double *shift = nullptr);
+// Blobs of the bodies of a setup: the most and the fewest, and the most of those
+// whose blocks fit one CTA's shared memory (0: none).
+struct BodySizes {
+    int max_np = 0, min_np = 0x7fffffff, small_np = 0;
+    void add(int64_t np);
+};
 // Asynchronous setup of the blocks of nb bodies: start (nb+1, global blob
 // indices), poff (nb offsets into P).  A failing body p sets flags[flag_slot[p]]
-// = 2, or, without flag_slot, lowers flags[0] to p.  sizes: the bodies may be of
-// several sizes.
+// = 2, or, without flag_slot, lowers flags[0] to p.
 mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, const double *q,
-                              const int64_t *start, const int64_t *poff, double *P, int max_np,
-                              double a, double eta, int wall, int *flags, const int *flag_slot,
-                              cudaStream_t s, bool sizes, int schur = 1);
+                              const int64_t *start, const int64_t *poff, double *P,
+                              const BodySizes &sizes, double a, double eta, int wall, int *flags,
+                              const int *flag_slot, cudaStream_t s, int schur = 1);
 // Scratch that the setup of nb bodies of up to max_np blobs takes.
 size_t precond_scratch_bytes(int64_t nb, int max_np);
 constexpr int kSetupSmallRows = 128;  // rows of the blocks that take the small-body setup

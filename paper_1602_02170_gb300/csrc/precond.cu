@@ -582,12 +582,11 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
     SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base,
-    int schur, const int *__restrict__ order)
+    int schur, const int *__restrict__ order, int nmax)
 {
     extern __shared__ double sm[];
     __shared__ int bad, pfail;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nmax = scr.nmax;
     double *L = sm;                                       // rows of the lower triangle
     double *B = L + (size_t)nmax * (nmax + 1) / 2;        // n x 6
     double *pT = B + 6 * nmax;                            // the panel's columns, kPanel x nmax
@@ -599,6 +598,7 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
         const int64_t b0 = start[p];
         const int np = (int)(start[p + 1] - b0);
         const int n = 3 * np, m = n + 6;
+        if (n > nmax) continue;  // uniform; pc_factor_cluster_kernel's
         double *Pp = P + poff[p];
         const double qx = q[3 * p], qy = q[3 * p + 1], qz = q[3 * p + 2];
         __syncthreads();  // done with the previous body
@@ -743,18 +743,18 @@ __global__ void __launch_bounds__(256, 2) pc_factor_small_kernel(
     }
 }
 
-// Bodies from the largest to the smallest (a counting sort by blobs, at most
-// kSmemMaxRows / 3): CTAs start in this order, so that the long ones spread over
-// the SMs and the short ones fill in beside them.
+// Bodies from the largest to the smallest (a counting sort by blobs; those above
+// kSmemMaxRows rows, which the kernel skips, come first): CTAs start in this order,
+// so that the long ones spread over the SMs and the short ones fill in beside them.
 __global__ void __launch_bounds__(1024) pc_order_kernel(int64_t nb, const int64_t *__restrict__ start,
                                                         int *__restrict__ order)
 {
-    constexpr int kMax = kSmemMaxRows / 3;
-    __shared__ int count[kMax + 2];
-    for (int b = threadIdx.x; b < kMax + 2; b += blockDim.x) count[b] = 0;
+    constexpr int kMax = kSmemMaxRows / 3 + 1;
+    __shared__ int count[kMax + 1];
+    auto bin = [&](int64_t p) { return (int)min(start[p + 1] - start[p], (int64_t)kMax); };
+    for (int b = threadIdx.x; b <= kMax; b += blockDim.x) count[b] = 0;
     __syncthreads();
-    for (int64_t p = threadIdx.x; p < nb; p += blockDim.x)
-        atomicAdd(count + (int)(start[p + 1] - start[p]), 1);
+    for (int64_t p = threadIdx.x; p < nb; p += blockDim.x) atomicAdd(count + bin(p), 1);
     __syncthreads();
     if (threadIdx.x == 0)
         for (int b = kMax, at = 0; b >= 0; --b) {
@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(1024) pc_order_kernel(int64_t nb, const int64_
         }
     __syncthreads();
     for (int64_t p = threadIdx.x; p < nb; p += blockDim.x)
-        order[atomicAdd(count + (int)(start[p + 1] - start[p]), 1)] = (int)p;
+        order[atomicAdd(count + bin(p), 1)] = (int)p;
 }
 
 size_t factor_small_smem(int nmax)
@@ -832,7 +832,8 @@ template <bool SROWS, bool DF>
 __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc_factor_cluster_kernel(
     int64_t nb, const double *__restrict__ r, const double *__restrict__ q,
     const int64_t *__restrict__ start, const int64_t *__restrict__ poff, double *__restrict__ P,
-    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base, int schur)
+    SplitScratch scr, int *__restrict__ flag, const int *__restrict__ flag_slot, int64_t p_base, int schur,
+    int skip)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -860,6 +861,7 @@ __global__ void __cluster_dims__(kFacCluster, 1, 1) __launch_bounds__(256, 2) pc
         const int64_t b0 = start[p];
         const int np = (int)(start[p + 1] - b0);
         const int n = 3 * np, m = n + 6;
+        if (n <= skip) continue;  // uniform over the cluster; pc_factor_small_kernel's
         const int nown = n > rank ? (n - 1 - rank) / kFacCluster + 1 : 0;
         double *Pp = P + poff[p];
         const double qx = q[3 * p], qy = q[3 * p + 1], qz = q[3 * p + 2];
@@ -1679,15 +1681,14 @@ __global__ void __launch_bounds__(32 * kKeepWarps) pc_keep_factor_kernel(
     }
 }
 
-// sizes: the bodies are not all of one size.
 // Runs S1..S4 over groups of bodies whose scratch fits the cap (S1, S2, S3'
 // with `factored`).
 mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double *q,
-                      const int64_t *start, const int64_t *poff, double *P, int max_np, double a,
-                      double eta, int wall, int *flag, const int *flag_slot, int schur, cudaStream_t s,
-                      const double *shift, bool sizes, bool factored = false)
+                      const int64_t *start, const int64_t *poff, double *P, const BodySizes &sizes,
+                      double a, double eta, int wall, int *flag, const int *flag_slot, int schur,
+                      cudaStream_t s, const double *shift, bool factored = false)
 {
-    const int nmax = 3 * max_np;
+    const int max_np = sizes.max_np, nmax = 3 * max_np;
     const int64_t wsize = factored ? 0 : (int64_t)nmax * nmax, stride = split_stride(nmax, wsize);
     const int64_t cap_bytes = (int64_t)MB_SETUP_SCRATCH_MB << 20;
     const int64_t group = std::max<int64_t>(1, std::min<int64_t>(nb, cap_bytes / (8 * stride)));
@@ -1713,9 +1714,15 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
         // otherwise.  42-blob bodies, clusters: 97 us for 8, 118 for 32, 148 for
         // 40, 264 for 100.  A CTA per body in global memory, column by column,
         // took the whole setup of 300 bodies of 54, 80 and 100 blobs from 1.8, 3.6
-        // and 5.7 ms to 3.3, 7.2 and 11.6.
+        // and 5.7 ms to 3.3, 7.2 and 11.6.  Where many small bodies come with
+        // larger ones, each kernel takes its own: 2,000 bodies of 12 blobs and 5 of
+        // 60 take 0.72 ms, with clusters for all 2.4.  The kernels run one after the
+        // other, so below four CTAs an SM the clusters take all (60 bodies of 42 blobs
+        // and 4 of 54: 0.91 ms against 0.96).
         const bool df = nmax <= kSetupSmallRows;  // double-float S3 and S4
-        if (!lsmem || ng * kFacCluster <= 2 * (int64_t)ctx->sm_count) {
+        const bool waves = ng * kFacCluster > (lsmem ? 2 : 4) * (int64_t)ctx->sm_count;
+        const int small_rows = waves ? 3 * sizes.small_np : 0;
+        if (small_rows < nmax) {
             const size_t csm = factor_cluster_smem(nmax, lsmem);
             auto fk = df ? pc_factor_cluster_kernel<true, true>
                          : lsmem ? pc_factor_cluster_kernel<true, false>
@@ -1723,26 +1730,29 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
             MB_CUDA_TRY(ctx, cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)csm));
             fk<<<(int)ng * kFacCluster, 256, csm, s>>>(ng, r, q + 3 * g0, st, po, P, scr, flag,
-                                                       flag_slot, g0, schur);
-        } else {
-            const size_t fsmem = factor_small_smem(nmax);
+                                                       flag_slot, g0, schur, small_rows);
+            count_launch();
+        }
+        if (small_rows > 0) {
+            const size_t fsmem = factor_small_smem(small_rows);
             auto factor = df ? pc_factor_small_kernel<true> : pc_factor_small_kernel<false>;
             MB_CUDA_TRY(ctx, cudaFuncSetAttribute(factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)fsmem));
             int *order = nullptr;
-            if (sizes && ng > ctx->sm_count) {
+            if (sizes.min_np < max_np && ng > ctx->sm_count) {
                 order = (int *)(scr.base + stride * group);
                 pc_order_kernel<<<1, 1024, 0, s>>>(ng, st, order);
                 count_launch();
             }
             factor<<<(unsigned)std::min<int64_t>(ng, 1 << 30), 256, fsmem, s>>>(
-                ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur, order);
+                ng, r, q + 3 * g0, st, po, P, scr, flag, flag_slot, g0, schur, order, small_rows);
+            count_launch();
         }
         if (factored) {
             const int panels = (int)ceil_div(nmax, kFacPanel);
             pc_keep_factor_kernel<<<(unsigned)std::min<int64_t>(ceil_div(ng * panels, kKeepWarps), 1 << 30),
                                     32 * kKeepWarps, 0, s>>>(ng, st, po, P, scr, panels);
-            count_launch(3);
+            count_launch(2);
             MB_CUDA_TRY(ctx, cudaGetLastError());
             continue;
         }
@@ -1769,7 +1779,7 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
                 const int gp = (int)std::min<int64_t>(ng * tiles, 1 << 30);
                 pc_product_df_kernel<<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles, schur);
             }
-            count_launch(4);
+            count_launch(3);
             MB_CUDA_TRY(ctx, cudaGetLastError());
             continue;
         } else if (nmax <= 256)
@@ -1778,7 +1788,7 @@ mb_status setup_split(mb_context *ctx, int64_t nb, const double *r, const double
             pc_trinv_kernel<16><<<gt, 256, 0, s>>>(ng, st, po, P, scr, col_groups);
         const int gp = (int)std::min<int64_t>(ng * tiles, 16 * (int64_t)ctx->sm_count);
         pc_product_kernel<<<gp, 256, 0, s>>>(ng, st, po, P, scr, tiles, schur);
-        count_launch(4);
+        count_launch(3);
         MB_CUDA_TRY(ctx, cudaGetLastError());
     }
     return MB_OK;
@@ -1866,12 +1876,11 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
         return set_err(ctx, MB_EINVAL, "blob_start[0] must be 0 and blob_start[n_b] = N");
     std::vector<int64_t> off(nb + 1);
     off[0] = 0;
-    int max_np = 0, min_np = 0x7fffffff;
+    BodySizes sizes;
     for (int64_t p = 0; p < nb; ++p) {
         const int64_t np = hstart[p + 1] - hstart[p];
         if (np < 1) return set_err(ctx, MB_EINVAL, "body %lld has no blobs", (long long)p);
-        max_np = std::max<int>(max_np, (int)np);
-        min_np = std::min<int>(min_np, (int)np);
+        sizes.add(np);
         off[p + 1] = off[p] + (3 * np + 6) * (3 * np + 6);
     }
     MB_TRY(ensure(ctx, ctx->pinv, sizeof(double) * off[nb], "preconditioner"));
@@ -1885,7 +1894,7 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
     const int big = 0x7fffffff;
     MB_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->flag.ptr, &big, sizeof(int), cudaMemcpyHostToDevice, s));
 
-    const int nmax = 3 * max_np;
+    const int nmax = 3 * sizes.max_np;
     const bool lsmem = nmax <= kSmemMaxRows;
     const size_t small = sizeof(double) * (13 * (size_t)nmax + 72);
     const size_t smem = small + (lsmem ? sizeof(double) * (size_t)nmax * nmax : 0);
@@ -1916,8 +1925,9 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
     auto launch = [&](auto kern) -> mb_status {
         if (nmax <= kSplitMaxRowsSmem)
             return setup_split(ctx, nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,
-                               (const int64_t *)ctx->pinv_off.ptr, (double *)ctx->pinv.ptr, max_np,
-                               a, eta, wall, (int *)ctx->flag.ptr, nullptr, schur, s, shift, min_np < max_np, factored);
+                               (const int64_t *)ctx->pinv_off.ptr, (double *)ctx->pinv.ptr, sizes,
+                               a, eta, wall, (int *)ctx->flag.ptr, nullptr, schur, s, shift,
+                               factored);
         MB_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
         kern<<<grid, kSetupThreads, smem, s>>>(nb, r, q, (const int64_t *)ctx->blob_start_copy.ptr,
@@ -1941,7 +1951,7 @@ mb_status precond_setup(mb_context *ctx, int64_t nb, int64_t n, const double *r,
     MB_TRY(wait_stream(ctx, s, "preconditioner setup"));
     ctx->pc_nb = nb;
     ctx->pc_n = n;
-    ctx->pc_max_np = max_np;
+    ctx->pc_max_np = sizes.max_np;
     ctx->pc_doubles = off[nb];
     ctx->pc_f32_ready = false;
     ctx->pc_kind = MB_PRECOND_WALL;
@@ -1963,12 +1973,19 @@ size_t precond_scratch_bytes(int64_t nb, int max_np)
                             (size_t)MB_SETUP_SCRATCH_MB << 20);
 }
 
-mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, const double *q,
-                              const int64_t *start, const int64_t *poff, double *P, int max_np,
-                              double a, double eta, int wall, int *flags, const int *flag_slot,
-                              cudaStream_t s, bool sizes, int schur)
+void BodySizes::add(int64_t np)
 {
-    const int nmax = 3 * max_np;
+    max_np = std::max<int>(max_np, (int)np);
+    min_np = std::min<int>(min_np, (int)np);
+    if (3 * np <= kSmemMaxRows) small_np = std::max<int>(small_np, (int)np);
+}
+
+mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, const double *q,
+                              const int64_t *start, const int64_t *poff, double *P,
+                              const BodySizes &sizes, double a, double eta, int wall, int *flags,
+                              const int *flag_slot, cudaStream_t s, int schur)
+{
+    const int nmax = 3 * sizes.max_np;
     const bool lsmem = nmax <= kSmemMaxRows;
     const size_t small = sizeof(double) * (13 * (size_t)nmax + 72);
     const size_t smem = small + (lsmem ? sizeof(double) * (size_t)nmax * nmax : 0);
@@ -1985,8 +2002,8 @@ mb_status precond_setup_range(mb_context *ctx, int64_t nb, const double *r, cons
     }
     auto launch = [&](auto kern) -> mb_status {
         if (nmax <= kSplitMaxRowsSmem)
-            return setup_split(ctx, nb, r, q, start, poff, P, max_np, a, eta, wall, flags,
-                               flag_slot, schur, s, nullptr, sizes);
+            return setup_split(ctx, nb, r, q, start, poff, P, sizes, a, eta, wall, flags, flag_slot,
+                               schur, s, nullptr);
         MB_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem));
         kern<<<grid, kSetupThreads, smem, s>>>(nb, r, q, start, poff, k, scale, P, scratch, stride,
@@ -2093,12 +2110,11 @@ mb_status precond_setup_shared(mb_context *ctx, int64_t nb, int64_t n, const dou
                                      cudaMemcpyDeviceToDevice, s));
     const int big = 0x7fffffff;
     MB_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->flag.ptr, &big, sizeof(int), cudaMemcpyHostToDevice, s));
-    int max_ref_np = 0;
-    for (int64_t t = 0; t < ns; ++t)
-        max_ref_np = std::max<int>(max_ref_np, (int)(rstart[t + 1] - rstart[t]));
+    BodySizes sizes;
+    for (int64_t t = 0; t < ns; ++t) sizes.add(rstart[t + 1] - rstart[t]);
     MB_TRY(precond_setup_range(ctx, ns, dref, dref + 3 * rstart[ns], dstart, doff,
-                               (double *)ctx->pinv.ptr, max_ref_np, a, eta, 0,
-                               (int *)ctx->flag.ptr, nullptr, s, true, schur));
+                               (double *)ctx->pinv.ptr, sizes, a, eta, 0, (int *)ctx->flag.ptr,
+                               nullptr, s, schur));
     int first_bad = big;
     MB_CUDA_TRY(ctx, cudaMemcpyAsync(&first_bad, ctx->flag.ptr, sizeof(int),
                                      cudaMemcpyDeviceToHost, s));

@@ -1319,7 +1319,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
         for (size_t i = 0; i < admitted.size();) {
             const Req *first = admitted[i], *prev = first;
             int64_t nb = first->prob.n_bodies, nblob = first->prob.n_blobs;
-            int max_np = first->max_np, min_np = max_np;
+            int max_np = first->max_np;
             size_t end = i + 1;
             const size_t room = ctx->budget > ctx->held ? ctx->budget - ctx->held : 0;
             for (; end < admitted.size(); ++end) {
@@ -1342,6 +1342,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
             count_launch(2);
             // the run's blob ranges (over its requests' own, which hold one
             // entry more each) and preconditioner offsets
+            BodySizes sizes;
             std::vector<int64_t> po, bs;
             po.reserve(nb);
             bs.reserve(nb + 1);
@@ -1353,7 +1354,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
                     bs.push_back(rq->blob_off + rq->hstart[p]);
                     const int64_t np = rq->hstart[p + 1] - rq->hstart[p];
                     acc += (3 * np + 6) * (3 * np + 6);
-                    min_np = std::min(min_np, (int)np);
+                    sizes.add(np);
                 }
             }
             bs.push_back(b1);
@@ -1364,9 +1365,9 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
             // the copies read host vectors: make them complete before these go out of scope
             MB_CUDA_TRY(ctx, cudaStreamSynchronize(s));
             MB_TRY(precond_setup_range(ctx, nb, r, q + 3 * first->body_off,
-                                       bstart + first->start_off, poff + first->body_off, P, max_np,
+                                       bstart + first->start_off, poff + first->body_off, P, sizes,
                                        prm.a, prm.eta, prm.wall, st.bad,
-                                       body_slot + first->body_off, s, min_np < max_np));
+                                       body_slot + first->body_off, s));
         }
         std::vector<Seg> segs;
         std::vector<int> seg_off, list;

@@ -510,3 +510,24 @@ def test_preconditioner_form_by_use(ctx):
         u = host(ctx.mobility_matvec(r, lam, a, 1.0, True, "fp64"))
         assert rel_l2(u, host(ctx.K_apply(r, dev(q), start, torch.cat([U, W], dim=1)))) <= 1e-8
         assert rel_l2(host(ctx.KT_apply(r, dev(q), start, lam)), np.concatenate([F, T], axis=1)) <= 1e-8
+
+
+@pytest.mark.parametrize("counts", [[4] * 200 + [54], [60] + [53, 12] * 40, [15, 75, 3, 42, 100] * 35])
+def test_preconditioner_small_beside_large_bodies(ctx, counts):
+    """Enough bodies that small ones take a CTA each, beside some above 160 rows,
+    which take clusters: explicit and (from as many bodies as SMs on) factored
+    forms, each body against the oracle's direct solve.  The bar is that of the
+    other preconditioner tests."""
+    rng = np.random.default_rng(len(counts))
+    a, nbod = 0.2, len(counts)
+    start = np.concatenate([[0], np.cumsum(counts)]).astype(np.int64)
+    q = np.stack([5.0 * (np.arange(nbod) % 20), 5.0 * (np.arange(nbod) // 20), np.full(nbod, 2.5)], axis=1)
+    r = np.concatenate([q[p] + 2.2 * a * np.stack([np.arange(c) % 3, np.arange(c) // 3 % 3,
+                                                   np.arange(c) // 9], axis=1) for p, c in enumerate(counts)])
+    r = r + rng.uniform(-0.02, 0.02, r.shape)
+    w, g = rng.standard_normal(r.shape), rng.standard_normal((nbod, 6))
+    ctx.precond_setup(dev(r), dev(q), dev(start, torch.int64), a, 1.0, True)
+    lam, UO = ctx.precond_apply(dev(w), dev(g))
+    lam_ref, UO_ref = O.precond_apply(r, q, start, a, 1.0, True, w, g)
+    assert rel_l2(host(lam), lam_ref) <= 1e-9
+    assert rel_l2(host(UO), UO_ref) <= 1e-9
