@@ -56,12 +56,10 @@ __device__ __forceinline__ int tile_body_of(const TileBodies &tb, int64_t i)
     return lo;
 }
 
-// 1 / d in FP64 for d > 0: the FP32 reciprocal and one step of third order
-// y (1 + e + e^2), e = 1 - d y (|e| < 2^-22); arguments outside the FP32
-// range take the division.
-__device__ __forceinline__ double rcp_pos(double d)
+// 1 / d in FP64 for 1e-30 < d < 1e30: the FP32 reciprocal and one step of third
+// order y (1 + e + e^2), e = 1 - d y (|e| < 2^-22).
+__device__ __forceinline__ double rcp_mid(double d)
 {
-    if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
     const double y = (double)(1.0f / (float)d);
     const double e = fma(-d, y, 1.0);
     return fma(y, fma(e, e, e), y);
@@ -69,12 +67,22 @@ __device__ __forceinline__ double rcp_pos(double d)
 
 // R = (s^2 - v.v) I + 2 v v^T + 2 s [v]_x of the normalised quaternion:
 // with t = 2 / |theta|^2, (t s^2 - 1) I + t (v v^T + s [v]_x); R row-major,
-// then q, in m[0..11].
+// then q, in m[0..11].  Quaternions far from unit length, whose t may be out of
+// range, are normalised first.
 __device__ __forceinline__ void body_frame(const double *__restrict__ th,
                                            const double *__restrict__ q, double *m)
 {
-    const double s = th[0], x = th[1], y = th[2], z = th[3];
-    const double t = 2.0 * rcp_pos(fma(s, s, fma(x, x, fma(y, y, z * z))));
+    double s = th[0], x = th[1], y = th[2], z = th[3], t = 2.0;
+    const double n2 = fma(s, s, fma(x, x, fma(y, y, z * z)));
+    if (n2 > 1e-30 && n2 < 1e30) {
+        t *= rcp_mid(n2);
+    } else {
+        const double inv = rsqrt(n2);
+        s *= inv;
+        x *= inv;
+        y *= inv;
+        z *= inv;
+    }
     const double ts = t * s, tx = t * x, ty = t * y, tz = t * z, d = fma(ts, s, -1.0);
     m[0] = fma(tx, x, d);
     m[1] = fma(tx, y, -ts * z);

@@ -46,3 +46,14 @@ def test_kinematics_by_body_sizes(ctx, name):
     FT = host(ctx.KT_apply(dev(r), dev(q), S, dev(lam)))
     F, T = O.KT_apply(lam, r, q, start)
     assert np.abs(FT - np.concatenate([F, T], 1)).max() <= 1e-11
+
+
+@pytest.mark.parametrize("scale", [1e-155, 1e-100, 1e-16, 1e-14, 1e14, 1e16, 1e100, 1e153])
+def test_blob_build_from_quaternions_of_any_length(ctx, scale):
+    """Quaternions are normalised whatever their length.  At 1e-155 the squares
+    are denormal, good to 5e-14 of their sum: 1e-12 for offsets of a few units."""
+    q, theta, start, rho, _ = _case([7] * 50, 3)
+    S = torch.as_tensor(start, device="cuda")
+    r = host(ctx.blob_positions(dev(q), dev(theta * scale), S, dev(rho)))
+    unit = theta / np.linalg.norm(theta, axis=1, keepdims=True)
+    assert np.abs(r - O.blob_positions(q, unit, start, rho)).max() <= 1e-12
