@@ -174,3 +174,31 @@ def test_batch_singular_request_among_joint_setups(ctx):
     with pytest.raises(mb.MBError) as ei:
         ctx.solve_batch([_prob(s) for s in susp], A, 1.0, True, tol=1e-10, prec="mixed")
     assert ei.value.name == "MB_ESINGULAR" and "problem 1" in str(ei.value)
+
+
+def test_batch_after_a_batch_within_a_small_budget():
+    """A context keeps its last batch's buffers; where the budget does not hold
+    the next batch beside them, though by itself it fits, they go."""
+    def shells(nb, per, a, seed):
+        s = I.sphere_suspension(seed, nb, per, a, 4.0 * nb ** 0.5, 1.5, 4.0)
+        return [_prob(s)], s.a
+
+    first, a1 = shells(300, 12, 0.3, 1)    # a large basis, little scratch
+    second, a2 = shells(10, 162, 0.1, 2)   # a small basis, much scratch
+    run1 = lambda c: c.solve_batch(first, a1, 1.0, True, tol=1e-6, restart=150, prec="mixed")
+    run2 = lambda c: c.solve_batch(second, a2, 1.0, True, tol=1e-6, restart=20, prec="mixed")
+    need = []
+    for run in (run1, run2):
+        with mb.Context(0) as c:
+            want = run(c)
+            need.append(c.workspace_bytes())
+    budget = max(need) + (1 << 20)
+    with mb.Context(0) as c:
+        run1(c)
+        run2(c)
+        assert c.workspace_bytes() > budget  # beside the kept buffers it would not fit
+    with mb.Context(0, budget) as c:
+        run1(c)
+        (U, W, lam, info), = run2(c)
+        assert info["converged"] == 1 and c.workspace_bytes() <= budget
+    assert rel_l2(host(lam), host(want[0][2])) <= 1e-5
