@@ -13,6 +13,7 @@
 //     P_p^-1 = [[M_p^-1 - Q_p N_p Q_p^T, -Q_p N_p], [-N_p Q_p^T, -N_p]],
 // so that one application is one batched FP64 GEMV per body.
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 #include <unordered_map>
 #include <vector>
@@ -1212,10 +1213,10 @@ __global__ void __launch_bounds__(256) pc_trinv_kernel(
 // G and N in the scratch) as double-float pairs packed in the 8 bytes of an
 // FP64 number.
 // A 32 x 32 tile of double-float numbers in shared memory: hi and lo parts in
-// rows of kTileLd floats (pairs of columns stay 8-byte aligned, and two rows
-// apart by one start 2 banks apart); row 32 stays zero.
+// rows of kTileLd floats (pairs of columns, read as float2, stay 8-byte aligned,
+// and two rows apart by one start 2 banks apart); row 32 stays zero.
 constexpr int kTileLd = kTile + 2;
-struct DfTile {
+struct __align__(16) DfTile {
     float hi[(kTile + 1) * kTileLd], lo[(kTile + 1) * kTileLd];
     __device__ __forceinline__ dfl at(int r, int c) const
     {
@@ -1238,6 +1239,9 @@ struct DfTile {
         *(float2 *)(lo + r * kTileLd + 2 * c2) = v.lo;
     }
 };
+static_assert(alignof(DfTile) % alignof(float2) == 0 && offsetof(DfTile, lo) % alignof(float2) == 0 &&
+                  sizeof(float) * kTileLd % alignof(float2) == 0,
+              "pair() reads aligned float2s");
 
 // acc += A X for rows r, r + 16 and the column pair c2 of 32 x 32 tiles
 // (threads c2 = tid % 16, r = tid / 16 of 256).
