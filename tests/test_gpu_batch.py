@@ -202,3 +202,22 @@ def test_batch_after_a_batch_within_a_small_budget():
         (U, W, lam, info), = run2(c)
         assert info["converged"] == 1 and c.workspace_bytes() <= budget
     assert rel_l2(host(lam), host(want[0][2])) <= 1e-5
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64", "df64"])
+@pytest.mark.parametrize("bodies", [[1, 2, 1], [20, 1, 33], [90, 70]])
+def test_batch_residuals(ctx, bodies, prec):
+    """The saddle system's residual by separate FP64 products: the solves' 1e-10
+    of |b|, as much again for the engine's own products (double-float: 1e-13 of
+    velocities below |b|) and the loss between estimated and true residuals."""
+    tol = 1e-10
+    susp = [I.mixed_suspension(70 + k, nb) for k, nb in enumerate(bodies)]
+    res = ctx.solve_batch([_prob(s) for s in susp], A, 1.0, True, tol=tol, prec=prec)
+    for s, (U, W, lam, info) in zip(susp, res):
+        p = _prob(s)
+        r = ctx.blob_positions(p["q"], p["theta"], p["blob_start"], p["rho"])
+        top = ctx.mobility_matvec(r, lam, A, 1.0, True, "fp64") - ctx.K_apply(
+            r, p["q"], p["blob_start"], torch.cat([U, W], dim=1))
+        b = torch.cat([p["F"], p["T"]], dim=1)
+        low = ctx.KT_apply(r, p["q"], p["blob_start"], lam) - b
+        assert float((top.norm() ** 2 + low.norm() ** 2).sqrt() / b.norm()) <= 2 * tol

@@ -57,3 +57,19 @@ def test_blob_build_from_quaternions_of_any_length(ctx, scale):
     r = host(ctx.blob_positions(dev(q), dev(theta * scale), S, dev(rho)))
     unit = theta / np.linalg.norm(theta, axis=1, keepdims=True)
     assert np.abs(r - O.blob_positions(q, unit, start, rho)).max() <= 1e-12
+
+
+def test_rotation_matrices_to_the_last_bits(ctx):
+    """The frame of a body from the rows of the identity: 2 / |theta|^2 to two ulp,
+    two more products and a sum at size 1 or 2, so 8 x 2^-53 an entry."""
+    rng = np.random.default_rng(4)
+    nb = 4000
+    theta = rng.standard_normal((nb, 4)) * 10.0 ** rng.uniform(-20, 20, (nb, 1))
+    S = torch.as_tensor(3 * np.arange(nb + 1), device="cuda")
+    r = host(ctx.blob_positions(dev(np.zeros((nb, 3))), dev(theta), S, dev(np.tile(np.eye(3), (nb, 1)))))
+    L = np.longdouble
+    s, x, y, z = (theta.astype(L) / np.sqrt((theta.astype(L) ** 2).sum(1, keepdims=True))).T
+    R = np.stack([1 - 2 * (y * y + z * z), 2 * (x * y + s * z), 2 * (x * z - s * y),
+                  2 * (x * y - s * z), 1 - 2 * (x * x + z * z), 2 * (y * z + s * x),
+                  2 * (x * z + s * y), 2 * (y * z - s * x), 1 - 2 * (x * x + y * y)], axis=1)
+    assert np.abs(r.reshape(nb, 9) - R).max() <= 8 * 2.0 ** -53

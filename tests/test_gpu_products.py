@@ -238,3 +238,41 @@ def test_noalloc_every_size_and_in_place(ctx, n, wall):
     assert np.abs(got - ref).max() <= TOL["fp32"] * np.abs(ref).max()
     mb.mobility_matvec_noalloc(R, F, 0.5, 1.0, wall, out=F)
     assert np.abs(host(F) - got).max() <= 1e-14 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("wall", [True, False])
+@pytest.mark.parametrize("n", [4095, 4096, 4097])
+def test_fp32_symmetric_blocks_where_they_grow(ctx, n, wall):
+    """Blocks of 64 blobs below 4,096 blobs, of 128 from there on; the last one
+    is nearly empty at 4,097."""
+    r, f = _cloud(n, n)
+    got = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, wall, "fp32"))
+    assert ctx.pair_variant(n, wall) == 3
+    ref = host(ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, wall, "fp64"))
+    assert np.abs(got - ref).max() <= TOL["fp32"] * np.abs(ref).max()
+
+
+def test_fp32_variant_of_large_products(ctx):
+    r, f = _cloud(20000, 20000)
+    ctx.mobility_matvec(dev(r), dev(f), 0.5, 1.0, True, "fp32")
+    assert ctx.pair_variant(20000, True) == 3
+
+
+def test_fp64_reciprocal_square_root_to_the_last_bits(ctx):
+    """One blob far smaller than every distance, points beside it: u = 3a/4 / r (and
+    (a / r)^2 of it) in units of 1 / (6 pi eta a).  Distances of 26 bits have exact
+    squares, so u carries the reciprocal square root's rounding (one ulp allowed)
+    and those of two products: 2 ulp.  r^2 runs over the FP32 exponents, where the
+    estimate is an FP32 one, and beyond both ends of them."""
+    rng = np.random.default_rng(2)
+    a = 2.0 ** -80
+    e = np.concatenate([rng.integers(-72, 73, 6000), np.tile([-64, -63, 62, 63, 64], 800)])
+    y = np.ldexp(rng.integers(2 ** 25, 2 ** 26, len(e)).astype(np.float64), e - 25)
+    y[-10:] = np.ldexp(1.0, [-64, -63, -62, 62, 63, 64, -1, 0, 1, 2])
+    x = np.zeros((len(y), 3))
+    x[:, 1] = y
+    got = host(ctx.mobility_eval(dev(x), dev(np.zeros((1, 3))), dev([[1.0, 0.0, 0.0]]), a, 1.0, False, "fp64"))
+    L = np.longdouble
+    ref = L(1.0 / (6.0 * np.pi * 1.0 * a)) * (L(0.75 * a) / L(1) / y.astype(L) + L(0.5) * L(a) ** 3 / y.astype(L) ** 3)
+    assert np.abs(got[:, 0] / ref - 1).max() <= 2 * 2.0 ** -52
+    assert np.all(got[:, 1:] == 0)
