@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(NT, NT == kNT ? (NP == 1 ? 3 : 2) : 16) pair_f
 // 1.3e-7 (1.4e-7) without; 2,100 blobs in shells of 42 without 1.35e-7 / 1.15e-7
 // (1.25e-7).  9,003 blobs 134 -> 136 us with the wall, 76 -> 87 without.
 constexpr int kBoxBlobs = 256;
+constexpr int kSymBoxNT = kBoxBlobs / 2;  // the only blocks that come sorted: one a box
 constexpr int64_t kSymNT64MinN = 4096, kSymNT128MinN = 12000;
 
 struct SortGrid {
@@ -249,29 +250,37 @@ __global__ void __launch_bounds__(NT, 512 / NT) pair_sym_kernel(
 {
     __shared__ float4 sP[kX2SmemFloat4PerSource * NT];
     __shared__ float sRev[3 * NT * (NT / 32)];
-    constexpr int kPer = kBoxBlobs / (2 * NT);  // this kernel's blocks per box
-    const float far2 = box ? fmaxf(grid->far2, 1.5625f * k.four_a2) : 0.f;
-    const float vfar2 = 0.25f * kVeryFarRadii * kVeryFarRadii * k.four_a2;
+    float far2 = 0.f, vfar2 = 0.f;
+    if (NT == kSymBoxNT && box) {
+        far2 = fmaxf(grid->far2, 1.5625f * k.four_a2);
+        vfar2 = 0.25f * kVeryFarRadii * kVeryFarRadii * k.four_a2;
+    }
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         int64_t I, J;
         triangle_pair(item >> 1, I, J);
         const int half = (int)(item & 1);
-        int level = kNear;  // the same in every thread
-        if (box && I / kPer != J / kPer) {
-            const float *bi = box + 6 * (I / kPer), *bj = box + 6 * (J / kPer);
-            float d2 = 0.f;
+        if constexpr (NT == kSymBoxNT) {
+            int level = kNear;  // the same in every thread
+            if (box && I != J) {
+                const float *bi = box + 6 * I, *bj = box + 6 * J;
+                float d2 = 0.f;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const float g = fmaxf(fmaxf(bj[c] - bi[3 + c], bi[c] - bj[3 + c]), 0.f);
-                d2 = fmaf(g, g, d2);
+                for (int c = 0; c < 3; ++c) {
+                    const float g = fmaxf(fmaxf(bj[c] - bi[3 + c], bi[c] - bj[3 + c]), 0.f);
+                    d2 = fmaf(g, g, d2);
+                }
+                if (d2 > far2) level = d2 > vfar2 ? kVeryFar : kFar;
             }
-            if (d2 > far2) level = d2 > vfar2 ? kVeryFar : kFar;
+            if (level == kVeryFar) {
+                x2sym_item<WALL, NT, kVeryFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half);
+                continue;
+            }
+            if (level == kFar) {
+                x2sym_item<WALL, NT, kFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half);
+                continue;
+            }
         }
-        if (level == kVeryFar)
-            x2sym_item<WALL, NT, kVeryFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
-        else if (level == kFar)
-            x2sym_item<WALL, NT, kFar>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
-        else x2sym_item<WALL, NT, kNear>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half, half + 1);
+        x2sym_item<WALL, NT, kNear>(sP, sRev, hi, lo, f, n, I, J, k, u, scale, half);
     }
 }
 
@@ -731,6 +740,7 @@ void f32_launch(int v, const Plan &p, cudaStream_t s, const float4 *hi, const fl
 // (2^10 .. 2^kSortBits): blocks of 512 blobs span a few dozen cells, and the
 // per-tile count tables stay small.
 constexpr int64_t kSortMinN = 16384;
+static_assert(kSortMinN >= kSymNT128MinN, "sorted blobs come in blocks of kSymBoxNT");
 constexpr int kSortBits = 15;         // most cell bits
 constexpr int kSortKeysSmem = 16384;  // keys staged per round of the scatter
 

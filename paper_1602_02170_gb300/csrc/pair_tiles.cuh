@@ -255,8 +255,8 @@ __device__ __forceinline__ SrcX2 load_sym(const float4 *sP, int slot)
     return q;
 }
 
-// Symmetric packed item over block pair (I, J), I <= J, blocks of 2*NT blobs
-// (two targets per thread, as in x2_item with NP = 1).  Each unordered pair
+// Symmetric packed item over half of block pair (I, J), I <= J, blocks of 2*NT
+// blobs (two targets per thread, as in x2_item with NP = 1; NT sources).  Each unordered pair
 // is evaluated once.  Forward contributions accumulate in the thread's
 // registers (tile sums folded Kahan-style).  Reverse contributions use a
 // rotating schedule inside each group of 32 staged sources: at step t lane l
@@ -268,7 +268,6 @@ __device__ __forceinline__ SrcX2 load_sym(const float4 *sP, int slot)
 // over all ordered pairs.  u must be zeroed beforehand and receives
 // scale * M f.
 //
-// Sources [sub0, sub1) NT of block J (two halves of NT blobs).
 // LEVEL: how far apart the blocks' bounding boxes are known to be (mob_coefs2).
 // From kFar on the separations take the hi parts alone, whose rounding then
 // moves a separation by at most 2^-18 of itself.
@@ -278,9 +277,10 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
                                            const float4 *__restrict__ lo,
                                            const double *__restrict__ f, int64_t n, int64_t I,
                                            int64_t J, const MobConsts2 &k,
-                                           double *__restrict__ u, double scale, int sub0 = 0,
-                                           int sub1 = 2)
+                                           double *__restrict__ u, double scale, int half)
 {
+    const int64_t j0 = J * 2 * NT + half * NT;
+    if (j0 >= n) return;
     constexpr int NW = NT / 32;
     // Blocks of 64 and 128 blobs: FP32 sums over 16 steps instead of 32 to 64,
     // and but for blocks of 128 with the wall one rounding a term
@@ -306,106 +306,102 @@ __device__ __forceinline__ void x2sym_item(float4 *__restrict__ sP, float *__res
     for (int t = 0; t < 2; ++t)
 #pragma unroll
         for (int c = 0; c < 3; ++c) sum[t][c] = comp[t][c] = 0.f;
-    for (int sub = sub0; sub < sub1; ++sub) {
-        const int64_t j0 = J * 2 * NT + sub * NT;
-        if (j0 >= n) break;
-        __syncthreads();
-        {
-            const int64_t j = j0 + threadIdx.x;
-            const bool valid = j < n;
-            const int64_t jc = valid ? j : j0;
-            const float4 h = hi[jc], l = lo[jc];
-            const float fx = valid ? (float)f[3 * jc] : 0.f;
-            const float fy = valid ? (float)f[3 * jc + 1] : 0.f;
-            const float fz = valid ? (float)f[3 * jc + 2] : 0.f;
-            stage_sym<WALL>(sP, threadIdx.x, h, l, fx, fy, fz);
-        }
-        __syncthreads();
-        float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
-        auto fold = [&]() {
-            kahan_add(sum[0][0], comp[0][0], ax.x);
-            kahan_add(sum[0][1], comp[0][1], ay.x);
-            kahan_add(sum[0][2], comp[0][2], az.x);
-            kahan_add(sum[1][0], comp[1][0], ax.y);
-            kahan_add(sum[1][1], comp[1][1], ay.y);
-            kahan_add(sum[1][2], comp[1][2], az.y);
-            ax = ay = az = make_float2(0.f, 0.f);
-        };
-        if (diag) {
-            for (int s0 = 0; s0 < NT; s0 += FINE ? kRun : NT) {
+    __syncthreads();
+    {
+        const int64_t j = j0 + threadIdx.x;
+        const bool valid = j < n;
+        const int64_t jc = valid ? j : j0;
+        const float4 h = hi[jc], l = lo[jc];
+        const float fx = valid ? (float)f[3 * jc] : 0.f;
+        const float fy = valid ? (float)f[3 * jc + 1] : 0.f;
+        const float fz = valid ? (float)f[3 * jc + 2] : 0.f;
+        stage_sym<WALL>(sP, threadIdx.x, h, l, fx, fy, fz);
+    }
+    __syncthreads();
+    float2 ax = make_float2(0.f, 0.f), ay = ax, az = ax;
+    auto fold = [&]() {
+        kahan_add(sum[0][0], comp[0][0], ax.x);
+        kahan_add(sum[0][1], comp[0][1], ay.x);
+        kahan_add(sum[0][2], comp[0][2], az.x);
+        kahan_add(sum[1][0], comp[1][0], ax.y);
+        kahan_add(sum[1][1], comp[1][1], ay.y);
+        kahan_add(sum[1][2], comp[1][2], az.y);
+        ax = ay = az = make_float2(0.f, 0.f);
+    };
+    if (diag) {
+        for (int s0 = 0; s0 < NT; s0 += FINE ? kRun : NT) {
 #pragma unroll 2
-                for (int s = s0; s < s0 + (FINE ? kRun : NT); ++s) {
-                    const SrcX2 q = load_sym<WALL, true>(sP, s);
-                    const float2 dx = add2(add2(xh, q.nx), add2(xl, q.nxl));
-                    const float2 dy = add2(add2(yh, q.ny), add2(yl, q.nyl));
-                    const float2 dz = add2(fma2(q.z, k.m1, zh), add2(zl, q.nzl));
-                    const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
-                    const Mob<float2> m = mob_coefs2<WALL, kNear>(dz, dxy2, zh, q.z, q.zz, k);
+            for (int s = s0; s < s0 + (FINE ? kRun : NT); ++s) {
+                const SrcX2 q = load_sym<WALL, true>(sP, s);
+                const float2 dx = add2(add2(xh, q.nx), add2(xl, q.nxl));
+                const float2 dy = add2(add2(yh, q.ny), add2(yl, q.nyl));
+                const float2 dz = add2(fma2(q.z, k.m1, zh), add2(zl, q.nzl));
+                const float2 dxy2 = fma2(dy, dy, fma2(dx, dx, k.tiny));
+                const Mob<float2> m = mob_coefs2<WALL, kNear>(dz, dxy2, zh, q.z, q.zz, k);
+                mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
+            }
+            if (FINE) fold();
+        }
+    } else {
+        for (int g = 0; g < NT / 32; ++g) {
+            float2 rx = make_float2(0.f, 0.f), ry = rx, rz = rx;
+            float run[3] = {0.f, 0.f, 0.f};  // FINE: sums of the first run of steps
+            for (int t0 = 0; t0 < 32; t0 += kRun) {
+#pragma unroll 2
+                for (int t = t0; t < t0 + kRun; ++t) {
+                    const int s = g * 32 + ((lane + t) & 31);
+                    const SrcX2 q = load_sym<WALL, LEVEL == kNear>(sP, s);
+                    float2 dx = add2(xh, q.nx);
+                    float2 dy = add2(yh, q.ny);
+                    float2 dz = fma2(q.z, k.m1, zh);
+                    if (LEVEL == kNear) {
+                        dx = add2(dx, add2(xl, q.nxl));
+                        dy = add2(dy, add2(yl, q.nyl));
+                        dz = add2(dz, add2(zl, q.nzl));
+                    }
+                    const float2 dxy2 = fma2(dy, dy, LEVEL == kNear ? fma2(dx, dx, k.tiny)
+                                                                    : mul2(dx, dx));
+                    const Mob<float2> m = mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, q.z, q.zz, k);
                     mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
+                    mob_apply2<WALL, true, ONCE>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
+                    // hand the accumulator to lane - 1, which meets this source next step
+                    const int from = (lane + 1) & 31;
+                    rx.x = __shfl_sync(0xffffffffu, rx.x, from);
+                    rx.y = __shfl_sync(0xffffffffu, rx.y, from);
+                    ry.x = __shfl_sync(0xffffffffu, ry.x, from);
+                    ry.y = __shfl_sync(0xffffffffu, ry.y, from);
+                    rz.x = __shfl_sync(0xffffffffu, rz.x, from);
+                    rz.y = __shfl_sync(0xffffffffu, rz.y, from);
                 }
                 if (FINE) fold();
+                if (FINE && t0 == 0) {
+                    run[0] = rx.x + rx.y;
+                    run[1] = ry.x + ry.y;
+                    run[2] = rz.x + rz.y;
+                    rx = ry = rz = make_float2(0.f, 0.f);
+                }
             }
-        } else {
-            for (int g = 0; g < NT / 32; ++g) {
-                float2 rx = make_float2(0.f, 0.f), ry = rx, rz = rx;
-                float half[3] = {0.f, 0.f, 0.f};  // FINE: sums of the first run of steps
-                for (int t0 = 0; t0 < 32; t0 += kRun) {
-#pragma unroll 2
-                    for (int t = t0; t < t0 + kRun; ++t) {
-                        const int s = g * 32 + ((lane + t) & 31);
-                        const SrcX2 q = load_sym<WALL, LEVEL == kNear>(sP, s);
-                        float2 dx = add2(xh, q.nx);
-                        float2 dy = add2(yh, q.ny);
-                        float2 dz = fma2(q.z, k.m1, zh);
-                        if (LEVEL == kNear) {
-                            dx = add2(dx, add2(xl, q.nxl));
-                            dy = add2(dy, add2(yl, q.nyl));
-                            dz = add2(dz, add2(zl, q.nzl));
-                        }
-                        const float2 dxy2 = fma2(dy, dy, LEVEL == kNear ? fma2(dx, dx, k.tiny)
-                                                                        : mul2(dx, dx));
-                        const Mob<float2> m = mob_coefs2<WALL, LEVEL>(dz, dxy2, zh, q.z, q.zz, k);
-                        mob_apply2<WALL, false, ONCE>(m, dx, dy, dz, q.fx, q.fy, q.fz, ax, ay, az);
-                        mob_apply2<WALL, true, ONCE>(m, dx, dy, dz, fix, fiy, fiz, rx, ry, rz);
-                        // hand the accumulator to lane - 1, which meets this source next step
-                        const int from = (lane + 1) & 31;
-                        rx.x = __shfl_sync(0xffffffffu, rx.x, from);
-                        rx.y = __shfl_sync(0xffffffffu, rx.y, from);
-                        ry.x = __shfl_sync(0xffffffffu, ry.x, from);
-                        ry.y = __shfl_sync(0xffffffffu, ry.y, from);
-                        rz.x = __shfl_sync(0xffffffffu, rz.x, from);
-                        rz.y = __shfl_sync(0xffffffffu, rz.y, from);
-                    }
-                    if (FINE) fold();
-                    if (FINE && t0 == 0) {
-                        half[0] = rx.x + rx.y;
-                        half[1] = ry.x + ry.y;
-                        half[2] = rz.x + rz.y;
-                        rx = ry = rz = make_float2(0.f, 0.f);
-                    }
-                }
-                float *o3 = sRev + 3 * (warp * NT + g * 32 + lane);
-                const float2 rev[3] = {rx, ry, rz};
+            float *o3 = sRev + 3 * (warp * NT + g * 32 + lane);
+            const float2 rev[3] = {rx, ry, rz};
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    o3[c] = rev[c].x + rev[c].y;
-                    // after half a round lane l held the sums of source l + 16
-                    if (FINE) o3[c] += __shfl_xor_sync(0xffffffffu, half[c], 16);
-                }
+            for (int c = 0; c < 3; ++c) {
+                o3[c] = rev[c].x + rev[c].y;
+                // after half a round lane l held the sums of source l + 16
+                if (FINE) o3[c] += __shfl_xor_sync(0xffffffffu, run[c], 16);
             }
         }
-        if (!FINE) fold();
-        if (!diag) {
-            __syncthreads();
-            const int64_t j = j0 + threadIdx.x;
-            if (j < n) {
+    }
+    if (!FINE) fold();
+    if (!diag) {
+        __syncthreads();
+        const int64_t j = j0 + threadIdx.x;
+        if (j < n) {
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    float acc = 0.f;
+            for (int c = 0; c < 3; ++c) {
+                float acc = 0.f;
 #pragma unroll
-                    for (int w = 0; w < NW; ++w) acc += sRev[3 * (w * NT + threadIdx.x) + c];
-                    atomicAdd(u + 3 * j + c, scale * (double)acc);
-                }
+                for (int w = 0; w < NW; ++w) acc += sRev[3 * (w * NT + threadIdx.x) + c];
+                atomicAdd(u + 3 * j + c, scale * (double)acc);
             }
         }
     }

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) eng_sym_kernel(
         const int half = (int)(local & 1);
         int64_t I, J;
         triangle_pair(local >> 1, I, J);
-        x2sym_item<WALL, NT>(sP, sRev, P.hi, P.lo, P.f, P.n, I, J, k, P.y, scale, half, half + 1);
+        x2sym_item<WALL, NT>(sP, sRev, P.hi, P.lo, P.f, P.n, I, J, k, P.y, scale, half);
     }
 }
 
