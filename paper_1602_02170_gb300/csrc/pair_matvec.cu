@@ -1271,16 +1271,23 @@ constexpr int64_t kF64SumsMinN = 400;
 
 int f64_sums(int64_t n) { return n < kF64SumsMinN ? 1 : n < 32768 ? 8 : 16; }
 
-// One where the arrays don't fit the budget, or would have to be allocated
-// within a stream capture.
+// One where the arrays don't fit the budget, or in a capture of the caller's
+// where they would have to be allocated or, from kF64HeldMaxN blobs on, at all:
+// products of that size hold no workspace, which a later call may move, so that
+// their graphs stay valid.  (Graphs of smaller ones hold it, as those of FP32
+// products do; the solver's own are dropped when workspace moves.)
+constexpr int64_t kF64HeldMaxN = 8192;
+
 int f64_sums_held(mb_context *ctx, int64_t n, cudaStream_t s)
 {
     const int S = f64_sums(n);
     const size_t bytes = sizeof(double) * 3 * (size_t)n * S;
-    if (ctx->partial.bytes >= bytes) return S;
+    const bool held = ctx->partial.bytes >= bytes;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
-    return st == cudaStreamCaptureStatusNone && ensure_room(ctx, ctx->partial) >= bytes ? S : 1;
+    if (S > 1 && s != ctx->cap_stream && cudaStreamIsCapturing(s, &st) != cudaSuccess)
+        cudaGetLastError();
+    if (st != cudaStreamCaptureStatusNone) return held && n < kF64HeldMaxN ? S : 1;
+    return held || ensure_room(ctx, ctx->partial) >= bytes ? S : 1;
 }
 
 template <bool WALL, int C>

@@ -64,6 +64,37 @@ def test_fp64_sums_of_many_blobs(ctx):
     assert err <= 9e-16
 
 
+@pytest.mark.parametrize("n", [3000, 9000])
+def test_fp64_product_in_a_graph(n):
+    """A captured FP64 product, on a new context or after a first call, and (from
+    8,192 blobs on, whose graphs hold no workspace) after a larger product has
+    moved the context's.  1e-14: the last FP64 bits of sums of n terms."""
+    import torch
+
+    import paper_1602_02170_gb300 as mb
+
+    r, f = _cloud(n, n)
+    R, F = dev(r), dev(f)
+    for warm in (False, True):
+        with mb.Context(0) as c:
+            with mb.Context(0) as other:
+                want = host(other.mobility_matvec(R, F, 0.5, 1.0, True, "fp64"))
+            if warm:
+                c.mobility_matvec(R, F, 0.5, 1.0, True, "fp64")
+            out = torch.zeros_like(R)
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                c.mobility_matvec(R, F, 0.5, 1.0, True, "fp64", out=out)
+            if n >= 8192:
+                R2, F2 = (dev(v) for v in _cloud(1, 2 * n))
+                c.mobility_matvec(R2, F2, 0.5, 1.0, True, "fp64")
+            for _ in range(2):
+                out.zero_()
+                g.replay()
+                assert rel_l2(host(out), want) <= 1e-14
+
+
 @pytest.mark.parametrize("target", ["f", "r"])
 def test_fp64_product_in_place(ctx, target):
     """The velocities may overwrite the forces or the positions."""
