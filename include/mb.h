@@ -175,8 +175,11 @@ mb_status mb_measure_fma_rate(mb_context *ctx, mb_precision prec, double *flops_
  * memory makes the copies faster).  Mixing kinds is MB_EINVAL.  With the
  * wall, every z must be > 0 (blobs at z < a are computed as written but the
  * matrix need not be positive definite); this is not checked.  N = 0 is a
- * no-op.  u may be f or r.  MB_FP64 and MB_DF64 add partial sums with FP64
- * atomics, so results may differ between calls in the last FP64 bits.
+ * no-op.  u may be f or r.  MB_FP64, MB_DF64 and from 600 blobs on
+ * MB_FP32_KAHAN (unless a variant other than 3 is pinned) add partial sums with
+ * FP64 atomics, so results are equal from call to call to FP64 rounding only,
+ * and so are the solves that use these products.  The first call of a size may
+ * allocate workspace: make it before a stream capture.
  */
 mb_status mb_mobility_matvec(mb_context *ctx, const double *r, const double *f, int64_t n,
                              double a, double eta, int wall, mb_precision prec, double *u,
@@ -184,7 +187,8 @@ mb_status mb_mobility_matvec(mb_context *ctx, const double *r, const double *f, 
 
 /*
  * Choice of the FP32 pair-kernel variant used by this context:
- *   -1  by size (default): 3 from 600 blobs on, 4 below;
+ *   -1  by size (default): 3 from 600 blobs on, below 4 in the solver's steps
+ *       and one launch of thread-block clusters for a single product;
  *    0  scalar FP32 kernel, one target per thread;
  *    1  packed FP32 kernel (paired f32x2 arithmetic), two targets per thread;
  *    2  packed FP32 kernel, four targets per thread;
@@ -218,7 +222,8 @@ mb_status mb_context_set_wait_limit(mb_context *ctx, double seconds);
 /* The FP32 pair-kernel variant this context uses for N blobs with or
  * without the wall: the fixed variant if one was set, else the one chosen
  * by size once a matvec of that size class (half octaves of N, wall or not)
- * has run, else -1. */
+ * has run, else -1.  By size, 4 stands for the kernels below 600 blobs (see
+ * mb_context_set_pair_variant). */
 mb_status mb_context_pair_variant(const mb_context *ctx, int64_t n, int wall, int *variant);
 
 /*

@@ -325,7 +325,8 @@ class Context:
         self._check(self.L.mb_context_set_pair_variant(self.handle, int(variant)))
 
     def pair_variant(self, n: int, wall: bool = True) -> int:
-        """Variant used for N blobs (-1 before the first product of their size class)."""
+        """Variant used for N blobs (-1 before the first product of their size class;
+        4, chosen by size, stands for the kernels of fewer than 600 blobs)."""
         v = ctypes.c_int()
         self._check(self.L.mb_context_pair_variant(self.handle, int(n), int(bool(wall)),
                                                     ctypes.byref(v)))

@@ -68,7 +68,8 @@ struct mb_context {
 
     // matvec workspace
     mb::DevBuf pos_hi, pos_lo;   // packed float4 positions (FP32 path)
-    mb::DevBuf partial;          // per-source-chunk partial velocities (FP64)
+    mb::DevBuf partial;          // partial velocities (FP64): of source chunks, or the
+                                 // arrays that an FP64 product's sums are spread over
     mb::DevBuf stage_r, stage_f, stage_u;  // staging for host-pointer calls
     mb::DevBuf eval_hi, eval_lo;           // packed flow-evaluation points (FP32 path)
     mb::DevBuf render_r, render_f;         // refined blobs of a flow rendering

@@ -381,9 +381,9 @@ void launch_small(const double *r, const double *f, int64_t n, double a, double 
 // use, so a warp or two per scheduler keep it busy and what matters is that
 // every scheduler gets the same number of pair steps: the items are far more
 // than the warps in flight and the hardware deals them out as CTAs end.
-// launch_f64sym picks C.  2,730 blobs: 1,276 -> 632 us against every ordered
-// pair once in one-warp CTAs; 16,384 blobs: 28.3 -> 21.3 ms against 256-thread
-// symmetric items of the ungrouped formula (1.36 TFLOP/s in the method's 108
+// launch_f64sym picks C.  2,730 blobs: 1,274 -> 619 us against every ordered
+// pair once in one-warp CTAs; 16,384 blobs: 28.3 -> 20.6 ms against 256-thread
+// symmetric items of the ungrouped formula (1.41 TFLOP/s in the method's 108
 // flop per ordered pair, of 1.06 measured: each pair is evaluated once).
 // u: S arrays of 3 n (f64_sums), block J's items adding to the targets in array
 // J mod S and block I's to the sources in array I mod S.
@@ -1198,11 +1198,12 @@ mb_status f32_run(mb_context *ctx, int v, const double *f, int64_t n, double a, 
     return MB_OK;
 }
 
-// The symmetric kernel from kSymMinN blobs on, one-warp CTAs that evaluate
-// every ordered pair below.  A mixed solve (us) of 336 / 504 / 672 / 1,344 /
-// 2,688 blobs takes 944 / 962 / 1,180 / 1,730 / 3,920 with the one and 982 /
-// 995 / 1,149 / 1,370 / 2,310 with the other: zeroing the sums and the atomics
-// cost two to three microseconds a step, and few pairs save less.
+// The symmetric kernel from kSymMinN blobs on; below, one-warp CTAs that evaluate
+// every ordered pair in a solver's steps, and the one-launch kernel for a product.
+// A mixed solve (us) of 336 / 504 / 672 / 1,344 / 2,688 blobs takes 944 / 962 /
+// 1,180 / 1,730 / 3,920 with every ordered pair and 982 / 995 / 1,149 / 1,370 /
+// 2,310 with the symmetric kernel: zeroing the sums and the atomics cost two to
+// three microseconds a step, and few pairs save less.
 constexpr int64_t kSymMinN = 600;
 static_assert(kSymMinN <= kSmallMaxN, "a product below kSymMinN takes the one-launch kernel");
 

@@ -412,20 +412,25 @@ __global__ void __launch_bounds__(256) precond_apply_kernel(
 }
 
 // ---------------------------------------------------------------------------
-// Split setup for bodies with 3 n_p <= kSplitMaxRows.  The single kernel
-// above runs every step of a body on one SM; here only the Cholesky does,
-// and the O(n^3) rest is spread over many CTAs:
+// Split setup for bodies with 3 n_p <= kSplitMaxRowsSmem.  The single kernel
+// above runs every step of a body on one SM; here the O(n^3) work is spread
+// over more:
 //   S1 pc_assemble_kernel  M_p's lower triangle written into P_p's n x n block
-//                          (warp per blob row and 32 columns);
-//   S2 pc_factor_kernel    one CTA per body: Cholesky M_p = L L^T carried out
+//                          (one 3 x 3 block a thread);
+//   S2 pc_factor_small_kernel    one CTA per body (many bodies up to kSmemMaxRows
+//      pc_factor_cluster_kernel  rows) or a cluster of CTAs (few bodies, and all
+//                          above that): Cholesky M_p = L L^T carried out
 //                          together with G = L^-1 K_p (the six K columns are
 //                          eliminated alongside), then S = G^T G = K^T M^-1 K,
 //                          N = S^-1; stores L^T in P_p's upper triangle;
-//   S3 pc_trinv_kernel     one warp per column c of W = L^-1 (forward
-//                          substitution in registers), with row c of
-//                          Q = M^-1 K = W^T G and of Q N, and P_p's border;
-//   S4 pc_product_kernel   P_p's n x n block = W^T W - (Q N) Q^T in 32 x 32
-//                          tiles through shared memory.
+//   S3 pc_trinv_df_kernel  (up to kSetupSmallRows rows) W = L^-1 by 32 x 32 tiles,
+//      pc_trinv_kernel     or one warp per column c of it (forward substitution
+//                          in registers), with row c of Q = M^-1 K = W^T G and
+//                          of Q N, and P_p's border;
+//   S4 pc_product_df_kernel, pc_product_df16_kernel, pc_product_kernel
+//                          P_p's n x n block = W^T W - (Q N) Q^T in 32 x 32
+//                          (or 16 x 16) tiles through shared memory.
+// The factored form ends after S2 (S3', pc_keep_factor_kernel).
 // Per-body scratch (stride kept uniform within a group of bodies):
 //   [W (nmax^2, row-major, zero above the diagonal near it) | G (6 nmax) |
 //    Q (6 nmax) | QN (6 nmax) | dW (nmax) | N (36)].
@@ -795,8 +800,7 @@ size_t factor_small_smem(int nmax)
 // no CTA writes an entry that another CTA reads between two barriers: the
 // barrier of panel q+1 separates the stage-C reads of panel q from the
 // owners' next writes of the same entries.  The outputs are those of
-// pc_factor_kernel up to rounding (here each entry takes its products in one
-// FMA chain).
+// pc_factor_small_kernel up to rounding.
 constexpr int kFacCluster = 8;
 
 size_t factor_cluster_smem(int nmax, bool srows)
@@ -2334,7 +2338,8 @@ static void precond_apply_impl(mb_context *ctx, const double *w, const double *g
         // symv_rows for whole or half blocks (one body an SM or more).  Shorter
         // pieces of rows walked column by column read DRAM in short strips: 60
         // bodies of 154 blobs 77 us against 49 by a warp per row, 40 of 300 blobs
-        // 227 against 105.
+        // 227 against 105.  (Blocks here have at most 2,229 + 6 rows, what the setup's
+        // shared memory holds, so x and symv_rows' sums stay below 48 KB.)
         const auto kern = chunks <= 2 ? precond_apply_kernel<double, true>
                                       : precond_apply_kernel<double, false>;
         kern<<<grid, 256, sizeof(double) * m, s>>>(

@@ -1573,6 +1573,7 @@ mb_status Engine::step(cudaStream_t s, int *n_running, int *n_queued)
         // precond apply for bodies of active slots: Z_j = P^-1 V_j
         int max_np = 1;
         for (int sl : arn) max_np = std::max(max_np, running[sl]->max_np);
+        // (with symv_rows' sums below 48 KB: the setup holds at most 2,229 rows a body)
         const int pc_smem = (int)sizeof(double) * (3 * max_np + 6);
         const int pc_grid = (int)std::min<int64_t>(b_cap, 8 * (int64_t)ctx->sm_count);
         eng_precond_apply_kernel<<<pc_grid, 256, pc_smem, s>>>(body_slot, body_b0, body_b1, poff, 0,
