@@ -74,6 +74,7 @@ mb_status ensure(mb_context *ctx, DevBuf &buf, size_t bytes, const char *what)
     }
     if (e != cudaSuccess) {
         buf.ptr = nullptr;
+        cudaGetLastError();  // callers may go on with less
         return cuda_err(ctx, e, what);
     }
     buf.bytes = grow;

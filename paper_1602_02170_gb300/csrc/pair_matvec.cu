@@ -1376,9 +1376,14 @@ mb_status matvec_packed(mb_context *ctx, const double *r, const double *f, int64
     }
     // FP64: u (or, of several sums or deferred, the sums that a launch or the
     // caller adds and scales) zeroed, then one launch over the block-pair triangle
-    const int S = f64_sums_held(ctx, n, s);
+    int S = f64_sums_held(ctx, n, s);
+    const size_t one = sizeof(double) * 3 * (size_t)n;
+    if (S > 1 && ensure(ctx, ctx->partial, S * one, "matvec partials") != MB_OK) {
+        ctx->err.clear();  // the device has less left than the budget: one array does
+        S = 1;
+    }
     const bool sums = defer || S > 1;
-    const size_t bytes = sizeof(double) * 3 * (size_t)n * S;
+    const size_t bytes = S * one;
     if (sums) MB_TRY(ensure(ctx, ctx->partial, bytes, "matvec partials"));
     double *uk = sums ? (double *)ctx->partial.ptr : u;
     const double sk = sums ? 1.0 : scale;
